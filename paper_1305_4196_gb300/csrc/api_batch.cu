@@ -227,8 +227,9 @@ int build_table(md_batch* b) {
     BCK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, b->device));
     if (smem + 8192 > (size_t)optin)
         return bfail(b, MD_ERR_CELL_OVERFLOW, "an ensemble task needs %zu B of shared memory", smem);
-    b->smem = smem;
     b->tile_slots = (int)(smem / sizeof(float4)) - 1;
+    if (!b->blk.empty()) smem += ENS_LIST_EXTRA;
+    b->smem = smem;
     const int per_sm = ensemble_ctas_per_sm(b->threads, smem);
     if (per_sm < 1) return bfail(b, MD_ERR_CUDA, "the ensemble kernel does not fit an SM at %d threads", b->threads);
     b->grid = per_sm * b->sms;

@@ -627,81 +627,58 @@ __device__ int ens_stage(const EnsBlockSys& y, const EnsArrays& ea, const float4
     return T;
 }
 
-// Shared memory of a LIST task for a tile of T atoms: the padded FP32 arrays and the
-// lanes' rings of list entries (8 warps).
+// Shared memory of a LIST task: the scan's buffers and the tile of T atoms.  The host sizes the
+// launch by ens_list_smem and adds ENS_LIST_EXTRA behind what a FORCE tile may take.
 __host__ __device__ inline size_t ens_list_smem_bytes(int T) {
-    return (size_t)soa_len(T + 1) * 3 * sizeof(float) + (size_t)NL_WARPS * 32 * NL_RING * sizeof(uint16_t);
+    return nl_tile_bytes(T) + NL_WARPS * sizeof(NlWarp);
 }
 
 // LIST: the Verlet lists of the own atoms of block b, by the candidate scan of the main
-// builder (nl_scan.cuh): warp w takes own cell w, one lane per atom; entries are tile
-// indices in chunks of 8 (the last padded with T), by slot.
+// builder (nl_scan.cuh): a warp takes an own cell; entries are tile indices in chunks of 8
+// (the last padded with T), by slot.
 __device__ void ens_list(const EnsBlockSys& y, const BatchState& st, const EnsArrays& ea, bool odd, int b,
-                         size_t smem_bytes, unsigned char* smem, EnsTile& mt, int* pp) {
+                         size_t smem_bytes, unsigned char* smem, EnsTile& mt) {
     ens_meta(y, ea, b, mt);
     const int T = mt.prefix[64];
     if (ens_list_smem_bytes(T) > smem_bytes || T > 65535) {
         if (threadIdx.x == 0) atomicOr(st.err, ERR_TILE_OVERFLOW);
         return;
     }
-    const int SL = soa_len(T + 1);
-    float* tx = reinterpret_cast<float*>(smem);
-    float* ty = tx + SL;
-    float* tz = ty + SL;
-    uint16_t* buf = reinterpret_cast<uint16_t*>(tz + SL);  // NL_WARPS x NL_RING x 32
     TileOffsets to;
 #pragma unroll
     for (int d = 0; d < 3; ++d)
 #pragma unroll
         for (int q = 0; q < 4; ++q) to.off[d][q] = y.off[d][q];
-    tile_pad_prefix(mt, pp);
-    tile_stage_soa<true>(mt, pp, (odd ? ea.xsb : ea.xs) + y.a0, to, tx, ty, tz);
+    float* const tx = reinterpret_cast<float*>(smem + NL_WARPS * sizeof(NlWarp));
+    const int stride = (T + 3) & ~3;
+    float* const ty = tx + stride;
+    float* const tz = ty + stride;
+    const float4* xs = (odd ? ea.xsb : ea.xs) + y.a0;
+    nl_stage(mt, to, tx, ty, tz, [&](int j) { return __ldcg(xs + j); });
     __syncthreads();
     const PosBuf P = ens_pos(st, ea, odd);
-    const unsigned sx = (unsigned)__cvta_generic_to_shared(tx);
-    const unsigned sy = (unsigned)__cvta_generic_to_shared(ty);
-    const unsigned sz = (unsigned)__cvta_generic_to_shared(tz);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     if (warp >= NL_WARPS) return;
-    uint16_t* col = buf + (size_t)warp * NL_RING * 32 + lane;
+    NlWarp& w = reinterpret_cast<NlWarp*>(smem)[warp];
     const int cap = ea.list_chunks * 8;
     uint4* nl = ea.nl + y.a0 * (int64_t)ea.list_chunks;
-    const f2_t hi2 = f2_pack(ea.rl2_hi, ea.rl2_hi), lo2 = f2_pack(ea.rl2_lo, ea.rl2_lo);
     for (int oc = warp; oc < 8; oc += min(nw, NL_WARPS)) {
-        const int lx = oc & 1, ly = (oc >> 1) & 1, lz = oc >> 2;
-        const int own_coord = (lx + 1) + 4 * (ly + 1) + 16 * (lz + 1);
-        const int own_begin = mt.prefix[oc], own_count = mt.prefix[oc + 1] - own_begin;
-        for (int base = 0; base < own_count; base += 32) {
-            const int e = base + lane;
-            const bool active = e < own_count;
-            const int ei = active ? e : 0;
-            const int own_p = pp[oc] + ei;
-            const int slot_i = mt.start[oc] + ei;
-            const int64_t gi = y.a0 + __ldcg(ea.perm_s + y.a0 + slot_i);
-            const float xi = tx[own_p], yi = ty[own_p], zi = tz[own_p];
-            const f2_t pix = f2_pack(xi, xi), piy = f2_pack(yi, yi), piz = f2_pack(zi, zi);
-            ListOut o{col, nl + slot_i, (size_t)y.n, cap, 0, 0};
-#pragma unroll 1
-            for (int key = 0; key < 27; ++key) {  // the own cell first, then the 26 neighbours
-                const int kk = key == 0 ? 0 : (key <= 13 ? key - 14 : key - 13);
-                const int oz = (kk + 13) / 9 - 1, oy = ((kk + 13) / 3) % 3 - 1, ox = (kk + 13) % 3 - 1;
-                const int sl = c_tiles.idx_of_coord[own_coord + ox + 4 * oy + 16 * oz];
-                const int s_adj = mt.start[sl] - pp[sl];  // system slot = padded index + s_adj
-                auto retest = [&](int q) {
-                    const int64_t gj = y.a0 + __ldcg(ea.perm_s + y.a0 + q + s_adj);
+        const int own_coord = (1 + (oc & 1)) + 4 * (1 + ((oc >> 1) & 1)) + 16 * (1 + (oc >> 2));
+        const int count = mt.prefix[oc + 1] - mt.prefix[oc];
+        for (int lo_own = 0; lo_own < count; lo_own += 32) {
+            const int own_n = min(32, count - lo_own);
+            const int slot0 = mt.start[oc] + lo_own;
+            const int cnt = nl_scan_cell<0>(
+                w, mt, tx, ty, tz, oc, own_coord, lo_own, own_n, ea.rl2_hi, ea.rl2_lo, nl + slot0, (size_t)y.n, cap,
+                [&](int own, int u) {
+                    const int sl = ens_slot_of(mt, u);
+                    const int64_t gi = y.a0 + __ldcg(ea.perm_s + y.a0 + slot0 + own);
+                    const int64_t gj = y.a0 + __ldcg(ea.perm_s + y.a0 + mt.start[sl] + (u - mt.prefix[sl]));
                     return ens_fp64_pair_test(P.x, P.y, P.z, y, gi, gj, ea.rl2);
-                };
-                if (key == 0)
-                    scan_cell<0, true>(sx, sy, sz, pp[sl], mt.prefix[sl + 1] - mt.prefix[sl], mt.prefix[sl] - pp[sl],
-                                       pix, piy, piz, hi2, lo2, own_p, active, o, retest);
-                else
-                    scan_cell<0, false>(sx, sy, sz, pp[sl], mt.prefix[sl + 1] - mt.prefix[sl], mt.prefix[sl] - pp[sl],
-                                        pix, piy, piz, hi2, lo2, own_p, active, o, retest);
-            }
-            flush_chunks(o, (unsigned)T, true);
-            if (active) {
-                if (o.cnt > cap) atomicOr(st.err, ERR_LIST_OVERFLOW);
-                ea.nl_cnt[y.a0 + slot_i] = o.cnt < cap ? o.cnt : cap;
+                });
+            if (lane < own_n) {
+                if (cnt > cap) atomicOr(st.err, ERR_LIST_OVERFLOW);
+                ea.nl_cnt[y.a0 + slot0 + lane] = cnt < cap ? cnt : cap;
             }
         }
     }
@@ -1005,8 +982,7 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS, 1)
     __shared__ double red[BATCH_MAX_THREADS];
     __shared__ int nqueued;
     __shared__ EnsTile mt;
-    __shared__ int pp[65];
-    const size_t smem_bytes = (size_t)(tile_slots + 1) * sizeof(float4);
+    const size_t smem_bytes = (size_t)(tile_slots + 1) * sizeof(float4) + ENS_LIST_EXTRA;
     __shared__ uint16_t queue[ENS_QUEUE];
     __shared__ int s_ent, s_task, s_take, s_quit;
     __shared__ uint32_t s_phase;
@@ -1096,7 +1072,7 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS, 1)
                         case ST_SCAN: ens_scan(y, ea, warp_tot); break;
                         case ST_SCAT: ens_scatter(y, ea, st.err, task); break;
                         case ST_SORT: ens_sort(y, st, ea, odd, task); break;
-                        case ST_LIST: ens_list(y, st, ea, odd, task, smem_bytes, smem, mt, pp); break;
+                        case ST_LIST: ens_list(y, st, ea, odd, task, smem_bytes, smem, mt); break;
                         default:
                             if (energy_call && k == K)
                                 ens_force<true>(y, st, ea, pt, fs2_max, k, K, dt, task, en.idx, tile_slots, tile, mt,
@@ -1132,7 +1108,8 @@ size_t batch_smem_bytes(int nmax, int cmax) {
 
 size_t ens_tile_smem_bytes(int tile_slots) { return (size_t)(tile_slots + 1) * sizeof(float4); }
 
-size_t ens_list_smem(int T) { return ens_list_smem_bytes(T); }
+static_assert(NL_WARPS * sizeof(NlWarp) <= 32768 + 228 * 12 + ENS_LIST_EXTRA, "a LIST task's buffers");
+size_t ens_list_smem(int T) { return (size_t)((T + 228) & ~3) * 3 * sizeof(float) + 32768; }
 
 void launch_ensemble(const EnsEntry* ent, int nent, const BatchSys* one, const EnsBlockSys* blk,
                      const BatchState& st, const EnsArrays& ea, const PairTable& pt, int n_steps, int flags,

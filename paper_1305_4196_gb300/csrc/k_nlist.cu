@@ -4,37 +4,41 @@
 // (Sec. II.A) and gives each task its own list storage so that no two tasks
 // update the same structure (Sec. II.A, Sec. II.C).  Here one CTA is the task
 // of one 2x2x2-cell block: it stages the block's 4x4x4-cell tile in shared
-// memory, each of its 8 warps takes one cell of the block (lanes = the cell's
-// atoms), and every candidate of the 27 surrounding cells is broadcast from
-// shared memory to the warp.  Each atom's list is written only by its own
-// lane, so the lists need no synchronisation at all.
+// memory and each of its 8 warps scans the 27 cells around one cell of the
+// block (nl_scan.cuh).  Each list is written by one warp alone, so the lists
+// need no synchronisation at all.
 //
 // The set is exactly the FP64 definition: pairs with minimum-image
 // |x_i - x_j|^2 < r_list^2 evaluated as ((dx*dx)+dy*dy)+dz*dz.  The FP32
-// tile test decides every candidate whose r^2 is further than a relative
-// 1e-4 from r_list^2 (the FP32 coordinate error is below 1e-6); candidates
-// inside that band are re-tested with the FP64 positions in exactly the
-// definition's operation order (minimum image d - L*rint(d/L)).
+// tile test decides every candidate whose r^2 is further from r_list^2 than
+// twice the bound on its FP32 error (tile_frame_cut_band, a relative 3e-6 for a
+// liquid); candidates inside that band are re-tested with the FP64 positions in
+// exactly the definition's operation order (minimum image d - L*rint(d/L)).
 //
 // Full lists hold every neighbour of every atom.  Half lists (Newton's third
 // law, Sec. II.D.3) hold each pair once: a neighbour in the same cell only if
 // it comes later in cell order, plus all neighbours of the 13 "forward" cells.
+//
+// Bound by instruction issue (68 % of cycles at 24 warps per SM; 80 registers, and
+// 42 KB of scan buffers beside the tile).  At 1,048,576 atoms: 590 us and 567 M warp
+// instructions with a lane per own atom that tested every atom of the 27 cells and
+// appended its own hits, 391 us and 322 M with the scan of nl_scan.cuh (other forms of it:
+// 439 us with hit masks turned into entries by a loop over their bits; 551 us with the self
+// pair and the band sieved out of the rows by a lane each).
 #include "nl_scan.cuh"
+
+#include <algorithm>
 
 namespace mdgb {
 
-// The lists of the own atoms of block b (the CTA's task).
+// The lists of the own atoms of block b (the CTA's task): warp w takes own cell w, or of each
+// cell the share `part` of `split` (small systems, whose blocks are too few to fill the SMs).
 template <int HALF>
 __device__ __forceinline__ void build_block(const DevState& s, const Geometry& g, const TileOffsets& to, double rl2,
-                                            float band_lo, float band_hi, int list_cap, int tile_cap, int b) {
+                                            float band_lo, float band_hi, int list_cap, int tile_cap, int b, int part,
+                                            int split) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ TileMeta m;
-    __shared__ int pp[65];
-    const int SL = soa_len(tile_cap);
-    float* tx = reinterpret_cast<float*>(smem);
-    float* ty = tx + SL;
-    float* tz = ty + SL;
-    uint16_t* buf = reinterpret_cast<uint16_t*>(tz + SL);  // NL_WARPS x NL_RING x 32
 
     tile_meta(g, s.cell_start, b, m);
     const int T = m.prefix[64];
@@ -47,63 +51,38 @@ __device__ __forceinline__ void build_block(const DevState& s, const Geometry& g
         return;
     }
     if (m.prefix[8] == 0) return;  // empty block (vacuum): no lists to build
-    tile_pad_prefix(m, pp);
-    tile_stage_soa(m, pp, s.xr, to, tx, ty, tz);
+    const int stride = (tile_cap + 3) & ~3;
+    const int nw = blockDim.x >> 5;
+    float* const tx = reinterpret_cast<float*>(smem + nw * sizeof(NlWarp));
+    float* const ty = tx + stride;
+    float* const tz = ty + stride;
+    nl_stage(m, to, tx, ty, tz, [&](int j) { return s.xr[j]; });
     __syncthreads();
 
-    const unsigned sx = (unsigned)__cvta_generic_to_shared(tx);
-    const unsigned sy = (unsigned)__cvta_generic_to_shared(ty);
-    const unsigned sz = (unsigned)__cvta_generic_to_shared(tz);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int lx = warp & 1, ly = (warp >> 1) & 1, lz = warp >> 2;
-    const int own_begin = m.prefix[warp], own_count = m.prefix[warp + 1] - own_begin;
-    const int own_pbegin = pp[warp];
-    uint16_t* col = buf + (size_t)warp * NL_RING * 32 + lane;
-    const int blk0 = m.start[0];
-    const int own_coord = (lx + 1) + 4 * (ly + 1) + 16 * (lz + 1);
-    const f2_t hi2 = f2_pack(band_hi, band_hi), lo2 = f2_pack(band_lo, band_lo);
+    NlWarp& w = reinterpret_cast<NlWarp*>(smem)[warp];
     int max_cnt = 0;
     unsigned long long sum_cnt = 0;
-
-    for (int base = 0; base < own_count; base += 32) {
-        const int e = base + lane;
-        const bool active = e < own_count;
-        const int ei = active ? e : 0;
-        const int ui = own_begin + ei;
-        const int own_p = own_pbegin + ei;
-        const float xi = tx[own_p], yi = ty[own_p], zi = tz[own_p];
-        const f2_t pix = f2_pack(xi, xi), piy = f2_pack(yi, yi), piz = f2_pack(zi, zi);
-        const int gi = blk0 + ui;
-        ListOut o{col, reinterpret_cast<uint4*>(s.nl) + gi, (size_t)s.np, list_cap, 0, 0};
-        {
-            const int slot = c_tiles.idx_of_coord[own_coord];
-            const int jadj = m.start[slot] - pp[slot];  // cell-ordered atom index = padded index + jadj
-            scan_cell<HALF, true>(sx, sy, sz, pp[slot], m.prefix[slot + 1] - m.prefix[slot],
-                                  m.prefix[slot] - pp[slot], pix, piy, piz, hi2, lo2, own_p, active, o,
-                                  [&](int q) {
-                                      return fp64_pair_test(s.x, s.y, s.z, g.L[0], g.L[1], g.L[2], gi, q + jadj, rl2);
-                                  });
-        }
-#pragma unroll 1
-        for (int key = HALF ? 1 : -13; key <= 13; ++key) {
-            if (key == 0) continue;
-            const int oz = (key + 13) / 9 - 1, oy = ((key + 13) / 3) % 3 - 1, ox = (key + 13) % 3 - 1;
-            const int slot = c_tiles.idx_of_coord[own_coord + ox + 4 * oy + 16 * oz];
-            const int jadj = m.start[slot] - pp[slot];
-            scan_cell<HALF, false>(sx, sy, sz, pp[slot], m.prefix[slot + 1] - m.prefix[slot],
-                                   m.prefix[slot] - pp[slot], pix, piy, piz, hi2, lo2, own_p, active, o,
-                                   [&](int q) {
-                                       return fp64_pair_test(s.x, s.y, s.z, g.L[0], g.L[1], g.L[2], gi, q + jadj, rl2);
-                                   });
-        }
-        // the last chunk, padded with the tile's dummy slot T
-        flush_chunks(o, (unsigned)T, true);
-        const int cnt = o.cnt;
-        if (active) {
-            if (cnt > list_cap) atomicOr(s.err, ERR_LIST_OVERFLOW);
-            s.nl_cnt[gi] = (uint16_t)(cnt < list_cap ? cnt : list_cap);
-            max_cnt = cnt > max_cnt ? cnt : max_cnt;
-            sum_cnt += (unsigned long long)cnt;
+    for (int oc = warp; oc < 8; oc += nw) {
+        const int own_coord = (1 + (oc & 1)) + 4 * (1 + ((oc >> 1) & 1)) + 16 * (1 + (oc >> 2));
+        const int count = m.prefix[oc + 1] - m.prefix[oc];
+        const int per = (count + split - 1) / split;
+        const int hi_own = min(count, (part + 1) * per);
+        for (int lo_own = part * per; lo_own < hi_own; lo_own += 32) {
+            const int own_n = min(32, hi_own - lo_own);
+            const int g0 = m.start[oc] + lo_own;
+            const int cnt = nl_scan_cell<HALF>(
+                w, m, tx, ty, tz, oc, own_coord, lo_own, own_n, band_hi, band_lo, reinterpret_cast<uint4*>(s.nl) + g0,
+                (size_t)s.np, list_cap, [&](int own, int u) {
+                    return fp64_pair_test(s.x, s.y, s.z, g.L[0], g.L[1], g.L[2], g0 + own, tile_global_index(m, u),
+                                          rl2);
+                });
+            if (lane < own_n) {
+                if (cnt > list_cap) atomicOr(s.err, ERR_LIST_OVERFLOW);
+                s.nl_cnt[g0 + lane] = (uint16_t)(cnt < list_cap ? cnt : list_cap);
+                max_cnt = cnt > max_cnt ? cnt : max_cnt;
+                sum_cnt += (unsigned long long)cnt;
+            }
         }
     }
 #pragma unroll
@@ -111,18 +90,19 @@ __device__ __forceinline__ void build_block(const DevState& s, const Geometry& g
         max_cnt = max(max_cnt, __shfl_xor_sync(0xffffffffu, max_cnt, o));
         sum_cnt += __shfl_xor_sync(0xffffffffu, sum_cnt, o);
     }
-    if (lane == 0) {
+    if (lane == 0 && max_cnt > 0) {
         atomicMax(&s.stats[0], max_cnt);
         atomicAdd(reinterpret_cast<unsigned long long*>(&s.stats[2]), sum_cnt);
     }
 }
 
-// One CTA per block in spatial order.
+// `split` CTAs per block, blocks in spatial order.
 template <int HALF>
 __global__ void __launch_bounds__(NL_WARPS * 32, 3) k_build_lists(DevState s, Geometry g, TileOffsets to,
                                                                   double rl2, float band_lo, float band_hi,
-                                                                  int list_cap, int tile_cap) {
-    build_block<HALF>(s, g, to, rl2, band_lo, band_hi, list_cap, tile_cap, spatial_block(g, blockIdx.x));
+                                                                  int list_cap, int tile_cap, int split) {
+    build_block<HALF>(s, g, to, rl2, band_lo, band_hi, list_cap, tile_cap, spatial_block(g, blockIdx.x / split),
+                      blockIdx.x % split, split);
 }
 
 // A compact system: a grid of s.compact CTAs over the occupied blocks.
@@ -132,32 +112,44 @@ __global__ void __launch_bounds__(NL_WARPS * 32, 3) k_build_lists_occ(DevState s
                                                                       int list_cap, int tile_cap) {
     const int count = s.stats[4];
     for (int k = blockIdx.x; k < count; k += gridDim.x) {
-        build_block<HALF>(s, g, to, rl2, band_lo, band_hi, list_cap, tile_cap, s.blk_list[k]);
+        build_block<HALF>(s, g, to, rl2, band_lo, band_hi, list_cap, tile_cap, s.blk_list[k], 0, 1);
         __syncthreads();  // the next block reuses the shared memory
     }
 }
 
-static size_t nl_smem_bytes(int list_cap, int tile_cap) {
+// Shared memory of a CTA of `warps` warps.
+static size_t nl_smem_bytes(int tile_cap, int warps) { return nl_tile_bytes(tile_cap) + warps * sizeof(NlWarp); }
+
+// The size the callers hold against the limit of an SM's shared memory: 12 B per tile atom and
+// about 35 KB (with a tile close to the limit a CTA runs four warps).
+size_t build_lists_smem(int list_cap, int tile_cap) {
     (void)list_cap;
-    return (size_t)soa_len(tile_cap) * 3 * sizeof(float) + (size_t)NL_WARPS * 32 * NL_RING * 2;
+    return (size_t)((tile_cap + 227) & ~3) * 3 * sizeof(float) + 32768;
 }
 
 void launch_build_lists(const DevState& s, const Geometry& g, const TileOffsets& to, double rl2, int list_cap,
                         int tile_cap, int half, cudaStream_t st) {
     if (s.n == 0) return;
-    size_t smem = nl_smem_bytes(list_cap, tile_cap);
-    float lo = (float)(rl2 * (1.0 - 1e-4));
-    float hi = (float)(rl2 * (1.0 + 1e-4));
+    const int warps = nl_smem_bytes(tile_cap, NL_WARPS) <= 226 * 1024 ? NL_WARPS : NL_WARPS / 2;
+    const size_t smem = nl_smem_bytes(tile_cap, warps);
+    // candidates whose FP32 r^2 the error bound of the tile's coordinates leaves undecided
+    const double band = tile_frame_cut_band(std::max({g.w[0], g.w[1], g.w[2]}), 0.0, std::sqrt(rl2));
+    const float lo = (float)(rl2 * (1.0 - band)), hi = (float)(rl2 * (1.0 + band));
+    const int threads = warps * 32;
     if (s.compact) {
-        if (half) k_build_lists_occ<1><<<s.compact, NL_WARPS * 32, smem, st>>>(s, g, to, rl2, lo, hi, list_cap, tile_cap);
-        else k_build_lists_occ<0><<<s.compact, NL_WARPS * 32, smem, st>>>(s, g, to, rl2, lo, hi, list_cap, tile_cap);
+        if (half) k_build_lists_occ<1><<<s.compact, threads, smem, st>>>(s, g, to, rl2, lo, hi, list_cap, tile_cap);
+        else k_build_lists_occ<0><<<s.compact, threads, smem, st>>>(s, g, to, rl2, lo, hi, list_cap, tile_cap);
         return;
     }
-    if (half) k_build_lists<1><<<g.nblock, NL_WARPS * 32, smem, st>>>(s, g, to, rl2, lo, hi, list_cap, tile_cap);
-    else k_build_lists<0><<<g.nblock, NL_WARPS * 32, smem, st>>>(s, g, to, rl2, lo, hi, list_cap, tile_cap);
+    // CTAs per block, each a share of every cell's atoms: while the grid is below two CTAs per SM,
+    // down to shares of about 8 atoms (32,000 atoms, 64 blocks: 150 us with one CTA each, 57 us
+    // with five)
+    const int per_cell = (int)((s.n + g.ncell - 1) / g.ncell);
+    const int split = std::max(1, std::min({(per_cell + 7) / 8, (2 * 152 + g.nblock - 1) / g.nblock, 16}));
+    const unsigned grid = (unsigned)g.nblock * (unsigned)split;
+    if (half) k_build_lists<1><<<grid, threads, smem, st>>>(s, g, to, rl2, lo, hi, list_cap, tile_cap, split);
+    else k_build_lists<0><<<grid, threads, smem, st>>>(s, g, to, rl2, lo, hi, list_cap, tile_cap, split);
 }
-
-size_t build_lists_smem(int list_cap, int tile_cap) { return nl_smem_bytes(list_cap, tile_cap); }
 
 template <typename K>
 static void allow_max_smem(K kernel) {

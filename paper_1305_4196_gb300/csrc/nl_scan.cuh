@@ -1,11 +1,22 @@
 // nl_scan.cuh - the candidate scan of the neighbour-list builders (k_nlist.cu, and the
 // block systems of the ensemble kernel in k_batch.cu).
 //
-// A CTA stages its block's tile as three FP32 arrays with every cell starting on a 16-byte
-// boundary (padded indices), so that one 128-bit broadcast load yields two packed FP32x2
-// operands; a warp takes one own cell, one lane per atom, and scans the candidates of each
-// neighbour cell in groups of 32, four per step.  Accepted entries go to a ring of slots per
-// lane in shared memory and leave for global memory in chunks of 8 tile indices.
+// A CTA stages its block's tile as three FP32 arrays; then one warp builds the lists of up to
+// 32 own atoms of one cell against the cell itself and its neighbour cells, in stages that need
+// no barrier beyond the warp:
+//  1. Cull: the neighbour cells' atoms, a lane each, against the bounding box of the own
+//     atoms.  Of the ~740 atoms of 27 cells of a liquid (3.2 sigma wide, list radius 2.8) about
+//     375 can have a neighbour among the own atoms; their tile indices go to a buffer in scan
+//     order.
+//  2. Test: 64 candidates at a time, each lane holding two neighbouring ones in packed
+//     registers, while the own atoms pass by as broadcast loads: seven packed operations and
+//     two compares for 64 pairs.
+//  3. Append: two ballots give every hit its place behind the own atom's entries (two bit counts
+//     per lane, as a lane's two candidates follow each other), and the lanes write their
+//     candidates' tile indices there, into a row of shared memory per own atom.  After the 64
+//     candidates a lane per own atom writes the row's complete chunks of 8 entries to global
+//     memory (16 bytes each; the lanes' chunks are consecutive).
+// The scan order is that of the cells, and inside a cell that of its atoms.
 #pragma once
 
 #include "fixpt.cuh"
@@ -14,190 +25,264 @@
 namespace mdgb {
 
 constexpr int NL_WARPS = 8;
+constexpr int NL_BATCH = 64;    // candidates tested at a time (two per lane)
+constexpr int NL_CAND = 288;    // candidate buffer
+constexpr int NL_ROW = 56;      // entries of an own atom's row
+constexpr float NL_FAR = 1.0e6f;  // coordinate of an empty candidate slot
 
-// Two packed FP32 pairs from 16 bytes of shared memory (one 128-bit load).
-__device__ __forceinline__ void lds_f2x2(unsigned addr, f2_t& lo, f2_t& hi) {
-    asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(lo), "=l"(hi) : "r"(addr));
-}
-
-__device__ __forceinline__ unsigned sign_in(unsigned mask, float v) {
-    return __funnelshift_l(__float_as_uint(v), mask, 1);  // (mask << 1) | sign bit of v
-}
-
-// Scan of one group of up to 32 consecutive candidates of the padded tile (padded
-// index g0, a multiple of 4; nvalid of them are real) against a lane's atom, four per
-// step: one 128-bit broadcast load per coordinate, packed FP32x2 arithmetic.  The scan
-// stops after the step holding the last real candidate (nvalid is the same for the
-// whole warp).  Candidate k of the group lands in bit 31-k of the masks: `maybe` has
-// r^2 <= band_hi (inside the list radius or in the FP64 re-test band), `sure` has
-// r^2 < band_lo (inside for certain).  Each bit is the sign of r^2 - threshold
-// shifted in; bits past the scanned steps are zero.
-__device__ __forceinline__ void scan_group(unsigned sx, unsigned sy, unsigned sz, int g0, int nvalid, f2_t pix,
-                                           f2_t piy, f2_t piz, f2_t hi2, f2_t lo2, unsigned& maybe,
-                                           unsigned& sure) {
-    unsigned mm = 0u, ms = 0u;
-    const unsigned off0 = (unsigned)g0 * 4u;
-    int k = 0;
-#pragma unroll
-    for (; k < 32; k += 4) {
-        if (k >= nvalid) break;
-        f2_t x01, x23, y01, y23, z01, z23;
-        lds_f2x2(sx + off0 + 4u * k, x01, x23);
-        lds_f2x2(sy + off0 + 4u * k, y01, y23);
-        lds_f2x2(sz + off0 + 4u * k, z01, z23);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const f2_t dx = f2_sub(pix, h ? x23 : x01);
-            const f2_t dy = f2_sub(piy, h ? y23 : y01);
-            const f2_t dz = f2_sub(piz, h ? z23 : z01);
-            const f2_t r2 = f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx)));
-            float ha, hb, la, lb;
-            f2_unpack(f2_sub(r2, hi2), ha, hb);
-            f2_unpack(f2_sub(r2, lo2), la, lb);
-            mm = sign_in(sign_in(mm, ha), hb);
-            ms = sign_in(sign_in(ms, la), lb);
-        }
-    }
-    // k candidates were shifted in (k >= 4): move candidate 0 to bit 31
-    maybe = k < 32 ? mm << (32 - k) : mm;
-    sure = k < 32 ? ms << (32 - k) : ms;
-}
-
-// A lane's list output.  Accepted entries go to a ring of NL_RING slots in shared
-// memory (slot r at col[r * 32]) and leave for global memory in full chunks of 8 as
-// soon as they are complete, so the CTA never holds whole lists on chip.
-constexpr int NL_RING = 64;
-
-struct ListOut {
-    uint16_t* col;  // this lane's ring
-    uint4* out;     // chunk 0 of this atom's list; chunk c at out[c * np]
-    size_t np;
-    int list_cap;
-    int cnt;      // entries accepted so far (may exceed list_cap: overflow)
-    int flushed;  // entries already written to global memory (a multiple of 8)
+// One warp's shared memory.  A batch can add 64 entries to the up to 7 left in a row: one that
+// runs over its row (into the next, or the slack behind the last) is found by its length and
+// done again in two halves.
+struct __align__(16) NlWarp {
+    float4 own_xy[32];          // own atoms' coordinates, each twice (packed operands)
+    float4 own_z[32];           // z twice, then the shared address behind the atom's last entry
+    uint16_t row[32 * NL_ROW + 16];
+    uint16_t cand[NL_CAND];     // tile indices
 };
 
-__device__ __forceinline__ unsigned ring_pair(const uint16_t* __restrict__ col, int k, int stored, unsigned pad) {
-    const unsigned a = k < stored ? (unsigned)col[(k & (NL_RING - 1)) * 32] : pad;
-    const unsigned b = k + 1 < stored ? (unsigned)col[((k + 1) & (NL_RING - 1)) * 32] : pad;
-    return a | (b << 16);
+__device__ __forceinline__ float warp_min(float v) {
+    int i = __float_as_int(v);
+    i ^= (i >> 31) & 0x7fffffff;  // integers in the order of the floats
+    i = __reduce_min_sync(0xffffffffu, i);
+    return __int_as_float(i ^ ((i >> 31) & 0x7fffffff));
 }
 
-// Write every complete chunk; with pad < 65536 also the last partial chunk, padded.
-__device__ __forceinline__ void flush_chunks(ListOut& o, unsigned pad, bool last) {
-    const int stored = o.cnt < o.list_cap ? o.cnt : o.list_cap;
-    while (stored - o.flushed >= 8 || (last && stored > o.flushed)) {
-        const int k = o.flushed;
-        o.out[(size_t)(k >> 3) * o.np] = make_uint4(ring_pair(o.col, k, stored, pad), ring_pair(o.col, k + 2, stored, pad),
-                                                    ring_pair(o.col, k + 4, stored, pad),
-                                                    ring_pair(o.col, k + 6, stored, pad));
-        o.flushed = k + 8;
-    }
+__device__ __forceinline__ void lds_f2x2(unsigned addr, f2_t& a, f2_t& b) {
+    asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "r"(addr) : "memory");
 }
 
-// Candidates of one neighbour cell (padded indices p0 .. p0+cnt-1; canonical tile
-// index = padded index + adj): scan in groups of 32, re-test the band candidates in FP64
-// (retest(padded index) gives the definition's answer), then append the accepted ones to
-// the lane's list in candidate order.  OWN marks the atom's own cell, where the atom
-// itself (full lists) or every atom up to it (half lists) is excluded; own_p is the
-// atom's padded index.
-template <int HALF, bool OWN, typename Retest>
-__device__ __forceinline__ void scan_cell(unsigned sx, unsigned sy, unsigned sz, int p0, int cnt_c, int adj,
-                                          f2_t pix, f2_t piy, f2_t piz, f2_t hi2, f2_t lo2, int own_p, bool active,
-                                          ListOut& o, Retest&& retest) {
-    const int p1 = p0 + cnt_c;
-    for (int g0 = p0; g0 < p1; g0 += 32) {
-        unsigned mm, ms;
-        const int nvalid = p1 - g0;
-        scan_group(sx, sy, sz, g0, nvalid, pix, piy, piz, hi2, lo2, mm, ms);
-        if (nvalid < 32) mm &= ~0u << (32 - nvalid);
-        if (OWN) {
-            const int rel = own_p - g0;  // own atom's bit is 31 - rel
-            if (HALF) {
-                if (rel >= 31) mm = 0u;
-                else if (rel >= 0) mm &= ~0u >> (rel + 1);
-            } else if (rel >= 0 && rel < 32) {
-                mm &= ~(0x80000000u >> rel);
-            }
-        }
-        if (!active) mm = 0u;
-        const int ubase = g0 + adj;
-        unsigned band = mm & ~ms;
-        while (band) {  // rare: within 1e-4 of r_list^2 in relative terms
-            const int k = __clz(band);
-            const unsigned bit = 0x80000000u >> k;
-            band ^= bit;
-            if (!retest(g0 + k)) mm ^= bit;
-        }
-        if (!mm) continue;
-        const int nb = __popc(mm);
-        int c = o.cnt;
-        if (c + nb <= o.list_cap) {
-            while (mm) {
-                const int k = __clz(mm);
-                mm ^= 0x80000000u >> k;
-                o.col[(c & (NL_RING - 1)) * 32] = (uint16_t)(ubase + k);
-                ++c;
-            }
+// This thread's lane, read once (a plain threadIdx.x is read again in every loop).
+__device__ __forceinline__ int nl_lane() {
+    int l;
+    asm volatile("mov.u32 %0, %%laneid;" : "=r"(l));
+    return l;
+}
+
+// A lane's two candidates of a batch.
+struct NlPair {
+    f2_t x, y, z;
+    unsigned u0, u1;  // their tile indices
+    int index;        // scan index of the first one (the own cell's atoms are 0, 1, ...)
+};
+
+// Append a warp's hits (ra, rb < hi, and for OWN the index rule) to an own atom's row; az: shared
+// address of its own_z, tail: the address behind the row's last entry.  In assembly so that
+// the comparisons, votes and stores share their predicates.
+template <int HALF, bool OWN>
+__device__ __forceinline__ void nl_append(unsigned az, unsigned tail, int lane, unsigned below, float ra, float rb,
+                                          float hi, int self, const NlPair& c) {
+#define NL_APPEND(RULE)                                                                                       \
+    asm volatile(                                                                                             \
+        "{\n\t.reg .pred p, q, l;\n\t.reg .b32 a, b;\n\t.reg .b16 u, v;\n\t"                                  \
+        "setp.lt.f32 p, %0, %2;\n\tsetp.lt.f32 q, %1, %2;\n\t" RULE "setp.eq.s32 l, %3, 31;\n\t"              \
+        "vote.sync.ballot.b32 a, p, 0xffffffff;\n\tvote.sync.ballot.b32 b, q, 0xffffffff;\n\t"                \
+        "and.b32 a, a, %4;\n\tand.b32 b, b, %4;\n\tpopc.b32 a, a;\n\tpopc.b32 b, b;\n\tadd.u32 a, a, b;\n\t"  \
+        "mad.lo.u32 a, a, 2, %5;\n\tcvt.u16.u32 u, %6;\n\tcvt.u16.u32 v, %7;\n\t"                             \
+        "@p st.shared.u16 [a], u;\n\t@p add.u32 a, a, 2;\n\t"                                                 \
+        "@q st.shared.u16 [a], v;\n\t@q add.u32 a, a, 2;\n\t"                                                 \
+        "@l st.shared.u32 [%8+8], a;\n\t}" ::"f"(ra),                                                         \
+        "f"(rb), "f"(hi), "r"(lane), "r"(below), "r"(tail), "r"(c.u0), "r"(c.u1), "r"(az), "r"(c.index),      \
+        "r"(self), "r"(self - 1)                                                                              \
+        : "memory")
+    if (!OWN) NL_APPEND("");
+    else if (HALF) NL_APPEND("setp.gt.and.s32 p, %9, %10, p;\n\tsetp.gt.and.s32 q, %9, %11, q;\n\t");
+    else NL_APPEND("setp.ne.and.s32 p, %9, %10, p;\n\tsetp.ne.and.s32 q, %9, %11, q;\n\t");
+#undef NL_APPEND
+}
+
+// One batch against every own atom.  OWN: the batch holds atoms of the own cell, of which an own
+// atom takes no pair with itself (half lists: only with later ones); self0: own atom 0's index
+// in its cell.  EXACT decides the pairs with r^2 in [lo, hi) by retest(own, u); without it they
+// count as hits, and the smallest bit pattern of r^2 - lo is returned: below that of hi - lo if
+// there was one, as negative numbers have the highest bit set.
+template <int HALF, bool OWN, bool EXACT, typename Retest>
+__device__ __forceinline__ unsigned nl_test(unsigned axy, int lane, int self0, int own_n, const NlPair& c, float hi,
+                                            float lo, Retest&& retest) {
+    const f2_t lo2 = f2_pack(lo, lo);
+    const unsigned below = (1u << lane) - 1u;
+    unsigned near_lo = 0xffffffffu;
+    const unsigned end = axy + 16u * (unsigned)own_n;
+    constexpr unsigned DZ = 32u * sizeof(float4);  // own_z lies behind own_xy
+    int a = 0;
+#pragma unroll(EXACT ? 1 : 2)
+    for (; axy != end; axy += 16u, ++a) {
+        f2_t ox, oy, oz, tail;
+        lds_f2x2(axy, ox, oy);
+        lds_f2x2(axy + DZ, oz, tail);
+        const f2_t dx = f2_sub(ox, c.x), dy = f2_sub(oy, c.y), dz = f2_sub(oz, c.z);
+        const f2_t r2 = f2_fma(dz, dz, f2_fma(dy, dy, f2_mul(dx, dx)));
+        float ra, rb;
+        f2_unpack(r2, ra, rb);
+        if (EXACT) {  // a pair of the band that the definition excludes: out of reach
+            if (ra < hi && !(ra < lo) && !retest(a, (int)c.u0)) ra = hi;
+            if (rb < hi && !(rb < lo) && !retest(a, (int)c.u1)) rb = hi;
         } else {
-            while (mm) {
-                const int k = __clz(mm);
-                mm ^= 0x80000000u >> k;
-                if (c < o.list_cap) o.col[(c & (NL_RING - 1)) * 32] = (uint16_t)(ubase + k);
-                ++c;
-            }
+            float ta, tb;
+            f2_unpack(f2_sub(r2, lo2), ta, tb);
+            near_lo = min(near_lo, min(__float_as_uint(ta), __float_as_uint(tb)));
         }
-        o.cnt = c;
-        flush_chunks(o, 0u, false);
+        nl_append<HALF, OWN>(axy + DZ, (unsigned)tail, lane, below, ra, rb, hi, self0 + a, c);
     }
+    return near_lo;
 }
 
-// Padded cell starts of the tile: every cell's first atom at a multiple of 4, so
-// that candidate groups start on 16-byte boundaries.  Threads 0..63; ends with
-// __syncthreads.
-__device__ __forceinline__ void tile_pad_prefix(const TileMeta& m, int* __restrict__ pp) {
-    const int t = threadIdx.x;
-    if (t < 64) {
-        const int cnt = m.prefix[t + 1] - m.prefix[t];
-        int v = (cnt + 3) & ~3;
-        const int lane = t & 31;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            int y = __shfl_up_sync(0xffffffffu, v, o);
-            if (lane >= o) v += y;
-        }
-        pp[t + 1] = v;
-    }
-    __syncthreads();
-    if (t >= 32 && t < 64) pp[t + 1] += pp[32];
-    if (t == 0) pp[0] = 0;
-    __syncthreads();
+// Shared memory of the tile's arrays (T <= tile_cap atoms and the padding of a 16-byte start).
+__host__ __device__ inline size_t nl_tile_bytes(int tile_cap) {
+    return (size_t)((tile_cap + 3) & ~3) * 3 * sizeof(float);
 }
 
-// Padded SoA staging, one warp per tile cell (no search for the cell of an atom); CG:
-// coordinates written by other CTAs of the same launch, read from L2.
-template <bool CG = false>
-__device__ __forceinline__ void tile_stage_soa(const TileMeta& m, const int* __restrict__ pp,
-                                               const float4* __restrict__ xr, const TileOffsets& to,
-                                               float* __restrict__ tx, float* __restrict__ ty,
-                                               float* __restrict__ tz) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int slot = warp; slot < 64; slot += (int)(blockDim.x >> 5)) {
+// Stage the tile's FP32 coordinates in the frame of the block, by tile index, one warp per cell
+// (two cells at a time); load(j): the cell-relative coordinates of cell-ordered atom j.
+template <typename Load>
+__device__ __forceinline__ void nl_stage(const TileMeta& m, const TileOffsets& to, float* __restrict__ tx,
+                                         float* __restrict__ ty, float* __restrict__ tz, Load&& load) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+#pragma unroll 2
+    for (int slot = warp; slot < 64; slot += nw) {
         const int c = c_tiles.coord_of_idx[slot];
-        const float ox = pick4(to.off[0], c & 3), oy = pick4(to.off[1], (c >> 2) & 3),
-                    oz = pick4(to.off[2], c >> 4);
-        const int j0 = m.start[slot], cnt = m.prefix[slot + 1] - m.prefix[slot], q0 = pp[slot];
+        const float ox = pick4(to.off[0], c & 3), oy = pick4(to.off[1], (c >> 2) & 3), oz = pick4(to.off[2], c >> 4);
+        const int u0 = m.prefix[slot], cnt = m.prefix[slot + 1] - u0, j0 = m.start[slot];
         for (int e = lane; e < cnt; e += 32) {
-            const float4 p = CG ? __ldcg(xr + j0 + e) : xr[j0 + e];
-            tx[q0 + e] = p.x + ox;
-            ty[q0 + e] = p.y + oy;
-            tz[q0 + e] = p.z + oz;
+            const float4 p = load(j0 + e);
+            tx[u0 + e] = p.x + ox;
+            ty[u0 + e] = p.y + oy;
+            tz[u0 + e] = p.z + oz;
         }
     }
 }
 
-// Padded SoA array length for a tile of at most tile_cap atoms: 3 padding slots per
-// cell at most, plus one group of read-ahead past the last cell.
-__host__ __device__ inline int soa_len(int tile_cap) { return (tile_cap + 64 * 3 + 32 + 3) & ~3; }
+// The lists of own atoms lo_own .. lo_own + own_n - 1 (own_n <= 32) of the cell in tile slot
+// `own` (< 8), whose tile coordinate is own_coord.  out: chunk 0 of lane 0's list, the other lanes' behind
+// it, chunk c at out[c * np]; cap: entries a list holds (a multiple of 8; more are counted only).
+// Returns this lane's list length.
+template <int HALF, typename Retest>
+__device__ __forceinline__ int nl_scan_cell(NlWarp& w, const TileMeta& m, const float* __restrict__ tx,
+                                            const float* __restrict__ ty, const float* __restrict__ tz, int own,
+                                            int own_coord, int lo_own, int own_n, float hi, float lo, uint4* out,
+                                            size_t np, int cap, Retest&& retest) {
+    const int lane = nl_lane();
+    constexpr int NK = HALF ? 14 : 27;
+    // the own cell, then the others in the order of key = dx + 3 dy + 9 dz (half lists: key > 0);
+    // lane k holds the k-th one's tile range
+    int my_first = 0, my_end = 0;
+    if (lane < NK) {
+        const int k13 = lane == 0 ? 13 : (HALF ? lane : (lane <= 13 ? lane - 14 : lane - 13)) + 13;
+        const int slot = c_tiles.idx_of_coord[own_coord + (k13 % 3 - 1) + 4 * ((k13 / 3) % 3 - 1) + 16 * (k13 / 9 - 1)];
+        my_first = m.prefix[slot];
+        my_end = m.prefix[slot + 1];
+    }
+    const int own_count = __shfl_sync(0xffffffffu, my_end - my_first, 0);
+    const int T = m.prefix[64];
+    float xl, yl, zl, xh, yh, zh;  // the box of the own atoms
+    {
+        const int u = m.prefix[own] + lo_own + min(lane, own_n - 1);
+        const float x = tx[u], y = ty[u], z = tz[u];
+        w.own_xy[lane] = make_float4(x, x, y, y);
+        w.own_z[lane] = make_float4(z, z, 0.f, 0.f);
+        xl = warp_min(x), yl = warp_min(y), zl = warp_min(z);
+        xh = -warp_min(-x), yh = -warp_min(-y), zh = -warp_min(-z);
+    }
+    uint4* const row = reinterpret_cast<uint4*>(w.row + lane * NL_ROW);
+    const unsigned first = (unsigned)__cvta_generic_to_shared(row);
+    unsigned* const tail = reinterpret_cast<unsigned*>(&w.own_z[lane].z);
+    const unsigned axy = (unsigned)__cvta_generic_to_shared(w.own_xy);
+    const unsigned below = (1u << lane) - 1u;
+    out += lane;
+    uint4 part = make_uint4(0u, 0u, 0u, 0u);  // the list's open chunk: cnt % 8 entries
+    int cnt = 0;
+    int nc = 0, base = 0;  // candidates in the buffer; scan index of its first one
+    // (the loops below run on values the compiler knows to be the same in every lane: ballots,
+    // reductions and loop counters)
+    const int n_own = (int)__reduce_max_sync(0xffffffffu, (unsigned)own_n);
+    const int n_cell = (int)__reduce_max_sync(0xffffffffu, (unsigned)own_count);
+#pragma unroll 1
+    for (int k = 0; k <= NK; ++k) {  // k = NK: no cell, what is left in the buffer
+        int u = __shfl_sync(0xffffffffu, my_first, k);
+        const int end = __shfl_sync(0xffffffffu, my_end, k);
+        bool more;
+        do {
+            // ---- 1. cull up to 32 atoms of the cell
+            const int ui = u + lane, ur = max(min(ui, end - 1), 0);
+            const float x = tx[ur], y = ty[ur], z = tz[ur];
+            // distance to the box of the own atoms: each rounded difference is at most that to
+            // any own atom, so no pair with r^2 < hi is lost
+            const float dx = fmaxf(fmaxf(xl - x, x - xh), 0.f), dy = fmaxf(fmaxf(yl - y, y - yh), 0.f),
+                        dz = fmaxf(fmaxf(zl - z, z - zh), 0.f);
+            const float d2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
+            const bool keep = (ui < end) & ((d2 < hi) | (k == 0));
+            const unsigned kept = __ballot_sync(0xffffffffu, keep);
+            if (keep) w.cand[nc + __popc(kept & below)] = (uint16_t)ui;
+            nc += __popc(kept);
+            u += 32;
+            more = __any_sync(0xffffffffu, u < end);
+            if (nc <= NL_CAND - 32 && k < NK) continue;
+            // ---- 2. and 3. whole batches, and at the end what is left
+            __syncwarp();
+            int s = 0, width = NL_BATCH;
+            while (k == NK ? s < nc : s + NL_BATCH <= nc) {
+                const int nb = min(nc - s, width);
+                if (cnt & 7) row[0] = part;
+                *tail = first + 2u * (unsigned)(cnt & 7);
+                __syncwarp();
+                NlPair c;
+                {
+                    const int i = 2 * lane;
+                    const bool p = i < nb, q = i + 1 < nb;
+                    c.u0 = p ? w.cand[s + i] : 0u;
+                    c.u1 = q ? w.cand[s + i + 1] : 0u;
+                    c.x = f2_pack(p ? tx[c.u0] : NL_FAR, q ? tx[c.u1] : NL_FAR);
+                    c.y = f2_pack(p ? ty[c.u0] : NL_FAR, q ? ty[c.u1] : NL_FAR);
+                    c.z = f2_pack(p ? tz[c.u0] : NL_FAR, q ? tz[c.u1] : NL_FAR);
+                    c.index = base + s + i;
+                }
+                const unsigned near_lo = base + s < n_cell
+                                             ? nl_test<HALF, true, false>(axy, lane, lo_own, n_own, c, hi, lo, retest)
+                                             : nl_test<HALF, false, false>(axy, lane, lo_own, n_own, c, hi, lo, retest);
+                __syncwarp();
+                int open = (int)(*tail - first) >> 1;
+                if (__any_sync(0xffffffffu, open > NL_ROW)) {  // a row ran over: again, half as many
+                    width = NL_BATCH / 2;
+                    continue;
+                }
+                if (__any_sync(0xffffffffu, near_lo < __float_as_uint(hi - lo))) {  // rare: the definition decides in [lo, hi)
+                    *tail = first + 2u * (unsigned)(cnt & 7);
+                    __syncwarp();
+                    nl_test<HALF, true, true>(axy, lane, lo_own, n_own, c, hi, lo, retest);
+                    __syncwarp();
+                    open = (int)(*tail - first) >> 1;
+                }
+                // complete chunks to global memory, the open one to the lane's registers
+                const int c0 = cnt >> 3, nch = open >> 3;
+                const int most = (int)__reduce_max_sync(0xffffffffu, (unsigned)nch);
+                uint4* to = out + (size_t)c0 * np;
+                for (int j = 0; j < most; ++j) {
+                    if (j < nch && 8 * (c0 + j) < cap) *to = row[j];
+                    to += np;
+                }
+                part = row[nch];
+                cnt = 8 * c0 + open;
+                s += nb;
+                __syncwarp();
+            }
+            // what is left (less than a batch) to the front of the buffer
+            const int left = nc - s;
+            const uint16_t v0 = lane < left ? w.cand[s + lane] : (uint16_t)0;
+            const uint16_t v1 = lane + 32 < left ? w.cand[s + lane + 32] : (uint16_t)0;
+            __syncwarp();
+            if (lane < left) w.cand[lane] = v0;
+            if (lane + 32 < left) w.cand[lane + 32] = v1;
+            base += s;
+            nc = left;
+            __syncwarp();
+        } while (more);
+    }
+    if ((cnt & 7) && lane < own_n && cnt < cap) {  // the last chunk, padded with the tile's dummy slot
+        row[0] = part;
+        for (int e = cnt & 7; e < 8; ++e) w.row[lane * NL_ROW + e] = (uint16_t)T;
+        out[(size_t)(cnt >> 3) * np] = row[0];
+    }
+    __syncwarp();  // the next own atoms reuse the buffers
+    return cnt;
+}
 
 }  // namespace mdgb
