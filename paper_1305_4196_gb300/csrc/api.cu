@@ -528,6 +528,11 @@ double fill_pair_table(PairTable& pt, const double* eps, const double* sigma, co
         pt.sig2_d[t] = sg * sg;
         pt.eps_d[t] = e;
         pt.rc2_d[t] = rc_t * rc_t;
+        const double sg6 = sg * sg * sg * sg * sg * sg;
+        pt.lj_a_d[t] = 48.0 * e * sg6 * sg6;
+        pt.lj_b_d[t] = 24.0 * e * sg6;
+        pt.lj_a12_d[t] = 4.0 * e * sg6 * sg6;
+        pt.lj_b6_d[t] = 4.0 * e * sg6;
         pt.sig2_f[t] = (float)(sg * sg);
         pt.c48_f[t] = (float)(48.0 * e * 2048.0);
         pt.c24_f[t] = (float)(24.0 * e * 2048.0);

@@ -9,9 +9,19 @@
 //    of j in shared memory; one launch per colour class of blocks, whose tiles are disjoint
 //    (the barrier-separated waves of Sec. II.B).
 //
-// On GB300 the FP64 pipe bounds these kernels (the list and coordinates stream through
-// with DRAM nearly idle), so the pair arithmetic is kept to few FP64 operations: one
-// reciprocal of r^2 per pair serves both (sigma/r)^2 and f/r.
+// On GB300 the FP64 pipe bounds these kernels: an SM takes 16 cycles for a warp's FP64
+// operation, while it issues 64 others (the list and coordinates stream through with DRAM
+// nearly idle).  So the full-list kernel spends other instructions to save FP64 ones:
+//  * the list entries are tested in FP32 first, on the upper halves of the tile's coordinates,
+//    and only those that may lie inside the cutoff go to a queue in shared memory; the lanes
+//    of a warp then take their queues in step (a 76-entry list holds 55 inside, and the
+//    longest of 32 lanes about 62, where a masked loop runs all 80 padded entries);
+//  * 17 FP64 operations per pair: three differences, three for r^2, one reciprocal by a cubic
+//    step from an FP32 seed (three), five for f / r = inv^4 (a inv^3 - b), three sums; the
+//    exact cutoff test compares bit patterns.
+// Every result is that of FP64 arithmetic throughout.  At 360,703 atoms a force evaluation took
+// 1.38 ms and one with energy and virial 2.11 ms with 22 operations for each of the 80 padded
+// entries, and takes 0.80 and 1.27 ms; the FP64 pipe is 87 % busy.
 #include "fixpt.cuh"
 #include "tile.cuh"
 
@@ -37,18 +47,89 @@ __device__ __forceinline__ double rcp_nr(double x) {
     return y;
 }
 
+// The FP32 number of a double's upper half (20 mantissa bits, truncated; 0 below FP32's range).
+__device__ __forceinline__ float upper_f32(double x) {
+    const int h = __double2hiint(x);
+    const int t = max((h & 0x7fffffff) - (896 << 20), 0);
+    return __int_as_float((h & (int)0x80000000) | (t << 3));
+}
+
+// 1/x to within about an ulp in three FP64 operations, for x well inside FP32's range
+// (2^-100 .. 2^126): from an FP32 seed y (error e = 1 - x y of 2^-22) one step y (1 + e + e^2) of
+// Householder's third-order iteration leaves e^3.  Other x, zero among them, take rcp_nr.
+static __device__ __noinline__ double rcp_nr_far(double x) { return rcp_nr(x); }  // (a call: not computed for every x)
+
+__device__ __forceinline__ double rcp_cubic(double x) {
+    const unsigned h = (unsigned)__double2hiint(x) - (896u << 20);  // exponent as FP32 has it
+    if (h - (27u << 20) >= (226u << 20)) return rcp_nr_far(x);
+    const float xf = __int_as_float((int)__funnelshift_l((unsigned)__double2loint(x), h, 3));
+    const int yf = __float_as_int(rcp_approx(xf));
+    const double y = __hiloint2double((yf >> 3) + (896 << 20), yf << 29);
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
 // ---------------------------------------------------------------- full list
+constexpr int FQ = 16;  // queue slots per thread: up to 8 waiting and a chunk
+
+__host__ __device__ constexpr size_t fp64_queue_bytes(int threads) { return (size_t)threads * FQ * sizeof(uint16_t); }
+
 template <bool EV>
+struct Fp64Sums {
+    double f[3] = {0, 0, 0};
+    double pe = 0, w[6] = {0, 0, 0, 0, 0, 0};
+};
+
+// One pair: r^2 and the cutoff decision in FP64, and the force of an inside pair.
+template <bool SINGLE, bool EV>
+__device__ __forceinline__ void fp64_pair(const PairTable& pt, const double* __restrict__ tx,
+                                          const double* __restrict__ ty, const double* __restrict__ tz,
+                                          const int* __restrict__ tsp, int u, double xi, double yi, double zi, int si,
+                                          Fp64Sums<EV>& a) {
+    const double dx = xi - tx[u], dy = yi - ty[u], dz = zi - tz[u];
+    const double r2 = dx * dx + dy * dy + dz * dz;
+    const int t = SINGLE ? 0 : si * pt.nsp + tsp[u];
+    const double inv = rcp_cubic(r2);
+    const double inv2 = inv * inv, inv3 = inv2 * inv;
+    double fr = fma(SINGLE ? pt.lj_a_d[0] : pt.lj_a_d[t], inv3, -(SINGLE ? pt.lj_b_d[0] : pt.lj_b_d[t])) * (inv2 * inv2);
+    // r^2 >= 0 compares like its bits
+    const bool in = __double_as_longlong(r2) < __double_as_longlong(SINGLE ? pt.rc2_d[0] : pt.rc2_d[t]);
+    if (!in) fr = 0.0;
+    if (EV) {
+        const double px = fr * dx, py = fr * dy, pz = fr * dz;
+        a.f[0] += px;
+        a.f[1] += py;
+        a.f[2] += pz;
+        // 4 eps (s6^2 - s6) = inv^3 (a inv^3 / 12 - b / 6)
+        const double e = fma(SINGLE ? pt.lj_a12_d[0] : pt.lj_a12_d[t], inv3, -(SINGLE ? pt.lj_b6_d[0] : pt.lj_b6_d[t]));
+        a.pe = fma(in ? inv3 : 0.0, e, a.pe);
+        a.w[0] = fma(dx, px, a.w[0]);
+        a.w[1] = fma(dy, py, a.w[1]);
+        a.w[2] = fma(dz, pz, a.w[2]);
+        a.w[3] = fma(dx, py, a.w[3]);
+        a.w[4] = fma(dx, pz, a.w[4]);
+        a.w[5] = fma(dy, pz, a.w[5]);
+    } else {
+        a.f[0] = fma(fr, dx, a.f[0]);
+        a.f[1] = fma(fr, dy, a.f[1]);
+        a.f[2] = fma(fr, dz, a.f[2]);
+    }
+}
+
+// LPA lanes per atom, lane q of them with chunks q, q + LPA, ... of the list; `split` CTAs share
+// one block, each staging the tile and taking every split-th group of own atoms.  rc2_test: r_cut^2
+// plus the bound on the FP32 test's error, largest over the species pairs.  QUEUE = false evaluates
+// every entry (a tile that leaves no room for the queues).
+template <bool SINGLE, bool EV, int LPA, bool QUEUE>
 __global__ void __launch_bounds__(F_THREADS) k_force_fp64_full(DevState s, Geometry g, PairTable pt, int tile_cap,
-                                                               int split) {
+                                                               int split, float rc2_test) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ TileMeta m;
     double* tx = reinterpret_cast<double*>(smem);
     double* ty = tx + tile_cap;
     double* tz = ty + tile_cap;
     int* tsp = reinterpret_cast<int*>(tz + tile_cap);
-    // split CTAs share one block (small systems): each stages the tile and takes every
-    // split-th group of F_THREADS own atoms
+    uint16_t* const queue = reinterpret_cast<uint16_t*>(tsp + tile_cap) + threadIdx.x;
     const int b = spatial_block(g, blockIdx.x / split), part = blockIdx.x % split;
     tile_meta(g, s.cell_start, b, m);
     const int T = m.prefix[64];
@@ -56,54 +137,89 @@ __global__ void __launch_bounds__(F_THREADS) k_force_fp64_full(DevState s, Geome
         if (threadIdx.x == 0) atomicOr(s.err, ERR_TILE_OVERFLOW);
         return;
     }
+    const int nown = m.prefix[8];
+    const int per = blockDim.x / LPA;  // own atoms at a time
+    if (part * per >= nown) return;
     tile_stage_f64(s, g, m, b, tx, ty, tz, tsp);
     __syncthreads();
     const int blk0 = m.start[0];
-    const int nown = m.prefix[8];
     const int64_t n = s.n;
-    const int np = s.np;
-    for (int ui = part * blockDim.x + threadIdx.x; ui < nown; ui += split * blockDim.x) {
-        const int gi = blk0 + ui;
-        const double xi = tx[ui], yi = ty[ui], zi = tz[ui];
-        const int si = tsp[ui];
-        const int nch = (s.nl_cnt[gi] + 7) >> 3;
-        double fx = 0, fy = 0, fz = 0, pe = 0, w0 = 0, w1 = 0, w2 = 0, w3 = 0, w4 = 0, w5 = 0;
-        MDGB_FOR_EACH_NEIGHBOUR(reinterpret_cast<const uint4*>(s.nl) + gi, np, nch, {
-            const double dx = xi - tx[u], dy = yi - ty[u], dz = zi - tz[u];
-            const double r2 = dx * dx + dy * dy + dz * dz;
-            const int t = si * pt.nsp + tsp[u];
-            if (r2 < pt.rc2_d[t]) {
-                const double inv = rcp_nr(r2);
-                const double sr2 = pt.sig2_d[t] * inv;
-                const double s6 = sr2 * sr2 * sr2;
-                const double e = pt.eps_d[t];
-                const double fr = 24.0 * e * (2.0 * s6 * s6 - s6) * inv;
-                fx += fr * dx;
-                fy += fr * dy;
-                fz += fr * dz;
-                if (EV) {
-                    pe += 4.0 * e * (s6 * s6 - s6);
-                    w0 += dx * (fr * dx);
-                    w1 += dy * (fr * dy);
-                    w2 += dz * (fr * dz);
-                    w3 += dx * (fr * dy);
-                    w4 += dx * (fr * dz);
-                    w5 += dy * (fr * dz);
+    const size_t np = s.np;
+    const int lq = threadIdx.x % LPA;
+    for (int u0 = part * per; u0 < nown; u0 += split * per) {
+        const int ui = u0 + (int)threadIdx.x / LPA;
+        const bool active = ui < nown;
+        const int gi = blk0 + (active ? ui : 0);
+        const double xi = tx[active ? ui : 0], yi = ty[active ? ui : 0], zi = tz[active ? ui : 0];
+        const int si = SINGLE ? 0 : tsp[active ? ui : 0];
+        const int nch = active ? (s.nl_cnt[gi] + 7) >> 3 : 0;
+        const uint4* lp = reinterpret_cast<const uint4*>(s.nl) + gi;
+        Fp64Sums<EV> a;
+        if (QUEUE) {
+            const float xf = upper_f32(xi), yf = upper_f32(yi), zf = upper_f32(zi);
+            int head = 0, tail = 0;
+            uint4 nxt = make_uint4(0u, 0u, 0u, 0u);
+            if (lq < nch) nxt = __ldcs(lp + (size_t)lq * np);
+            for (int c = lq; __any_sync(0xffffffffu, c < nch); c += LPA) {
+                const uint4 cur = nxt;
+                if (c + LPA < nch) nxt = __ldcs(lp + (size_t)(c + LPA) * np);
+                if (c < nch) {
+                    const unsigned wd[4] = {cur.x, cur.y, cur.z, cur.w};
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) {
+                        const int u = (int)((wd[e >> 1] >> ((e & 1) * 16)) & 0xffffu);
+                        const float dx = xf - upper_f32(tx[u]), dy = yf - upper_f32(ty[u]), dz = zf - upper_f32(tz[u]);
+                        if (fmaf(dz, dz, fmaf(dy, dy, dx * dx)) < rc2_test) {
+                            queue[(tail & (FQ - 1)) * F_THREADS] = (uint16_t)u;
+                            ++tail;
+                        }
+                    }
+                }
+                // in step while every lane has an entry, or some lane too many for the next chunk
+                while (__any_sync(0xffffffffu, tail - head > FQ - 8) || __all_sync(0xffffffffu, tail > head)) {
+                    if (tail > head) {
+                        fp64_pair<SINGLE, EV>(pt, tx, ty, tz, tsp, queue[(head & (FQ - 1)) * F_THREADS], xi, yi, zi, si,
+                                              a);
+                        ++head;
+                    }
                 }
             }
-        })
-        if (!(isfinite(fx) && isfinite(fy) && isfinite(fz))) atomicOr(s.err, ERR_NONFINITE);
-        s.f[gi] = fx;
-        s.f[n + gi] = fy;
-        s.f[2 * n + gi] = fz;
+            while (__any_sync(0xffffffffu, tail > head)) {
+                if (tail > head) {
+                    fp64_pair<SINGLE, EV>(pt, tx, ty, tz, tsp, queue[(head & (FQ - 1)) * F_THREADS], xi, yi, zi, si, a);
+                    ++head;
+                }
+            }
+        } else {
+            for (int c = lq; c < nch; c += LPA) {
+                const uint4 cur = __ldcs(lp + (size_t)c * np);
+                const unsigned wd[4] = {cur.x, cur.y, cur.z, cur.w};
+#pragma unroll 1
+                for (int e = 0; e < 8; ++e)
+                    fp64_pair<SINGLE, EV>(pt, tx, ty, tz, tsp, (int)((wd[e >> 1] >> ((e & 1) * 16)) & 0xffffu), xi, yi,
+                                          zi, si, a);
+            }
+        }
+#pragma unroll
+        for (int o = LPA / 2; o > 0; o >>= 1) {
+#pragma unroll
+            for (int d = 0; d < 3; ++d) a.f[d] += __shfl_xor_sync(0xffffffffu, a.f[d], o);
+            if (EV) {
+                a.pe += __shfl_xor_sync(0xffffffffu, a.pe, o);
+#pragma unroll
+                for (int d = 0; d < 6; ++d) a.w[d] += __shfl_xor_sync(0xffffffffu, a.w[d], o);
+            }
+        }
+        if (!active) continue;
+        if (!(isfinite(a.f[0]) && isfinite(a.f[1]) && isfinite(a.f[2]))) atomicOr(s.err, ERR_NONFINITE);
+        if (lq) continue;
+        s.f[gi] = a.f[0];
+        s.f[n + gi] = a.f[1];
+        s.f[2 * n + gi] = a.f[2];
         if (EV) {
-            s.pe_atom_d[gi] = 0.5 * pe;
-            s.vir_atom_d[gi] = 0.5 * w0;
-            s.vir_atom_d[n + gi] = 0.5 * w1;
-            s.vir_atom_d[2 * n + gi] = 0.5 * w2;
-            s.vir_atom_d[3 * n + gi] = 0.5 * w3;
-            s.vir_atom_d[4 * n + gi] = 0.5 * w4;
-            s.vir_atom_d[5 * n + gi] = 0.5 * w5;
+            s.pe_atom_d[gi] = 0.5 * a.pe;
+#pragma unroll
+            for (int d = 0; d < 6; ++d) s.vir_atom_d[d * n + gi] = 0.5 * a.w[d];
         }
     }
 }
@@ -196,22 +312,62 @@ __global__ void __launch_bounds__(F_THREADS) k_force_fp64_half(DevState s, Geome
 }
 
 // ---------------------------------------------------------------- launchers
+using Fp64Full = void (*)(DevState, Geometry, PairTable, int, int, float);
+
+template <bool SINGLE, bool EV, bool QUEUE>
+static Fp64Full full_of(int lpa) {
+    switch (lpa) {
+        case 1: return k_force_fp64_full<SINGLE, EV, 1, QUEUE>;
+        case 2: return k_force_fp64_full<SINGLE, EV, 2, QUEUE>;
+        case 4: return k_force_fp64_full<SINGLE, EV, 4, QUEUE>;
+        default: return k_force_fp64_full<SINGLE, EV, 8, QUEUE>;
+    }
+}
+
+static Fp64Full full_kernel(bool single, bool ev, bool queue, int lpa) {
+    if (single) {
+        if (ev) return queue ? full_of<true, true, true>(lpa) : full_of<true, true, false>(lpa);
+        return queue ? full_of<true, false, true>(lpa) : full_of<true, false, false>(lpa);
+    }
+    if (ev) return queue ? full_of<false, true, true>(lpa) : full_of<false, true, false>(lpa);
+    return queue ? full_of<false, false, true>(lpa) : full_of<false, false, false>(lpa);
+}
+
+static void launch_full(const DevState& s, const Geometry& g, const PairTable& pt, int tile_cap, int split, int lpa,
+                        int with_energy, float rc2_test, size_t smem, cudaStream_t st) {
+    // (the FP32 test needs r_cut^2 well inside FP32's range)
+    const bool queue = smem + fp64_queue_bytes(F_THREADS) <= 226 * 1024 && rc2_test > 1e-24f && rc2_test < 1e30f;
+    if (queue) smem += fp64_queue_bytes(F_THREADS);
+    const unsigned grid = (unsigned)g.nblock * (unsigned)split;
+    full_kernel(pt.nsp == 1, with_energy != 0, queue, lpa)<<<grid, F_THREADS, smem, st>>>(s, g, pt, tile_cap, split,
+                                                                                        rc2_test);
+}
+
 void launch_forces_fp64(const DevState& s, const Geometry& g, const PairTable& pt, int tile_cap, int half,
                         int with_energy, cudaStream_t st) {
     if (s.n == 0) return;
     const size_t smem = force_smem_bytes(0, half, with_energy, tile_cap);
     if (!half) {
-        // CTAs per block: about one own atom per thread while the grid is below two CTAs per SM
+        // Lanes per atom and CTAs per block: more of both while the grid is below two CTAs per SM
+        // (4,000 atoms have 8 blocks: 197 us with 16 CTAs and one lane, 46 us with 128 and eight).
         const int sms = g_sm_count > 0 ? g_sm_count : 152;
         const int64_t per_block = (s.n + g.nblock - 1) / g.nblock;
-        int split = (int)std::min<int64_t>((per_block + F_THREADS - 1) / F_THREADS, (2 * sms + g.nblock - 1) / g.nblock);
-        split = std::max(1, std::min(split, 8));
-        const unsigned grid = (unsigned)g.nblock * (unsigned)split;
-        if (with_energy) {
-            k_force_fp64_full<true><<<grid, F_THREADS, smem, st>>>(s, g, pt, tile_cap, split);
-        } else {
-            k_force_fp64_full<false><<<grid, F_THREADS, smem, st>>>(s, g, pt, tile_cap, split);
+        int lpa = 1;
+        int64_t split = 1;
+        for (; lpa <= 8; lpa *= 2) {
+            split = std::max<int64_t>(1, (per_block * lpa + F_THREADS - 1) / F_THREADS);
+            if (g.nblock * split >= 2 * sms) break;
         }
+        lpa = std::min(lpa, 8);
+        if (lpa == 1) split = std::min<int64_t>(split, (2 * sms + g.nblock - 1) / g.nblock);
+        // the FP32 test's error: coordinates up to two cells from the block centre, cut to 20 bits
+        const double wmax = std::max({g.w[0], g.w[1], g.w[2]});
+        double rc2 = 0.0;
+        for (int t = 0; t < pt.nsp * pt.nsp; ++t) rc2 = std::max(rc2, pt.rc2_d[t]);
+        const double e_d = 3.0 * wmax * 0x1p-19;
+        const double rc = std::sqrt(rc2);
+        const float rc2_test = (float)((rc2 + 2.0 * std::sqrt(3.0) * rc * e_d + 3.0 * e_d * e_d) * (1.0 + 1e-6));
+        launch_full(s, g, pt, tile_cap, (int)split, lpa, with_energy, rc2_test, smem, st);
         return;
     }
     cudaMemsetAsync(s.f, 0, sizeof(double) * 3 * (size_t)s.n, st);
@@ -238,8 +394,8 @@ static void allow_max_smem(K kernel) {
 void init_force_fp64_kernels() {
     int dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&g_sm_count, cudaDevAttrMultiProcessorCount, dev);
-    allow_max_smem(k_force_fp64_full<false>);
-    allow_max_smem(k_force_fp64_full<true>);
+    for (int k = 0; k < 8; ++k)
+        for (int lpa = 1; lpa <= 8; lpa *= 2) allow_max_smem(full_kernel(k & 1, k & 2, k & 4, lpa));
     allow_max_smem(k_force_fp64_half<false>);
     allow_max_smem(k_force_fp64_half<true>);
 }

@@ -57,6 +57,9 @@ struct PairTable {
     int nsp;
     float sig2_f[MAX_PAIR], c48_f[MAX_PAIR], c24_f[MAX_PAIR], c4_f[MAX_PAIR], rc2_f[MAX_PAIR];
     double sig_d[MAX_PAIR], sig2_d[MAX_PAIR], eps_d[MAX_PAIR], rc2_d[MAX_PAIR];
+    // f / r = inv^4 (lj_a_d inv^3 - lj_b_d) with inv = 1/r^2: 48 eps sigma^12 and 24 eps sigma^6; a
+    // twelfth and a sixth of them for the energy
+    double lj_a_d[MAX_PAIR], lj_b_d[MAX_PAIR], lj_a12_d[MAX_PAIR], lj_b6_d[MAX_PAIR];
     double hdtm[MAX_SPECIES];  // (dt/2) / m per species
     double hdtm_q[MAX_SPECIES];  // (dt/2) / m * 2^-32: half kick per unit of Q31.32 force
     double mass[MAX_SPECIES];

@@ -250,22 +250,27 @@ __device__ __forceinline__ void tile_stage_f64(const DevState& s, const Geometry
     int bx, by, bz;
     block_coords(g, b, bx, by, bz);
     const int T = m.prefix[64];
-    for (int u = threadIdx.x; u < T; u += blockDim.x) {
-        const int slot = tile_slot_of(m, u);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const double cx = (2.0 * bx + 1.0) * g.w[0], cy = (2.0 * by + 1.0) * g.w[1], cz = (2.0 * bz + 1.0) * g.w[2];
+#pragma unroll 2
+    for (int slot = warp; slot < 64; slot += nw) {  // one warp per tile cell
         const int c = c_tiles.coord_of_idx[slot];
-        const int j = m.start[slot] + (u - m.prefix[slot]);
-        const int t3[3] = {c & 3, (c >> 2) & 3, c >> 4};
-        const int b3[3] = {bx, by, bz};
-        const double* X[3] = {s.x, s.y, s.z};
-        double* out[3] = {tx_, ty_, tz_};
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            const int raw = 2 * b3[d] - 1 + t3[d];
-            const double shift = raw < 0 ? -g.L[d] : (raw >= g.nc[d] ? g.L[d] : 0.0);
-            const double centre = (2.0 * b3[d] + 1.0) * g.w[d];
-            out[d][u] = (X[d][j] + shift) - centre;
+        const int rx = 2 * bx - 1 + (c & 3), ry = 2 * by - 1 + ((c >> 2) & 3), rz = 2 * bz - 1 + (c >> 4);
+        const int u0 = m.prefix[slot], cnt = m.prefix[slot + 1] - u0, j0 = m.start[slot];
+        for (int e = lane; e < cnt; e += 32) {
+            double x = s.x[j0 + e], y = s.y[j0 + e], z = s.z[j0 + e];
+            const int sp = s.species[j0 + e];
+            if (rx < 0) x -= g.L[0];
+            else if (rx >= g.nc[0]) x += g.L[0];
+            if (ry < 0) y -= g.L[1];
+            else if (ry >= g.nc[1]) y += g.L[1];
+            if (rz < 0) z -= g.L[2];
+            else if (rz >= g.nc[2]) z += g.L[2];
+            tx_[u0 + e] = x - cx;
+            ty_[u0 + e] = y - cy;
+            tz_[u0 + e] = z - cz;
+            tsp[u0 + e] = sp;
         }
-        tsp[u] = s.species[j];
     }
     if (threadIdx.x == 0) {
         tx_[T] = ty_[T] = tz_[T] = 1.0e4;
