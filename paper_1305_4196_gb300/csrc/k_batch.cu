@@ -579,7 +579,9 @@ __device__ void ens_meta(const EnsBlockSys& y, const EnsArrays& ea, int b, EnsTi
     const int bx = b % y.nb[0], t_ = b / y.nb[0], by = t_ % y.nb[1], bz = t_ / y.nb[1];
     const int t = threadIdx.x;
     if (t < 64) {
-        const int c = c_tiles.coord_of_idx[t];
+        const int c = tile_coord_of(t);
+        mt.coord[t] = (int8_t)c;
+        mt.slot[c] = (int8_t)t;
         int cx = 2 * bx - 1 + (c & 3), cy = 2 * by - 1 + ((c >> 2) & 3), cz = 2 * bz - 1 + (c >> 4);
         cx += cx < 0 ? y.nc[0] : (cx >= y.nc[0] ? -y.nc[0] : 0);
         cy += cy < 0 ? y.nc[1] : (cy >= y.nc[1] ? -y.nc[1] : 0);
@@ -613,12 +615,17 @@ __device__ int ens_stage(const EnsBlockSys& y, const EnsArrays& ea, const float4
         if (threadIdx.x == 0) atomicOr(err, ERR_TILE_OVERFLOW);
         return -1;
     }
+    TileOffsets to;
+#pragma unroll
+    for (int d = 0; d < 3; ++d)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) to.off[d][q] = y.off[d][q];
     // all threads over the tile's atoms (its cell by binary search), so that the L2 loads of
     // a task overlap
     for (int u = threadIdx.x; u < T; u += blockDim.x) {
         const int sl = ens_slot_of(mt, u);
-        const int c = c_tiles.coord_of_idx[sl];
-        const float ox = pick4(y.off[0], c & 3), oy = pick4(y.off[1], (c >> 2) & 3), oz = pick4(y.off[2], c >> 4);
+        const int c = mt.coord[sl];
+        const float ox = pick4(to.off[0], c & 3), oy = pick4(to.off[1], (c >> 2) & 3), oz = pick4(to.off[2], c >> 4);
         const float4 p = __ldcg(xs + y.a0 + mt.start[sl] + (u - mt.prefix[sl]));
         tile[u] = make_float4(p.x + ox, p.y + oy, p.z + oz, 0.0f);
     }

@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(G_THREADS) k_force_backward(DevState s, Geomet
     } else {
         const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
         for (int slot = warp; slot < 64; slot += nw) {
-            const int c = c_tiles.coord_of_idx[slot];
+            const int c = m.coord[slot];
             const float ox = pick4(to.off[0], c & 3), oy = pick4(to.off[1], (c >> 2) & 3),
                         oz = pick4(to.off[2], c >> 4);
             const int u0 = m.prefix[slot], cnt = m.prefix[slot + 1] - u0, j0 = m.start[slot];

@@ -83,7 +83,7 @@ __global__ void __launch_bounds__(AF_WARPS * 32) k_build_sched(DevState s, Geome
         return;
     }
     for (int slot = warp; slot < 64; slot += AF_WARPS) {  // the tile's FP32 coordinates, as everywhere
-        const int c = c_tiles.coord_of_idx[slot];
+        const int c = m.coord[slot];
         const float ox = pick4(to.off[0], c & 3), oy = pick4(to.off[1], (c >> 2) & 3),
                     oz = pick4(to.off[2], c >> 4);
         const int j0 = m.start[slot], u0 = m.prefix[slot], cnt = m.prefix[slot + 1] - u0;
@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(AF_WARPS * 32) k_build_sched(DevState s, Geome
     }
     __syncthreads();
 
-    const int own_c = c_tiles.coord_of_idx[warp];
+    const int own_c = m.coord[warp];
     const int cx = own_c & 3, cy = (own_c >> 2) & 3, cz = own_c >> 4;
     const int own0 = m.prefix[warp], nw = m.prefix[warp + 1] - own0;
     const int blk0 = m.start[0];
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(AF_WARPS * 32) k_build_sched(DevState s, Geome
         for (int p = 0; p < AF_PHASES; ++p) {
             int dx, dy, dz;
             af_offset(p, dx, dy, dz);
-            const int ts = c_tiles.idx_of_coord[(cx + dx) + 4 * (cy + dy) + 16 * (cz + dz)];
+            const int ts = m.slot[(cx + dx) + 4 * (cy + dy) + 16 * (cz + dz)];
             const int t0 = m.prefix[ts], mt = m.prefix[ts + 1] - t0;
             if (mt > AF_MAX_CELL) {
                 if (lane == 0) atomicOr(s.err, ERR_CELL_DENSE);

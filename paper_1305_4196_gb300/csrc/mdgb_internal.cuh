@@ -248,6 +248,8 @@ struct TileOffsets {
 struct TileMeta {
     int prefix[65];  // tile slot -> first tile index (prefix[64] = tile size)
     int start[64];   // tile slot -> first global (cell-ordered) atom index
+    int8_t coord[64];  // tile slot -> tile coordinate (tx + 4 ty + 16 tz)
+    int8_t slot[64];   // tile coordinate -> tile slot
 };
 
 // Device state shared by the kernels (all arrays in cell order unless noted).
@@ -272,6 +274,7 @@ struct DevState {
                             // nl[((k / 8) * np + s) * 8 + k % 8]; the last chunk is padded with the
                             // tile's dummy slot (a point far outside every cutoff)
     uint16_t *nl_cnt;       // list length per atom
+    int nl_chunks;          // chunks of 8 entries the list matrix holds for each atom
     float *pe_atom_f;       // per-atom energy share (mixed, on demand)
     float *vir_atom_f;      // per-atom virial share, 6 x n (mixed, on demand)
     double *pe_atom_d;      // FP64 path
@@ -321,6 +324,12 @@ struct StepOut {
 void launch_forces_mixed_fused(const DevState& s, const Geometry& g, const PairTable& pt, const TileOffsets& to,
                                int tile_cap, int mode, StepOut out, double dt, double lim2, cudaStream_t st);
 enum { FUSE_KICK = 1, FUSE_KICK_KICK_DRIFT = 2 };  // modes of launch_forces_mixed_fused
+// The same tasks with several CTAs per block and lanes per atom (k_force_split.cu), for systems
+// of few blocks; false where one CTA per block is the better form (nothing is launched).
+bool launch_forces_mixed_split(const DevState& s, const Geometry& g, const PairTable& pt, const TileOffsets& to,
+                               int tile_cap, float fs2_max, bool with_energy, int mode, StepOut out, double dt,
+                               float lim2_f, size_t smem, cudaStream_t st);
+void init_force_split_kernels();
 // TB-SMA forces (full lists, mixed): the density pass writes emb[i] = 1/sqrt(rho_i) (0 for an
 // atom without neighbours), the force pass the Q31.32 forces; with_energy also writes the
 // per-atom energies and virial shares.  Two launches.

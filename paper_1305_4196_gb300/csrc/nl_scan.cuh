@@ -139,7 +139,7 @@ __device__ __forceinline__ void nl_stage(const TileMeta& m, const TileOffsets& t
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
 #pragma unroll 2
     for (int slot = warp; slot < 64; slot += nw) {
-        const int c = c_tiles.coord_of_idx[slot];
+        const int c = m.coord[slot];
         const float ox = pick4(to.off[0], c & 3), oy = pick4(to.off[1], (c >> 2) & 3), oz = pick4(to.off[2], c >> 4);
         const int u0 = m.prefix[slot], cnt = m.prefix[slot + 1] - u0, j0 = m.start[slot];
         for (int e = lane; e < cnt; e += 32) {
@@ -167,7 +167,7 @@ __device__ __forceinline__ int nl_scan_cell(NlWarp& w, const TileMeta& m, const 
     int my_first = 0, my_end = 0;
     if (lane < NK) {
         const int k13 = lane == 0 ? 13 : (HALF ? lane : (lane <= 13 ? lane - 14 : lane - 13)) + 13;
-        const int slot = c_tiles.idx_of_coord[own_coord + (k13 % 3 - 1) + 4 * ((k13 / 3) % 3 - 1) + 16 * (k13 / 9 - 1)];
+        const int slot = m.slot[own_coord + (k13 % 3 - 1) + 4 * ((k13 / 3) % 3 - 1) + 16 * (k13 / 9 - 1)];
         my_first = m.prefix[slot];
         my_end = m.prefix[slot + 1];
     }

@@ -69,11 +69,29 @@ static_assert(count_tile_receivers() == TILE_RECV_CELLS, "half-shell targets of 
 __host__ __device__ inline int half_recv_cap(int tile_cap) { return ((tile_cap * 11 + 15) / 16 + 31) & ~31; }
 __host__ __device__ inline int tile_cap_for_recv(int recv) { return (recv * 16 + 10) / 11; }
 
-static __constant__ TileTables c_tiles = make_tile_tables();
+// Tile coordinate of slot t, from the table as 2-bit digits in immediate operands: an indexed read
+// of constant memory takes some 600 cycles here, which every CTA would wait for before its
+// first load (and once per cell while staging; those read TileMeta instead).
+__host__ __device__ constexpr unsigned long long tile_digits(int axis, int half) {
+    constexpr TileTables t = make_tile_tables();
+    unsigned long long v = 0;
+    for (int k = 0; k < 32; ++k)
+        v |= (unsigned long long)((t.coord_of_idx[32 * half + k] >> (2 * axis)) & 3) << (2 * k);
+    return v;
+}
 
-// Cell id of tile slot t of the block with coordinates (bx, by, bz).
-__device__ __forceinline__ int tile_cell_id(const Geometry& g, int bx, int by, int bz, int t) {
-    const int c = c_tiles.coord_of_idx[t];
+__device__ __forceinline__ int tile_coord_of(int t) {
+    constexpr unsigned long long x0 = tile_digits(0, 0), x1 = tile_digits(0, 1), y0 = tile_digits(1, 0),
+                                 y1 = tile_digits(1, 1), z0 = tile_digits(2, 0), z1 = tile_digits(2, 1);
+    const int sh = 2 * (t & 31);
+    const bool lo = t < 32;
+    const int x = (int)((lo ? x0 : x1) >> sh) & 3, y = (int)((lo ? y0 : y1) >> sh) & 3,
+              z = (int)((lo ? z0 : z1) >> sh) & 3;
+    return x + 4 * y + 16 * z;
+}
+
+// Cell id at tile coordinate c of the block with coordinates (bx, by, bz).
+__device__ __forceinline__ int tile_cell_id(const Geometry& g, int bx, int by, int bz, int c) {
     const int tx = c & 3, ty = (c >> 2) & 3, tz = c >> 4;
     int cx = 2 * bx - 1 + tx, cy = 2 * by - 1 + ty, cz = 2 * bz - 1 + tz;
     cx += cx < 0 ? g.nc[0] : (cx >= g.nc[0] ? -g.nc[0] : 0);
@@ -89,10 +107,13 @@ __device__ __forceinline__ void tile_meta(const Geometry& g, const int32_t* __re
     if (t < 64) {
         int bx, by, bz;
         block_coords(g, b, bx, by, bz);
-        int id = tile_cell_id(g, bx, by, bz, t);
+        const int c = tile_coord_of(t);
+        int id = tile_cell_id(g, bx, by, bz, c);
         int st = cell_start[id];
         int cnt = cell_start[id + 1] - st;
         m.start[t] = st;
+        m.coord[t] = (int8_t)c;
+        m.slot[c] = (int8_t)t;
         // inclusive scan of the 64 counts over two warps
         int lane = t & 31;
         int v = cnt;
@@ -119,10 +140,13 @@ __device__ __forceinline__ void tile_meta_warp(const Geometry& g, const int32_t*
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const int t = lane + 32 * h;
-        const int id = tile_cell_id(g, bx, by, bz, t);
+        const int c = tile_coord_of(t);
+        const int id = tile_cell_id(g, bx, by, bz, c);
         const int st = cell_start[id];
         int v = cell_start[id + 1] - st;
         m.start[t] = st;
+        m.coord[t] = (int8_t)c;
+        m.slot[c] = (int8_t)t;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int y = __shfl_up_sync(0xffffffffu, v, o);
@@ -170,16 +194,19 @@ __device__ __forceinline__ int tile_global_index(const TileMeta& m, int u) {
     return m.start[slot] + (u - m.prefix[slot]);
 }
 
-// o[t] for t in 0..3 without dynamic indexing (which would copy the table to local memory)
+// o[t] for t in 0..3, where o = (-3/2, -1/2, 1/2, 3/2) w: by two selects (dynamic indexing would
+// copy the table to local memory, and nested conditions compile to branches: 600 cycles for
+// the six offsets of two tile cells)
 __device__ __forceinline__ float pick4(const float (&o)[4], int t) {
-    return t == 0 ? o[0] : (t == 1 ? o[1] : (t == 2 ? o[2] : o[3]));
+    const float a = ((t + 1) & 2) ? o[2] : o[3];  // t = 1, 2: the inner cells
+    return __int_as_float(__float_as_int(a) ^ (t < 2 ? (int)0x80000000 : 0));
 }
 
 // Block-frame FP32 coordinates of tile index u, the same additions as the staging below.
 __device__ __forceinline__ float4 tile_coord(const TileMeta& m, const TileOffsets& to, const float4* __restrict__ xr,
                                              int u) {
     const int slot = tile_slot_of(m, u);
-    const int c = c_tiles.coord_of_idx[slot];
+    const int c = m.coord[slot];
     const float4 p = xr[m.start[slot] + (u - m.prefix[slot])];
     return make_float4(p.x + pick4(to.off[0], c & 3), p.y + pick4(to.off[1], (c >> 2) & 3),
                        p.z + pick4(to.off[2], c >> 4), p.w);
@@ -192,9 +219,9 @@ __device__ __forceinline__ void tile_stage_f32_cells(const TileMeta& m, const fl
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     for (int slot = warp; slot < 64; slot += 2 * nw) {
         const int slot2 = slot + nw;
-        const int c = c_tiles.coord_of_idx[slot];
+        const int c = m.coord[slot];
         const int u0 = m.prefix[slot], cnt = m.prefix[slot + 1] - u0, j0 = m.start[slot];
-        const int c2 = slot2 < 64 ? c_tiles.coord_of_idx[slot2] : 0;
+        const int c2 = slot2 < 64 ? m.coord[slot2] : 0;
         const int v0 = slot2 < 64 ? m.prefix[slot2] : 0;
         const int cnt2 = slot2 < 64 ? m.prefix[slot2 + 1] - v0 : 0;
         const int k0 = slot2 < 64 ? m.start[slot2] : 0;
@@ -230,7 +257,7 @@ __device__ __forceinline__ void tile_stage_f32(const TileMeta& m, const float4* 
     const int T = m.prefix[64];
     for (int u = threadIdx.x; u < T; u += blockDim.x) {
         int slot = tile_slot_of(m, u);
-        int c = c_tiles.coord_of_idx[slot];
+        int c = m.coord[slot];
         int j = m.start[slot] + (u - m.prefix[slot]);
         float4 p = xr[j];
         p.x += pick4(to.off[0], c & 3);
@@ -254,7 +281,7 @@ __device__ __forceinline__ void tile_stage_f64(const DevState& s, const Geometry
     const double cx = (2.0 * bx + 1.0) * g.w[0], cy = (2.0 * by + 1.0) * g.w[1], cz = (2.0 * bz + 1.0) * g.w[2];
 #pragma unroll 2
     for (int slot = warp; slot < 64; slot += nw) {  // one warp per tile cell
-        const int c = c_tiles.coord_of_idx[slot];
+        const int c = m.coord[slot];
         const int rx = 2 * bx - 1 + (c & 3), ry = 2 * by - 1 + ((c >> 2) & 3), rz = 2 * bz - 1 + (c >> 4);
         const int u0 = m.prefix[slot], cnt = m.prefix[slot + 1] - u0, j0 = m.start[slot];
         for (int e = lane; e < cnt; e += 32) {
