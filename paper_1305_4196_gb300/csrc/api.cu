@@ -247,6 +247,7 @@ int alloc_lists(md_system* s, int cap, bool keep = false) {
                            cudaMemcpyDeviceToDevice, s->stream));
     dfree(s, s->st[0].nl);
     s->st[0].nl = s->st[1].nl = s->st[2].nl = nl;
+    for (int k = 0; k < 3; ++k) s->st[k].nl_chunks = cap / 8;
     s->list_cap = cap;
     s->graphs_valid = false;
     return MD_OK;
