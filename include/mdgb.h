@@ -171,9 +171,10 @@ int md_forces(md_system *s, double *f_out, int device_ptrs);
 /*
  * Integrate n_steps velocity-Verlet steps: v += dt F/(2m); x += dt v;
  * rebuild lists if the policy says so; F = F(x); v += dt F/(2m).
- * Steps run as CUDA-graph launches (the rebuild decision taken on the device in a
- * conditional node per step; graphs of 8 steps where possible, else one step per
- * graph); the host reads the device status once per
+ * Steps run as one CUDA-graph launch per chunk of up to 200 steps (the rebuild decision
+ * taken on the device in a conditional node per step, the steps in a while node and a
+ * remainder; with md_set_timing on, graphs of 8 steps or one, whose force kernels
+ * event nodes can bracket); the host reads the device status once per
  * chunk of up to 200 steps.  If a rebuild inside a chunk outgrows the
  * list or tile capacity, the chunk is redone from a snapshot of its starting
  * state after the capacities have been regrown (md_info.n_redos counts these).

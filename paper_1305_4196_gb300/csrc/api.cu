@@ -12,9 +12,13 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <map>
 #include <vector>
 
 using namespace mdgb;
+
+// words of the device's status block: err, rebuild flag, 8 statistics, 6 unused, 3 control words of 64 bits
+constexpr int STATUS_WORDS = 22, STATUS_CTRL = 16;
 
 struct md_system {
     int device = 0;
@@ -37,7 +41,9 @@ struct md_system {
             *slot_src = nullptr, *sorted_src = nullptr, *scan_scratch = nullptr;
     double *partials = nullptr, *out8 = nullptr;
     int nparts = 0;
-    uint32_t* h_flags = nullptr;  // pinned: [0] err, [1] rebuild flag, [2..5] stats
+    // pinned mirror of the device's status block, read with one copy: [0] err, [1] rebuild flag,
+    // [2..9] stats, then the control words (d_ctrl)
+    uint32_t* h_flags = nullptr;
     bool has_state = false, lists_valid = false, forces_valid = false;
     int64_t n_builds = 0, n_steps = 0, list_entries = 0;
     int max_list = 0, max_tile = 0;
@@ -64,6 +70,9 @@ struct md_system {
     // MULTI_STEPS kick-kick-drift steps from buffer 0 in one graph (even: back in buffer 0),
     // for md_step calls without timing events: fewer graph launches per step
     StepGraph g_multi;
+    // the steps of a chunk in one graph, by what its loop of LOOP_STEPS steps leaves over
+    // (2 * steps + 1 if the closing step of a call follows); see capture_loop
+    std::map<int, StepGraph> g_loop;
     float4* xr_alt = nullptr;
     int potential = 0;       // 0: Lennard-Jones pair table; 1: TB-SMA many-body (md_set_tbsma)
     TBTable tb{};
@@ -74,8 +83,10 @@ struct md_system {
     bool graph_timing = false;
     bool use_graphs = true;  // MDGB_NO_GRAPHS=1 at md_create: host-launched steps (profilers see every kernel)
     bool no_fuse = false;    // MDGB_NO_FUSE=1 at md_create: separate force and integration kernels
-    long long* d_ctrl = nullptr;  // [0] step counter, [1] builds done inside graphs
-    long long* h_ctrl = nullptr;  // pinned mirror
+    // control words of the step graphs, in the status block: [0] step counter, [1] builds done
+    // inside graphs, [2] loop passes left
+    long long* d_ctrl = nullptr;
+    long long* h_ctrl = nullptr;  // pinned, for the copy to the device
     bool snapshot_first = true;
     int compact = 0;          // grid of the occupied-block loops of a mostly empty system (see do_build)
     bool no_compact = false;  // MDGB_NO_COMPACT=1 at md_create: one CTA per block always
@@ -254,12 +265,17 @@ int alloc_lists(md_system* s, int cap, bool keep = false) {
 }
 
 int sync_flags(md_system* s) {
-    CK(cudaMemcpyAsync(s->h_flags, s->st[0].err, sizeof(uint32_t), cudaMemcpyDeviceToHost, s->stream));
-    CK(cudaMemcpyAsync(s->h_flags + 1, s->st[0].rebuild_flag, sizeof(int32_t), cudaMemcpyDeviceToHost, s->stream));
-    CK(cudaMemcpyAsync(s->h_flags + 2, s->st[0].stats, 5 * sizeof(int32_t), cudaMemcpyDeviceToHost, s->stream));
+    CK(cudaMemcpyAsync(s->h_flags, s->st[0].err, STATUS_WORDS * sizeof(uint32_t), cudaMemcpyDeviceToHost, s->stream));
     CK(cudaStreamSynchronize(s->stream));
     drain_events(s);
     return MD_OK;
+}
+
+// Builds done inside graphs since the control words were written, as of the last sync_flags.
+long long builds_in_graphs(const md_system* s) {
+    long long b;
+    std::memcpy(&b, s->h_flags + STATUS_CTRL + 2, sizeof(b));
+    return b;
 }
 
 int check_err(md_system* s, uint32_t mask) {
@@ -780,6 +796,153 @@ int capture_fused_multi(md_system* s, md_system::StepGraph& out) {
     return MD_OK;
 }
 
+// ---- whole chunks in one graph
+//
+// A conditional node at the top level of a graph costs 8.6 us, one inside the body of another
+// about 2 us (measured around an empty kernel; a kernel node alone 1.3 us), and a pass of a
+// while node 5.7 us.  So a chunk of steps is one graph: a while node whose body holds LOOP_STEPS
+// steps, each with its own conditional rebuild, and an if node (always taken) with the steps left
+// over.  Against a graph per step and 8-step graphs of top-level conditions this takes
+// about 7 us off every step.
+constexpr int LOOP_STEPS = 4;  // even: fused steps are back in coordinate buffer 0
+
+// A conditional node behind `tail` (or, while capturing on cs, behind what is captured); its body.
+int add_conditional(md_system* s, cudaGraph_t g, std::vector<cudaGraphNode_t>& tail, cudaGraphConditionalHandle h,
+                    cudaGraphConditionalNodeType type, cudaGraph_t* body) {
+    alignas(cudaGraphNodeParams) unsigned char cp_raw[sizeof(cudaGraphNodeParams)];
+    std::memset(cp_raw, 0, sizeof(cp_raw));  // all reserved bytes must be zero
+    cudaGraphNodeParams& cp = *reinterpret_cast<cudaGraphNodeParams*>(cp_raw);
+    cp.type = cudaGraphNodeTypeConditional;
+    cp.conditional.handle = h;
+    cp.conditional.type = type;
+    cp.conditional.size = 1;
+    cudaGraphNode_t node;
+    CK(cudaGraphAddNode(&node, g, tail.empty() ? nullptr : tail.data(), nullptr, tail.size(), &cp));
+    tail.assign(1, node);
+    *body = cp.conditional.phGraph_out[0];
+    return MD_OK;
+}
+
+// What `enqueue` puts on cap_stream, appended to graph g behind tail.
+template <typename F>
+int append_captured(md_system* s, cudaGraph_t g, std::vector<cudaGraphNode_t>& tail, F&& enqueue) {
+    cudaStream_t cs = s->cap_stream;
+    CK(cudaStreamBeginCaptureToGraph(cs, g, tail.empty() ? nullptr : tail.data(), nullptr, tail.size(),
+                                     cudaStreamCaptureModeThreadLocal));
+    enqueue(cs);
+    cudaStreamCaptureStatus status;
+    const cudaGraphNode_t* deps = nullptr;
+    size_t ndeps = 0;
+    cudaGraph_t cg = nullptr;
+    CK(cudaStreamGetCaptureInfo(cs, &status, nullptr, &cg, &deps, nullptr, &ndeps));
+    tail.assign(deps, deps + ndeps);
+    CK(cudaStreamEndCapture(cs, &g));
+    return MD_OK;
+}
+
+// One step: step control -> IF(rebuild){binning, gather, copy back, list build on buffer p} -> forces
+// and what follows them.  mid: another step of the chunk follows (fused: kick-kick-drift into the
+// other buffer; else the separate integration); otherwise the step ends its forces, fused ones
+// with the closing kick.
+int append_step(md_system* s, cudaGraph_t g, std::vector<cudaGraphNode_t>& tail, int p, bool mid) {
+    const DevState a = view(s, p);
+    cudaGraphConditionalHandle h;
+    CK(cudaGraphConditionalHandleCreate(&h, g, 0, cudaGraphCondAssignDefault));
+    int rc = append_captured(s, g, tail, [&](cudaStream_t cs) {
+        launch_step_ctrl(s->rebuild == MD_REBUILD_EVERY_K ? 1 : 0, s->rebuild_k, a.rebuild_flag, s->d_ctrl,
+                         s->d_ctrl + 1, a.err, h, cs);
+    });
+    if (rc) return rc;
+    cudaGraph_t body = nullptr;
+    if ((rc = add_conditional(s, g, tail, h, cudaGraphCondTypeIf, &body))) return rc;
+    std::vector<cudaGraphNode_t> none;
+    rc = append_captured(s, body, none, [&](cudaStream_t cs) {
+        enqueue_bin(s, a, cs);
+        cudaMemsetAsync(a.stats, 0, 4 * sizeof(int32_t), cs);
+        enqueue_lists(s, a, cs);
+        launch_count_build(s->d_ctrl + 1, cs);
+    });
+    if (rc) return rc;
+    return append_captured(s, g, tail, [&](cudaStream_t cs) {
+        if (fused(s)) {
+            launch_forces_mixed_fused(a, s->g, s->pt, s->to, s->tile_cap, mid ? FUSE_KICK_KICK_DRIFT : FUSE_KICK,
+                                      step_out(s, 1 - p), s->dt, s->lim2, cs);
+        } else {
+            enqueue_forces(s, 0, cs);
+            if (mid) launch_integrate(a, s->g, s->pt, INT_KICK_KICK_DRIFT, mixed(s), s->dt, s->lim2, cs);
+        }
+    });
+}
+
+// The graph of a chunk: d_ctrl[2] passes of LOOP_STEPS mid steps, `left` more of them, and with
+// `closing` a step that is not followed by another.
+int capture_loop(md_system* s, int left, bool closing, md_system::StepGraph& out) {
+    destroy_graph(out);
+    CK(cudaGraphCreate(&out.graph, 0));
+    cudaGraph_t g = out.graph;
+    // fused steps alternate between the position buffers; the others work in buffer 0
+    const auto buffer = [&](int step) { return fused(s) ? step & 1 : 0; };
+    std::vector<cudaGraphNode_t> tail;
+    cudaGraphConditionalHandle hw;
+    CK(cudaGraphConditionalHandleCreate(&hw, g, 0, cudaGraphCondAssignDefault));
+    int rc = append_captured(s, g, tail, [&](cudaStream_t cs) { launch_loop_ctrl(s->d_ctrl + 2, 0, hw, cs); });
+    if (rc) return rc;
+    cudaGraph_t body = nullptr;
+    if ((rc = add_conditional(s, g, tail, hw, cudaGraphCondTypeWhile, &body))) return rc;
+    std::vector<cudaGraphNode_t> btail;
+    for (int j = 0; j < LOOP_STEPS; ++j)
+        if ((rc = append_step(s, body, btail, buffer(j), true))) return rc;
+    if ((rc = append_captured(s, body, btail, [&](cudaStream_t cs) { launch_loop_ctrl(s->d_ctrl + 2, 1, hw, cs); })))
+        return rc;
+    if (left > 0 || closing) {
+        cudaGraphConditionalHandle hi;
+        CK(cudaGraphConditionalHandleCreate(&hi, g, 1, cudaGraphCondAssignDefault));
+        if ((rc = add_conditional(s, g, tail, hi, cudaGraphCondTypeIf, &body))) return rc;
+        btail.clear();
+        for (int j = 0; j < left; ++j)
+            if ((rc = append_step(s, body, btail, buffer(j), true))) return rc;
+        if (closing && (rc = append_step(s, body, btail, buffer(left), false))) return rc;
+    }
+    CKL();
+    CK(cudaGraphInstantiate(&out.exec, g, 0));
+    return MD_OK;
+}
+
+void destroy_loops(md_system* s) {
+    for (auto& e : s->g_loop) destroy_graph(e.second);
+    s->g_loop.clear();
+}
+
+// Launch n_mid steps that are followed by another and, with `closing`, one that is not.
+int launch_loop(md_system* s, int n_mid, bool closing) {
+    if (!(s->graphs_valid && s->graph_tile_cap == s->tile_cap && s->graph_list_cap == s->list_cap && !s->graph_timing)) {
+        destroy_loops(s);
+        s->graphs_valid = true;
+        s->graph_tile_cap = s->tile_cap;
+        s->graph_list_cap = s->list_cap;
+        s->graph_timing = false;
+    }
+    const int passes = n_mid / LOOP_STEPS, left = n_mid % LOOP_STEPS;
+    // (a program that varies its step counts meets at most 2 * LOOP_STEPS kinds of rest)
+    md_system::StepGraph& gr = s->g_loop[2 * left + (closing ? 1 : 0)];
+    if (!gr.exec) {
+        const int rc = capture_loop(s, left, closing, gr);
+        if (rc) {
+            destroy_loops(s);
+            return rc;
+        }
+    }
+    s->h_ctrl[0] = s->n_steps;
+    s->h_ctrl[1] = 0;
+    s->h_ctrl[2] = passes;
+    CK(cudaMemcpyAsync(s->d_ctrl, s->h_ctrl, 3 * sizeof(long long), cudaMemcpyHostToDevice, s->stream));
+    CK(cudaGraphLaunch(gr.exec, s->stream));
+    const int steps = n_mid + (closing ? 1 : 0);
+    s->launches += 1 + passes + (fused(s) ? 2 : 1 + force_kernels(s)) * steps + (fused(s) ? 0 : n_mid);
+    s->force_evals += steps;
+    return MD_OK;
+}
+
 int ensure_graphs(md_system* s) {
     if (s->graphs_valid && s->graph_tile_cap == s->tile_cap && s->graph_list_cap == s->list_cap &&
         s->graph_timing == s->timing)
@@ -878,15 +1041,17 @@ int run_steps_direct_fused(md_system* s, int len, bool first, bool last) {
 int run_chunk_fused(md_system* s, int len, bool first, bool last) {
     int rc;
     if (!s->use_graphs) return run_steps_direct_fused(s, len, first, last);
-    if ((rc = ensure_graphs(s))) return rc;
+    if (s->timing && (rc = ensure_graphs(s))) return rc;
     const DevState a = view(s, 0);
     launch_copy_state(s->st[2], a, s->stream);
     CKL();
     s->launches += 1;
     s->snapshot_first = first;
-    s->h_ctrl[0] = s->n_steps;
-    s->h_ctrl[1] = 0;
-    CK(cudaMemcpyAsync(s->d_ctrl, s->h_ctrl, 2 * sizeof(long long), cudaMemcpyHostToDevice, s->stream));
+    if (s->timing) {  // (launch_loop writes them otherwise)
+        s->h_ctrl[0] = s->n_steps;
+        s->h_ctrl[1] = 0;
+        CK(cudaMemcpyAsync(s->d_ctrl, s->h_ctrl, 2 * sizeof(long long), cudaMemcpyHostToDevice, s->stream));
+    }
     if (first) {
         // the displacement flag of a later chunk's first step comes from the previous one
         CK(cudaMemsetAsync(a.rebuild_flag, 0, sizeof(int32_t), s->stream));
@@ -896,7 +1061,11 @@ int run_chunk_fused(md_system* s, int len, bool first, bool last) {
     }
     int p = 0;
     const int n_kkd = last ? len - 1 : len;  // steps that end with the next opening kick and drift
-    for (int k = 0; k < len; ++k) {
+    if (!s->timing) {
+        if ((rc = launch_loop(s, n_kkd, last))) return rc;
+        p = n_kkd & 1;
+    }
+    for (int k = 0; s->timing && k < len; ++k) {  // with timing on: graphs that can hold event nodes
         if (s->g_multi.exec && p == 0 && k + MULTI_STEPS <= n_kkd) {
             if (s->timing) {
                 const auto& gm = s->g_multi;
@@ -928,12 +1097,11 @@ int run_chunk_fused(md_system* s, int len, bool first, bool last) {
         if (kkd) p ^= 1;
     }
     if (p && (rc = positions_to_buffer0(s))) return rc;
-    CK(cudaMemcpyAsync(s->h_ctrl, s->d_ctrl, 2 * sizeof(long long), cudaMemcpyDeviceToHost, s->stream));
     if ((rc = sync_flags(s))) return rc;
     const uint32_t e = s->h_flags[0];
     if (e & ERR_TILE_OVERFLOW) return MD_ERR_CELL_OVERFLOW;  // the chunk is redone: nothing of it counts
     if (e & ERR_LIST_OVERFLOW) return MD_ERR_LIST_OVERFLOW;
-    const long long builds = s->h_ctrl[1];
+    const long long builds = builds_in_graphs(s);
     s->launches += builds * 10;  // binning (8), list build, build counter
     if (builds > 0) {
         s->n_builds += builds;
@@ -949,18 +1117,27 @@ int run_chunk_fused(md_system* s, int len, bool first, bool last) {
 int run_chunk(md_system* s, int len, bool first) {
     int rc;
     if (!s->use_graphs) return run_steps_direct(s, len, first);
-    if ((rc = ensure_graphs(s))) return rc;
+    if (s->timing && (rc = ensure_graphs(s))) return rc;
     const DevState& a = s->st[0];
     // snapshot of the chunk's starting state (for a redo after a capacity overflow)
     launch_copy_state(s->st[2], a, s->stream);
     CKL();
     s->launches += 1;
     s->snapshot_first = first;
-    s->h_ctrl[0] = s->n_steps;
-    s->h_ctrl[1] = 0;
-    CK(cudaMemcpyAsync(s->d_ctrl, s->h_ctrl, 2 * sizeof(long long), cudaMemcpyHostToDevice, s->stream));
+    if (s->timing) {  // (launch_loop writes them otherwise)
+        s->h_ctrl[0] = s->n_steps;
+        s->h_ctrl[1] = 0;
+        CK(cudaMemcpyAsync(s->d_ctrl, s->h_ctrl, 2 * sizeof(long long), cudaMemcpyHostToDevice, s->stream));
+    }
     CK(cudaMemsetAsync(a.rebuild_flag, 0, sizeof(int32_t), s->stream));
-    for (int k = 0; k < len; ++k) {
+    if (!s->timing) {
+        launch_integrate(a, s->g, s->pt, first ? INT_KICK_DRIFT : INT_KICK_KICK_DRIFT, mixed(s), s->dt, s->lim2,
+                         s->stream);
+        CKL();
+        s->launches += 1;
+        if ((rc = launch_loop(s, len - 1, true))) return rc;
+    }
+    for (int k = 0; s->timing && k < len; ++k) {  // with timing on: graphs that can hold event nodes
         md_system::StepGraph& gr = (first && k == 0) ? s->g_first : s->g_mid;
         if (s->timing && gr.ev_a && gr.ev_b) {
             auto ev = take_events(s);
@@ -972,12 +1149,11 @@ int run_chunk(md_system* s, int len, bool first) {
         s->launches += 2 + force_kernels(s);  // integrate, step control, forces
         s->force_evals += 1;
     }
-    CK(cudaMemcpyAsync(s->h_ctrl, s->d_ctrl, 2 * sizeof(long long), cudaMemcpyDeviceToHost, s->stream));
     if ((rc = sync_flags(s))) return rc;
     const uint32_t e = s->h_flags[0];
     if (e & ERR_TILE_OVERFLOW) return MD_ERR_CELL_OVERFLOW;  // the chunk is redone: nothing of it counts
     if (e & ERR_LIST_OVERFLOW) return MD_ERR_LIST_OVERFLOW;
-    const long long builds = s->h_ctrl[1];
+    const long long builds = builds_in_graphs(s);
     s->launches += builds * 10;  // binning (8), list build, build counter
     if (builds > 0) {
         s->n_builds += builds;
@@ -1143,10 +1319,13 @@ int md_create(int64_t n, const double box[3], double r_cut, double skin, const m
         return bail(rc);
     if ((rc = dalloc(s, &d0.cell_start, (size_t)g.ncell + 1)) || (rc = dalloc(s, &d0.centre, 3 * (size_t)g.ncell)) ||
         (rc = dalloc(s, &d0.nl_cnt, n)) ||
-        (rc = dalloc(s, &d0.err, 1)) || (rc = dalloc(s, &d0.rebuild_flag, 1)) || (rc = dalloc(s, &d0.stats, 8)) ||
+        (rc = dalloc(s, &d0.err, STATUS_WORDS)) ||
         (rc = dalloc(s, &d0.blk_list, (size_t)g.nblock)) ||
         (p->list_kind == MD_LIST_HALF_ATOMIC_FREE && (rc = dalloc(s, &d0.af_steps, (size_t)g.nblock * 8 * 14 * 2))))
         return bail(rc);
+    d0.rebuild_flag = reinterpret_cast<int32_t*>(d0.err) + 1;
+    d0.stats = reinterpret_cast<int32_t*>(d0.err) + 2;
+    s->d_ctrl = reinterpret_cast<long long*>(d0.err + STATUS_CTRL);
     if (p->precision == MD_MIXED) {
         if ((rc = dalloc(s, &d0.fq, 3 * (size_t)n)) || (rc = dalloc(s, &d0.pe_atom_f, n)) ||
             (rc = dalloc(s, &d0.vir_atom_f, 6 * (size_t)n)) || (rc = dalloc(s, &s->xr_alt, n)) ||
@@ -1178,7 +1357,6 @@ int md_create(int64_t n, const double box[3], double r_cut, double skin, const m
         d1.pe_atom_d = d0.pe_atom_d;
         d1.vir_atom_d = d0.vir_atom_d;
     }
-    if ((rc = dalloc(s, &s->d_ctrl, 2))) return bail(rc);
     if (cudaStreamCreateWithFlags(&s->cap_stream, cudaStreamNonBlocking) != cudaSuccess) return bail(MD_ERR_CUDA);
     if ((rc = alloc_lists(s, lc))) return bail(rc);
     if ((rc = dalloc(s, &s->atom_cell, n)) || (rc = dalloc(s, &s->cell_count, g.ncell)) ||
@@ -1188,11 +1366,9 @@ int md_create(int64_t n, const double box[3], double r_cut, double skin, const m
         return bail(rc);
     s->nparts = 592;
     if ((rc = dalloc(s, &s->partials, 8 * (size_t)s->nparts)) || (rc = dalloc(s, &s->out8, 8))) return bail(rc);
-    if (cudaMallocHost(&s->h_flags, 16 * sizeof(uint32_t)) != cudaSuccess) return bail(MD_ERR_CUDA);
-    if (cudaMallocHost(&s->h_ctrl, 2 * sizeof(long long)) != cudaSuccess) return bail(MD_ERR_CUDA);
-    if (cudaMemsetAsync(d0.err, 0, sizeof(uint32_t), s->stream) != cudaSuccess ||
-        cudaMemsetAsync(s->d_ctrl, 0, 2 * sizeof(long long), s->stream) != cudaSuccess ||
-        cudaMemsetAsync(d0.rebuild_flag, 0, sizeof(int32_t), s->stream) != cudaSuccess ||
+    if (cudaMallocHost(&s->h_flags, STATUS_WORDS * sizeof(uint32_t)) != cudaSuccess) return bail(MD_ERR_CUDA);
+    if (cudaMallocHost(&s->h_ctrl, 3 * sizeof(long long)) != cudaSuccess) return bail(MD_ERR_CUDA);
+    if (cudaMemsetAsync(d0.err, 0, STATUS_WORDS * sizeof(uint32_t), s->stream) != cudaSuccess ||
         cudaStreamSynchronize(s->stream) != cudaSuccess)
         return bail(MD_ERR_CUDA);
     *out = s;
@@ -1323,6 +1499,8 @@ int md_step(md_system* s, int32_t n_steps) {
         launch_integrate(s->st[0], s->g, s->pt, INT_KICK, mixed(s), s->dt, s->lim2, s->stream);
         CKL();
         s->launches += 1;
+    } else if (s->use_graphs) {
+        return MD_OK;  // nothing was launched since the last chunk's status was read
     }
     rc = sync_flags(s);
     if (rc) return rc;
@@ -1650,6 +1828,7 @@ void md_destroy(md_system* s) {
     for (auto& row : s->g_fused)
         for (auto& gr : row) destroy_graph(gr);
     destroy_graph(s->g_multi);
+    destroy_loops(s);
     if (s->cap_stream) cudaStreamDestroy(s->cap_stream);
     if (prev >= 0 && prev != s->device) cudaSetDevice(prev);
     delete s;

@@ -111,6 +111,18 @@ __global__ void k_step_ctrl(int policy, int every_k, int32_t* rebuild_flag, long
     cudaGraphSetConditional(handle, rebuild ? 1u : 0u);
 }
 
+// The while node over a chunk's steps: another pass as long as some are left; done: the passes
+// that just ended.
+__global__ void k_loop_ctrl(long long* passes_left, int done, cudaGraphConditionalHandle handle) {
+    const long long left = *passes_left - done;
+    *passes_left = left;
+    cudaGraphSetConditional(handle, left > 0 ? 1u : 0u);
+}
+
+void launch_loop_ctrl(long long* passes_left, int done, cudaGraphConditionalHandle handle, cudaStream_t st) {
+    k_loop_ctrl<<<1, 1, 0, st>>>(passes_left, done, handle);
+}
+
 __global__ void k_count_build(long long* n_builds) { *n_builds += 1; }
 
 void launch_step_ctrl(int policy, int every_k, int32_t* rebuild_flag, long long* step_counter,

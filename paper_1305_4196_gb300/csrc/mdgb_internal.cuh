@@ -306,6 +306,7 @@ void launch_gather(const DevState& s, const DevState& scratch, const Geometry& g
 void launch_classify_blocks(const DevState& s, const Geometry& g, cudaStream_t st);
 void launch_step_ctrl(int policy, int every_k, int32_t* rebuild_flag, long long* step_counter,
                       long long* n_builds, uint32_t* err, cudaGraphConditionalHandle handle, cudaStream_t st);
+void launch_loop_ctrl(long long* passes_left, int done, cudaGraphConditionalHandle handle, cudaStream_t st);
 void launch_count_build(long long* n_builds, cudaStream_t st);
 void launch_copy_state(const DevState& dst, const DevState& src, cudaStream_t st);
 void launch_build_lists(const DevState& s, const Geometry& g, const TileOffsets& to, double rl2, int list_cap,
