@@ -70,3 +70,24 @@ def test_close_pairs_leave_their_lanes():
     e = np.sqrt(((F - Fr) ** 2).sum(1)) / np.maximum(mag, np.sqrt(np.median(mag) ** 2))
     assert e.max() <= 2e-5
     s.close()
+
+
+@pytest.mark.parametrize("two", [False, True])
+@pytest.mark.parametrize("n,rho", [(1501, 0.8442), (4999, 1.3), (13001, 0.75), (61001, 0.8442)])
+def test_half_list_lanes(n, rho, two):
+    """Four lanes per atom in the colour launches: blocks of more own atoms than lanes (several
+    rounds), counted reaction sums in whole-box tiles, ordinary blocks."""
+    w = W.fcc_vacancies(n, rho, 0.8, seed=n)
+    P = KA if two else O.LJParams.single()
+    sp = W.species_shuffle(w.n, 0.2, 5) if two else w.species
+    s = M.System(w.n, w.box, r_cut=float(P.rc.max()), skin=0.3, eps=P.eps, sigma=P.sig, mass=P.mass,
+                 rcut=P.rc if two else None, list_kind=M.MD_LIST_HALF_COLOUR8)
+    s.set_state(w.pos, w.vel, sp)
+    F = s.forces()
+    Fr = (O.lj_forces(w.pos, w.box, P, sp) if two else O.lj_forces(w.pos, w.box, P))[0]
+    mag = np.sqrt((Fr ** 2).sum(1))
+    e = np.sqrt(((F - Fr) ** 2).sum(1)) / np.maximum(mag, np.sqrt((mag ** 2).mean()))
+    assert e.max() <= 2e-5
+    q = np.rint(F * 2.0 ** 32).astype(np.int64)
+    assert np.array_equal(q.sum(0), np.zeros(3, np.int64))  # every reaction is the exact negative
+    s.close()
