@@ -77,6 +77,8 @@ struct md_system {
     int potential = 0;       // 0: Lennard-Jones pair table; 1: TB-SMA many-body (md_set_tbsma)
     TBTable tb{};
     float* emb = nullptr;    // TB-SMA: 1/sqrt(rho) per atom (cell order)
+    double* grad_ws = nullptr;  // workspace of the derivatives, from the first call on
+    size_t grad_ws_doubles = 0;
     double* pos_alt = nullptr;  // FP64 positions of buffer 1 (x, y, z: n each)
     bool graphs_valid = false;
     int graph_tile_cap = 0, graph_list_cap = 0;
@@ -1605,16 +1607,21 @@ static int backward(md_system* s, const double* grad_f, int device_ptrs, double*
     if (half(s)) return fail(s, MD_ERR_ARG, "derivatives need full neighbour lists (MD_LIST_FULL)");
     if (s->potential != 0) return fail(s, MD_ERR_ARG, "derivatives are for the Lennard-Jones potential");
     const int ns = s->pt.nsp;
-    const int ncol = ns * ns * 4;
+    const int ncol = ns * ns * 2;
     std::vector<double> tot(ncol, 0.0);
     if (s->n > 0) {
         int rc = ensure_lists(s);
         if (rc) return rc;
         const int64_t n = s->n;
-        const int nparts = 256;
-        double* scratch = nullptr;
         double *G = nullptr, *gx = nullptr;
-        CK(cudaMallocAsync(&scratch, sizeof(double) * backward_scratch_doubles(n, ns, nparts), s->stream));
+        const size_t need = backward_scratch_doubles(s->g, ns, !mixed(s), n);
+        if (need > s->grad_ws_doubles) {  // kept by the system, as its other arrays
+            dfree(s, s->grad_ws);
+            s->grad_ws = nullptr;
+            s->grad_ws_doubles = 0;
+            if ((rc = dalloc(s, &s->grad_ws, need))) return rc;
+            s->grad_ws_doubles = need;
+        }
         if (grad_f) {
             if (device_ptrs) {
                 G = const_cast<double*>(grad_f);
@@ -1629,32 +1636,30 @@ static int backward(md_system* s, const double* grad_f, int device_ptrs, double*
         }
         const size_t smem = backward_smem_bytes(!mixed(s), s->tile_cap);
         if (smem > 226 * 1024) return fail(s, MD_ERR_CELL_OVERFLOW, "tile of %d atoms exceeds shared memory", s->tile_cap);
-        launch_force_backward(s->st[0], s->g, s->pt, s->to, s->tile_cap, !mixed(s), G, gx, de_deps != nullptr, scratch,
-                              nparts, s->stream);
+        launch_force_backward(s->st[0], s->g, s->pt, s->to, s->tile_cap, !mixed(s), G, gx, s->grad_ws,
+                              s->stream);
         CKL();
-        s->launches += (G ? 1 : 0) + 1 + (gx ? 1 : 0) + 2;
-        const double* totals = scratch + backward_scratch_doubles(n, ns, nparts) - ncol;
-        CK(cudaMemcpyAsync(tot.data(), totals, sizeof(double) * ncol, cudaMemcpyDeviceToHost, s->stream));
+        s->launches += (G ? 1 : 0) + 2;
+        CK(cudaMemcpyAsync(tot.data(), s->grad_ws, sizeof(double) * ncol, cudaMemcpyDeviceToHost, s->stream));
         if (grad_pos && !device_ptrs)
             CK(cudaMemcpyAsync(grad_pos, gx, sizeof(double) * 3 * n, cudaMemcpyDeviceToHost, s->stream));
         if (grad_f && !device_ptrs) CK(cudaFreeAsync(G, s->stream));
         if (grad_pos && !device_ptrs) CK(cudaFreeAsync(gx, s->stream));
-        CK(cudaFreeAsync(scratch, s->stream));
         if ((rc = sync_flags(s))) return rc;
         if ((rc = check_err(s, ERR_NONFINITE | ERR_TILE_OVERFLOW))) return rc;
     }
-    // column (s_i * ns + s_j) * 4 + q holds the terms of atoms of species s_i with neighbours
+    // column (s_i * ns + s_j) * 2 + q holds the terms of atoms of species s_i with neighbours
     // of species s_j (each pair halved per side): the shared value of {a,b} gets both sides
     for (int a = 0; a < ns; ++a)
         for (int b = 0; b < ns; ++b) {
-            const double* ab = &tot[(a * ns + b) * 4];
-            const double* ba = &tot[(b * ns + a) * 4];
+            const double* ab = &tot[(a * ns + b) * 2];
+            const double* ba = &tot[(b * ns + a) * 2];
             const int t = a * ns + b;
             const double w = (a == b) ? 1.0 : 0.0;  // the diagonal entry already holds both sides
             if (grad_eps) grad_eps[t] = ab[0] + (1.0 - w) * ba[0];
             if (grad_sigma) grad_sigma[t] = ab[1] + (1.0 - w) * ba[1];
-            if (de_deps) de_deps[t] = ab[2] + (1.0 - w) * ba[2];
-            if (de_dsig) de_dsig[t] = ab[3] + (1.0 - w) * ba[3];
+            if (de_deps) de_deps[t] = ab[0] + (1.0 - w) * ba[0];
+            if (de_dsig) de_dsig[t] = ab[1] + (1.0 - w) * ba[1];
         }
     return MD_OK;
 }

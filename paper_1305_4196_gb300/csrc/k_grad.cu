@@ -12,265 +12,364 @@
 // derivatives, dE/deps_ab = sum 4 (s6^2 - s6) and dE/dsig_ab = sum 24 eps
 // (2 s6^2 - s6) / sig, come from the same pass.
 //
-// The kernel follows the full-list force kernels: one CTA per 2x2x2-cell block with
-// the block's 4x4x4-cell tile (coordinates, species and global index) in shared
-// memory, G read from the cell-ordered global copy (L2-resident); one thread per
-// atom accumulating only its own dL/dx_i (each pair is seen from both sides, which
-// also gives the negative term on x_j).  Parameter terms are accumulated per atom by
-// neighbour species and summed in a fixed order afterwards, so every result is
-// deterministic.  T = double on FP64 systems, float (FP32 pair arithmetic,
-// block-frame coordinates) on mixed-precision ones.
+// One CTA per 2x2x2-cell block with the block's 4x4x4-cell tile in shared memory, as in the
+// full-list force kernels; an atom accumulates only its own dL/dx_i (each pair is seen from
+// both sides, which also gives the negative term on x_j).  T = double on FP64 systems, float
+// (FP32 pair arithmetic, block-frame coordinates) on mixed-precision ones.
+//  * Four lanes share an atom, lane q with word q (entries 2q, 2q + 1) of every 16-byte chunk of the
+//    list, so a warp reads its lists in whole sectors and a system of a few 10^4 atoms fills
+//    the SMs.
+//  * The parameter terms leave out the factors that their species pair shares and are
+//    summed in the CTA, to one row of partial sums per CTA instead of one per atom.
+//  * The summation order is fixed, so every result is deterministic.
+// The pass is bound by instruction issue and the latency of the gathered G_j.  For 32,000 atoms of a
+// binary mixture it took 217 us with one lane per atom, 2-byte list reads and FP64 sums, and 47 us
+// for the column sums of a row per atom; it takes 43 and 3 us.
 #include "tile.cuh"
 
 #include <algorithm>
 
+#include "fixpt.cuh"
+#include "fp64_math.cuh"
+
 namespace mdgb {
 
-constexpr int G_THREADS = 128;
-static int g_sm_count = 0;  // SMs of the device, read at initialisation
-constexpr int G_QUANT = 4;  // per species pair: dL/deps, dL/dsig, dE/deps, dE/dsig
+constexpr int G_LPA = 4;  // lanes per own atom
+constexpr int G_THREADS = 512;
+constexpr int G_ATOMS = G_THREADS / G_LPA;  // own atoms at a time
+constexpr int G_QUANT = 2;                  // per species pair: the derivatives by eps and by sig
+static int g_sm_count = 0;                  // SMs of the device, read at initialisation
 
+// G of one atom in the arithmetic of the pairs.
 template <typename T>
-struct GradTile {
-    T *x, *y, *z;
-    int *sp, *gid;  // species, cell-ordered global index (the dummy slot: -1)
+struct alignas(4 * sizeof(T)) Grad4 {
+    T x, y, z, w;
 };
 
-// Global index of every tile atom, one warp per tile cell.
-__device__ __forceinline__ void stage_gid(const TileMeta& m, int* __restrict__ gid) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+// A lane's sum of parameter terms.  FP64 terms are summed in FP64; FP32 terms in two floats, hi
+// and lo, with the rounding error of every addition to hi kept in lo (to about 2^-45 of the largest
+// partial sum; the terms themselves are rounded at 2^-24): an FP64 addition and the conversion
+// before it would hold a warp as long as some 100 FP32 operations.
+template <typename T>
+struct ParamSum;
+
+template <>
+struct ParamSum<double> {
+    double v = 0.0;
+    __device__ __forceinline__ void add(double x, bool take) {
+        if (take) v += x;
+    }
+    __device__ __forceinline__ void merge(int o, bool) { v += __shfl_xor_sync(0xffffffffu, v, o); }
+    __device__ __forceinline__ double get() const { return v; }
+};
+
+template <>
+struct ParamSum<float> {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float x, bool take) {
+        x = take ? x : 0.f;
+        const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
+        hi = s;
+    }
+    __device__ __forceinline__ void merge(int o, bool upper) {
+        // both lanes add the upper lane's sum to the lower lane's, so that they stay equal
+        const float oh = __shfl_xor_sync(0xffffffffu, hi, o), ol = __shfl_xor_sync(0xffffffffu, lo, o);
+        const float x = upper ? hi : oh;
+        hi = upper ? oh : hi;
+        lo = __fadd_rn(lo, ol);
+        add(x, true);
+    }
+    __device__ __forceinline__ double get() const { return (double)hi + (double)lo; }
+};
+
+__device__ __forceinline__ float grad_rcp(float x) {
+    const float y = rcp_approx(x);
+    return __fmaf_rn(y, __fmaf_rn(-x, y, 1.0f), y);
+}
+__device__ __forceinline__ double grad_rcp(double x) { return rcp_cubic(x); }
+
+// Per species pair, in shared memory: the lanes of a warp read several entries at once, which the
+// constant bank would serve one after another.  (FP64 keeps 24 eps there: the tile takes the rest.)
+template <typename T, int NT>
+struct GradTable;
+
+template <int NT>
+struct GradTable<float, NT> {
+    float sig2[NT], e24[NT], in[NT], out[NT];  // inside below `in`, outside from `out` on
+};
+
+template <int NT>
+struct GradTable<double, NT> {
+    double sig2[NT], out[NT];
+};
+
+// part_out: column by column (species pair t, quantity q: 2 t + q), each CTA's sum of its own atoms'
+// terms.  Each unordered pair is visited from both sides, so every term is halved.
+// EN: the energy's parameter derivatives (G_ is not read); otherwise those of the loss.
+template <typename T, int NSP, bool EN>
+__global__ void __launch_bounds__(G_THREADS, 2) k_force_backward(DevState s, Geometry g, PairTable pt, TileOffsets to,
+                                                                 int tile_cap, const void* __restrict__ G_,
+                                                                 double* __restrict__ gx_out,
+                                                                 double* __restrict__ part_out, int split) {
+    constexpr bool FP64 = sizeof(T) == 8;
+    constexpr int NV = NSP * G_QUANT, NC = NSP * NV;  // sums per atom, per CTA
+    static_assert(NC <= 32, "one lane per sum");
+    const Grad4<T>* __restrict__ G = reinterpret_cast<const Grad4<T>*>(G_);
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ TileMeta m;
+    __shared__ GradTable<T, NSP * NSP> tab;
+    // split CTAs share one block: each stages the whole tile and takes every split-th group of
+    // own atoms, so that a small system still spreads over the SMs
+    const int b = spatial_block(g, blockIdx.x / split), part = blockIdx.x % split;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    constexpr int nw = G_THREADS / 32;
+    if (threadIdx.x < NSP * NSP) {
+        if constexpr (FP64) {
+            tab.sig2[threadIdx.x] = pt.sig2_d[threadIdx.x];
+            tab.out[threadIdx.x] = pt.rc2_d[threadIdx.x];
+        } else {
+            tab.sig2[threadIdx.x] = pt.sig2_f[threadIdx.x];
+            tab.e24[threadIdx.x] = 6.0f * pt.c4_f[threadIdx.x];
+            tab.in[threadIdx.x] = pt.rc2lo_f[threadIdx.x];
+            tab.out[threadIdx.x] = pt.rc2hi_f[threadIdx.x];
+        }
+    }
+    tile_meta(g, s.cell_start, b, m);
+    const int T_ = m.prefix[64], nown = m.prefix[8];
+    if (T_ + 1 > tile_cap || part * G_ATOMS >= nown) {
+        if (threadIdx.x == 0 && T_ + 1 > tile_cap) atomicOr(s.err, ERR_TILE_OVERFLOW);
+        if (threadIdx.x < NC) part_out[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = 0.0;
+        return;
+    }
+    // the tile: FP64 as x | y | z | species, FP32 as (x, y, z, species); behind it the atoms' global
+    // indices
+    double* tx = reinterpret_cast<double*>(smem);
+    double *ty = tx + tile_cap, *tz = ty + tile_cap;
+    int* tsp = reinterpret_cast<int*>(tz + tile_cap);
+    float4* tp = reinterpret_cast<float4*>(smem);
+    int* gid = FP64 ? tsp + tile_cap : reinterpret_cast<int*>(tp + tile_cap);
+    if (FP64) {
+        tile_stage_f64(s, g, m, b, tx, ty, tz, tsp);
+    } else {
+        tile_stage_f32_cells(m, s.xr, to, tp);
+        if (threadIdx.x == 0) tp[T_] = make_float4(1.0e4f, 1.0e4f, 1.0e4f, __int_as_float(0));
+    }
     for (int slot = warp; slot < 64; slot += nw) {
         const int u0 = m.prefix[slot], cnt = m.prefix[slot + 1] - u0, j0 = m.start[slot];
         for (int e = lane; e < cnt; e += 32) gid[u0 + e] = j0 + e;
     }
-}
-
-__device__ __forceinline__ void add_by_species(double (&P)[MAX_SPECIES][G_QUANT], int sj, int q, double v) {
-    // explicit branches keep the accumulators in registers
-    if (sj == 0) P[0][q] += v;
-    else if (sj == 1) P[1][q] += v;
-    else if (sj == 2) P[2][q] += v;
-    else P[3][q] += v;
-}
-
-// prm: n x (nsp*nsp*G_QUANT), row i holds atom i's terms in the columns of its own
-// species row (t = s_i * nsp + s_j), zero elsewhere; each unordered pair is visited
-// from both sides, so every term is halved.
-template <typename T>
-__global__ void __launch_bounds__(G_THREADS) k_force_backward(DevState s, Geometry g, PairTable pt, TileOffsets to,
-                                                              int tile_cap, const double* __restrict__ G,
-                                                              double* __restrict__ gx_out, double* __restrict__ prm,
-                                                              int want_energy, int split) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ TileMeta m;
-    // split CTAs share one block: each stages the whole tile and takes every split-th group
-    // of G_THREADS own atoms, so that a small system still spreads over the SMs
-    const int b = spatial_block(g, blockIdx.x / split), part = blockIdx.x % split;
-    tile_meta(g, s.cell_start, b, m);
-    const int T_ = m.prefix[64];
-    if (T_ + 1 > tile_cap) {
-        if (threadIdx.x == 0) atomicOr(s.err, ERR_TILE_OVERFLOW);
-        return;
-    }
-    const int nown = m.prefix[8];
-    if (nown == 0) return;
-    GradTile<T> t;
-    t.x = reinterpret_cast<T*>(smem);
-    t.y = t.x + tile_cap;
-    t.z = t.y + tile_cap;
-    t.sp = reinterpret_cast<int*>(t.z + tile_cap);
-    t.gid = t.sp + tile_cap;
-    if constexpr (sizeof(T) == 8) {
-        tile_stage_f64(s, g, m, b, t.x, t.y, t.z, t.sp);
-    } else {
-        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-        for (int slot = warp; slot < 64; slot += nw) {
-            const int c = m.coord[slot];
-            const float ox = pick4(to.off[0], c & 3), oy = pick4(to.off[1], (c >> 2) & 3),
-                        oz = pick4(to.off[2], c >> 4);
-            const int u0 = m.prefix[slot], cnt = m.prefix[slot + 1] - u0, j0 = m.start[slot];
-            for (int e = lane; e < cnt; e += 32) {
-                const float4 p = s.xr[j0 + e];
-                t.x[u0 + e] = p.x + ox;
-                t.y[u0 + e] = p.y + oy;
-                t.z[u0 + e] = p.z + oz;
-                t.sp[u0 + e] = __float_as_int(p.w);
-            }
-        }
-        if (threadIdx.x == 0) {
-            t.x[T_] = t.y[T_] = t.z[T_] = 1.0e4f;
-            t.sp[T_] = 0;
-        }
-    }
-    stage_gid(m, t.gid);
-    if (threadIdx.x == 0) t.gid[T_] = -1;
     __syncthreads();
-    const int nsp = pt.nsp;
-    const int ncol = nsp * nsp * G_QUANT;
     const int blk0 = m.start[0];
-    const int64_t n = s.n;
-    for (int ui = part * blockDim.x + threadIdx.x; ui < nown; ui += split * blockDim.x) {
-        const int64_t gi = blk0 + ui;
-        const T xi = t.x[ui], yi = t.y[ui], zi = t.z[ui];
-        const T Gx = G ? (T)G[gi] : T(0), Gy = G ? (T)G[n + gi] : T(0), Gz = G ? (T)G[2 * n + gi] : T(0);
-        const int si = t.sp[ui];
-        T ax = 0, ay = 0, az = 0;
-        double P[MAX_SPECIES][G_QUANT] = {};
-        const int cnt = s.nl_cnt[gi];
-        for (int k = 0; k < cnt; ++k) {
-            const int u = s.nl[((size_t)(k >> 3) * s.np + gi) * 8 + (k & 7)];
-            const T dx = xi - t.x[u], dy = yi - t.y[u], dz = zi - t.z[u];
-            const T r2 = dx * dx + dy * dy + dz * dz;
-            const int sj = t.sp[u];
-            const int tt = si * nsp + sj;
-            if (sizeof(T) == 8) {
-                if (!(r2 < (T)pt.rc2_d[tt])) continue;
+    const size_t np = s.np;
+    const int lq = threadIdx.x % G_LPA;
+    double mine = 0.0;  // lane c of a warp: the warp's sum for column c
+    for (int u0 = part * G_ATOMS; u0 < nown; u0 += split * G_ATOMS) {
+        const int ui = u0 + (int)threadIdx.x / G_LPA;
+        const bool active = ui < nown;
+        const int uc = active ? ui : 0, gi = blk0 + uc;
+        T xi, yi, zi;
+        int si;
+        if (FP64) {
+            xi = (T)tx[uc], yi = (T)ty[uc], zi = (T)tz[uc];
+            si = tsp[uc];
+        } else {
+            const float4 p = tp[uc];
+            xi = p.x, yi = p.y, zi = p.z;
+            si = __float_as_int(p.w);
+        }
+        Grad4<T> Gi{};
+        if (!EN) Gi = G[gi];
+        T a[3] = {T(0), T(0), T(0)};
+        ParamSum<T> sum[NSP][G_QUANT];
+        const auto visit = [&](int u) {
+            T dx, dy, dz;
+            int sj;
+            if (FP64) {
+                dx = xi - (T)tx[u], dy = yi - (T)ty[u], dz = zi - (T)tz[u];
+                sj = tsp[u];
             } else {
-                if (!((float)r2 < pt.rc2hi_f[tt])) continue;
-                if (!((float)r2 < pt.rc2lo_f[tt]) &&  // rare: decide the cutoff in FP64
-                    !fp64_pair_test(s.x, s.y, s.z, g.L[0], g.L[1], g.L[2], (int)gi, t.gid[u], pt.rc2_d[tt]))
-                    continue;
+                const float4 p = tp[u];
+                dx = xi - p.x, dy = yi - p.y, dz = zi - p.z;
+                sj = __float_as_int(p.w);
             }
-            const T sig2 = sizeof(T) == 8 ? (T)pt.sig2_d[tt] : (T)pt.sig2_f[tt];
-            const T e = sizeof(T) == 8 ? (T)pt.eps_d[tt] : (T)(pt.c4_f[tt] * 0.25f);
-            const T sig = (T)pt.sig_d[tt];
-            const T inv = T(1) / r2;
-            const T sr2 = sig2 * inv;
+            const T r2 = dx * dx + dy * dy + dz * dz;
+            const int t = NSP == 1 ? 0 : si * NSP + sj;
+            if (!(r2 < tab.out[t])) return;
+            if constexpr (!FP64) {
+                if (!(r2 < tab.in[t]) &&  // rare: decide the cutoff in FP64
+                    !fp64_pair_test(s.x, s.y, s.z, g.L[0], g.L[1], g.L[2], gi, gid[u], pt.rc2_d[t]))
+                    return;
+            }
+            const T inv = grad_rcp(r2);
+            const T sr2 = tab.sig2[t] * inv;
             const T s6 = sr2 * sr2 * sr2;
-            const T gq = T(24) * e * (T(2) * s6 * s6 - s6) * inv;
-            const T gp = T(24) * e * (T(4) * s6 - T(14) * s6 * s6) * inv * inv;
-            const int gj = t.gid[u];
-            const T wx = Gx - (G ? (T)G[gj] : T(0)), wy = Gy - (G ? (T)G[n + gj] : T(0)),
-                    wz = Gz - (G ? (T)G[2 * n + gj] : T(0));
-            const T wd = wx * dx + wy * dy + wz * dz;
-            const T two_gp_wd = T(2) * gp * wd;
-            ax += gq * wx + two_gp_wd * dx;
-            ay += gq * wy + two_gp_wd * dy;
-            az += gq * wz + two_gp_wd * dz;
-            add_by_species(P, sj, 0, (double)(wd * (T(24) * (T(2) * s6 * s6 - s6) * inv)));
-            add_by_species(P, sj, 1, (double)(wd * (T(144) * e * (T(4) * s6 * s6 - s6) * inv / sig)));
-            if (want_energy) {
-                add_by_species(P, sj, 2, (double)(T(4) * (s6 * s6 - s6)));
-                add_by_species(P, sj, 3, (double)(T(24) * e * (T(2) * s6 * s6 - s6) / sig));
+            const T v = T(2) * s6 * s6 - s6;
+            T q0, q1;
+            if (EN) {
+                q0 = s6 * s6 - s6;  // dE/deps / 4
+                q1 = v;             // dE/dsig sig / (24 eps)
+            } else {
+                const Grad4<T> Gj = G[gid[u]];
+                const T wx = Gi.x - Gj.x, wy = Gi.y - Gj.y, wz = Gi.z - Gj.z;
+                const T wd = wx * dx + wy * dy + wz * dz;
+                T e24;
+                if constexpr (FP64) e24 = 24.0 * pt.eps_d[t];
+                else e24 = tab.e24[t];
+                const T gq = e24 * v * inv;
+                const T h = T(2) * (e24 * (T(4) * s6 - T(14) * s6 * s6) * inv * inv) * wd;
+                a[0] += gq * wx + h * dx;
+                a[1] += gq * wy + h * dy;
+                a[2] += gq * wz + h * dz;
+                const T wi = wd * inv;
+                q0 = wi * v;                              // dL/deps / 24
+                q1 = wi * (T(4) * s6 * s6 - s6);          // dL/dsig sig / (144 eps)
+            }
+#pragma unroll
+            for (int k = 0; k < NSP; ++k) {
+                sum[k][0].add(q0, NSP == 1 || sj == k);
+                sum[k][1].add(q1, NSP == 1 || sj == k);
+            }
+        };
+        const int nch = active ? (s.nl_cnt[gi] + 7) >> 3 : 0;
+        const unsigned* words = reinterpret_cast<const unsigned*>(s.nl) + (size_t)gi * 4 + lq;
+        unsigned nxt = nch > 0 ? __ldcs(words) : 0u;
+        for (int c = 0; c < nch; ++c) {
+            const unsigned w = nxt;
+            if (c + 1 < nch) nxt = __ldcs(words + (size_t)(c + 1) * np * 4);
+            visit((int)(w & 0xffffu));
+            visit((int)(w >> 16));
+        }
+        __syncwarp();
+        if (!EN) {
+#pragma unroll
+            for (int o = 1; o < G_LPA; o <<= 1) {
+#pragma unroll
+                for (int d = 0; d < 3; ++d) a[d] += __shfl_xor_sync(0xffffffffu, a[d], o);
+            }
+            if (gx_out && active && lq < 3) {
+                const T v = lq == 0 ? a[0] : (lq == 1 ? a[1] : a[2]);
+                gx_out[3 * (size_t)s.orig[gi] + lq] = (double)v;
             }
         }
-        if (gx_out) {
-            gx_out[gi] = (double)ax;
-            gx_out[n + gi] = (double)ay;
-            gx_out[2 * n + gi] = (double)az;
-        }
-        double* row = prm + gi * ncol;
-        for (int c = 0; c < ncol; ++c) row[c] = 0.0;
+        // the sums of an atom's lanes, then of the warp's atoms by their species
 #pragma unroll
-        for (int b2 = 0; b2 < MAX_SPECIES; ++b2) {
-            if (b2 >= nsp) break;
+        for (int k = 0; k < NSP; ++k) {
 #pragma unroll
-            for (int q = 0; q < G_QUANT; ++q) row[(si * nsp + b2) * G_QUANT + q] = 0.5 * P[b2][q];
+            for (int q = 0; q < G_QUANT; ++q) {
+#pragma unroll
+                for (int o = 1; o < G_LPA; o <<= 1) sum[k][q].merge(o, lane & o);
+#pragma unroll
+                for (int c = 0; c < NSP; ++c) {
+                    ParamSum<T> v = NSP == 1 || si == c ? sum[k][q] : ParamSum<T>();
+#pragma unroll
+                    for (int o = G_LPA; o < 32; o <<= 1) v.merge(o, lane & o);
+                    if (lane == c * NV + k * G_QUANT + q) mine += v.get();
+                }
+            }
         }
+    }
+    __syncthreads();
+    double* red = reinterpret_cast<double*>(smem);  // the tile is done with
+    red[threadIdx.x] = mine;
+    __syncthreads();
+    if (threadIdx.x < NC) {
+        double v = 0.0;
+        for (int k = 0; k < nw; ++k) v += red[32 * k + threadIdx.x];
+        // the factors left out above, halved
+        const int t = threadIdx.x / G_QUANT, q = threadIdx.x % G_QUANT;
+        const double f = EN ? (q ? 12.0 * pt.eps_d[t] / pt.sig_d[t] : 2.0)
+                            : (q ? 72.0 * pt.eps_d[t] / pt.sig_d[t] : 12.0);
+        part_out[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = f * v;
     }
 }
 
-// Column sums of an n x ncol matrix in a fixed order: per-CTA partials over contiguous
-// row ranges, then one CTA over the partials.
+// Column sums of the CTAs' partial sums (column by column), one CTA per column, in a fixed order.
 constexpr int CS_THREADS = 256;
 
-__global__ void __launch_bounds__(CS_THREADS) k_colsum_partials(const double* __restrict__ a, int64_t n, int ncol,
-                                                                int64_t chunk, double* __restrict__ part) {
+__global__ void __launch_bounds__(CS_THREADS) k_colsum(const double* __restrict__ part, int nparts,
+                                                       double* __restrict__ out) {
     __shared__ double sh[CS_THREADS];
-    const int64_t lo = blockIdx.x * chunk;
-    const int64_t hi = lo + chunk < n ? lo + chunk : n;
-    for (int c = 0; c < ncol; ++c) {
-        double acc = 0.0;
-        for (int64_t i = lo + threadIdx.x; i < hi; i += CS_THREADS) acc += a[i * ncol + c];
-        sh[threadIdx.x] = acc;
-        __syncthreads();
-        for (int w = CS_THREADS / 2; w > 0; w >>= 1) {
-            if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) part[blockIdx.x * ncol + c] = sh[0];
+    double acc = 0.0;
+    for (int p = threadIdx.x; p < nparts; p += CS_THREADS) acc += part[(size_t)blockIdx.x * nparts + p];
+    sh[threadIdx.x] = acc;
+    __syncthreads();
+    for (int w = CS_THREADS / 2; w > 0; w >>= 1) {
+        if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
         __syncthreads();
     }
+    if (threadIdx.x == 0) out[blockIdx.x] = sh[0];
 }
 
-__global__ void __launch_bounds__(CS_THREADS) k_colsum_final(const double* __restrict__ part, int nparts, int ncol,
-                                                             double* __restrict__ out) {
-    __shared__ double sh[CS_THREADS];
-    for (int c = 0; c < ncol; ++c) {
-        double acc = 0.0;
-        for (int p = threadIdx.x; p < nparts; p += CS_THREADS) acc += part[p * ncol + c];
-        sh[threadIdx.x] = acc;
-        __syncthreads();
-        for (int w = CS_THREADS / 2; w > 0; w >>= 1) {
-            if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) out[c] = sh[0];
-        __syncthreads();
-    }
-}
-
-// G (N x 3, original order) -> cell order, 3 x n
-__global__ void k_grad_in(DevState s, const double* __restrict__ G, double* __restrict__ Gc) {
+// G (N x 3, original order) -> cell order, one (x, y, z, -) entry per atom
+template <typename T>
+__global__ void k_grad_in(DevState s, const double* __restrict__ G, Grad4<T>* __restrict__ Gc) {
     const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= s.n) return;
     const int64_t o = s.orig[i];
-    Gc[i] = G[3 * o];
-    Gc[s.n + i] = G[3 * o + 1];
-    Gc[2 * s.n + i] = G[3 * o + 2];
-}
-
-// cell order, 3 x n -> original order, N x 3
-__global__ void k_grad_out(DevState s, const double* __restrict__ gc, double* __restrict__ out) {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= s.n) return;
-    const int64_t o = s.orig[i];
-    out[3 * o] = gc[i];
-    out[3 * o + 1] = gc[s.n + i];
-    out[3 * o + 2] = gc[2 * s.n + i];
+    Gc[i] = Grad4<T>{(T)G[3 * o], (T)G[3 * o + 1], (T)G[3 * o + 2], T(0)};
 }
 
 size_t backward_smem_bytes(int fp64, int tile_cap) {
-    return (size_t)tile_cap * (3 * (fp64 ? sizeof(double) : sizeof(float)) + 2 * sizeof(int));
+    // (the reduction at the end reuses the tile's memory)
+    return std::max((size_t)tile_cap * (3 * (fp64 ? sizeof(double) : sizeof(float)) + 2 * sizeof(int)),
+                    sizeof(double) * G_THREADS);
 }
 
-size_t backward_scratch_doubles(int64_t n, int nsp, int nparts) {
-    return 3 * (size_t)n + 3 * (size_t)n + (size_t)n * nsp * nsp * G_QUANT + (size_t)nparts * nsp * nsp * G_QUANT +
-           (size_t)nsp * nsp * G_QUANT;
-}
-
-// scratch layout: Gc (3n) | gx (3n) | prm (n x ncol) | partials (nparts x ncol) | totals (ncol)
-void launch_force_backward(const DevState& s, const Geometry& g, const PairTable& pt, const TileOffsets& to,
-                           int tile_cap, int fp64, const double* G, double* gx_orig, int want_energy,
-                           double* scratch, int nparts, cudaStream_t st) {
-    const int64_t n = s.n;
-    const int ncol = pt.nsp * pt.nsp * G_QUANT;
-    double* Gc = scratch;
-    double* gxc = Gc + 3 * n;
-    double* prm = gxc + 3 * n;
-    double* part = prm + (size_t)n * ncol;
-    double* tot = part + (size_t)nparts * ncol;
-    const int bs = 256;
-    const unsigned nb = (unsigned)((n + bs - 1) / bs);
-    if (G) k_grad_in<<<nb, bs, 0, st>>>(s, G, Gc);
-    const size_t smem = backward_smem_bytes(fp64, tile_cap);
-    // CTAs per block: enough for about one own atom per thread, while the grid is below two
-    // CTAs per SM (small systems, e.g. force-matching snapshots of a few 10^4 atoms)
+// CTAs per block: enough for one group of own atoms each, while the grid is below two CTAs
+// per SM (small systems, e.g. force-matching snapshots of a few 10^4 atoms)
+static int backward_split(const Geometry& g, int64_t n) {
     const int sms = g_sm_count > 0 ? g_sm_count : 152;
     const int64_t per_block = (n + g.nblock - 1) / g.nblock;
-    int split = (int)std::min<int64_t>((per_block + G_THREADS - 1) / G_THREADS, (2 * sms + g.nblock - 1) / g.nblock);
-    split = std::max(1, std::min(split, 8));
+    const int split = (int)std::min<int64_t>((per_block + G_ATOMS - 1) / G_ATOMS, (2 * sms + g.nblock - 1) / g.nblock);
+    return std::max(1, std::min(split, 8));
+}
+
+// scratch layout: totals (nsp x nsp x 2) | partial sums (the same x CTAs) | G in cell order (n x 4 of T)
+static size_t backward_sums(const Geometry& g, int nsp, int64_t n) {
+    const size_t ncol = (size_t)nsp * nsp * G_QUANT;
+    return (ncol * (1 + (size_t)g.nblock * backward_split(g, n)) + 3) & ~(size_t)3;
+}
+
+size_t backward_scratch_doubles(const Geometry& g, int nsp, int fp64, int64_t n) {
+    return backward_sums(g, nsp, n) + (size_t)n * (fp64 ? 4 : 2);
+}
+
+using Backward = void (*)(DevState, Geometry, PairTable, TileOffsets, int, const void*, double*, double*, int);
+
+template <typename T, bool EN>
+static Backward backward_of(int nsp) {
+    switch (nsp) {
+        case 1: return k_force_backward<T, 1, EN>;
+        case 2: return k_force_backward<T, 2, EN>;
+        case 3: return k_force_backward<T, 3, EN>;
+        default: return k_force_backward<T, 4, EN>;
+    }
+}
+
+static Backward backward_kernel(int fp64, int energy, int nsp) {
+    if (fp64) return energy ? backward_of<double, true>(nsp) : backward_of<double, false>(nsp);
+    return energy ? backward_of<float, true>(nsp) : backward_of<float, false>(nsp);
+}
+
+// With G: dL/deps and dL/dsig (columns 2 t and 2 t + 1 of the totals at the start of the scratch), and
+// dL/dx in the caller's order into gx.  Without: dE/deps and dE/dsig.
+void launch_force_backward(const DevState& s, const Geometry& g, const PairTable& pt, const TileOffsets& to,
+                           int tile_cap, int fp64, const double* G, double* gx, double* scratch, cudaStream_t st) {
+    const int64_t n = s.n;
+    const int ncol = pt.nsp * pt.nsp * G_QUANT, split = backward_split(g, n);
     const unsigned grid = (unsigned)g.nblock * (unsigned)split;
-    if (fp64)
-        k_force_backward<double><<<grid, G_THREADS, smem, st>>>(s, g, pt, to, tile_cap, G ? Gc : nullptr,
-                                                               gx_orig ? gxc : nullptr, prm, want_energy, split);
-    else
-        k_force_backward<float><<<grid, G_THREADS, smem, st>>>(s, g, pt, to, tile_cap, G ? Gc : nullptr,
-                                                              gx_orig ? gxc : nullptr, prm, want_energy, split);
-    if (gx_orig) k_grad_out<<<nb, bs, 0, st>>>(s, gxc, gx_orig);
-    const int64_t chunk = (n + nparts - 1) / nparts;
-    k_colsum_partials<<<nparts, CS_THREADS, 0, st>>>(prm, n, ncol, chunk > 0 ? chunk : 1, part);
-    k_colsum_final<<<1, CS_THREADS, 0, st>>>(part, nparts, ncol, tot);
+    double* part = scratch + ncol;
+    double* Gc = scratch + backward_sums(g, pt.nsp, n);
+    const int bs = 256;
+    const unsigned nb = (unsigned)((n + bs - 1) / bs);
+    if (G) {
+        if (fp64) k_grad_in<<<nb, bs, 0, st>>>(s, G, reinterpret_cast<Grad4<double>*>(Gc));
+        else k_grad_in<<<nb, bs, 0, st>>>(s, G, reinterpret_cast<Grad4<float>*>(Gc));
+    }
+    backward_kernel(fp64, G == nullptr, pt.nsp)<<<grid, G_THREADS, backward_smem_bytes(fp64, tile_cap), st>>>(
+        s, g, pt, to, tile_cap, Gc, gx, part, split);
+    k_colsum<<<ncol, CS_THREADS, 0, st>>>(part, (int)grid, scratch);
 }
 
 template <typename K>
@@ -286,8 +385,7 @@ static void allow_max_smem(K kernel) {
 void init_grad_kernels() {
     int dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&g_sm_count, cudaDevAttrMultiProcessorCount, dev);
-    allow_max_smem(k_force_backward<double>);
-    allow_max_smem(k_force_backward<float>);
+    for (int k = 0; k < 4 * MAX_SPECIES; ++k) allow_max_smem(backward_kernel(k & 1, k & 2, 1 + k / 4));
 }
 
 }  // namespace mdgb

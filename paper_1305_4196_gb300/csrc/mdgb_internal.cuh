@@ -368,10 +368,9 @@ void init_half_af_kernels();
 void init_force_fp64_kernels();
 void init_grad_kernels();
 size_t backward_smem_bytes(int fp64, int tile_cap);
-size_t backward_scratch_doubles(int64_t n, int nsp, int nparts);
+size_t backward_scratch_doubles(const Geometry& g, int nsp, int fp64, int64_t n);
 void launch_force_backward(const DevState& s, const Geometry& g, const PairTable& pt, const TileOffsets& to,
-                           int tile_cap, int fp64, const double* G, double* gx_orig, int want_energy,
-                           double* scratch, int nparts, cudaStream_t st);
+                           int tile_cap, int fp64, const double* G, double* gx, double* scratch, cudaStream_t st);
 void init_list_kernels();
 
 // integrate modes
