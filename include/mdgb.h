@@ -182,7 +182,7 @@ int md_forces(md_system *s, double *f_out, int device_ptrs);
  * performs the velocity-Verlet updates around it (closing kick, and unless it
  * is the last step of the call, the next opening kick and drift): the same
  * operations as separate kernels, with the positions (FP32 and FP64)
- * double-buffered.  After md_set_tbsma the integration runs as separate kernels.
+ * double-buffered; after md_set_tbsma it does so in the second of the two force passes.
  * With the environment variable MDGB_NO_GRAPHS=1 set when the system is
  * created, the same kernels are launched from the host instead and the rebuild
  * flag is read after every step (slower; for profilers that do not follow

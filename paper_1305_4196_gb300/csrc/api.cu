@@ -174,7 +174,7 @@ void enqueue_lists(const md_system* s, const DevState& a, cudaStream_t st) {
     else launch_build_lists(a, s->g, s->to, s->rl2, s->list_cap, s->tile_cap, half(s), st);
 }
 // md_step runs the full-list mixed path with velocity Verlet fused into the force kernel
-bool fused(const md_system* s) { return mixed(s) && !half(s) && !s->no_fuse && s->potential == 0; }
+bool fused(const md_system* s) { return mixed(s) && !half(s) && !s->no_fuse; }
 // kernels per force evaluation: 8 colour launches (half lists), two passes (TB-SMA), else one
 int force_kernels(const md_system* s) { return half(s) ? 8 : (s->potential == 1 ? 2 : 1); }
 
@@ -194,6 +194,13 @@ DevState view(const md_system* s, int p) {
 StepOut step_out(const md_system* s, int p) {
     const DevState v = view(s, p);
     return StepOut{v.xr, v.x, v.y, v.z};
+}
+// Forces of the state a with what follows them in a fused step (mode).
+void enqueue_fused(const md_system* s, const DevState& a, int mode, const StepOut& out, cudaStream_t st) {
+    if (s->potential == 1)
+        launch_tbsma(a, s->g, s->pt, s->tb, s->to, s->tile_cap, s->emb, 0, mode, out, s->dt, s->lim2, st);
+    else
+        launch_forces_mixed_fused(a, s->g, s->pt, s->to, s->tile_cap, mode, out, s->dt, s->lim2, st);
 }
 // Positions of buffer 1 back into buffer 0 (a chunk of fused steps that ended in buffer 1).
 int positions_to_buffer0(md_system* s) {
@@ -490,7 +497,8 @@ int do_build(md_system* s, int p = 0) {
 
 void enqueue_forces(md_system* s, int with_energy, cudaStream_t st) {
     const DevState& a = s->st[0];
-    if (s->potential == 1) launch_tbsma(a, s->g, s->tb, s->to, s->tile_cap, s->emb, with_energy, st);
+    if (s->potential == 1) launch_tbsma(a, s->g, s->pt, s->tb, s->to, s->tile_cap, s->emb, with_energy, FUSE_FORCE_ONLY, StepOut{},
+                                        s->dt, s->lim2, st);
     else if (mixed(s) && af(s)) launch_forces_half_af(a, s->g, s->pt, s->to, s->tile_cap, fs2_max_of(s->pt), with_energy, st);
     else if (mixed(s)) launch_forces_mixed(a, s->g, s->pt, s->to, s->tile_cap, half(s), with_energy, st);
     else launch_forces_fp64(a, s->g, s->pt, s->tile_cap, half(s), with_energy, st);
@@ -507,7 +515,8 @@ int do_forces(md_system* s, int with_energy) {
     if (s->potential == 1) {
         if (tbsma_smem_bytes(s->tile_cap) > 226 * 1024)
             return fail(s, MD_ERR_CELL_OVERFLOW, "tile of %d atoms exceeds shared memory", s->tile_cap);
-        launch_tbsma(a, s->g, s->tb, s->to, s->tile_cap, s->emb, with_energy, s->stream);
+        launch_tbsma(a, s->g, s->pt, s->tb, s->to, s->tile_cap, s->emb, with_energy, FUSE_FORCE_ONLY, StepOut{},
+                     s->dt, s->lim2, s->stream);
     } else if (mixed(s)) {
         if (fsmem(s, with_energy, s->tile_cap) > 226 * 1024)
             return fail(s, MD_ERR_CELL_OVERFLOW, "tile of %d atoms exceeds shared memory", s->tile_cap);
@@ -708,12 +717,12 @@ int capture_fused(md_system* s, bool kkd, int p, md_system::StepGraph& out) {
         CK(cudaEventRecordWithFlags(ev.first, cs, cudaEventRecordExternal));
         CK(cudaStreamGetCaptureInfo(cs, &status, nullptr, &cg, &deps, nullptr, &ndeps));
         out.ev_a = ndeps ? deps[0] : nullptr;
-        launch_forces_mixed_fused(a, s->g, s->pt, s->to, s->tile_cap, mode, step_out(s, 1 - p), s->dt, s->lim2, cs);
+        enqueue_fused(s, a, mode, step_out(s, 1 - p), cs);
         CK(cudaEventRecordWithFlags(ev.second, cs, cudaEventRecordExternal));
         CK(cudaStreamGetCaptureInfo(cs, &status, nullptr, &cg, &deps, nullptr, &ndeps));
         out.ev_b = ndeps ? deps[0] : nullptr;
     } else {
-        launch_forces_mixed_fused(a, s->g, s->pt, s->to, s->tile_cap, mode, step_out(s, 1 - p), s->dt, s->lim2, cs);
+        enqueue_fused(s, a, mode, step_out(s, 1 - p), cs);
     }
     CK(cudaStreamEndCapture(cs, &g));
     CK(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
@@ -774,8 +783,7 @@ int capture_fused_multi(md_system* s, md_system::StepGraph& out) {
             CK(cudaStreamGetCaptureInfo(cs, &status, nullptr, &cg, &deps, nullptr, &ndeps));
             out.ev_multi_a.push_back(ndeps ? deps[0] : nullptr);
         }
-        launch_forces_mixed_fused(a, s->g, s->pt, s->to, s->tile_cap, FUSE_KICK_KICK_DRIFT, step_out(s, 1 - p), s->dt,
-                                  s->lim2, cs);
+        enqueue_fused(s, a, FUSE_KICK_KICK_DRIFT, step_out(s, 1 - p), cs);
         if (timed) {
             auto ev = take_events(s);
             s->ev_free.push_back(ev);
@@ -867,8 +875,7 @@ int append_step(md_system* s, cudaGraph_t g, std::vector<cudaGraphNode_t>& tail,
     if (rc) return rc;
     return append_captured(s, g, tail, [&](cudaStream_t cs) {
         if (fused(s)) {
-            launch_forces_mixed_fused(a, s->g, s->pt, s->to, s->tile_cap, mid ? FUSE_KICK_KICK_DRIFT : FUSE_KICK,
-                                      step_out(s, 1 - p), s->dt, s->lim2, cs);
+            enqueue_fused(s, a, mid ? FUSE_KICK_KICK_DRIFT : FUSE_KICK, step_out(s, 1 - p), cs);
         } else {
             enqueue_forces(s, 0, cs);
             if (mid) launch_integrate(a, s->g, s->pt, INT_KICK_KICK_DRIFT, mixed(s), s->dt, s->lim2, cs);
@@ -940,7 +947,7 @@ int launch_loop(md_system* s, int n_mid, bool closing) {
     CK(cudaMemcpyAsync(s->d_ctrl, s->h_ctrl, 3 * sizeof(long long), cudaMemcpyHostToDevice, s->stream));
     CK(cudaGraphLaunch(gr.exec, s->stream));
     const int steps = n_mid + (closing ? 1 : 0);
-    s->launches += 1 + passes + (fused(s) ? 2 : 1 + force_kernels(s)) * steps + (fused(s) ? 0 : n_mid);
+    s->launches += 1 + passes + (1 + force_kernels(s)) * steps + (fused(s) ? 0 : n_mid);
     s->force_evals += steps;
     return MD_OK;
 }
@@ -1019,15 +1026,13 @@ int run_steps_direct_fused(md_system* s, int len, bool first, bool last) {
             ev = take_events(s);
             CK(cudaEventRecord(ev.first, s->stream));
         }
-        launch_forces_mixed_fused(view(s, p), s->g, s->pt, s->to, s->tile_cap,
-                                  kkd ? FUSE_KICK_KICK_DRIFT : FUSE_KICK, step_out(s, 1 - p), s->dt, s->lim2,
-                                  s->stream);
+        enqueue_fused(s, view(s, p), kkd ? FUSE_KICK_KICK_DRIFT : FUSE_KICK, step_out(s, 1 - p), s->stream);
         CKL();
         if (ev.second) {
             CK(cudaEventRecord(ev.second, s->stream));
             s->ev_force.push_back(ev);
         }
-        s->launches += 1;
+        s->launches += force_kernels(s);
         s->force_evals += 1;
         if (kkd) p ^= 1;
     }
@@ -1042,6 +1047,8 @@ int run_steps_direct_fused(md_system* s, int len, bool first, bool last) {
 // alternate between the two FP32 buffers and end the chunk in buffer 0.
 int run_chunk_fused(md_system* s, int len, bool first, bool last) {
     int rc;
+    if (s->potential == 1 && tbsma_smem_bytes(s->tile_cap) > 226 * 1024)
+        return fail(s, MD_ERR_CELL_OVERFLOW, "tile of %d atoms exceeds shared memory", s->tile_cap);
     if (!s->use_graphs) return run_steps_direct_fused(s, len, first, last);
     if (s->timing && (rc = ensure_graphs(s))) return rc;
     const DevState a = view(s, 0);
@@ -1080,7 +1087,7 @@ int run_chunk_fused(md_system* s, int len, bool first, bool last) {
                 }
             }
             CK(cudaGraphLaunch(s->g_multi.exec, s->stream));  // MULTI_STEPS steps; back in buffer 0
-            s->launches += 2 * MULTI_STEPS;
+            s->launches += (1 + force_kernels(s)) * MULTI_STEPS;
             s->force_evals += MULTI_STEPS;
             k += MULTI_STEPS - 1;
             continue;
@@ -1094,7 +1101,7 @@ int run_chunk_fused(md_system* s, int len, bool first, bool last) {
             s->ev_force.push_back(ev);
         }
         CK(cudaGraphLaunch(gr.exec, s->stream));
-        s->launches += 2;  // step control, fused force kernel
+        s->launches += 1 + force_kernels(s);  // step control, fused forces
         s->force_evals += 1;
         if (kkd) p ^= 1;
     }
@@ -1592,6 +1599,8 @@ int md_set_tbsma(md_system* s, double A, double xi, double p, double q, double r
     const double band = tile_frame_cut_band(wmax, 0.5 * s->skin, r_cut);
     tb.rc2lo_f = (float)(r_cut * r_cut * (1.0 - band));
     tb.rc2hi_f = (float)(r_cut * r_cut * (1.0 + band));
+    tb.rc2_f = (float)(r_cut * r_cut);
+    tb.band_f = std::max(tb.rc2hi_f - tb.rc2_f, tb.rc2_f - tb.rc2lo_f);  // (exact: neighbouring numbers)
     s->potential = 1;
     s->forces_valid = false;
     s->graphs_valid = false;

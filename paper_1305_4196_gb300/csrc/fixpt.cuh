@@ -202,4 +202,16 @@ __device__ __forceinline__ void fix_add2(FixAcc& acc, f2_t fs2, f2_t d, f2_t mag
     acc.lo += __float_as_uint(t2a) + __float_as_uint(t2b);
 }
 
+// The same for d = 1.
+__device__ __forceinline__ void fix_add2_one(FixAcc& acc, f2_t v, f2_t magic2, f2_t two21) {
+    const f2_t t1 = f2_add(v, magic2);
+    const f2_t r = f2_add(v, f2_sub(magic2, t1));
+    const f2_t t2 = f2_fma(r, two21, magic2);
+    float t1a, t1b, t2a, t2b;
+    f2_unpack(t1, t1a, t1b);
+    f2_unpack(t2, t2a, t2b);
+    acc.hi += __float_as_uint(t1a) + __float_as_uint(t1b);
+    acc.lo += __float_as_uint(t2a) + __float_as_uint(t2b);
+}
+
 }  // namespace mdgb

@@ -111,6 +111,7 @@ struct TBTable {
     float r0, kp, lp, kq, lq;  // FP32 forms of the two exponentials
     float c_rep, c_band;       // 2 p / r0, q / r0
     float rc2lo_f, rc2hi_f;    // the FP64 decision band around r_cut^2
+    float rc2_f, band_f;       // the same as a distance: |r^2 - rc2_f| <= band_f holds all of it
     double rc2_d;              // r_cut^2
 };
 
@@ -324,7 +325,7 @@ struct StepOut {
 };
 void launch_forces_mixed_fused(const DevState& s, const Geometry& g, const PairTable& pt, const TileOffsets& to,
                                int tile_cap, int mode, StepOut out, double dt, double lim2, cudaStream_t st);
-enum { FUSE_KICK = 1, FUSE_KICK_KICK_DRIFT = 2 };  // modes of launch_forces_mixed_fused
+enum { FUSE_FORCE_ONLY = 0, FUSE_KICK = 1, FUSE_KICK_KICK_DRIFT = 2 };  // modes of the fused force launches
 // The same tasks with several CTAs per block and lanes per atom (k_force_split.cu), for systems
 // of few blocks; false where one CTA per block is the better form (nothing is launched).
 bool launch_forces_mixed_split(const DevState& s, const Geometry& g, const PairTable& pt, const TileOffsets& to,
@@ -334,8 +335,9 @@ void init_force_split_kernels();
 // TB-SMA forces (full lists, mixed): the density pass writes emb[i] = 1/sqrt(rho_i) (0 for an
 // atom without neighbours), the force pass the Q31.32 forces; with_energy also writes the
 // per-atom energies and virial shares.  Two launches.
-void launch_tbsma(const DevState& s, const Geometry& g, const TBTable& tb, const TileOffsets& to, int tile_cap,
-                  float* emb, int with_energy, cudaStream_t st);
+void launch_tbsma(const DevState& s, const Geometry& g, const PairTable& pt, const TBTable& tb, const TileOffsets& to,
+                  int tile_cap, float* emb, int with_energy, int mode, StepOut out, double dt, double lim2,
+                  cudaStream_t st);
 size_t tbsma_smem_bytes(int tile_cap);
 // Colour-schedule race detector: blocks [block0, block0 + nblocks) tag their tile atoms.
 void launch_colour_tags(const DevState& s, const Geometry& g, int block0, int nblocks, int32_t* tags,

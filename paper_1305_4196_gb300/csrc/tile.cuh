@@ -213,9 +213,12 @@ __device__ __forceinline__ float4 tile_coord(const TileMeta& m, const TileOffset
 }
 
 // Stage the block-frame FP32 coordinates of the tile, one warp per tile cell (lanes
-// over the cell's atoms, two cells per step so that two loads are in flight).
+// over the cell's atoms, two cells per step so that two loads are in flight).  W: the .w
+// entries from w (one value per atom, read from L2) in place of the species bits.
+template <bool W = false>
 __device__ __forceinline__ void tile_stage_f32_cells(const TileMeta& m, const float4* __restrict__ xr,
-                                                     const TileOffsets& to, float4* __restrict__ tile) {
+                                                     const TileOffsets& to, float4* __restrict__ tile,
+                                                     const float* __restrict__ w = nullptr) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     for (int slot = warp; slot < 64; slot += 2 * nw) {
         const int slot2 = slot + nw;
@@ -233,20 +236,13 @@ __device__ __forceinline__ void tile_stage_f32_cells(const TileMeta& m, const fl
             float4 p = make_float4(0.f, 0.f, 0.f, 0.f), q = p;
             if (e < cnt) p = xr[j0 + e];
             if (e < cnt2) q = xr[k0 + e];
+            if (W) {
+                if (e < cnt) p.w = __ldcg(w + j0 + e);
+                if (e < cnt2) q.w = __ldcg(w + k0 + e);
+            }
             if (e < cnt) tile[u0 + e] = make_float4(p.x + ox, p.y + oy, p.z + oz, p.w);
             if (e < cnt2) tile[v0 + e] = make_float4(q.x + ox2, q.y + oy2, q.z + oz2, q.w);
         }
-    }
-}
-
-// One FP32 value per tile atom into the .w of its tile entry (a single-species tile does
-// not need the species there), one warp per tile cell.
-__device__ __forceinline__ void tile_stage_w(const TileMeta& m, const float* __restrict__ v,
-                                             float4* __restrict__ tile) {
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int slot = warp; slot < 64; slot += nw) {
-        const int u0 = m.prefix[slot], cnt = m.prefix[slot + 1] - u0, j0 = m.start[slot];
-        for (int e = lane; e < cnt; e += 32) tile[u0 + e].w = v[j0 + e];
     }
 }
 
