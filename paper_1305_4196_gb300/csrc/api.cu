@@ -1239,11 +1239,6 @@ int md_create(int64_t n, const double box[3], double r_cut, double skin, const m
     if (rc) return bail(rc);
     cudaGetDevice(&s->device);
     s->stream = static_cast<cudaStream_t>(p->stream);
-    init_force_kernels();
-    init_list_kernels();
-    init_grad_kernels();
-    init_tbsma_kernels();
-    init_half_af_kernels();
     {
         const char* ng = std::getenv("MDGB_NO_GRAPHS");
         s->use_graphs = !(ng && ng[0] && ng[0] != '0');
@@ -1258,6 +1253,10 @@ int md_create(int64_t n, const double box[3], double r_cut, double skin, const m
     s->np = round_up((int)std::max<int64_t>(n, 1), 64);
     s->precision = p->precision;
     s->list_kind = p->list_kind;
+    // (those of md_set_tbsma and of the derivatives at their first use)
+    init_force_kernels(mixed(s), half(s), p->n_species == 1);
+    init_list_kernels(half(s));
+    if (af(s)) init_half_af_kernels();
     s->rebuild = p->rebuild;
     s->rebuild_k = p->rebuild_k;
     s->dt = p->dt;
@@ -1582,6 +1581,7 @@ int md_set_tbsma(md_system* s, double A, double xi, double p, double q, double r
     if (!(xi * xi * std::exp(2.0 * q) < 2000.0)) return fail(s, MD_ERR_ARG, "xi^2 exp(2q) must be below 2000");
     DeviceGuard dg(s->device);
     if (!s->emb) {
+        init_tbsma_kernels();
         int rc = dalloc(s, &s->emb, (size_t)std::max<int64_t>(s->n, 1));
         if (rc) return rc;
     }
@@ -1625,6 +1625,7 @@ static int backward(md_system* s, const double* grad_f, int device_ptrs, double*
         double *G = nullptr, *gx = nullptr;
         const size_t need = backward_scratch_doubles(s->g, ns, !mixed(s), n);
         if (need > s->grad_ws_doubles) {  // kept by the system, as its other arrays
+            init_grad_kernels(!mixed(s), ns);
             dfree(s, s->grad_ws);
             s->grad_ws = nullptr;
             s->grad_ws_doubles = 0;

@@ -464,31 +464,30 @@ static void allow_max_smem(K kernel) {
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
 }
 
-void init_force_kernels() {
-    allow_max_smem(k_force_mixed_full<true, false, FM_FORCE>);
-    allow_max_smem(k_force_mixed_full<true, true, FM_FORCE>);
-    allow_max_smem(k_force_mixed_full<false, false, FM_FORCE>);
-    allow_max_smem(k_force_mixed_full<false, true, FM_FORCE>);
-    allow_max_smem(k_force_mixed_full<true, false, FM_KICK>);
-    allow_max_smem(k_force_mixed_full<false, false, FM_KICK>);
-    allow_max_smem(k_force_mixed_full<true, false, FM_KKD>);
-    allow_max_smem(k_force_mixed_full<false, false, FM_KKD>);
-    allow_max_smem(k_force_mixed_occ<true, false, FM_FORCE>);
-    allow_max_smem(k_force_mixed_occ<true, true, FM_FORCE>);
-    allow_max_smem(k_force_mixed_occ<false, false, FM_FORCE>);
-    allow_max_smem(k_force_mixed_occ<false, true, FM_FORCE>);
-    allow_max_smem(k_force_mixed_occ<true, false, FM_KICK>);
-    allow_max_smem(k_force_mixed_occ<false, false, FM_KICK>);
-    allow_max_smem(k_force_mixed_occ<true, false, FM_KKD>);
-    allow_max_smem(k_force_mixed_occ<false, false, FM_KKD>);
-    allow_max_smem(k_force_mixed_half<true, false, 1>);
-    allow_max_smem(k_force_mixed_half<true, false, 4>);
-    allow_max_smem(k_force_mixed_half<true, true, 1>);
-    allow_max_smem(k_force_mixed_half<false, false, 1>);
-    allow_max_smem(k_force_mixed_half<false, false, 4>);
-    allow_max_smem(k_force_mixed_half<false, true, 1>);
-    init_force_split_kernels();
-    init_force_fp64_kernels();
+template <bool SINGLE>
+static void init_force_kernels_of(int half) {
+    if (half) {
+        allow_max_smem(k_force_mixed_half<SINGLE, false, 1>);
+        allow_max_smem(k_force_mixed_half<SINGLE, false, 4>);
+        allow_max_smem(k_force_mixed_half<SINGLE, true, 1>);
+        return;
+    }
+    allow_max_smem(k_force_mixed_full<SINGLE, false, FM_FORCE>);
+    allow_max_smem(k_force_mixed_full<SINGLE, true, FM_FORCE>);
+    allow_max_smem(k_force_mixed_full<SINGLE, false, FM_KICK>);
+    allow_max_smem(k_force_mixed_full<SINGLE, false, FM_KKD>);
+    allow_max_smem(k_force_mixed_occ<SINGLE, false, FM_FORCE>);
+    allow_max_smem(k_force_mixed_occ<SINGLE, true, FM_FORCE>);
+    allow_max_smem(k_force_mixed_occ<SINGLE, false, FM_KICK>);
+    allow_max_smem(k_force_mixed_occ<SINGLE, false, FM_KKD>);
+    init_force_split_kernels(SINGLE);
+}
+
+// The kernels that a system of this kind launches (each costs its creation some microseconds).
+void init_force_kernels(int mixed, int half, int single) {
+    if (!mixed) init_force_fp64_kernels(half, single);
+    else if (single) init_force_kernels_of<true>(half);
+    else init_force_kernels_of<false>(half);
 }
 
 // |fs2 * d| < 2^22 (the exact range of the two-part split) is guaranteed when |fs2| < 2^22 / r_cut

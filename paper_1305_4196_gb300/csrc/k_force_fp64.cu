@@ -354,13 +354,16 @@ static void allow_max_smem(K kernel) {
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
 }
 
-void init_force_fp64_kernels() {
+void init_force_fp64_kernels(int half, int single) {
     int dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&g_sm_count, cudaDevAttrMultiProcessorCount, dev);
-    for (int k = 0; k < 8; ++k)
-        for (int lpa = 1; lpa <= 8; lpa *= 2) allow_max_smem(full_kernel(k & 1, k & 2, k & 4, lpa));
-    allow_max_smem(k_force_fp64_half<false>);
-    allow_max_smem(k_force_fp64_half<true>);
+    if (half) {
+        allow_max_smem(k_force_fp64_half<false>);
+        allow_max_smem(k_force_fp64_half<true>);
+        return;
+    }
+    for (int k = 0; k < 4; ++k)
+        for (int lpa = 1; lpa <= 8; lpa *= 2) allow_max_smem(full_kernel(single, k & 1, k & 2, lpa));
 }
 
 }  // namespace mdgb

@@ -196,14 +196,12 @@ int g_sm_count = 0;  // SMs of the device, read at initialisation (never during 
 
 }  // namespace
 
-void init_force_split_kernels() {
+void init_force_split_kernels(int single) {
     int dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&g_sm_count, cudaDevAttrMultiProcessorCount, dev);
-    for (int single = 0; single < 2; ++single) {
-        allow_max_smem(split_kernel(single, true, FM_FORCE, 1));
-        for (int mode = FM_FORCE; mode <= FM_KKD; ++mode)
-            for (int lpa = 2; lpa <= 8; lpa *= 2) allow_max_smem(split_kernel(single, false, mode, lpa));
-    }
+    allow_max_smem(split_kernel(single, true, FM_FORCE, 1));
+    for (int mode = FM_FORCE; mode <= FM_KKD; ++mode)
+        for (int lpa = 2; lpa <= 8; lpa *= 2) allow_max_smem(split_kernel(single, false, mode, lpa));
 }
 
 bool launch_forces_mixed_split(const DevState& s, const Geometry& g, const PairTable& pt, const TileOffsets& to,

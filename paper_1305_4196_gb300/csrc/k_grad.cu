@@ -382,10 +382,10 @@ static void allow_max_smem(K kernel) {
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
 }
 
-void init_grad_kernels() {
+void init_grad_kernels(int fp64, int nsp) {
     int dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&g_sm_count, cudaDevAttrMultiProcessorCount, dev);
-    for (int k = 0; k < 4 * MAX_SPECIES; ++k) allow_max_smem(backward_kernel(k & 1, k & 2, 1 + k / 4));
+    for (int energy = 0; energy < 2; ++energy) allow_max_smem(backward_kernel(fp64, energy, nsp));
 }
 
 }  // namespace mdgb

@@ -161,11 +161,14 @@ static void allow_max_smem(K kernel) {
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
 }
 
-void init_list_kernels() {
-    allow_max_smem(k_build_lists<0>);
-    allow_max_smem(k_build_lists<1>);
-    allow_max_smem(k_build_lists_occ<0>);
-    allow_max_smem(k_build_lists_occ<1>);
+void init_list_kernels(int half) {
+    if (half) {
+        allow_max_smem(k_build_lists<1>);
+        allow_max_smem(k_build_lists_occ<1>);
+    } else {
+        allow_max_smem(k_build_lists<0>);
+        allow_max_smem(k_build_lists_occ<0>);
+    }
 }
 
 // ---------------------------------------------------------------- export

@@ -331,7 +331,7 @@ enum { FUSE_FORCE_ONLY = 0, FUSE_KICK = 1, FUSE_KICK_KICK_DRIFT = 2 };  // modes
 bool launch_forces_mixed_split(const DevState& s, const Geometry& g, const PairTable& pt, const TileOffsets& to,
                                int tile_cap, float fs2_max, bool with_energy, int mode, StepOut out, double dt,
                                float lim2_f, size_t smem, cudaStream_t st);
-void init_force_split_kernels();
+void init_force_split_kernels(int single);
 // TB-SMA forces (full lists, mixed): the density pass writes emb[i] = 1/sqrt(rho_i) (0 for an
 // atom without neighbours), the force pass the Q31.32 forces; with_energy also writes the
 // per-atom energies and virial shares.  Two launches.
@@ -357,7 +357,7 @@ void launch_cells_out(const DevState& s, const Geometry& g, int32_t* cells, cuda
 void launch_pairs_out(const DevState& s, const Geometry& g, int half, unsigned long long* counter,
                       int32_t* pairs, long long cap, cudaStream_t st);
 
-void init_force_kernels();
+void init_force_kernels(int mixed, int half, int single);
 float fs2_max_of(const PairTable& pt);  // largest |fs2| the two-part split takes (k_force.cu)
 // atom-free half lists (k_half_af.cu)
 void launch_build_sched(const DevState& s, const Geometry& g, const TileOffsets& to, double rl2, int list_cap,
@@ -367,13 +367,13 @@ void launch_forces_half_af(const DevState& s, const Geometry& g, const PairTable
 size_t af_sched_smem_bytes(int tile_cap);
 size_t af_force_smem_bytes(int tile_cap);
 void init_half_af_kernels();
-void init_force_fp64_kernels();
-void init_grad_kernels();
+void init_force_fp64_kernels(int half, int single);
+void init_grad_kernels(int fp64, int nsp);
 size_t backward_smem_bytes(int fp64, int tile_cap);
 size_t backward_scratch_doubles(const Geometry& g, int nsp, int fp64, int64_t n);
 void launch_force_backward(const DevState& s, const Geometry& g, const PairTable& pt, const TileOffsets& to,
                            int tile_cap, int fp64, const double* G, double* gx, double* scratch, cudaStream_t st);
-void init_list_kernels();
+void init_list_kernels(int half);
 
 // integrate modes
 enum { INT_KICK_DRIFT = 0, INT_KICK_KICK_DRIFT = 1, INT_KICK = 2 };
