@@ -26,6 +26,7 @@ constexpr int NBUCKET = 5;  // one-CTA systems: [.., 512), [512, 1024), [1024, 2
 const int BUCKET_HI[NBUCKET] = {512, 1024, 2048, 4096, BATCH_MAX_ATOMS + 1};
 constexpr long long DEFAULT_BUDGET = 1LL << 34;  // cycles without work before a CTA gives up (~9 s)
 constexpr int DEFAULT_ONE_CTA_MAX = 2048;
+constexpr int ENS_SHARE_CTAS = 2;  // CTAs per SM that a launch usually has
 
 int bucket_of(int64_t n) {
     for (int k = 0; k < NBUCKET; ++k)
@@ -190,7 +191,11 @@ int build_table(md_batch* b) {
     for (int k = 0; k < b->nsys; ++k) order[k] = k;
     // the longest tasks first: one-CTA systems by size, then block systems by size
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) { return b->n[x] > b->n[y]; });
-    std::vector<EnsEntry> e_one, e_blk;
+    // A one-CTA system of more than half of a CTA's share of all atoms is shared out as tasks (an
+    // atom costs about the same on every path), if that makes more than one.
+    const int64_t share = b->ntot / std::max(1, ENS_SHARE_CTAS * b->sms) / 2;
+    int64_t s0 = 0;
+    std::vector<EnsEntry> e_one, e_shared, e_blk;
     for (int k : order) {
         if (b->n[k] == 0) continue;
         if (is_block(b, k)) {
@@ -208,16 +213,24 @@ int build_table(md_batch* b) {
             if (b->n[k] > BATCH_MAX_ATOMS)
                 return bfail(b, MD_ERR_BOX_TOO_SMALL, "system %d: %lld atoms in a box of fewer than 6 (r_cut + skin) per side",
                              k, (long long)b->n[k]);
-            const BatchSys y1 = make_sys(b, k, b->R[bucket_of(b->n[k])]);
+            BatchSys y1 = make_sys(b, k, b->R[bucket_of(b->n[k])]);
             if (y1.ncell > BATCH_MAX_CELLS) return bfail(b, MD_ERR_CELL_OVERFLOW, "system %d: too many cells", k);
             b->nmax = std::max(b->nmax, y1.n);
             b->cmax = std::max(b->cmax, y1.ncell);
-            e_one.push_back(EnsEntry{0, (int)b->one.size(), 0, 0, 0});
+            if (y1.n > share && y1.n > ENS_SHARED_CHUNK) {
+                y1.s0 = s0;
+                s0 += y1.ncell + 1;
+                e_shared.push_back(
+                    EnsEntry{2, (int)b->one.size(), (y1.n + ENS_SHARED_CHUNK - 1) / ENS_SHARED_CHUNK, 0, 0});
+            } else {
+                e_one.push_back(EnsEntry{0, (int)b->one.size(), 0, 0, 0});
+            }
             b->one.push_back(y1);
         }
     }
     b->nmax = (b->nmax + 7) & ~7;
-    b->ent = e_one;
+    b->ent = e_shared;
+    b->ent.insert(b->ent.end(), e_one.begin(), e_one.end());
     b->ent.insert(b->ent.end(), e_blk.begin(), e_blk.end());
     // shared memory: the larger of the one-CTA layout and the tile; the tile takes what is left
     size_t smem = b->one.empty() ? 0 : batch_smem_bytes(b->nmax, b->cmax);
@@ -233,10 +246,10 @@ int build_table(md_batch* b) {
     const int per_sm = ensemble_ctas_per_sm(b->threads, smem);
     if (per_sm < 1) return bfail(b, MD_ERR_CUDA, "the ensemble kernel does not fit an SM at %d threads", b->threads);
     b->grid = per_sm * b->sms;
-    // initial scheduler words: one-CTA systems at their task, block systems at START
+    // initial scheduler words: one-CTA systems at their task, the others at START
     std::vector<unsigned long long> init(b->ent.size(), 0ull);
     for (size_t e = 0; e < b->ent.size(); ++e)
-        if (b->ent[e].kind == 1) init[e] = (unsigned long long)ENS_START << 32;
+        if (b->ent[e].kind != 0) init[e] = (unsigned long long)ENS_START << 32;
     // the block systems' lists and coordinates belong to the old table
     if (b->ea.valid) BCK(cudaMemsetAsync(b->ea.valid, 0, sizeof(int32_t) * (size_t)b->nsys, b->stream));
     if (b->ea.rebuild) BCK(cudaMemsetAsync(b->ea.rebuild, 0, sizeof(int32_t) * (size_t)b->nsys, b->stream));
@@ -459,7 +472,7 @@ int md_batch_create(int32_t n_systems, const int64_t* n_atoms, const double* box
     b->n.assign(n_atoms, n_atoms + n_systems);
     b->box.assign(boxes, boxes + 3 * n_systems);
     b->a0.resize(n_systems);
-    int64_t cells_max = 0, nblk_max = 0;
+    int64_t cells_max = 0, nblk_max = 0, starts_max = 0;
     double band = 0.0, rho_max = 0.0;
     for (int k = 0; k < n_systems; ++k) {
         if (b->n[k] < 0 || b->n[k] > 0x7fffffffLL) return bail(MD_ERR_ARG);
@@ -474,6 +487,7 @@ int md_batch_create(int32_t n_systems, const int64_t* n_atoms, const double* box
         for (int R = 1; R <= 2; ++R) {
             const BatchSys y = make_sys(b, k, R);
             band = std::max(band, cell_frame_cut_band(std::max(y.w[0], std::max(y.w[1], y.w[2])), R, r_cut));
+            if (R == 2 && b->n[k] > ENS_SHARED_CHUNK && b->n[k] <= BATCH_MAX_ATOMS) starts_max += y.ncell + 1;
         }
         EnsBlockSys y;
         if (make_blk(b, k, y)) {
@@ -512,7 +526,8 @@ int md_batch_create(int32_t n_systems, const int64_t* n_atoms, const double* box
         (rc = balloc(b, &ea.valid, ns)) || (rc = balloc(b, &b->d_sys_of, nt)) || (rc = balloc(b, &b->d_box, 3 * ns)) ||
         (rc = balloc(b, &ea.pe_atom, nt)) ||
         (rc = balloc(b, &ea.count, (size_t)cells_max)) || (rc = balloc(b, &ea.cursor, (size_t)cells_max)) ||
-        (rc = balloc(b, &ea.cstart, (size_t)(cells_max + nblk_max))) || (rc = balloc(b, &ea.ctl, ns)) ||
+        (rc = balloc(b, &ea.cstart, (size_t)(cells_max + nblk_max))) ||
+        (rc = balloc(b, &ea.cstart1, (size_t)starts_max)) || (rc = balloc(b, &ea.ctl, ns)) ||
         (rc = balloc(b, &ea.done, ns)) || (rc = balloc(b, &ea.g_done, 1)) || (rc = balloc(b, &b->d_ctl_init, ns)) ||
         (rc = balloc(b, &b->d_ent, ns)) || (rc = balloc(b, &b->d_one, ns)) || (rc = balloc(b, &b->d_blk, ns)))
         return bail(rc);
@@ -657,7 +672,7 @@ int md_batch_set_wait_budget(md_batch* b, int64_t budget_cycles, int32_t held_sy
     if (held_system >= 0)
         for (size_t e = 0; e < b->ent.size(); ++e) {
             const EnsEntry& en = b->ent[e];
-            const int id = en.kind == 0 ? b->one[en.idx].id : b->blk[en.idx].id;
+            const int id = en.kind == 1 ? b->blk[en.idx].id : b->one[en.idx].id;
             if (id == held_system) b->hold = (int)e;
         }
     drop_graph(b);

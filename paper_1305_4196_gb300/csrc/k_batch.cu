@@ -78,29 +78,45 @@ struct Smem {
     int* warp_tot;        // 32
 };
 
+struct PosBuf {
+    double *x, *y, *z;
+};
+
+__device__ __forceinline__ PosBuf ens_pos(const BatchState& st, const EnsArrays& ea, bool odd) {
+    return odd ? PosBuf{ea.xa, ea.ya, ea.za} : PosBuf{st.x, st.y, st.z};
+}
+
+// Data of a one-CTA system is read through L1; a shared system's (below) from L2, where other CTAs
+// of the launch wrote it.
+template <bool SHARED, typename T>
+__device__ __forceinline__ T ld_state(const T* p) {
+    return SHARED ? __ldcg(p) : *p;
+}
+
 // Wrap every atom into the box (one box length at most, counted in the image
 // counters), find its cell, and sort the atoms into cells, within a cell in index
 // order; write the slot-ordered FP32 coordinates.
-__device__ void batch_bin(const BatchSys& y, BatchState st, Smem& sm) {
+template <bool SHARED>
+__device__ void batch_bin(const BatchSys& y, BatchState st, const PosBuf& P, Smem& sm) {
     const int n = y.n, m = y.ncell;
     for (int k = threadIdx.x; k < m; k += blockDim.x) sm.ccount[k] = 0;
     __syncthreads();
     for (int a = threadIdx.x; a < n; a += blockDim.x) {
         const int64_t g = y.a0 + a;
-        double* X[3] = {st.x, st.y, st.z};
+        double* X[3] = {P.x, P.y, P.z};
         int32_t* I[3] = {st.ix, st.iy, st.iz};
         int c[3];
         uint32_t bad = 0;
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            double x = X[d][g];
+            double x = ld_state<SHARED>(X[d] + g);
             if (x >= y.L[d]) {
                 x = __dsub_rn(x, y.L[d]);
-                I[d][g] += 1;
+                I[d][g] = ld_state<SHARED>(I[d] + g) + 1;
                 X[d][g] = x;
             } else if (x < 0.0) {
                 x = __dadd_rn(x, y.L[d]);
-                I[d][g] -= 1;
+                I[d][g] = ld_state<SHARED>(I[d] + g) - 1;
                 X[d][g] = x;
             }
             if (!(x >= 0.0 && x <= y.L[d])) bad |= isfinite(x) ? ERR_ESCAPE : ERR_NONFINITE;
@@ -133,9 +149,9 @@ __device__ void batch_bin(const BatchSys& y, BatchState st, Smem& sm) {
             int rank = 0;
             for (int f = 0; f < cnt; ++f) rank += (int)sm.perm[s0 + f] < mine;
             const int64_t g = y.a0 + mine;
-            sm.px[s0 + rank] = __double2float_rn(st.x[g] - ox);
-            sm.py[s0 + rank] = __double2float_rn(st.y[g] - oy);
-            sm.pz[s0 + rank] = __double2float_rn(st.z[g] - oz);
+            sm.px[s0 + rank] = __double2float_rn(ld_state<SHARED>(P.x + g) - ox);
+            sm.py[s0 + rank] = __double2float_rn(ld_state<SHARED>(P.y + g) - oy);
+            sm.pz[s0 + rank] = __double2float_rn(ld_state<SHARED>(P.z + g) - oz);
             sm.scell[s0 + rank] = (uint16_t)id;
             sm.cell[mine] = (uint16_t)(s0 + rank);
         }
@@ -159,16 +175,38 @@ __device__ __forceinline__ void slot_cell(const BatchSys& y, const Smem& sm, int
 
 __device__ __forceinline__ int wrap_cell(int c, int nc) { return c < 0 ? c + nc : (c >= nc ? c - nc : c); }
 
+template <bool SHARED>
+__device__ __forceinline__ bool ens_fp64_pair_test(const double* __restrict__ x, const double* __restrict__ y,
+                                                   const double* __restrict__ z, double Lx, double Ly, double Lz,
+                                                   int64_t i, int64_t j, double r2max) {
+    const double dx = mic_rn(__dsub_rn(ld_state<SHARED>(x + i), ld_state<SHARED>(x + j)), Lx);
+    const double dy = mic_rn(__dsub_rn(ld_state<SHARED>(y + i), ld_state<SHARED>(y + j)), Ly);
+    const double dz = mic_rn(__dsub_rn(ld_state<SHARED>(z + i), ld_state<SHARED>(z + j)), Lz);
+    const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+    return r2 < r2max;
+}
+
 // Exact force on the atom of slot p, one candidate at a time: a pair whose FP32 r^2 lies in
 // the band around r_cut^2 is decided in FP64 by the definition, a large term is rounded in
 // FP64 (fix_term_wide); every other term is the one the packed loop would add.
-template <bool ENERGY>
-__device__ __noinline__ void batch_force_exact(const BatchSys& y, const BatchState& st, const PairTable& pt,
-                                               float fs2_max, const Smem& sm, float* __restrict__ pe_out, int p) {
+struct ExactForce {
+    long long qx, qy, qz;
+    float pe;
+};
+
+// Atom of slot p of a system, from the arrays of this CTA or those of the launch.
+template <bool SHARED>
+__device__ __forceinline__ int slot_atom(const BatchSys& y, const EnsArrays& ea, const Smem& sm, int p) {
+    return SHARED ? __ldcg(ea.perm_s + y.a0 + p) : (int)sm.perm[p];
+}
+
+template <bool ENERGY, bool SHARED>
+__device__ __noinline__ ExactForce batch_force_exact(const BatchSys& y, const BatchState& st, const EnsArrays& ea,
+                                                     const PosBuf& P, const PairTable& pt, float fs2_max,
+                                                     const Smem& sm, int p) {
     const int R = y.R;
     const float sig2 = pt.sig2_f[0], c48 = pt.c48_f[0], c24 = pt.c24_f[0], c4 = pt.c4_f[0];
-    const int a = sm.perm[p];
-    const int64_t g = y.a0 + a;
+    const int64_t g = y.a0 + slot_atom<SHARED>(y, ea, sm, p);
     int cx, cy, cz;
     slot_cell(y, sm, p, cx, cy, cz);
     const float xi = sm.px[p], yi = sm.py[p], zi = sm.pz[p];
@@ -188,7 +226,8 @@ __device__ __noinline__ void batch_force_exact(const BatchSys& y, const BatchSta
                     const float r2 = fmaf(ez, ez, fmaf(ey, ey, ex * ex));
                     if (!(r2 < pt.rc2hi_f[0])) continue;
                     if (!(r2 < pt.rc2lo_f[0]) &&
-                        !fp64_pair_test(st.x, st.y, st.z, y.L[0], y.L[1], y.L[2], g, y.a0 + sm.perm[q], pt.rc2_d[0]))
+                        !ens_fp64_pair_test<SHARED>(P.x, P.y, P.z, y.L[0], y.L[1], y.L[2], g,
+                                                    y.a0 + slot_atom<SHARED>(y, ea, sm, q), pt.rc2_d[0]))
                         continue;
                     const float inv = rcp_approx(r2);
                     const float s2 = sig2 * inv;
@@ -202,19 +241,17 @@ __device__ __noinline__ void batch_force_exact(const BatchSys& y, const BatchSta
                 }
             }
     fix_wide_count_ok(nwide, st.err);
-    st.fq[g] = qx;
-    st.fq[st.ntot + g] = qy;
-    st.fq[2 * st.ntot + g] = qz;
-    if (ENERGY) pe_out[a] = 0.5f * pe;
+    return ExactForce{qx, qy, qz, pe};
 }
 
-// Force on every atom (fixed point into st.fq); with energy, also its half pair energies
-// (FP32 per atom, neighbours in slot order: deterministic).  Two candidates per step:
+// Force on the atoms of slots lo .. hi - 1 (to done(slot, atom, force, pair energy)); with energy,
+// also its pair energies (FP32 per atom, neighbours in slot order: deterministic).  Two candidates per step:
 // the pair (q, q+1) with q even, masked to the cell's range and away from the atom itself.
-template <bool ENERGY>
-__device__ void batch_forces(const BatchSys& y, BatchState st, const PairTable& pt, float fs2_max, Smem& sm,
-                             float* __restrict__ pe_out) {
-    const int n = y.n, R = y.R;
+template <bool ENERGY, bool SHARED, typename Done>
+__device__ __forceinline__ void batch_forces(const BatchSys& y, const BatchState& st, const EnsArrays& ea,
+                                             const PosBuf& P, const PairTable& pt, float fs2_max, Smem& sm, int lo,
+                                             int hi, Done&& done) {
+    const int R = y.R;
     const f2_t magic2 = f2_pack(MAGIC, MAGIC), two21 = f2_pack(TWO21, TWO21);
     const f2_t sig2 = f2_pack(pt.sig2_f[0], pt.sig2_f[0]), c48 = f2_pack(pt.c48_f[0], pt.c48_f[0]);
     const f2_t nc24 = f2_pack(-pt.c24_f[0], -pt.c24_f[0]);
@@ -224,7 +261,7 @@ __device__ void batch_forces(const BatchSys& y, BatchState st, const PairTable& 
     const unsigned spz = (unsigned)__cvta_generic_to_shared(sm.pz);
     if (threadIdx.x == 0) *sm.nqueued = 0;
     __syncthreads();
-    for (int p = threadIdx.x; p < n; p += blockDim.x) {
+    for (int p = lo + (int)threadIdx.x; p < hi; p += blockDim.x) {
         int cx, cy, cz;
         slot_cell(y, sm, p, cx, cy, cz);
         const float xi = sm.px[p], yi = sm.py[p], zi = sm.pz[p];
@@ -282,17 +319,15 @@ __device__ void batch_forces(const BatchSys& y, BatchState st, const PairTable& 
             sm.queue[atomicAdd(sm.nqueued, 1)] = (uint16_t)p;
             continue;
         }
-        const int a = sm.perm[p];
-        const int64_t g = y.a0 + a;
-        st.fq[g] = fix_final(ax, nterms);
-        st.fq[st.ntot + g] = fix_final(ay, nterms);
-        st.fq[2 * st.ntot + g] = fix_final(az, nterms);
-        if (ENERGY) pe_out[a] = 0.5f * pe;
+        done(p, slot_atom<SHARED>(y, ea, sm, p), fix_final(ax, nterms), fix_final(ay, nterms), fix_final(az, nterms), pe);
     }
     __syncthreads();
     const int nq = *sm.nqueued;
-    for (int k = threadIdx.x; k < nq; k += blockDim.x)
-        batch_force_exact<ENERGY>(y, st, pt, fs2_max, sm, pe_out, sm.queue[k]);
+    for (int k = threadIdx.x; k < nq; k += blockDim.x) {
+        const int p = sm.queue[k];
+        const ExactForce e = batch_force_exact<ENERGY, SHARED>(y, st, ea, P, pt, fs2_max, sm, p);
+        done(p, slot_atom<SHARED>(y, ea, sm, p), e.qx, e.qy, e.qz, e.pe);
+    }
 }
 
 // v += k F (FP64, F in Q31.32); with drift also x += dt v
@@ -334,18 +369,13 @@ __device__ double block_sum(double v, double* sh) {
 // ---------------------------------------------------------------- one-CTA systems
 namespace {
 
-// The whole call for a system held by one CTA: flags BATCH_HAVE_FORCES (st.fq holds F at
-// the current positions), BATCH_ENERGY (potential and kinetic energy at the end).
-__device__ void run_one_system(const BatchSys& y, const BatchState& st, const PairTable& pt, int n_steps, int flags,
-                               double dt, float fs2_max, int nmax, int cmax, float* __restrict__ pe_atom,
-                               double* __restrict__ pe_out, double* __restrict__ ke_out, unsigned char* smem,
-                               int* warp_tot, int* nqueued, double* red) {
-    if (y.n == 0) return;
+// The shared memory of a one-CTA or shared system; false (flagged) when it does not fit.
+__device__ __forceinline__ bool batch_smem(const BatchSys& y, const BatchState& st, int nmax, int cmax,
+                                           unsigned char* smem, int* warp_tot, int* nqueued, Smem& sm) {
     if (y.n > nmax || y.ncell > cmax) {  // the host sizes the launch for its systems
         if (threadIdx.x == 0) atomicOr(st.err, ERR_TILE_OVERFLOW);
-        return;
+        return false;
     }
-    Smem sm;
     const int np2 = nmax + 2;  // even: the three coordinate arrays stay 8-byte aligned
     sm.px = reinterpret_cast<float*>(smem);
     sm.py = sm.px + np2;
@@ -358,29 +388,51 @@ __device__ void run_one_system(const BatchSys& y, const BatchState& st, const Pa
     sm.cstart = reinterpret_cast<int*>(smem + batch_smem_ints_offset(nmax));
     sm.ccount = sm.cstart + cmax + 1;
     sm.warp_tot = warp_tot;
-    if (!(flags & BATCH_HAVE_FORCES) || n_steps == 0) {
-        batch_bin(y, st, sm);
-        batch_forces<false>(y, st, pt, fs2_max, sm, nullptr);
+    return true;
+}
+
+// The whole call for a system held by one CTA: flags BATCH_HAVE_FORCES (st.fq holds F at
+// the current positions), BATCH_ENERGY (potential and kinetic energy at the end, from the
+// last force evaluation).
+__device__ void run_one_system(const BatchSys& y, const BatchState& st, const EnsArrays& ea, const PairTable& pt,
+                               int n_steps, int flags, double dt, float fs2_max, int nmax, int cmax,
+                               double* __restrict__ pe_out, double* __restrict__ ke_out, unsigned char* smem,
+                               int* warp_tot, int* nqueued, double* red) {
+    if (y.n == 0) return;
+    Smem sm;
+    if (!batch_smem(y, st, nmax, cmax, smem, warp_tot, nqueued, sm)) return;
+    const PosBuf P{st.x, st.y, st.z};
+    const bool energy = (flags & BATCH_ENERGY) != 0;
+    const bool forces_first = !(flags & BATCH_HAVE_FORCES) || n_steps == 0;
+    for (int step = forces_first ? -1 : 0; step < n_steps; ++step) {
+        if (step >= 0) {
+            batch_kick(y, st, pt, dt, true);  // opening half kick and drift
+            __syncthreads();
+        }
+        batch_bin<false>(y, st, P, sm);
+        const auto store = [&](int, int a, long long qx, long long qy, long long qz, float pe) {
+            const int64_t g = y.a0 + a;
+            st.fq[g] = qx;
+            st.fq[st.ntot + g] = qy;
+            st.fq[2 * st.ntot + g] = qz;
+            if (energy) ea.pe_atom[g] = 0.5f * pe;
+        };
+        if (energy && step == n_steps - 1)
+            batch_forces<true, false>(y, st, ea, P, pt, fs2_max, sm, 0, y.n, store);
+        else
+            batch_forces<false, false>(y, st, ea, P, pt, fs2_max, sm, 0, y.n, store);
         __syncthreads();
+        if (step >= 0) {
+            batch_kick(y, st, pt, dt, false);  // closing half kick
+            __syncthreads();
+        }
     }
-    for (int step = 0; step < n_steps; ++step) {
-        batch_kick(y, st, pt, dt, true);  // opening half kick and drift
-        __syncthreads();
-        batch_bin(y, st, sm);
-        batch_forces<false>(y, st, pt, fs2_max, sm, nullptr);
-        __syncthreads();
-        batch_kick(y, st, pt, dt, false);  // closing half kick
-        __syncthreads();
-    }
-    if (flags & BATCH_ENERGY) {
-        batch_bin(y, st, sm);
-        batch_forces<true>(y, st, pt, fs2_max, sm, pe_atom + y.a0);
-        __syncthreads();
+    if (energy) {
         double pe = 0.0, ke = 0.0;
         const double m = pt.mass[0];
         for (int a = threadIdx.x; a < y.n; a += blockDim.x) {
             const int64_t g = y.a0 + a;
-            pe += (double)pe_atom[g];
+            pe += (double)ea.pe_atom[g];
             ke += 0.5 * m * (st.vx[g] * st.vx[g] + st.vy[g] * st.vy[g] + st.vz[g] * st.vz[g]);
         }
         pe = block_sum(pe, red);
@@ -389,6 +441,109 @@ __device__ void run_one_system(const BatchSys& y, const BatchState& st, const Pa
             pe_out[y.id] = pe;
             ke_out[y.id] = ke;
         }
+    }
+}
+
+// ---------------------------------------------------------------- shared systems
+// A one-CTA system that would keep its CTA busy long after the others have run out of work is
+// advanced by the same operations in phases of tasks (so with the same results, bit for bit; which
+// form it takes only decides who computes what).  Phase p = 8 k + s of time step k is stage
+//   KICK  (atom chunks; only k = 0)  the opening half kick and drift with the forces of the
+//                       previous call, into the other position buffers;
+//   BIN   (one task)    the cells, and the coordinates by slot, to the arrays of the launch;
+//   FORCE (slot chunks) all of these into shared memory; the forces of the chunk's atoms, the
+//                       closing half kick of step k - 1, the opening one of step k and the drift
+//                       into the other position buffers (for k < K).
+// Then FINAL and ESUM, as for the block systems.
+
+// BIN of step k (positions in the odd / even buffers)
+__device__ void shared_bin(const BatchSys& y, const BatchState& st, const EnsArrays& ea, bool odd, Smem& sm) {
+    batch_bin<true>(y, st, ens_pos(st, ea, odd), sm);
+    for (int p = threadIdx.x; p < y.n; p += blockDim.x) {
+        ea.xs[y.a0 + p] = make_float4(sm.px[p], sm.py[p], sm.pz[p], __int_as_float((int)sm.scell[p]));
+        ea.perm_s[y.a0 + p] = sm.perm[p];
+    }
+    for (int c = threadIdx.x; c <= y.ncell; c += blockDim.x) ea.cstart1[y.s0 + c] = sm.cstart[c];
+}
+
+// One atom after its force (q) at step k of K, or with the previous call's force at step 0 (KICK).
+__device__ __forceinline__ void shared_update(const BatchSys& y, const BatchState& st, const EnsArrays& ea,
+                                              const PairTable& pt, int k, int K, double dt, int64_t g, long long qx,
+                                              long long qy, long long qz) {
+    if (K == 0) return;
+    const double hq = pt.hdtm_q[0];
+    double vx = __ldcg(st.vx + g), vy = __ldcg(st.vy + g), vz = __ldcg(st.vz + g);
+    if (k > 0) {  // closing half kick of step k - 1
+        vx = fma(hq, (double)qx, vx);
+        vy = fma(hq, (double)qy, vy);
+        vz = fma(hq, (double)qz, vz);
+    }
+    if (k < K) {  // opening half kick of step k
+        vx = fma(hq, (double)qx, vx);
+        vy = fma(hq, (double)qy, vy);
+        vz = fma(hq, (double)qz, vz);
+    }
+    st.vx[g] = vx;
+    st.vy[g] = vy;
+    st.vz[g] = vz;
+    if (k == K) return;
+    const bool odd = (k & 1) != 0;
+    const PosBuf P = ens_pos(st, ea, odd), Pn = ens_pos(st, ea, !odd);
+    Pn.x[g] = fma(dt, vx, __ldcg(P.x + g));
+    Pn.y[g] = fma(dt, vy, __ldcg(P.y + g));
+    Pn.z[g] = fma(dt, vz, __ldcg(P.z + g));
+}
+
+__device__ void shared_kick(const BatchSys& y, const BatchState& st, const EnsArrays& ea, const PairTable& pt, int K,
+                            double dt, int task) {
+    const int lo = task * ENS_SHARED_CHUNK, hi = min(y.n, lo + ENS_SHARED_CHUNK);
+    for (int a = lo + (int)threadIdx.x; a < hi; a += blockDim.x) {
+        const int64_t g = y.a0 + a;
+        shared_update(y, st, ea, pt, 0, K, dt, g, __ldcg(st.fq + g), __ldcg(st.fq + st.ntot + g),
+                      __ldcg(st.fq + 2 * st.ntot + g));
+    }
+}
+
+template <bool ENERGY>
+__device__ void shared_force(const BatchSys& y, const BatchState& st, const EnsArrays& ea, const PairTable& pt,
+                             float fs2_max, int k, int K, double dt, int task, Smem& sm) {
+    const float4* xs = ea.xs + y.a0;
+#pragma unroll 4
+    for (int p = threadIdx.x; p < y.n; p += blockDim.x) {
+        const float4 v = __ldcg(xs + p);
+        sm.px[p] = v.x;
+        sm.py[p] = v.y;
+        sm.pz[p] = v.z;
+        sm.scell[p] = (uint16_t)__float_as_int(v.w);
+    }
+    for (int c = threadIdx.x; c <= y.ncell; c += blockDim.x) sm.cstart[c] = __ldcg(ea.cstart1 + y.s0 + c);
+    if (threadIdx.x == 0) {  // slot n, as in batch_bin
+        sm.px[y.n] = sm.py[y.n] = sm.pz[y.n] = 1.0e4f;
+        sm.scell[y.n] = 0;
+    }
+    // (batch_forces begins with a barrier)
+    const int lo = task * ENS_SHARED_CHUNK, hi = min(y.n, lo + ENS_SHARED_CHUNK);
+    batch_forces<ENERGY, true>(y, st, ea, ens_pos(st, ea, (k & 1) != 0), pt, fs2_max, sm, lo, hi,
+                               [&](int, int a, long long qx, long long qy, long long qz, float pe) {
+                                   const int64_t g = y.a0 + a;
+                                   if (k == K) {
+                                       st.fq[g] = qx;
+                                       st.fq[st.ntot + g] = qy;
+                                       st.fq[2 * st.ntot + g] = qz;
+                                       if (ENERGY) ea.pe_atom[g] = 0.5f * pe;
+                                   }
+                                   shared_update(y, st, ea, pt, k, K, dt, g, qx, qy, qz);
+                               });
+}
+
+// FINAL (odd K): the second buffers' positions into the first.
+__device__ void shared_final(const BatchSys& y, const BatchState& st, const EnsArrays& ea, int task) {
+    const int lo = task * ENS_SHARED_CHUNK, hi = min(y.n, lo + ENS_SHARED_CHUNK);
+    for (int a = lo + (int)threadIdx.x; a < hi; a += blockDim.x) {
+        const int64_t g = y.a0 + a;
+        st.x[g] = __ldcg(ea.xa + g);
+        st.y[g] = __ldcg(ea.ya + g);
+        st.z[g] = __ldcg(ea.za + g);
     }
 }
 
@@ -427,19 +582,9 @@ __device__ void run_one_system(const BatchSys& y, const BatchState& st, const Pa
 // No task waits for anything: the scheduler only hands out tasks of phases that are ready.
 // Data written by one task and read by another goes through L2 (__ldcg), never through a
 // CTA's L1.
-enum { ST_BIN = 0, ST_SCAN = 1, ST_SCAT = 2, ST_SORT = 3, ST_LIST = 4, ST_FORCE = 5 };
+enum { ST_BIN = 0, ST_SCAN = 1, ST_SCAT = 2, ST_SORT = 3, ST_LIST = 4, ST_FORCE = 5, ST_KICK = 6 };
 
 __device__ __forceinline__ uint32_t ens_p_end(int K) { return 8u * (uint32_t)(K + 1); }  // FINAL; ESUM after it
-
-__device__ __forceinline__ bool ens_fp64_pair_test(const double* __restrict__ x, const double* __restrict__ y,
-                                                   const double* __restrict__ z, const EnsBlockSys& s, int64_t i,
-                                                   int64_t j, double r2max) {
-    const double dx = mic_rn(__dsub_rn(__ldcg(x + i), __ldcg(x + j)), s.L[0]);
-    const double dy = mic_rn(__dsub_rn(__ldcg(y + i), __ldcg(y + j)), s.L[1]);
-    const double dz = mic_rn(__dsub_rn(__ldcg(z + i), __ldcg(z + j)), s.L[2]);
-    const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-    return r2 < r2max;
-}
 
 // Wrap one coordinate into [0, L) (one box length at most, counted in the image counter)
 // and return its cell index; out-of-box or non-finite coordinates set *bad.
@@ -454,14 +599,6 @@ __device__ __forceinline__ int ens_wrap_cell(double& x, int32_t& img, double L, 
     if (!(x >= 0.0 && x <= L)) bad |= isfinite(x) ? ERR_ESCAPE : ERR_NONFINITE;
     const int c = (int)(x * inv_w);
     return c < 0 ? 0 : (c >= nc ? nc - 1 : c);
-}
-
-struct PosBuf {
-    double *x, *y, *z;
-};
-
-__device__ __forceinline__ PosBuf ens_pos(const BatchState& st, const EnsArrays& ea, bool odd) {
-    return odd ? PosBuf{ea.xa, ea.ya, ea.za} : PosBuf{st.x, st.y, st.z};
 }
 
 // BIN: wrap the positions of the odd / even buffer in place, cells and counts.
@@ -681,7 +818,7 @@ __device__ void ens_list(const EnsBlockSys& y, const BatchState& st, const EnsAr
                     const int sl = ens_slot_of(mt, u);
                     const int64_t gi = y.a0 + __ldcg(ea.perm_s + y.a0 + slot0 + own);
                     const int64_t gj = y.a0 + __ldcg(ea.perm_s + y.a0 + mt.start[sl] + (u - mt.prefix[sl]));
-                    return ens_fp64_pair_test(P.x, P.y, P.z, y, gi, gj, ea.rl2);
+                    return ens_fp64_pair_test<true>(P.x, P.y, P.z, y.L[0], y.L[1], y.L[2], gi, gj, ea.rl2);
                 });
             if (lane < own_n) {
                 if (cnt > cap) atomicOr(st.err, ERR_LIST_OVERFLOW);
@@ -873,7 +1010,7 @@ __device__ void ens_force(const EnsBlockSys& y, const BatchState& st, const EnsA
             if (!(r2 < pt.rc2lo_f[0])) {
                 const int sl = ens_slot_of(mt, q);
                 const int64_t gj = y.a0 + __ldcg(ea.perm_s + y.a0 + mt.start[sl] + (q - mt.prefix[sl]));
-                if (!ens_fp64_pair_test(P.x, P.y, P.z, y, gi, gj, pt.rc2_d[0])) continue;
+                if (!ens_fp64_pair_test<true>(P.x, P.y, P.z, y.L[0], y.L[1], y.L[2], gi, gj, pt.rc2_d[0])) continue;
             }
             const float inv = rcp_approx(r2);
             const float inv2 = __fmul_rn(inv, inv);
@@ -893,7 +1030,8 @@ __device__ void ens_force(const EnsBlockSys& y, const BatchState& st, const EnsA
     }
 }
 
-__device__ void ens_esum(const EnsBlockSys& y, const BatchState& st, const EnsArrays& ea, const PairTable& pt,
+template <typename Sys>
+__device__ void ens_esum(const Sys& y, const BatchState& st, const EnsArrays& ea, const PairTable& pt,
                          double* pe_out, double* ke_out, double* red) {
     double pe = 0.0, ke = 0.0;
     const double m = pt.mass[0];
@@ -918,6 +1056,7 @@ __device__ __forceinline__ int ens_ntasks(const EnsEntry& e, uint32_t p, int K) 
     const uint32_t pe = ens_p_end(K);
     if (p == pe) return e.n_atom_chunks;  // FINAL
     if (p == pe + 1) return 1;             // ESUM
+    if (e.kind == 2) return (p & 7) == ST_BIN ? 1 : e.n_atom_chunks;  // FORCE, KICK
     switch (p & 7) {
         case ST_BIN: return e.n_atom_chunks;
         case ST_SCAN: return 1;
@@ -932,6 +1071,15 @@ __device__ __forceinline__ uint32_t ens_next_phase(const EnsEntry& e, uint32_t p
                                                   const EnsArrays& ea) {
     if (e.kind == 0) return ENS_DONE;
     const uint32_t pe = ens_p_end(K);
+    if (e.kind == 2) {
+        if (p == ENS_START) return (flags & BATCH_HAVE_FORCES) && K > 0 ? ST_KICK : ST_BIN;
+        if (p == pe) return (flags & BATCH_ENERGY) ? pe + 1 : ENS_DONE;
+        if (p == pe + 1) return ENS_DONE;
+        const uint32_t k = p >> 3;
+        if ((p & 7) == ST_BIN) return 8u * k + ST_FORCE;
+        if ((p & 7) == ST_FORCE && (int)k == K) return (K & 1) ? pe : ((flags & BATCH_ENERGY) ? pe + 1 : ENS_DONE);
+        return 8u * (k + 1) + ST_BIN;
+    }
     volatile int* rebuild = ea.rebuild + e.idx;
     volatile int* valid = ea.valid + e.idx;
     if (p == ENS_START) {
@@ -1059,8 +1207,28 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS, 1)
         const EnsEntry en = ent[e];
         for (int task = task0; task < task0 + take; ++task) {
             if (en.kind == 0) {
-                run_one_system(one[en.idx], st, pt, K, flags, dt, fs2_max, nmax, cmax, ea.pe_atom, pe_out, ke_out, smem,
+                run_one_system(one[en.idx], st, ea, pt, K, flags, dt, fs2_max, nmax, cmax, pe_out, ke_out, smem,
                                warp_tot, &nqueued, red);
+            } else if (en.kind == 2) {
+                const BatchSys& y = one[en.idx];
+                const uint32_t pend = ens_p_end(K);
+                const int k = (int)(p >> 3);
+                Smem sm;
+                if (!batch_smem(y, st, nmax, cmax, smem, warp_tot, &nqueued, sm) || p == ENS_START) {
+                    // flagged, or only the decision of ens_next_phase
+                } else if (p == pend) {
+                    shared_final(y, st, ea, task);
+                } else if (p == pend + 1) {
+                    ens_esum(y, st, ea, pt, pe_out, ke_out, red);
+                } else if ((p & 7) == ST_BIN) {
+                    shared_bin(y, st, ea, (k & 1) != 0, sm);
+                } else if ((p & 7) == ST_KICK) {
+                    shared_kick(y, st, ea, pt, K, dt, task);
+                } else if (energy_call && k == K) {
+                    shared_force<true>(y, st, ea, pt, fs2_max, k, K, dt, task, sm);
+                } else {
+                    shared_force<false>(y, st, ea, pt, fs2_max, k, K, dt, task, sm);
+                }
             } else {
                 const EnsBlockSys& y = blk[en.idx];
                 const uint32_t pend = ens_p_end(K);

@@ -18,6 +18,7 @@ struct BatchSys {
     int nc[3];         // cells per dimension, each at least r_cut / R wide
     int ncell;
     int R;             // neighbour range in cells
+    int64_t s0;        // first of its ncell + 1 cell starts in cstart1 (a shared system)
     double L[3], w[3], inv_w[3];
     float wf[3];       // cell width in FP32 (the shift of a neighbour cell)
 };
@@ -38,7 +39,8 @@ struct EnsBlockSys {
 
 // One entry of the launch's work table: a system and the task counts of its phases.
 struct EnsEntry {
-    int kind;          // 0: one CTA for the whole call (BatchSys), 1: block tasks (EnsBlockSys)
+    int kind;          // 0: one CTA for the whole call (BatchSys), 1: block tasks (EnsBlockSys),
+                       // 2: the one-CTA operations shared out as tasks (BatchSys)
     int idx;           // index into the BatchSys or EnsBlockSys array
     int n_atom_chunks, n_cell_chunks, nblock;
 };
@@ -71,6 +73,7 @@ struct EnsArrays {
     float rl2_lo, rl2_hi;        // r_list^2 (1 -/+ 1e-4): candidates in between are re-tested in FP64
     int32_t *count, *cursor;     // cells of all block systems
     int32_t* cstart;             // cells + one per block system
+    int32_t* cstart1;            // cell starts of the shared systems
     float* pe_atom;              // ntot: half pair energies per atom (energy calls)
     unsigned long long* ctl;     // per entry: (phase << 32) | next task
     int32_t* done;               // per entry: tasks of the current phase completed
@@ -79,6 +82,7 @@ struct EnsArrays {
 };
 
 constexpr int ENS_ATOM_CHUNK = 2048;  // atoms per binning / scatter / wrap task
+constexpr int ENS_SHARED_CHUNK = 512; // atoms per task of a shared system
 constexpr int ENS_CELL_CHUNK = 64;    // cells per in-cell ordering task
 constexpr uint32_t ERR_TIMEOUT = 64u; // a CTA found no work for longer than its budget
 constexpr uint32_t ENS_DONE = 0xffffffffu, ENS_HOLD = 0xfffffffeu, ENS_START = 0xfffffffdu;
