@@ -520,7 +520,7 @@ int md_batch_create(int32_t n_systems, const int64_t* n_atoms, const double* box
         (rc = balloc(b, &b->d_pe, ns)) || (rc = balloc(b, &b->d_ke, ns)) || (rc = balloc(b, &b->d_aos, 3 * nt)) ||
         (rc = balloc(b, &ea.xa, nt)) || (rc = balloc(b, &ea.ya, nt)) || (rc = balloc(b, &ea.za, nt)) ||
         (rc = balloc(b, &ea.cell_of, nt)) || (rc = balloc(b, &ea.perm_u, nt)) || (rc = balloc(b, &ea.perm_s, nt)) ||
-        (rc = balloc(b, &ea.scell, nt)) || (rc = balloc(b, &ea.xs, nt)) || (rc = balloc(b, &ea.xsb, nt)) ||
+        (rc = balloc(b, &ea.xs, nt)) || (rc = balloc(b, &ea.xsb, nt)) ||
         (rc = balloc(b, &ea.xs_ref, nt)) || (rc = balloc(b, &ea.nl_cnt, nt)) ||
         (rc = balloc(b, &ea.nl, nt * (size_t)ea.list_chunks)) || (rc = balloc(b, &ea.rebuild, ns)) ||
         (rc = balloc(b, &ea.valid, ns)) || (rc = balloc(b, &b->d_sys_of, nt)) || (rc = balloc(b, &b->d_box, 3 * ns)) ||

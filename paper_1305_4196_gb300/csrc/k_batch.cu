@@ -186,13 +186,32 @@ __device__ __forceinline__ bool ens_fp64_pair_test(const double* __restrict__ x,
     return r2 < r2max;
 }
 
-// Exact force on the atom of slot p, one candidate at a time: a pair whose FP32 r^2 lies in
+// Exact force on the atom of slot p by a warp, its lanes over the candidates of a cell: a pair whose FP32 r^2 lies in
 // the band around r_cut^2 is decided in FP64 by the definition, a large term is rounded in
 // FP64 (fix_term_wide); every other term is the one the packed loop would add.
 struct ExactForce {
     long long qx, qy, qz;
     float pe;
 };
+
+// The lanes' exact sums, added up on every lane.
+__device__ __forceinline__ void warp_sum(long long& qx, long long& qy, long long& qz, int& nwide) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        qx += __shfl_xor_sync(0xffffffffu, qx, o);
+        qy += __shfl_xor_sync(0xffffffffu, qy, o);
+        qz += __shfl_xor_sync(0xffffffffu, qz, o);
+    }
+    nwide = (int)__reduce_add_sync(0xffffffffu, (unsigned)nwide);
+}
+
+// pe + a b of lane 0, then of lane 1, ... (FP32 sums keep the order of their terms)
+__device__ __forceinline__ float warp_sum_in_order(float pe, float a, float b) {
+#pragma unroll 4
+    for (int l = 0; l < 32; ++l)
+        pe = __fmaf_rn(__shfl_sync(0xffffffffu, a, l), __shfl_sync(0xffffffffu, b, l), pe);
+    return pe;
+}
 
 // Atom of slot p of a system, from the arrays of this CTA or those of the launch.
 template <bool SHARED>
@@ -220,27 +239,34 @@ __device__ __noinline__ ExactForce batch_force_exact(const BatchSys& y, const Ba
                                y.nc[0] * (wrap_cell(cy + dy, y.nc[1]) + y.nc[1] * wrap_cell(cz + dz, y.nc[2]));
                 const float sx = (float)dx * y.wf[0], sy = (float)dy * y.wf[1], sz = (float)dz * y.wf[2];
                 const int q1 = sm.cstart[id + 1];
-                for (int q = sm.cstart[id]; q < q1; ++q) {
-                    if (q == p) continue;
-                    const float ex = xi - (sm.px[q] + sx), ey = yi - (sm.py[q] + sy), ez = zi - (sm.pz[q] + sz);
-                    const float r2 = fmaf(ez, ez, fmaf(ey, ey, ex * ex));
-                    if (!(r2 < pt.rc2hi_f[0])) continue;
-                    if (!(r2 < pt.rc2lo_f[0]) &&
-                        !ens_fp64_pair_test<SHARED>(P.x, P.y, P.z, y.L[0], y.L[1], y.L[2], g,
-                                                    y.a0 + slot_atom<SHARED>(y, ea, sm, q), pt.rc2_d[0]))
-                        continue;
-                    const float inv = rcp_approx(r2);
-                    const float s2 = sig2 * inv;
-                    const float s6 = s2 * s2 * s2;
-                    const float fs2 = __fmul_rn(__fmul_rn(__fmaf_rn(c48, s6, -c24), s6), inv);  // (|f|/r) * 2^11
-                    qx += fix_term_any(fs2, ex, fs2_max, st.err);
-                    qy += fix_term_any(fs2, ey, fs2_max, st.err);
-                    qz += fix_term_any(fs2, ez, fs2_max, st.err);
-                    nwide += fabsf(fs2) < fs2_max ? 0 : 1;
-                    if (ENERGY) pe += c4 * s6 * (s6 - 1.0f);
+                for (int q0 = sm.cstart[id]; q0 < q1; q0 += 32) {
+                    const int q = q0 + ((int)threadIdx.x & 31);
+                    float ea0 = 0.f, ea1 = 0.f;  // factors of this lane's pair energy
+                    if (q < q1 && q != p) {
+                        const float ex = xi - (sm.px[q] + sx), ey = yi - (sm.py[q] + sy), ez = zi - (sm.pz[q] + sz);
+                        const float r2 = fmaf(ez, ez, fmaf(ey, ey, ex * ex));
+                        bool in = r2 < pt.rc2hi_f[0];
+                        if (in && !(r2 < pt.rc2lo_f[0]))
+                            in = ens_fp64_pair_test<SHARED>(P.x, P.y, P.z, y.L[0], y.L[1], y.L[2], g,
+                                                            y.a0 + slot_atom<SHARED>(y, ea, sm, q), pt.rc2_d[0]);
+                        if (in) {
+                            const float inv = rcp_approx(r2);
+                            const float s2 = sig2 * inv;
+                            const float s6 = s2 * s2 * s2;
+                            const float fs2 = __fmul_rn(__fmul_rn(__fmaf_rn(c48, s6, -c24), s6), inv);  // (|f|/r) * 2^11
+                            qx += fix_term_any(fs2, ex, fs2_max, st.err);
+                            qy += fix_term_any(fs2, ey, fs2_max, st.err);
+                            qz += fix_term_any(fs2, ez, fs2_max, st.err);
+                            nwide += fabsf(fs2) < fs2_max ? 0 : 1;
+                            ea0 = __fmul_rn(c4, s6);
+                            ea1 = __fsub_rn(s6, 1.0f);
+                        }
+                    }
+                    if (ENERGY) pe = warp_sum_in_order(pe, ea0, ea1);
                 }
             }
-    fix_wide_count_ok(nwide, st.err);
+    warp_sum(qx, qy, qz, nwide);
+    if ((threadIdx.x & 31) == 0) fix_wide_count_ok(nwide, st.err);
     return ExactForce{qx, qy, qz, pe};
 }
 
@@ -323,10 +349,10 @@ __device__ __forceinline__ void batch_forces(const BatchSys& y, const BatchState
     }
     __syncthreads();
     const int nq = *sm.nqueued;
-    for (int k = threadIdx.x; k < nq; k += blockDim.x) {
+    for (int k = threadIdx.x >> 5; k < nq; k += blockDim.x >> 5) {
         const int p = sm.queue[k];
         const ExactForce e = batch_force_exact<ENERGY, SHARED>(y, st, ea, P, pt, fs2_max, sm, p);
-        done(p, slot_atom<SHARED>(y, ea, sm, p), e.qx, e.qy, e.qz, e.pe);
+        if ((threadIdx.x & 31) == 0) done(p, slot_atom<SHARED>(y, ea, sm, p), e.qx, e.qy, e.qz, e.pe);
     }
 }
 
@@ -684,7 +710,6 @@ __device__ void ens_sort(const EnsBlockSys& y, const BatchState& st, const EnsAr
             const int64_t g = y.a0 + mine;
             const int64_t sl = y.a0 + s0 + rank;
             ea.perm_s[sl] = mine;
-            ea.scell[sl] = c;
             const float4 q = make_float4(__double2float_rn(__ldcg(P.x + g) - ox), __double2float_rn(__ldcg(P.y + g) - oy),
                                          __double2float_rn(__ldcg(P.z + g) - oz), 0.0f);
             xs[sl] = q;
@@ -742,33 +767,29 @@ __device__ void ens_meta(const EnsBlockSys& y, const EnsArrays& ea, int b, EnsTi
     __syncthreads();
 }
 
-// Fill the tile of block b from the FP32 coordinates xs (by slot) in the frame of the block;
-// returns the tile size T, or -1 if it exceeds tile_slots.  Ends with __syncthreads.
-__device__ int ens_stage(const EnsBlockSys& y, const EnsArrays& ea, const float4* xs, int b, int tile_slots,
-                         float4* tile, EnsTile& mt, uint32_t* err) {
-    ens_meta(y, ea, b, mt);
-    const int T = mt.prefix[64];
-    if (T + 1 > tile_slots) {
-        if (threadIdx.x == 0) atomicOr(err, ERR_TILE_OVERFLOW);
-        return -1;
-    }
+// Fill the tile of a block (meta mt) from the FP32 coordinates xs (by slot) in the frame of the
+// block.  All threads over the tile's atoms, four at a time with their cells found by branch-free
+// searches, so that the L2 loads of a task overlap.  Ends with __syncthreads.
+__device__ __forceinline__ void ens_stage(const EnsBlockSys& y, const float4* __restrict__ xs, float4* tile,
+                                          const EnsTile& mt) {
     TileOffsets to;
 #pragma unroll
     for (int d = 0; d < 3; ++d)
 #pragma unroll
         for (int q = 0; q < 4; ++q) to.off[d][q] = y.off[d][q];
-    // all threads over the tile's atoms (its cell by binary search), so that the L2 loads of
-    // a task overlap
+    const int T = mt.prefix[64];
+#pragma unroll 4
     for (int u = threadIdx.x; u < T; u += blockDim.x) {
-        const int sl = ens_slot_of(mt, u);
+        int sl = 0;
+#pragma unroll
+        for (int h = 32; h > 0; h >>= 1) sl += mt.prefix[sl + h] <= u ? h : 0;
         const int c = mt.coord[sl];
         const float ox = pick4(to.off[0], c & 3), oy = pick4(to.off[1], (c >> 2) & 3), oz = pick4(to.off[2], c >> 4);
-        const float4 p = __ldcg(xs + y.a0 + mt.start[sl] + (u - mt.prefix[sl]));
+        const float4 p = __ldcg(xs + mt.start[sl] + (u - mt.prefix[sl]));
         tile[u] = make_float4(p.x + ox, p.y + oy, p.z + oz, 0.0f);
     }
     if (threadIdx.x == 0) tile[T] = make_float4(1.0e4f, 1.0e4f, 1.0e4f, 0.0f);
     __syncthreads();
-    return T;
 }
 
 // Shared memory of a LIST task: the scan's buffers and the tile of T atoms.  The host sizes the
@@ -832,11 +853,12 @@ __device__ void ens_list(const EnsBlockSys& y, const BatchState& st, const EnsAr
 // loads overlap it.
 struct AtomState {
     double vx, vy, vz, x, y, z;
+    float4 ref;
 };
 
 __device__ __forceinline__ AtomState ens_load_state(const BatchState& st, const EnsArrays& ea, int k, int K,
-                                                    int64_t g) {
-    AtomState a{0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+                                                    int64_t g, int64_t sl) {
+    AtomState a{0.0, 0.0, 0.0, 0.0, 0.0, 0.0, make_float4(0.f, 0.f, 0.f, 0.f)};
     if (K == 0) return a;
     a.vx = __ldcg(st.vx + g);
     a.vy = __ldcg(st.vy + g);
@@ -846,15 +868,25 @@ __device__ __forceinline__ AtomState ens_load_state(const BatchState& st, const 
         a.x = __ldcg(P.x + g);
         a.y = __ldcg(P.y + g);
         a.z = __ldcg(P.z + g);
+        a.ref = __ldcg(ea.xs_ref + sl);
     }
     return a;
 }
 
-// Velocity Verlet for one own atom (slot, atom g, state a) after its force at step k of K.
+// Centres of a block's own cells (x, y, z of each), by the block's first threads.
+__device__ __forceinline__ void ens_centres(const EnsBlockSys& y, int b, double (&centre)[8][3]) {
+    if (threadIdx.x < 24) {
+        const int os = threadIdx.x / 3, d = threadIdx.x % 3;
+        const int bd = d == 0 ? b % y.nb[0] : (d == 1 ? (b / y.nb[0]) % y.nb[1] : b / (y.nb[0] * y.nb[1]));
+        centre[os][d] = (2 * bd + ((os >> d) & 1) + 0.5) * y.w[d];
+    }
+}
+
+// Velocity Verlet for one own atom (slot of own cell os, atom g, state a) after its force at step k of K.
 __device__ __forceinline__ void ens_epilogue(const EnsBlockSys& y, const BatchState& st, const EnsArrays& ea,
                                              const PairTable& pt, int k, int K, bool energy, double dt, int slot,
                                              int64_t g, long long qx, long long qy, long long qz, float pe,
-                                             int bidx, const AtomState& a) {
+                                             int bidx, const AtomState& a, const double (&centre)[3]) {
     if (k == K) {
         st.fq[g] = qx;
         st.fq[st.ntot + g] = qy;
@@ -887,34 +919,41 @@ __device__ __forceinline__ void ens_epilogue(const EnsBlockSys& y, const BatchSt
     Pn.y[g] = yv;
     Pn.z[g] = z;
     const int64_t sl = y.a0 + slot;
-    const int c = __ldcg(ea.scell + sl);
-    const int cx = c % y.nc[0], cy = (c / y.nc[0]) % y.nc[1], cz = c / (y.nc[0] * y.nc[1]);
-    const float4 q = make_float4(__double2float_rn(x - (cx + 0.5) * y.w[0]), __double2float_rn(yv - (cy + 0.5) * y.w[1]),
-                                 __double2float_rn(z - (cz + 0.5) * y.w[2]), 0.0f);
+    const float4 q = make_float4(__double2float_rn(x - centre[0]), __double2float_rn(yv - centre[1]),
+                                 __double2float_rn(z - centre[2]), 0.0f);
     (odd ? ea.xs : ea.xsb)[sl] = q;
-    const float4 r = __ldcg(ea.xs_ref + sl);
+    const float4 r = a.ref;
     const float ex = q.x - r.x, ey = q.y - r.y, ez = q.z - r.z;
     if (!(fmaf(ez, ez, fmaf(ey, ey, ex * ex)) <= ea.lim2_f)) ea.rebuild[bidx] = 1;
 }
 
 // Chunks 0 .. nch-1 of one list (chunk c at lp[c * stride]), two entries per call of body;
 // the chunks were written by other CTAs of the launch, so they are read from L2, two chunks
-// ahead of their use (a task holds few warps, so load latency is not hidden by others).
-template <typename Body>
-__device__ __forceinline__ void ens_for_each_pair(const uint4* __restrict__ lp, size_t stride, int nch, Body&& body) {
-    uint4 cur = make_uint4(0u, 0u, 0u, 0u), n1 = cur, n2 = cur;
-    if (nch > 0) cur = __ldcg(lp);
-    if (nch > 1) n1 = __ldcg(lp + stride);
-    for (int c = 0; c < nch; ++c) {
-        if (c + 2 < nch) n2 = __ldcg(lp + (size_t)(c + 2) * stride);
-        body((int)(cur.x & 0xffffu), (int)(cur.x >> 16));
-        body((int)(cur.y & 0xffffu), (int)(cur.y >> 16));
-        body((int)(cur.z & 0xffffu), (int)(cur.z >> 16));
-        body((int)(cur.w & 0xffffu), (int)(cur.w >> 16));
-        cur = n1;
-        n1 = n2;
+// ahead of their use (a task holds few warps, so load latency is not hidden by others), the first
+// two (of `chunks` that exist) before the length is known.
+struct EnsList {
+    const uint4* lp;
+    size_t stride;
+    uint4 c0, c1;
+    __device__ __forceinline__ EnsList(const uint4* lp_, size_t stride_, int chunks) : lp(lp_), stride(stride_) {
+        c0 = c1 = make_uint4(0u, 0u, 0u, 0u);
+        if (chunks > 0) c0 = __ldcg(lp);
+        if (chunks > 1) c1 = __ldcg(lp + stride);
     }
-}
+    template <typename Body>
+    __device__ __forceinline__ void walk(int nch, Body&& body) {
+        uint4 cur = c0, n1 = c1, n2 = c1;
+        for (int c = 0; c < nch; ++c) {
+            if (c + 2 < nch) n2 = __ldcg(lp + (size_t)(c + 2) * stride);
+            body((int)(cur.x & 0xffffu), (int)(cur.x >> 16));
+            body((int)(cur.y & 0xffffu), (int)(cur.y >> 16));
+            body((int)(cur.z & 0xffffu), (int)(cur.z >> 16));
+            body((int)(cur.w & 0xffffu), (int)(cur.w >> 16));
+            cur = n1;
+            n1 = n2;
+        }
+    }
+};
 
 // FORCE of block b at step k.  The pair step is the main path's one-species form: fs2 =
 // inv^4 (a inv^3 - b) with inv = 1/r^2, and the cutoff-band and large-force tests as two
@@ -923,23 +962,40 @@ template <bool ENERGY>
 __device__ void ens_force(const EnsBlockSys& y, const BatchState& st, const EnsArrays& ea, const PairTable& pt,
                           float fs2_max, int k, int K, double dt, int b, int bidx, int tile_slots, float4* tile,
                           EnsTile& mt, uint16_t* queue, int* nqueued) {
+    __shared__ double centre[8][3];
     const bool odd = (k & 1) != 0;
     if (threadIdx.x == 0) *nqueued = 0;
-    const int T = ens_stage(y, ea, odd ? ea.xsb : ea.xs, b, tile_slots, tile, mt, st.err);
-    if (T < 0) return;
+    ens_meta(y, ea, b, mt);
+    if (mt.prefix[64] + 1 > tile_slots) {
+        if (threadIdx.x == 0) atomicOr(st.err, ERR_TILE_OVERFLOW);
+        return;
+    }
     const unsigned tile_s = (unsigned)__cvta_generic_to_shared(tile);
     const uint4* nl = ea.nl + y.a0 * (int64_t)ea.list_chunks;
-    for (int u = threadIdx.x; u < mt.prefix[8]; u += blockDim.x) {
+    bool staged = false;
+    for (int r = 0; r < mt.prefix[8]; r += blockDim.x) {
+        const int u = r + (int)threadIdx.x;
+        const bool active = u < mt.prefix[8];
         int os = 0;
-        while (os < 7 && u >= mt.prefix[os + 1]) ++os;
-        const int slot = mt.start[os] + (u - mt.prefix[os]);
-        const float4 pi = tile[u];
-        const int nch = (__ldcg(ea.nl_cnt + y.a0 + slot) + 7) >> 3;
+#pragma unroll
+        for (int h = 4; h > 0; h >>= 1) os += mt.prefix[os + h] <= u ? h : 0;
+        const int slot = active ? mt.start[os] + (u - mt.prefix[os]) : 0;
+        // the list, the atom and its state: on their way while the tile is staged
+        const int cnt = __ldcg(ea.nl_cnt + y.a0 + slot);
+        EnsList list(nl + slot, (size_t)y.n, active ? ea.list_chunks : 0);
         const int64_t g = y.a0 + __ldcg(ea.perm_s + y.a0 + slot);
-        const AtomState as = ens_load_state(st, ea, k, K, g);
+        if (!staged) {
+            ens_centres(y, b, centre);
+            ens_stage(y, (odd ? ea.xsb : ea.xs) + y.a0, tile, mt);
+            staged = true;
+        }
+        if (!active) continue;
+        const AtomState as = ens_load_state(st, ea, k, K, g, y.a0 + slot);
+        const float4 pi = tile[u];
+        const int nch = (cnt + 7) >> 3;
         FixAcc ax{0u, 0u}, ay{0u, 0u}, az{0u, 0u};
         float pe = 0.f, mdist = 3.0e38f, mr2 = 3.0e38f;
-        ens_for_each_pair(nl + slot, (size_t)y.n, nch, [&](int u0, int u1) {
+        list.walk(nch, [&](int u0, int u1) {
             const float4 pa = lds_tile(tile_s, u0);
             const float4 pb = lds_tile(tile_s, u1);
             const f2_t ex = f2_pack(__fsub_rn(pi.x, pa.x), __fsub_rn(pi.x, pb.x));
@@ -981,14 +1037,15 @@ __device__ void ens_force(const EnsBlockSys& y, const BatchState& st, const EnsA
         }
         const int nterms = nch * 8;
         ens_epilogue(y, st, ea, pt, k, K, ENERGY, dt, slot, g, fix_final(ax, nterms), fix_final(ay, nterms),
-                     fix_final(az, nterms), pe, bidx, as);
+                     fix_final(az, nterms), pe, bidx, as, centre[os]);
     }
     __syncthreads();
-    // the exact pass: every entry one at a time, the same FP32 operations for ordinary pairs,
-    // FP64 decisions in the cutoff band, large terms rounded in FP64
+    // the exact pass, a warp per atom: the same FP32 operations for ordinary pairs, FP64 decisions
+    // in the cutoff band, large terms rounded in FP64; energies added in list order
     const PosBuf P = ens_pos(st, ea, odd);
     const int nq = min(*nqueued, ENS_QUEUE);
-    for (int j = threadIdx.x; j < nq; j += blockDim.x) {
+    const int lane = threadIdx.x & 31;
+    for (int j = threadIdx.x >> 5; j < nq; j += blockDim.x >> 5) {
         const int u = queue[j];
         int os = 0;
         while (os < 7 && u >= mt.prefix[os + 1]) ++os;
@@ -999,34 +1056,42 @@ __device__ void ens_force(const EnsBlockSys& y, const BatchState& st, const EnsA
         long long qx = 0, qy = 0, qz = 0;
         float pe = 0.f;
         int nwide = 0;
-        for (int e = 0; e < cnt; ++e) {
-            const uint4 ch = __ldcg(nl + (int64_t)(e >> 3) * y.n + slot);
-            const unsigned w = (e & 7) < 4 ? ((e & 7) < 2 ? ch.x : ch.y) : ((e & 7) < 6 ? ch.z : ch.w);
-            const int q = (int)((w >> (16 * (e & 1))) & 0xffffu);
-            const float4 pj = tile[q];
-            const float ex = __fsub_rn(pi.x, pj.x), ey = __fsub_rn(pi.y, pj.y), ez = __fsub_rn(pi.z, pj.z);
-            const float r2 = fmaf(ez, ez, fmaf(ey, ey, ex * ex));
-            if (!(r2 < pt.rc2hi_f[0])) continue;
-            if (!(r2 < pt.rc2lo_f[0])) {
-                const int sl = ens_slot_of(mt, q);
-                const int64_t gj = y.a0 + __ldcg(ea.perm_s + y.a0 + mt.start[sl] + (q - mt.prefix[sl]));
-                if (!ens_fp64_pair_test<true>(P.x, P.y, P.z, y.L[0], y.L[1], y.L[2], gi, gj, pt.rc2_d[0])) continue;
+        for (int e0 = 0; e0 < cnt; e0 += 32) {
+            const int e = e0 + lane;
+            float ea0 = 0.f, ea1 = 0.f;  // factors of this lane's pair energy
+            if (e < cnt) {
+                const int q = __ldcg(reinterpret_cast<const unsigned short*>(nl + (int64_t)(e >> 3) * y.n + slot) + (e & 7));
+                const float4 pj = tile[q];
+                const float ex = __fsub_rn(pi.x, pj.x), ey = __fsub_rn(pi.y, pj.y), ez = __fsub_rn(pi.z, pj.z);
+                const float r2 = fmaf(ez, ez, fmaf(ey, ey, ex * ex));
+                bool in = r2 < pt.rc2hi_f[0];
+                if (in && !(r2 < pt.rc2lo_f[0])) {
+                    const int sl = ens_slot_of(mt, q);
+                    const int64_t gj = y.a0 + __ldcg(ea.perm_s + y.a0 + mt.start[sl] + (q - mt.prefix[sl]));
+                    in = ens_fp64_pair_test<true>(P.x, P.y, P.z, y.L[0], y.L[1], y.L[2], gi, gj, pt.rc2_d[0]);
+                }
+                if (in) {
+                    const float inv = rcp_approx(r2);
+                    const float inv2 = __fmul_rn(inv, inv);
+                    const float inv3 = __fmul_rn(inv2, inv);
+                    const float fs2 = __fmul_rn(__fmaf_rn(pt.lj_a_f, inv3, -pt.lj_b_f), __fmul_rn(inv2, inv2));
+                    qx += fix_term_any(fs2, ex, fs2_max, st.err);
+                    qy += fix_term_any(fs2, ey, fs2_max, st.err);
+                    qz += fix_term_any(fs2, ez, fs2_max, st.err);
+                    nwide += fabsf(fs2) < fs2_max ? 0 : 1;
+                    const float s6 = __fmul_rn(pt.sig6_f, inv3);
+                    ea0 = __fmul_rn(pt.c4_f[0], s6);
+                    ea1 = __fsub_rn(s6, 1.0f);
+                }
             }
-            const float inv = rcp_approx(r2);
-            const float inv2 = __fmul_rn(inv, inv);
-            const float inv3 = __fmul_rn(inv2, inv);
-            const float fs2 = __fmul_rn(__fmaf_rn(pt.lj_a_f, inv3, -pt.lj_b_f), __fmul_rn(inv2, inv2));
-            qx += fix_term_any(fs2, ex, fs2_max, st.err);
-            qy += fix_term_any(fs2, ey, fs2_max, st.err);
-            qz += fix_term_any(fs2, ez, fs2_max, st.err);
-            nwide += fabsf(fs2) < fs2_max ? 0 : 1;
-            if (ENERGY) {
-                const float s6 = __fmul_rn(pt.sig6_f, inv3);
-                pe += pt.c4_f[0] * s6 * (s6 - 1.0f);
-            }
+            if (ENERGY) pe = warp_sum_in_order(pe, ea0, ea1);
         }
-        fix_wide_count_ok(nwide, st.err);
-        ens_epilogue(y, st, ea, pt, k, K, ENERGY, dt, slot, gi, qx, qy, qz, pe, bidx, ens_load_state(st, ea, k, K, gi));
+        warp_sum(qx, qy, qz, nwide);
+        if (lane == 0) {
+            fix_wide_count_ok(nwide, st.err);
+            ens_epilogue(y, st, ea, pt, k, K, ENERGY, dt, slot, gi, qx, qy, qz, pe, bidx,
+                         ens_load_state(st, ea, k, K, gi, y.a0 + slot), centre[os]);
+        }
     }
 }
 

@@ -59,7 +59,6 @@ struct EnsArrays {
     double *xa, *ya, *za;        // second position buffer (ntot)
     int32_t* cell_of;            // ntot: an atom's cell for the next binning
     int32_t *perm_u, *perm_s;    // ntot: slot -> atom within its system (unordered / ordered in a cell)
-    int32_t* scell;              // ntot: slot -> cell
     float4 *xs, *xsb;            // ntot: FP32 coordinates relative to the slot's build cell centre,
                                  // by slot, for even / odd steps
     float4* xs_ref;              // ntot: the same at the last build (skin/2 test)
