@@ -271,8 +271,8 @@ __device__ __noinline__ ExactForce batch_force_exact(const BatchSys& y, const Ba
 }
 
 // Force on the atoms of slots lo .. hi - 1 (to done(slot, atom, force, pair energy)); with energy,
-// also its pair energies (FP32 per atom, neighbours in slot order: deterministic).  Two candidates per step:
-// the pair (q, q+1) with q even, masked to the cell's range and away from the atom itself.
+// also its pair energies (FP32 per atom, neighbours in slot order: deterministic).  Candidates are
+// taken as pairs (q, q+1) with q even, masked to the cell's range and away from the atom itself.
 template <bool ENERGY, bool SHARED, typename Done>
 __device__ __forceinline__ void batch_forces(const BatchSys& y, const BatchState& st, const EnsArrays& ea,
                                              const PosBuf& P, const PairTable& pt, float fs2_max, Smem& sm, int lo,
@@ -304,40 +304,49 @@ __device__ __forceinline__ void batch_forces(const BatchSys& y, const BatchState
                     const float sxf = (float)dx * y.wf[0], syf = (float)dy * y.wf[1], szf = (float)dz * y.wf[2];
                     const f2_t sx = f2_pack(sxf, sxf), sy = f2_pack(syf, syf), sz = f2_pack(szf, szf);
                     const int c0 = sm.cstart[id], c1 = sm.cstart[id + 1];
-                    for (int q = c0 & ~1; q < c1; q += 2) {
-                        f2_t X, Y, Z;
-                        asm volatile("ld.shared.b64 %0, [%1];" : "=l"(X) : "r"(spx + 4u * (unsigned)q));
-                        asm volatile("ld.shared.b64 %0, [%1];" : "=l"(Y) : "r"(spy + 4u * (unsigned)q));
-                        asm volatile("ld.shared.b64 %0, [%1];" : "=l"(Z) : "r"(spz + 4u * (unsigned)q));
-                        const f2_t ex = f2_sub(pix, f2_add(X, sx));
-                        const f2_t ey = f2_sub(piy, f2_add(Y, sy));
-                        const f2_t ez = f2_sub(piz, f2_add(Z, sz));
-                        const f2_t r2 = f2_fma(ez, ez, f2_fma(ey, ey, f2_mul(ex, ex)));
-                        float r2a, r2b;
-                        f2_unpack(r2, r2a, r2b);
-                        const bool ina = (q >= c0) & (q != p) & (r2a < rc2_hi);
-                        const bool inb = (q + 1 < c1) & (q + 1 != p) & (r2b < rc2_hi);
-                        const f2_t inv = f2_pack(rcp_approx(r2a), rcp_approx(r2b));
-                        const f2_t s2 = f2_mul(sig2, inv);
-                        const f2_t s6 = f2_mul(f2_mul(s2, s2), s2);
-                        const f2_t fsv = f2_mul(f2_mul(f2_fma(c48, s6, nc24), s6), inv);
-                        float fa, fb;
-                        f2_unpack(fsv, fa, fb);
-                        fa = ina ? fa : 0.0f;
-                        fb = inb ? fb : 0.0f;
-                        bad |= (ina & !(r2a < rc2_lo)) | (inb & !(r2b < rc2_lo)) | !(fabsf(fa) < fs2_max) |
-                               !(fabsf(fb) < fs2_max);
-                        const f2_t fs2 = f2_pack(fa, fb);
-                        fix_add2(ax, fs2, ex, magic2, two21);
-                        fix_add2(ay, fs2, ey, magic2, two21);
-                        fix_add2(az, fs2, ez, magic2, two21);
-                        nterms += 2;
-                        nin += (int)ina + (int)inb;
-                        if (ENERGY) {
-                            float s6a, s6b;
-                            f2_unpack(s6, s6a, s6b);
-                            pe += (ina ? c4 * s6a * (s6a - 1.0f) : 0.0f) + (inb ? c4 * s6b * (s6b - 1.0f) : 0.0f);
+                    // two pairs of candidates at a time: their loads and chains overlap
+                    for (int q0 = c0 & ~1; q0 < c1; q0 += 4) {
+                        f2_t X[2], Y[2], Z[2];
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const unsigned at = 4u * (unsigned)(q0 + 2 * h < c1 ? q0 + 2 * h : q0);
+                            asm volatile("ld.shared.b64 %0, [%1];" : "=l"(X[h]) : "r"(spx + at));
+                            asm volatile("ld.shared.b64 %0, [%1];" : "=l"(Y[h]) : "r"(spy + at));
+                            asm volatile("ld.shared.b64 %0, [%1];" : "=l"(Z[h]) : "r"(spz + at));
                         }
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const int q = q0 + 2 * h;
+                            const f2_t ex = f2_sub(pix, f2_add(X[h], sx));
+                            const f2_t ey = f2_sub(piy, f2_add(Y[h], sy));
+                            const f2_t ez = f2_sub(piz, f2_add(Z[h], sz));
+                            const f2_t r2 = f2_fma(ez, ez, f2_fma(ey, ey, f2_mul(ex, ex)));
+                            float r2a, r2b;
+                            f2_unpack(r2, r2a, r2b);
+                            const bool ina = (h == 0 ? q >= c0 : q < c1) & (q != p) & (r2a < rc2_hi);
+                            const bool inb = (q + 1 < c1) & (q + 1 != p) & (r2b < rc2_hi);
+                            const f2_t inv = f2_pack(rcp_approx(r2a), rcp_approx(r2b));
+                            const f2_t s2 = f2_mul(sig2, inv);
+                            const f2_t s6 = f2_mul(f2_mul(s2, s2), s2);
+                            const f2_t fsv = f2_mul(f2_mul(f2_fma(c48, s6, nc24), s6), inv);
+                            float fa, fb;
+                            f2_unpack(fsv, fa, fb);
+                            fa = ina ? fa : 0.0f;
+                            fb = inb ? fb : 0.0f;
+                            bad |= (ina & !(r2a < rc2_lo)) | (inb & !(r2b < rc2_lo)) | !(fabsf(fa) < fs2_max) |
+                                   !(fabsf(fb) < fs2_max);
+                            const f2_t fs2 = f2_pack(fa, fb);
+                            fix_add2(ax, fs2, ex, magic2, two21);
+                            fix_add2(ay, fs2, ey, magic2, two21);
+                            fix_add2(az, fs2, ez, magic2, two21);
+                            nin += (int)ina + (int)inb;
+                            if (ENERGY) {
+                                float s6a, s6b;
+                                f2_unpack(s6, s6a, s6b);
+                                pe += (ina ? c4 * s6a * (s6a - 1.0f) : 0.0f) + (inb ? c4 * s6b * (s6b - 1.0f) : 0.0f);
+                            }
+                        }
+                        nterms += 4;
                     }
                 }
         bad |= nin > FIX_SPLIT_MAX_TERMS;  // the split sums could wrap: the exact 64-bit pass
