@@ -35,8 +35,10 @@ constexpr int FULL_THREADS = 256;  // CTA size of the full-list mixed kernel
 // Register cap of the full-list mixed kernel: 48 keeps 5 CTAs (40 warps) resident per SM.
 // The kernel is latency bound, and more resident warps beat longer per-thread schedules.
 #define MDGB_FULL_MAX_REGS 48
-// With several species the pair constants come from shared memory, and 48 registers spill.
-#define MDGB_FULL_MAX_REGS_SPECIES 64
+// With several species the pair constants come from shared memory, and 48 registers spill; so do the
+// seven sums of an energy and virial launch (1,048,576 atoms: 221 us at 48 registers, 182 at 56
+// and 64, 190 at 80).
+#define MDGB_FULL_MAX_REGS_WIDE 64
 // per-pair LJ in FP32: returns fs2 = (|f|/r) * 2^11 (not masked) and whether the FP32
 // r^2 is inside the cutoff
 template <bool SINGLE>
@@ -171,7 +173,7 @@ __device__ __forceinline__ void full_block(const DevState& s, const Geometry& g,
 }
 
 template <bool SINGLE, bool EV, int MODE>
-__global__ void __maxnreg__(SINGLE ? MDGB_FULL_MAX_REGS : MDGB_FULL_MAX_REGS_SPECIES) k_force_mixed_full(DevState s, Geometry g, PairTable pt,
+__global__ void __maxnreg__(SINGLE && !EV ? MDGB_FULL_MAX_REGS : MDGB_FULL_MAX_REGS_WIDE) k_force_mixed_full(DevState s, Geometry g, PairTable pt,
                                                                 TileOffsets to, int tile_cap, float fs2_max,
                                                                 StepOut out, double dt,
                                                                 float lim2_f) {
@@ -182,7 +184,7 @@ __global__ void __maxnreg__(SINGLE ? MDGB_FULL_MAX_REGS : MDGB_FULL_MAX_REGS_SPE
 // taking every gridDim-th entry of the list.  (A separate kernel: the loop in the
 // one-block kernel cost the dense case 10 % through its register allocation.)
 template <bool SINGLE, bool EV, int MODE>
-__global__ void __maxnreg__(SINGLE ? MDGB_FULL_MAX_REGS : MDGB_FULL_MAX_REGS_SPECIES) k_force_mixed_occ(DevState s, Geometry g, PairTable pt,
+__global__ void __maxnreg__(SINGLE && !EV ? MDGB_FULL_MAX_REGS : MDGB_FULL_MAX_REGS_WIDE) k_force_mixed_occ(DevState s, Geometry g, PairTable pt,
                                                                 TileOffsets to, int tile_cap, float fs2_max,
                                                                 StepOut out, double dt,
                                                                 float lim2_f) {
