@@ -13,15 +13,15 @@
 // operation, while it issues 64 others (the list and coordinates stream through with DRAM
 // nearly idle).  So the full-list kernel spends other instructions to save FP64 ones:
 //  * the list entries are tested in FP32 first, on the upper halves of the tile's coordinates,
-//    and only those that may lie inside the cutoff go to a queue in shared memory; the lanes
-//    of a warp then take their queues in step (a 76-entry list holds 55 inside, and the
-//    longest of 32 lanes about 62, where a masked loop runs all 80 padded entries);
+//    and only those that may lie inside the cutoff go to an atom's queue in shared memory; the
+//    lanes of a warp then take them in step, an atom's lanes side by side (a 76-entry list
+//    holds 55 inside, where a masked loop runs all 80 padded entries);
 //  * 17 FP64 operations per pair: three differences, three for r^2, one reciprocal by a cubic
 //    step from an FP32 seed (three), five for f / r = inv^4 (a inv^3 - b), three sums; the
 //    exact cutoff test compares bit patterns.
 // Every result is that of FP64 arithmetic throughout.  At 360,703 atoms a force evaluation took
 // 1.38 ms and one with energy and virial 2.11 ms with 22 operations for each of the 80 padded
-// entries, and takes 0.80 and 1.27 ms; the FP64 pipe is 87 % busy.
+// entries, and takes 0.78 and 1.25 ms; the FP64 pipe is 90 % busy.
 #include "fp64_math.cuh"
 #include "tile.cuh"
 
@@ -33,7 +33,7 @@ constexpr int F_THREADS = 256;
 static int g_sm_count = 0;  // SMs of the device, read at initialisation (never during a stream capture)
 
 // ---------------------------------------------------------------- full list
-constexpr int FQ = 16;  // queue slots per thread: up to 8 waiting and a chunk
+constexpr int FQ = 16;  // queue slots per lane; the lanes of an atom share theirs
 
 __host__ __device__ constexpr size_t fp64_queue_bytes(int threads) { return (size_t)threads * FQ * sizeof(uint16_t); }
 
@@ -79,7 +79,7 @@ __device__ __forceinline__ void fp64_pair(const PairTable& pt, const double* __r
     }
 }
 
-// LPA lanes per atom, lane q of them with chunks q, q + LPA, ... of the list; `split` CTAs share
+// LPA lanes per atom, which share its list and the queue of pairs to evaluate; `split` CTAs share
 // one block, each staging the tile and taking every split-th group of own atoms.  rc2_test: r_cut^2
 // plus the bound on the FP32 test's error, largest over the species pairs.  QUEUE = false evaluates
 // every entry (a tile that leaves no room for the queues).
@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(F_THREADS) k_force_fp64_full(DevState s, Geome
     double* ty = tx + tile_cap;
     double* tz = ty + tile_cap;
     int* tsp = reinterpret_cast<int*>(tz + tile_cap);
-    uint16_t* const queue = reinterpret_cast<uint16_t*>(tsp + tile_cap) + threadIdx.x;
+    uint16_t* const queues = reinterpret_cast<uint16_t*>(tsp + tile_cap);
     const int b = spatial_block(g, blockIdx.x / split), part = blockIdx.x % split;
     tile_meta(g, s.cell_start, b, m);
     const int T = m.prefix[64];
@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(F_THREADS) k_force_fp64_full(DevState s, Geome
     const int nown = m.prefix[8];
     const int per = blockDim.x / LPA;  // own atoms at a time
     if (part * per >= nown) return;
-    tile_stage_f64(s, g, m, b, tx, ty, tz, tsp);
+    tile_stage_f64(s, g, m, b, tx, ty, tz, tsp, split > 1 ? tile_needed(m, part, split, per) : TILE_ALL);
     __syncthreads();
     const int blk0 = m.start[0];
     const int64_t n = s.n;
@@ -119,40 +119,49 @@ __global__ void __launch_bounds__(F_THREADS) k_force_fp64_full(DevState s, Geome
         const uint4* lp = reinterpret_cast<const uint4*>(s.nl) + gi;
         Fp64Sums<EV> a;
         if (QUEUE) {
+            // The lanes of an atom share its queue, so that they evaluate the same number of pairs: lane q
+            // tests the list's words (two entries) q, q + LPA, ..., and takes every LPA-th pair.
+            constexpr int CAP = FQ * LPA;
+            constexpr unsigned GROUP = (1u << LPA) - 1u;
+            const int l0 = (int)(threadIdx.x & 31) & ~(LPA - 1);
+            const unsigned below = (1u << lq) - 1u;
+            uint16_t* const mine = queues + ((int)threadIdx.x - lq) * FQ;
+            const unsigned* const words = reinterpret_cast<const unsigned*>(s.nl) + (size_t)gi * 4;
+            const auto word = [&](int w) { return __ldcs(words + (size_t)(w >> 2) * np * 4 + (w & 3)); };
+            const int nw = nch * 4;
             const float xf = upper_f32(xi), yf = upper_f32(yi), zf = upper_f32(zi);
             int head = 0, tail = 0;
-            uint4 nxt = make_uint4(0u, 0u, 0u, 0u);
-            if (lq < nch) nxt = __ldcs(lp + (size_t)lq * np);
-            for (int c = lq; __any_sync(0xffffffffu, c < nch); c += LPA) {
-                const uint4 cur = nxt;
-                if (c + LPA < nch) nxt = __ldcs(lp + (size_t)(c + LPA) * np);
-                if (c < nch) {
-                    const unsigned wd[4] = {cur.x, cur.y, cur.z, cur.w};
+            const auto take = [&]() {
+                if (head + lq < tail)
+                    fp64_pair<SINGLE, EV>(pt, tx, ty, tz, tsp, mine[(head + lq) & (CAP - 1)], xi, yi, zi, si, a);
+                head = min(head + LPA, tail);
+            };
+            unsigned nxt = lq < nw ? word(lq) : 0u;
+            for (int w0 = 0; __any_sync(0xffffffffu, w0 < nw); w0 += LPA) {
+                const unsigned cur = nxt;
+                const int w = w0 + lq;
+                if (w + LPA < nw) nxt = word(w + LPA);
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        const int u = (int)((wd[e >> 1] >> ((e & 1) * 16)) & 0xffffu);
+                for (int h = 0; h < 2; ++h) {
+                    const int u = (int)((cur >> (16 * h)) & 0xffffu);
+                    bool near = false;
+                    if (w < nw) {
                         const float dx = xf - upper_f32(tx[u]), dy = yf - upper_f32(ty[u]), dz = zf - upper_f32(tz[u]);
-                        if (fmaf(dz, dz, fmaf(dy, dy, dx * dx)) < rc2_test) {
-                            queue[(tail & (FQ - 1)) * F_THREADS] = (uint16_t)u;
-                            ++tail;
-                        }
+                        near = fmaf(dz, dz, fmaf(dy, dy, dx * dx)) < rc2_test;
                     }
+                    const unsigned group = __ballot_sync(0xffffffffu, near) >> l0 & GROUP;
+                    if (near) mine[(tail + __popc(group & below)) & (CAP - 1)] = (uint16_t)u;
+                    tail += __popc(group);
                 }
-                // in step while every lane has an entry, or some lane too many for the next chunk
-                while (__any_sync(0xffffffffu, tail - head > FQ - 8) || __all_sync(0xffffffffu, tail > head)) {
-                    if (tail > head) {
-                        fp64_pair<SINGLE, EV>(pt, tx, ty, tz, tsp, queue[(head & (FQ - 1)) * F_THREADS], xi, yi, zi, si,
-                                              a);
-                        ++head;
-                    }
-                }
+                __syncwarp();
+                // in step while every atom has pairs for all its lanes, or some atom too many for the next words
+                while (__any_sync(0xffffffffu, tail - head > CAP - 2 * LPA) ||
+                       __all_sync(0xffffffffu, tail - head >= LPA))
+                    take();
+                __syncwarp();  // (before the next entries overwrite those just taken)
             }
-            while (__any_sync(0xffffffffu, tail > head)) {
-                if (tail > head) {
-                    fp64_pair<SINGLE, EV>(pt, tx, ty, tz, tsp, queue[(head & (FQ - 1)) * F_THREADS], xi, yi, zi, si, a);
-                    ++head;
-                }
-            }
+            while (__any_sync(0xffffffffu, tail > head)) take();
+            __syncwarp();
         } else {
             for (int c = lq; c < nch; c += LPA) {
                 const uint4 cur = __ldcs(lp + (size_t)c * np);
@@ -280,7 +289,6 @@ using Fp64Full = void (*)(DevState, Geometry, PairTable, int, int, float);
 template <bool SINGLE, bool EV, bool QUEUE>
 static Fp64Full full_of(int lpa) {
     switch (lpa) {
-        case 1: return k_force_fp64_full<SINGLE, EV, 1, QUEUE>;
         case 2: return k_force_fp64_full<SINGLE, EV, 2, QUEUE>;
         case 4: return k_force_fp64_full<SINGLE, EV, 4, QUEUE>;
         default: return k_force_fp64_full<SINGLE, EV, 8, QUEUE>;
@@ -311,18 +319,25 @@ void launch_forces_fp64(const DevState& s, const Geometry& g, const PairTable& p
     if (s.n == 0) return;
     const size_t smem = force_smem_bytes(0, half, with_energy, tile_cap);
     if (!half) {
-        // Lanes per atom and CTAs per block: more of both while the grid is below two CTAs per SM
-        // (4,000 atoms have 8 blocks: 197 us with 16 CTAs and one lane, 46 us with 128 and eight).
+        // CTAs per block: one where blocks suffice (two per SM), else the fewest that leave no SM with more
+        // than 1.2 times its share of the atoms (64 blocks over 152 SMs: 2 each).  Lanes per atom:
+        // eight while a CTA then takes its atoms in one pass, else four below one block per SM
+        // (23,328 atoms: 73 us, 89 with two); from there on two, and CTAs for one pass of
+        // them.  Against the same split with an own queue and whole 16-byte chunks per lane: 4,000 atoms
+        // (8 blocks) 29 us instead of 46, 10,976 (64) 47 / 75, 32,000 (64) 106 / 171, 55,296 (216)
+        // 173 / 212, 360,703 (2,016) 776 / 799.
         const int sms = g_sm_count > 0 ? g_sm_count : 152;
         const int64_t per_block = (s.n + g.nblock - 1) / g.nblock;
-        int lpa = 1;
         int64_t split = 1;
-        for (; lpa <= 8; lpa *= 2) {
-            split = std::max<int64_t>(1, (per_block * lpa + F_THREADS - 1) / F_THREADS);
-            if (g.nblock * split >= 2 * sms) break;
+        int lpa = 2;
+        if (g.nblock < 2 * sms) {
+            const auto share = [&](int64_t k) { return (g.nblock * k + sms - 1) / sms * (double)per_block / k; };
+            const double even = (double)s.n / sms;
+            while (split < 32 && share(split) > 1.2 * even) ++split;
+            if (per_block * 8 <= F_THREADS * split) lpa = 8;
+            else if (g.nblock < sms) lpa = 4;
+            else split = std::max(split, (per_block * 9 / 8 * lpa + F_THREADS - 1) / F_THREADS);  // (blocks differ)
         }
-        lpa = std::min(lpa, 8);
-        if (lpa == 1) split = std::min<int64_t>(split, (2 * sms + g.nblock - 1) / g.nblock);
         // the FP32 test's error: coordinates up to two cells from the block centre, cut to 20 bits
         const double wmax = std::max({g.w[0], g.w[1], g.w[2]});
         double rc2 = 0.0;
@@ -363,7 +378,7 @@ void init_force_fp64_kernels(int half, int single) {
         return;
     }
     for (int k = 0; k < 4; ++k)
-        for (int lpa = 1; lpa <= 8; lpa *= 2) allow_max_smem(full_kernel(single, k & 1, k & 2, lpa));
+        for (int lpa = 2; lpa <= 8; lpa *= 2) allow_max_smem(full_kernel(single, k & 1, k & 2, lpa));
 }
 
 }  // namespace mdgb

@@ -264,35 +264,83 @@ __device__ __forceinline__ void tile_stage_f32(const TileMeta& m, const float4* 
     }
 }
 
+constexpr unsigned long long TILE_ALL = ~0ull;
+constexpr int STAGE64_AHEAD = 4;
+
+// The tile cells (bit per slot) that the lists of a CTA's own atoms can reach, when CTAs share a block
+// and this one takes `per` own atoms from part * per on (and every split * per): the cells around
+// those own cells.  Every lane of a warp gets the mask.
+__device__ __forceinline__ unsigned long long tile_needed(const TileMeta& m, int part, int split, int per) {
+    const int lane = threadIdx.x & 31;
+    const int lo = part * per, hi = split * per >= m.prefix[8] ? lo + per : m.prefix[8];
+    const bool own = lane < 8 && m.prefix[lane & 7] < hi && m.prefix[(lane & 7) + 1] > lo;
+    const unsigned touched = __ballot_sync(0xffffffffu, own);  // own cell 1 + (o & 1), 1 + (o >> 1 & 1), 1 + (o >> 2)
+    unsigned half[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int c = m.coord[lane + 32 * h], x = c & 3, y = (c >> 2) & 3, z = c >> 4;
+        const unsigned near = (x == 0 ? 0x55u : (x == 3 ? 0xaau : 0xffu)) & (y == 0 ? 0x33u : (y == 3 ? 0xccu : 0xffu)) &
+                              (z == 0 ? 0x0fu : (z == 3 ? 0xf0u : 0xffu));
+        half[h] = __ballot_sync(0xffffffffu, (near & touched) != 0u);
+    }
+    return half[0] | ((unsigned long long)half[1] << 32);
+}
+
 // Stage the FP64 tile of block b: coordinates relative to the block centre (periodic
 // images shifted by one box length where the tile wraps), species, and a dummy slot T
-// far outside every cutoff.
+// far outside every cutoff.  Only the cells of `need` are filled.  One warp per tile cell, STAGE64_AHEAD
+// rows of 32 atoms on their way together (a CTA with an SM to itself waits for nothing else:
+// 31,000 cycles for the 4,000 atoms of a box of 4 cells per side with one row at a time).
 __device__ __forceinline__ void tile_stage_f64(const DevState& s, const Geometry& g, const TileMeta& m, int b,
                                                double* __restrict__ tx_, double* __restrict__ ty_,
-                                               double* __restrict__ tz_, int* __restrict__ tsp) {
+                                               double* __restrict__ tz_, int* __restrict__ tsp,
+                                               unsigned long long need = TILE_ALL) {
     int bx, by, bz;
     block_coords(g, b, bx, by, bz);
     const int T = m.prefix[64];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     const double cx = (2.0 * bx + 1.0) * g.w[0], cy = (2.0 * by + 1.0) * g.w[1], cz = (2.0 * bz + 1.0) * g.w[2];
-#pragma unroll 2
-    for (int slot = warp; slot < 64; slot += nw) {  // one warp per tile cell
-        const int c = m.coord[slot];
-        const int rx = 2 * bx - 1 + (c & 3), ry = 2 * by - 1 + ((c >> 2) & 3), rz = 2 * bz - 1 + (c >> 4);
-        const int u0 = m.prefix[slot], cnt = m.prefix[slot + 1] - u0, j0 = m.start[slot];
-        for (int e = lane; e < cnt; e += 32) {
-            double x = s.x[j0 + e], y = s.y[j0 + e], z = s.z[j0 + e];
-            const int sp = s.species[j0 + e];
-            if (rx < 0) x -= g.L[0];
-            else if (rx >= g.nc[0]) x += g.L[0];
-            if (ry < 0) y -= g.L[1];
-            else if (ry >= g.nc[1]) y += g.L[1];
-            if (rz < 0) z -= g.L[2];
-            else if (rz >= g.nc[2]) z += g.L[2];
-            tx_[u0 + e] = x - cx;
-            ty_[u0 + e] = y - cy;
-            tz_[u0 + e] = z - cz;
-            tsp[u0 + e] = sp;
+    // this warp's rows: (cell, first atom), cell by cell
+    int slot = warp, e0 = 0;
+    const auto next_cell = [&]() {
+        while (slot < 64 && !((need >> slot & 1) && e0 < m.prefix[slot + 1] - m.prefix[slot])) slot += nw, e0 = 0;
+    };
+    next_cell();
+    while (slot < 64) {
+        double x[STAGE64_AHEAD], y[STAGE64_AHEAD], z[STAGE64_AHEAD];
+        int sp[STAGE64_AHEAD], at[STAGE64_AHEAD], coord[STAGE64_AHEAD];
+#pragma unroll
+        for (int k = 0; k < STAGE64_AHEAD; ++k) {
+            at[k] = -1;
+            coord[k] = 21;  // (no wrap)
+            if (slot < 64) {
+                const int u0 = m.prefix[slot], e = e0 + lane;
+                coord[k] = m.coord[slot];
+                if (e < m.prefix[slot + 1] - u0) {
+                    const int j = m.start[slot] + e;
+                    at[k] = u0 + e;
+                    x[k] = s.x[j], y[k] = s.y[j], z[k] = s.z[j];
+                    sp[k] = s.species[j];
+                }
+                e0 += 32;
+                next_cell();
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < STAGE64_AHEAD; ++k) {
+            const int c = coord[k];
+            const int rx = 2 * bx - 1 + (c & 3), ry = 2 * by - 1 + ((c >> 2) & 3), rz = 2 * bz - 1 + (c >> 4);
+            if (at[k] < 0) continue;
+            if (rx < 0) x[k] -= g.L[0];
+            else if (rx >= g.nc[0]) x[k] += g.L[0];
+            if (ry < 0) y[k] -= g.L[1];
+            else if (ry >= g.nc[1]) y[k] += g.L[1];
+            if (rz < 0) z[k] -= g.L[2];
+            else if (rz >= g.nc[2]) z[k] += g.L[2];
+            tx_[at[k]] = x[k] - cx;
+            ty_[at[k]] = y[k] - cy;
+            tz_[at[k]] = z[k] - cz;
+            tsp[at[k]] = sp[k];
         }
     }
     if (threadIdx.x == 0) {

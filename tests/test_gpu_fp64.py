@@ -36,9 +36,9 @@ def check(pos, box, sp, P, r_cut, skin):
 @pytest.mark.parametrize("n,rho,close", [
     (2047, 0.8442, False),   # eight blocks, eight lanes per atom
     (8209, 1.86, True),      # a whole-box tile with no room for the queues
-    (21001, 0.8442, True),   # four lanes
-    (60001, 0.8442, False),  # two lanes
-    (150001, 0.8442, True),  # one lane, a CTA or more per block
+    (21001, 0.8442, True),   # four lanes, two CTAs per block
+    (60001, 0.8442, False),  # two lanes, three CTAs per block
+    (150001, 0.8442, True),  # two lanes, a CTA per block
 ])
 def test_forms_match_oracle(n, rho, close):
     w = W.fcc_vacancies(n, rho, 1.0, seed=n)
