@@ -334,6 +334,7 @@ void launch_forces_fp64(const DevState& s, const Geometry& g, const PairTable& p
             const auto share = [&](int64_t k) { return (g.nblock * k + sms - 1) / sms * (double)per_block / k; };
             const double even = (double)s.n / sms;
             while (split < 32 && share(split) > 1.2 * even) ++split;
+            split = std::max<int64_t>(split, sms / g.nblock);  // (up to a CTA per SM: blocks differ in size)
             if (per_block * 8 <= F_THREADS * split) lpa = 8;
             else if (g.nblock < sms) lpa = 4;
             else split = std::max(split, (per_block * 9 / 8 * lpa + F_THREADS - 1) / F_THREADS);  // (blocks differ)
