@@ -40,6 +40,7 @@ struct md_system {
     int32_t *atom_cell = nullptr, *cell_count = nullptr, *cursor = nullptr, *slot_key = nullptr,
             *slot_src = nullptr, *sorted_src = nullptr, *scan_scratch = nullptr;
     double *partials = nullptr, *out8 = nullptr;
+    unsigned* parts_done = nullptr;  // CTAs of the running energy reduction that have finished
     int nparts = 0;
     // pinned mirror of the device's status block, read with one copy: [0] err, [1] rebuild flag,
     // [2..9] stats, then the control words (d_ctrl)
@@ -1373,10 +1374,12 @@ int md_create(int64_t n, const double box[3], double r_cut, double skin, const m
         (rc = dalloc(s, &s->scan_scratch, scan_scratch_ints(g.ncell))))
         return bail(rc);
     s->nparts = 592;
-    if ((rc = dalloc(s, &s->partials, 8 * (size_t)s->nparts)) || (rc = dalloc(s, &s->out8, 8))) return bail(rc);
+    if ((rc = dalloc(s, &s->partials, 8 * (size_t)s->nparts + 1)) || (rc = dalloc(s, &s->out8, 8))) return bail(rc);
+    s->parts_done = reinterpret_cast<unsigned*>(s->partials + 8 * (size_t)s->nparts);
     if (cudaMallocHost(&s->h_flags, STATUS_WORDS * sizeof(uint32_t)) != cudaSuccess) return bail(MD_ERR_CUDA);
     if (cudaMallocHost(&s->h_ctrl, 3 * sizeof(long long)) != cudaSuccess) return bail(MD_ERR_CUDA);
     if (cudaMemsetAsync(d0.err, 0, STATUS_WORDS * sizeof(uint32_t), s->stream) != cudaSuccess ||
+        cudaMemsetAsync(s->parts_done, 0, sizeof(unsigned), s->stream) != cudaSuccess ||
         cudaStreamSynchronize(s->stream) != cudaSuccess)
         return bail(MD_ERR_CUDA);
     *out = s;
@@ -1694,9 +1697,10 @@ int md_energy_virial(md_system* s, double* pe, double* ke, double virial[6]) {
         int rc = ensure_lists(s);
         if (rc) return rc;
         if ((rc = do_forces(s, 1))) return rc;
-        launch_reduce_energy(s->st[s->cur], s->pt, mixed(s), s->partials, s->nparts, s->out8, s->stream);
+        launch_reduce_energy(s->st[s->cur], s->pt, mixed(s), s->partials, s->parts_done, s->nparts, s->out8,
+                             s->stream);
         CKL();
-        s->launches += 2;
+        s->launches += 1;
         CK(cudaMemcpyAsync(h, s->out8, sizeof(h), cudaMemcpyDeviceToHost, s->stream));
         if ((rc = sync_flags(s))) return rc;
         if ((rc = check_err(s, ERR_NONFINITE | ERR_TILE_OVERFLOW))) return rc;

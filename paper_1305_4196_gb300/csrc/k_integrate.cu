@@ -12,6 +12,8 @@
 // order: per-atom shares, then per-CTA FP64 partials, then one CTA.
 #include "mdgb_internal.cuh"
 
+#include <algorithm>
+
 namespace mdgb {
 
 __device__ __forceinline__ double force_of(const DevState& s, int mixed, int64_t i) {
@@ -157,68 +159,95 @@ void launch_copy_state(const DevState& dst, const DevState& src, cudaStream_t st
 }
 
 // ---------------------------------------------------------------- reductions
-// partial[b][0..7] = (PE, KE, W_xx, W_yy, W_zz, W_xy, W_xz, W_yz) over a contiguous chunk,
-// each thread summing a fixed strided subset in order, then a fixed-shape tree.
+// (PE, KE, W_xx, W_yy, W_zz, W_xy, W_xz, W_yz): partial[b][0..7] over a contiguous chunk, each thread
+// summing a fixed strided subset in order, then a fixed-shape tree; the CTA that finishes last
+// sums the partials in the same way.
+//
+// The FP64 pipe bounds this (an SM takes 16 cycles for a warp's FP64 addition or conversion), so a
+// thread adds its atoms' FP32 shares in two floats, hi and lo, with the rounding error of
+// every addition to hi kept in lo (to 2^-46 of the sum of its few atoms), and converts once: 54 -> 29 us
+// for 1,048,576 atoms (with the second launch that it saves).
 constexpr int RED_THREADS = 256;
 
-__global__ void __launch_bounds__(RED_THREADS) k_reduce_partials(DevState s, PairTable pt, int mixed,
-                                                                 int64_t chunk, double* __restrict__ partials) {
+struct FloatSum {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(float x) {
+        const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
+        hi = s;
+    }
+    // (a sum that is not finite stays what hi says)
+    __device__ __forceinline__ double get() const { return (double)hi + (isfinite(lo) ? (double)lo : 0.0); }
+};
+
+__device__ __forceinline__ void reduce_tree(double (&sh)[8][RED_THREADS], const double (&acc)[8]) {
+#pragma unroll
+    for (int c = 0; c < 8; ++c) sh[c][threadIdx.x] = acc[c];
+    __syncthreads();
+    for (int w = RED_THREADS / 2; w > 0; w >>= 1) {
+        if (threadIdx.x < w)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) sh[c][threadIdx.x] += sh[c][threadIdx.x + w];
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(RED_THREADS) k_reduce_energy(DevState s, PairTable pt, int mixed, int64_t chunk,
+                                                               double* __restrict__ partials,
+                                                               unsigned* __restrict__ finished,
+                                                               double* __restrict__ out8) {
     __shared__ double sh[8][RED_THREADS];
+    __shared__ bool last;
     const int64_t n = s.n;
     const int64_t lo = blockIdx.x * chunk;
     const int64_t hi = lo + chunk < n ? lo + chunk : n;
     double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    FloatSum f[7];
     for (int64_t i = lo + threadIdx.x; i < hi; i += RED_THREADS) {
-        const double m = pt.mass[s.species[i]];
         const double vx = s.vx[i], vy = s.vy[i], vz = s.vz[i];
-        acc[1] += 0.5 * m * (vx * vx + vy * vy + vz * vz);
+        if (pt.nsp == 1) acc[1] = fma(vx, vx, fma(vy, vy, fma(vz, vz, acc[1])));
+        else acc[1] += 0.5 * pt.mass[s.species[i]] * (vx * vx + vy * vy + vz * vz);
         if (mixed) {
-            acc[0] += (double)s.pe_atom_f[i];
+            f[0].add(s.pe_atom_f[i]);
 #pragma unroll
-            for (int c = 0; c < 6; ++c) acc[2 + c] += (double)s.vir_atom_f[c * n + i];
+            for (int c = 0; c < 6; ++c) f[1 + c].add(s.vir_atom_f[c * n + i]);
         } else {
             acc[0] += s.pe_atom_d[i];
 #pragma unroll
             for (int c = 0; c < 6; ++c) acc[2 + c] += s.vir_atom_d[c * n + i];
         }
     }
+    if (pt.nsp == 1) acc[1] *= 0.5 * pt.mass[0];
+    if (mixed) {
+        acc[0] = f[0].get();
 #pragma unroll
-    for (int c = 0; c < 8; ++c) sh[c][threadIdx.x] = acc[c];
-    __syncthreads();
-    for (int w = RED_THREADS / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-#pragma unroll
-            for (int c = 0; c < 8; ++c) sh[c][threadIdx.x] += sh[c][threadIdx.x + w];
-        __syncthreads();
+        for (int c = 0; c < 6; ++c) acc[2 + c] = f[1 + c].get();
     }
-    if (threadIdx.x < 8) partials[blockIdx.x * 8 + threadIdx.x] = sh[threadIdx.x][0];
-}
-
-__global__ void __launch_bounds__(RED_THREADS) k_reduce_final(const double* __restrict__ partials, int nparts,
-                                                               double* __restrict__ out8) {
-    __shared__ double sh[8][RED_THREADS];
-    double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int b = threadIdx.x; b < nparts; b += RED_THREADS)
-#pragma unroll
-        for (int c = 0; c < 8; ++c) acc[c] += partials[b * 8 + c];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) sh[c][threadIdx.x] = acc[c];
-    __syncthreads();
-    for (int w = RED_THREADS / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-#pragma unroll
-            for (int c = 0; c < 8; ++c) sh[c][threadIdx.x] += sh[c][threadIdx.x + w];
-        __syncthreads();
+    reduce_tree(sh, acc);
+    if (threadIdx.x < 8) {
+        __stcg(partials + blockIdx.x * 8 + threadIdx.x, sh[threadIdx.x][0]);
+        __threadfence();
     }
+    __syncthreads();
+    if (threadIdx.x == 0) last = atomicInc(finished, gridDim.x - 1) == gridDim.x - 1;  // (back to 0 for the next launch)
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+#pragma unroll
+    for (int c = 0; c < 8; ++c) acc[c] = 0.0;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += RED_THREADS)
+#pragma unroll
+        for (int c = 0; c < 8; ++c) acc[c] += __ldcg(partials + b * 8 + c);
+    reduce_tree(sh, acc);
     if (threadIdx.x < 8) out8[threadIdx.x] = sh[threadIdx.x][0];
 }
 
-void launch_reduce_energy(const DevState& s, const PairTable& pt, int mixed, double* partials, int nparts,
-                          double* out8, cudaStream_t st) {
-    int64_t chunk = (s.n + nparts - 1) / nparts;
-    if (chunk < 1) chunk = 1;
-    k_reduce_partials<<<nparts, RED_THREADS, 0, st>>>(s, pt, mixed, chunk, partials);
-    k_reduce_final<<<1, RED_THREADS, 0, st>>>(partials, nparts, out8);
+void launch_reduce_energy(const DevState& s, const PairTable& pt, int mixed, double* partials, unsigned* finished,
+                          int nparts, double* out8, cudaStream_t st) {
+    const int64_t want = (s.n + RED_THREADS - 1) / RED_THREADS;  // small systems: an atom per thread
+    const int parts = (int)std::max<int64_t>(1, std::min<int64_t>(nparts, want));
+    const int64_t chunk = std::max<int64_t>(1, (s.n + parts - 1) / parts);
+    k_reduce_energy<<<parts, RED_THREADS, 0, st>>>(s, pt, mixed, chunk, partials, finished, out8);
 }
 
 // ---------------------------------------------------------------- state I/O

@@ -347,8 +347,8 @@ void launch_forces_fp64(const DevState& s, const Geometry& g, const PairTable& p
                         int with_energy, cudaStream_t st);
 void launch_integrate(const DevState& s, const Geometry& g, const PairTable& pt, int mode, int mixed,
                       double dt, double lim2, cudaStream_t st);
-void launch_reduce_energy(const DevState& s, const PairTable& pt, int mixed, double* partials, int nparts,
-                          double* out8, cudaStream_t st);
+void launch_reduce_energy(const DevState& s, const PairTable& pt, int mixed, double* partials, unsigned* finished,
+                          int nparts, double* out8, cudaStream_t st);
 void launch_set_state(const DevState& s, const double* pos, const double* vel, const int32_t* species,
                       int nsp, cudaStream_t st);
 void launch_get_state(const DevState& s, double* pos, double* vel, int32_t* image, cudaStream_t st);
