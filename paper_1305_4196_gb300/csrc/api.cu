@@ -172,7 +172,7 @@ size_t fsmem(const md_system* s, int with_energy, int tile_cap) {
 }
 void enqueue_lists(const md_system* s, const DevState& a, cudaStream_t st) {
     if (af(s)) launch_build_sched(a, s->g, s->to, s->rl2, s->list_cap, s->tile_cap, st);
-    else launch_build_lists(a, s->g, s->to, s->rl2, s->list_cap, s->tile_cap, half(s), st);
+    else launch_build_lists(a, s->st[1], s->g, s->to, s->rl2, s->list_cap, s->tile_cap, half(s), st);
 }
 // md_step runs the full-list mixed path with velocity Verlet fused into the force kernel
 bool fused(const md_system* s) { return mixed(s) && !half(s) && !s->no_fuse; }
@@ -301,8 +301,10 @@ int check_err(md_system* s, uint32_t mask) {
     return fail(s, MD_ERR_ARG, "device error 0x%x", e);
 }
 
-// ---- binning: assign, count, scan, scatter, in-cell order, gather + copy back
-void enqueue_bin(md_system* s, const DevState& a, cudaStream_t st) {
+// ---- binning: assign, count, scan, scatter, in-cell order, gather.  The permuted state is then in
+// st[1], from where the list builder takes it to `a` (enqueue_lists has to follow; the other
+// builder, of the half lists without atomic operations, does not: copied back here).
+void enqueue_bin(md_system* s, const DevState& a, cudaStream_t st, bool copy_back) {
     const Geometry& g = s->g;
     cudaMemsetAsync(s->cell_count, 0, sizeof(int32_t) * g.ncell, st);
     cudaMemsetAsync(s->cursor, 0, sizeof(int32_t) * g.ncell, st);
@@ -310,15 +312,15 @@ void enqueue_bin(md_system* s, const DevState& a, cudaStream_t st) {
     launch_scan(s->cell_count, a.cell_start, g.ncell, s->scan_scratch, st);
     launch_scatter(a, s->atom_cell, a.cell_start, s->cursor, s->slot_key, s->slot_src, st);
     launch_cell_sort(g, a.cell_start, s->slot_key, s->slot_src, s->sorted_src, st);
-    launch_gather(a, s->st[1], g, s->sorted_src, s->atom_cell, st);
+    launch_gather(a, s->st[1], g, s->sorted_src, s->atom_cell, !mixed(s), copy_back, st);
     launch_classify_blocks(a, g, st);
 }
 
-int do_bin(md_system* s, int p = 0) {
+int do_bin(md_system* s, int p, bool copy_back) {
     if (s->n == 0) return MD_OK;
-    enqueue_bin(s, view(s, p), s->stream);
+    enqueue_bin(s, view(s, p), s->stream, copy_back);
     CKL();
-    s->launches += 8;
+    s->launches += copy_back ? 8 : 7;
     s->lists_valid = false;
     s->forces_valid = false;
     return MD_OK;
@@ -411,7 +413,7 @@ int do_build(md_system* s, int p = 0) {
         ev = take_events(s);
         CK(cudaEventRecord(ev.first, s->stream));
     }
-    int rc = do_bin(s, p);
+    int rc = do_bin(s, p, af(s));
     if (rc) return rc;
     if (s->n == 0) {
         s->lists_valid = true;
@@ -670,7 +672,7 @@ int capture_step(md_system* s, int mode, md_system::StepGraph& out) {
     CK(cudaStreamEndCapture(cs, &g));
     // the rebuild body
     CK(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-    enqueue_bin(s, a, cs);
+    enqueue_bin(s, a, cs, af(s));
     cudaMemsetAsync(a.stats, 0, 4 * sizeof(int32_t), cs);
     enqueue_lists(s, a, cs);
     launch_count_build(s->d_ctrl + 1, cs);
@@ -727,9 +729,9 @@ int capture_fused(md_system* s, bool kkd, int p, md_system::StepGraph& out) {
     }
     CK(cudaStreamEndCapture(cs, &g));
     CK(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-    enqueue_bin(s, a, cs);
+    enqueue_bin(s, a, cs, af(s));
     cudaMemsetAsync(a.stats, 0, 4 * sizeof(int32_t), cs);
-    launch_build_lists(a, s->g, s->to, s->rl2, s->list_cap, s->tile_cap, 0, cs);
+    enqueue_lists(s, a, cs);
     launch_count_build(s->d_ctrl + 1, cs);
     CK(cudaStreamEndCapture(cs, &body));
     CKL();
@@ -796,9 +798,9 @@ int capture_fused_multi(md_system* s, md_system::StepGraph& out) {
         tail.assign(deps, deps + ndeps);
         CK(cudaStreamEndCapture(cs, &g));
         CK(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-        enqueue_bin(s, a, cs);
+        enqueue_bin(s, a, cs, af(s));
         cudaMemsetAsync(a.stats, 0, 4 * sizeof(int32_t), cs);
-        launch_build_lists(a, s->g, s->to, s->rl2, s->list_cap, s->tile_cap, 0, cs);
+        enqueue_lists(s, a, cs);
         launch_count_build(s->d_ctrl + 1, cs);
         CK(cudaStreamEndCapture(cs, &body));
     }
@@ -851,7 +853,7 @@ int append_captured(md_system* s, cudaGraph_t g, std::vector<cudaGraphNode_t>& t
     return MD_OK;
 }
 
-// One step: step control -> IF(rebuild){binning, gather, copy back, list build on buffer p} -> forces
+// One step: step control -> IF(rebuild){binning, gather, list build on buffer p} -> forces
 // and what follows them.  mid: another step of the chunk follows (fused: kick-kick-drift into the
 // other buffer; else the separate integration); otherwise the step ends its forces, fused ones
 // with the closing kick.
@@ -868,7 +870,7 @@ int append_step(md_system* s, cudaGraph_t g, std::vector<cudaGraphNode_t>& tail,
     if ((rc = add_conditional(s, g, tail, h, cudaGraphCondTypeIf, &body))) return rc;
     std::vector<cudaGraphNode_t> none;
     rc = append_captured(s, body, none, [&](cudaStream_t cs) {
-        enqueue_bin(s, a, cs);
+        enqueue_bin(s, a, cs, af(s));
         cudaMemsetAsync(a.stats, 0, 4 * sizeof(int32_t), cs);
         enqueue_lists(s, a, cs);
         launch_count_build(s->d_ctrl + 1, cs);
@@ -1112,7 +1114,7 @@ int run_chunk_fused(md_system* s, int len, bool first, bool last) {
     if (e & ERR_TILE_OVERFLOW) return MD_ERR_CELL_OVERFLOW;  // the chunk is redone: nothing of it counts
     if (e & ERR_LIST_OVERFLOW) return MD_ERR_LIST_OVERFLOW;
     const long long builds = builds_in_graphs(s);
-    s->launches += builds * 10;  // binning (8), list build, build counter
+    s->launches += builds * (af(s) ? 10 : 9);  // binning (8, or 7 without the copy back), list build, build counter
     if (builds > 0) {
         s->n_builds += builds;
         s->max_list = (int)s->h_flags[2];
@@ -1164,7 +1166,7 @@ int run_chunk(md_system* s, int len, bool first) {
     if (e & ERR_TILE_OVERFLOW) return MD_ERR_CELL_OVERFLOW;  // the chunk is redone: nothing of it counts
     if (e & ERR_LIST_OVERFLOW) return MD_ERR_LIST_OVERFLOW;
     const long long builds = builds_in_graphs(s);
-    s->launches += builds * 10;  // binning (8), list build, build counter
+    s->launches += builds * (af(s) ? 10 : 9);  // binning (8, or 7 without the copy back), list build, build counter
     if (builds > 0) {
         s->n_builds += builds;
         s->max_list = (int)s->h_flags[2];
@@ -1431,7 +1433,7 @@ int md_bin_cells(md_system* s) {
     if (!s->has_state) return fail(s, MD_ERR_STATE, "no state");
     DeviceGuard dg(s->device);
     CK(cudaMemsetAsync(s->st[0].err, 0, sizeof(uint32_t), s->stream));
-    int rc = do_bin(s);
+    int rc = do_bin(s, 0, true);
     if (rc) return rc;
     rc = sync_flags(s);
     if (rc) return rc;

@@ -31,10 +31,23 @@
 
 namespace mdgb {
 
+// Atom i of the new order from the gather's copy to the state.
+__device__ __forceinline__ void copy_atom(const DevState& s, const DevState& d, int i) {
+    const double x = d.x[i], y = d.y[i], z = d.z[i], vx = d.vx[i], vy = d.vy[i], vz = d.vz[i];
+    const int ix = d.ix[i], iy = d.iy[i], iz = d.iz[i], sp = d.species[i], orig = d.orig[i];
+    s.x[i] = x, s.y[i] = y, s.z[i] = z;
+    s.vx[i] = vx, s.vy[i] = vy, s.vz[i] = vz;
+    s.ix[i] = ix, s.iy[i] = iy, s.iz[i] = iz;
+    s.species[i] = sp, s.orig[i] = orig;
+}
+
 // The lists of the own atoms of block b (the CTA's task): warp w takes own cell w, or of each
 // cell the share `part` of `split` (small systems, whose blocks are too few to fill the SMs).
+// d: the state in the new order as the gather left it; a warp copies its atoms to s behind their
+// lists, and the re-tests read d.
 template <int HALF>
-__device__ __forceinline__ void build_block(const DevState& s, const Geometry& g, const TileOffsets& to, double rl2,
+__device__ __forceinline__ void build_block(const DevState& s, const DevState& d, const Geometry& g,
+                                            const TileOffsets& to, double rl2,
                                             float band_lo, float band_hi, int list_cap, int tile_cap, int b, int part,
                                             int split) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -48,6 +61,8 @@ __device__ __forceinline__ void build_block(const DevState& s, const Geometry& g
     if (threadIdx.x == 0) atomicMax(&s.stats[1], need);
     if (need > tile_cap) {
         if (threadIdx.x == 0) atomicOr(s.err, ERR_TILE_OVERFLOW);
+        if (part == 0)
+            for (int u = threadIdx.x; u < m.prefix[8]; u += blockDim.x) copy_atom(s, d, m.start[0] + u);
         return;
     }
     if (m.prefix[8] == 0) return;  // empty block (vacuum): no lists to build
@@ -74,7 +89,7 @@ __device__ __forceinline__ void build_block(const DevState& s, const Geometry& g
             const int cnt = nl_scan_cell<HALF>(
                 w, m, tx, ty, tz, oc, own_coord, lo_own, own_n, band_hi, band_lo, reinterpret_cast<uint4*>(s.nl) + g0,
                 (size_t)s.np, list_cap, [&](int own, int u) {
-                    return fp64_pair_test(s.x, s.y, s.z, g.L[0], g.L[1], g.L[2], g0 + own, tile_global_index(m, u),
+                    return fp64_pair_test(d.x, d.y, d.z, g.L[0], g.L[1], g.L[2], g0 + own, tile_global_index(m, u),
                                           rl2);
                 });
             if (lane < own_n) {
@@ -82,6 +97,7 @@ __device__ __forceinline__ void build_block(const DevState& s, const Geometry& g
                 s.nl_cnt[g0 + lane] = (uint16_t)(cnt < list_cap ? cnt : list_cap);
                 max_cnt = cnt > max_cnt ? cnt : max_cnt;
                 sum_cnt += (unsigned long long)cnt;
+                copy_atom(s, d, g0 + lane);
             }
         }
     }
@@ -98,21 +114,22 @@ __device__ __forceinline__ void build_block(const DevState& s, const Geometry& g
 
 // `split` CTAs per block, blocks in spatial order.
 template <int HALF>
-__global__ void __launch_bounds__(NL_WARPS * 32, 3) k_build_lists(DevState s, Geometry g, TileOffsets to,
-                                                                  double rl2, float band_lo, float band_hi,
-                                                                  int list_cap, int tile_cap, int split) {
-    build_block<HALF>(s, g, to, rl2, band_lo, band_hi, list_cap, tile_cap, spatial_block(g, blockIdx.x / split),
+__global__ void __launch_bounds__(NL_WARPS * 32, 3) k_build_lists(DevState s, DevState d, Geometry g,
+                                                                  TileOffsets to, double rl2, float band_lo,
+                                                                  float band_hi, int list_cap, int tile_cap,
+                                                                  int split) {
+    build_block<HALF>(s, d, g, to, rl2, band_lo, band_hi, list_cap, tile_cap, spatial_block(g, blockIdx.x / split),
                       blockIdx.x % split, split);
 }
 
 // A compact system: a grid of s.compact CTAs over the occupied blocks.
 template <int HALF>
-__global__ void __launch_bounds__(NL_WARPS * 32, 3) k_build_lists_occ(DevState s, Geometry g, TileOffsets to,
-                                                                      double rl2, float band_lo, float band_hi,
-                                                                      int list_cap, int tile_cap) {
+__global__ void __launch_bounds__(NL_WARPS * 32, 3) k_build_lists_occ(DevState s, DevState d, Geometry g,
+                                                                      TileOffsets to, double rl2, float band_lo,
+                                                                      float band_hi, int list_cap, int tile_cap) {
     const int count = s.stats[4];
     for (int k = blockIdx.x; k < count; k += gridDim.x) {
-        build_block<HALF>(s, g, to, rl2, band_lo, band_hi, list_cap, tile_cap, s.blk_list[k], 0, 1);
+        build_block<HALF>(s, d, g, to, rl2, band_lo, band_hi, list_cap, tile_cap, s.blk_list[k], 0, 1);
         __syncthreads();  // the next block reuses the shared memory
     }
 }
@@ -127,7 +144,7 @@ size_t build_lists_smem(int list_cap, int tile_cap) {
     return (size_t)((tile_cap + 227) & ~3) * 3 * sizeof(float) + 32768;
 }
 
-void launch_build_lists(const DevState& s, const Geometry& g, const TileOffsets& to, double rl2, int list_cap,
+void launch_build_lists(const DevState& s, const DevState& d, const Geometry& g, const TileOffsets& to, double rl2, int list_cap,
                         int tile_cap, int half, cudaStream_t st) {
     if (s.n == 0) return;
     const int warps = nl_smem_bytes(tile_cap, NL_WARPS) <= 226 * 1024 ? NL_WARPS : NL_WARPS / 2;
@@ -137,8 +154,8 @@ void launch_build_lists(const DevState& s, const Geometry& g, const TileOffsets&
     const float lo = (float)(rl2 * (1.0 - band)), hi = (float)(rl2 * (1.0 + band));
     const int threads = warps * 32;
     if (s.compact) {
-        if (half) k_build_lists_occ<1><<<s.compact, threads, smem, st>>>(s, g, to, rl2, lo, hi, list_cap, tile_cap);
-        else k_build_lists_occ<0><<<s.compact, threads, smem, st>>>(s, g, to, rl2, lo, hi, list_cap, tile_cap);
+        if (half) k_build_lists_occ<1><<<s.compact, threads, smem, st>>>(s, d, g, to, rl2, lo, hi, list_cap, tile_cap);
+        else k_build_lists_occ<0><<<s.compact, threads, smem, st>>>(s, d, g, to, rl2, lo, hi, list_cap, tile_cap);
         return;
     }
     // CTAs per block, each a share of every cell's atoms: while the grid is below two CTAs per SM,
@@ -147,8 +164,8 @@ void launch_build_lists(const DevState& s, const Geometry& g, const TileOffsets&
     const int per_cell = (int)((s.n + g.ncell - 1) / g.ncell);
     const int split = std::max(1, std::min({(per_cell + 7) / 8, (2 * 152 + g.nblock - 1) / g.nblock, 16}));
     const unsigned grid = (unsigned)g.nblock * (unsigned)split;
-    if (half) k_build_lists<1><<<grid, threads, smem, st>>>(s, g, to, rl2, lo, hi, list_cap, tile_cap, split);
-    else k_build_lists<0><<<grid, threads, smem, st>>>(s, g, to, rl2, lo, hi, list_cap, tile_cap, split);
+    if (half) k_build_lists<1><<<grid, threads, smem, st>>>(s, d, g, to, rl2, lo, hi, list_cap, tile_cap, split);
+    else k_build_lists<0><<<grid, threads, smem, st>>>(s, d, g, to, rl2, lo, hi, list_cap, tile_cap, split);
 }
 
 template <typename K>

@@ -303,14 +303,14 @@ void launch_scatter(const DevState& s, const int32_t* atom_cell, const int32_t* 
 void launch_cell_sort(const Geometry& g, const int32_t* cell_start, const int32_t* slot_key,
                       const int32_t* slot_src, int32_t* sorted_src, cudaStream_t st);
 void launch_gather(const DevState& s, const DevState& scratch, const Geometry& g, const int32_t* sorted_src,
-                   const int32_t* atom_cell, cudaStream_t st);
+                   const int32_t* atom_cell, int fp64, bool copy_back, cudaStream_t st);
 void launch_classify_blocks(const DevState& s, const Geometry& g, cudaStream_t st);
 void launch_step_ctrl(int policy, int every_k, int32_t* rebuild_flag, long long* step_counter,
                       long long* n_builds, uint32_t* err, cudaGraphConditionalHandle handle, cudaStream_t st);
 void launch_loop_ctrl(long long* passes_left, int done, cudaGraphConditionalHandle handle, cudaStream_t st);
 void launch_count_build(long long* n_builds, cudaStream_t st);
 void launch_copy_state(const DevState& dst, const DevState& src, cudaStream_t st);
-void launch_build_lists(const DevState& s, const Geometry& g, const TileOffsets& to, double rl2, int list_cap,
+void launch_build_lists(const DevState& s, const DevState& d, const Geometry& g, const TileOffsets& to, double rl2, int list_cap,
                         int tile_cap, int half, cudaStream_t st);
 size_t build_lists_smem(int list_cap, int tile_cap);
 void launch_forces_mixed(const DevState& s, const Geometry& g, const PairTable& pt, const TileOffsets& to,
