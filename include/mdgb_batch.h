@@ -9,7 +9,8 @@
  *   - a system of at most one_cta_max atoms (2,048 unless md_batch_autotune picks
  *     1,024 or 4,096), or one whose box is under 6 (r_cut + skin) on a side, is one
  *     task: one CTA holds it in shared memory for all steps of the call (linked
- *     cells rebuilt every step, no list);
+ *     cells rebuilt every step, no list); where that would outlast the other work of
+ *     the call, the same operations are shared out as tasks, with the same results;
  *   - a larger system is advanced in phases of tasks that any CTA may take: when
  *     its Verlet lists are due (at the start of a call, and after a step in which
  *     some atom moved more than skin/2), binning in atom chunks, a scan of the cell
@@ -71,8 +72,8 @@ int md_batch_energies(md_batch *b, double *pe, double *ke);
 int md_batch_get_state(md_batch *b, double *pos, double *vel, int32_t *image, int device_ptrs);
 
 /*
- * How each system runs: path[k] = 0 (one CTA for the whole call) or 1 (block
- * tasks over many CTAs); threads[k], the CTA size of the launch; cell_range[k]
+ * How each system runs: path[k] = 0 (cells rebuilt every step, by one CTA for the
+ * whole call or by tasks) or 1 (block tasks over many CTAs); threads[k], the CTA size of the launch; cell_range[k]
  * (path 0: cells at least r_cut / cell_range wide; path 1: 1).  Host arrays of
  * n_systems; any may be NULL.
  */

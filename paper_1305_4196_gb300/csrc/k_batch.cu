@@ -3,7 +3,7 @@
 // The paper notes that its task functor can carry which copy of a system a task
 // works on, so that replicas share one schedule (Sec. II.C).  Here every call on an
 // ensemble is one launch of k_ensemble_run (at the end of this file), whose CTAs take
-// tasks from a device work table over all systems.  Two kinds of system:
+// tasks from a device work table over all systems.  Three kinds of system:
 //
 // A small system (a few hundred to a few thousand atoms) is one task: one CTA owns it
 // for all time steps of the call; its FP32 coordinates and linked cells live in shared
@@ -16,10 +16,13 @@
 //     with no branches, every pair force component added as rint(f * 2^32) through
 //     the main path's exact two-part integer split (forces do not depend on order);
 //     an atom with a pair in the FP64 cutoff band or a force beyond the split's range
-//     is finished after the loop by an exact scalar pass,
+//     is finished after the loop by a warp in an exact pass,
 //   * and integrates velocity Verlet in FP64.
 // There is no neighbour list: the cells are rebuilt every step, which for systems of
 // this size costs less than a list build would.
+//
+// One that would keep its CTA busy long after the others have run out of work is advanced by the
+// same operations in phases of tasks (the shared systems below).
 //
 // A larger system is advanced in phases of tasks that any CTA may take, with Verlet
 // lists (the block systems below).
@@ -601,7 +604,7 @@ __device__ void shared_final(const BatchSys& y, const BatchState& st, const EnsA
 //                        walks its list two entries per step in packed FP32x2 and adds every
 //                        pair force component as rint(f 2^32) through the exact two-part
 //                        split; an atom with a pair in the FP64 cutoff band or a force beyond
-//                        the split is finished by an exact scalar pass.  Then velocity Verlet
+//                        the split is finished by a warp in an exact pass.  Then velocity Verlet
 //                        in FP64: the closing half kick of step k - 1 and, for k < K, the
 //                        opening half kick and the drift of step k into the other position
 //                        buffers (other tasks of the phase still read this step's), and the
@@ -882,12 +885,12 @@ __device__ __forceinline__ AtomState ens_load_state(const BatchState& st, const 
     return a;
 }
 
-// Centres of a block's own cells (x, y, z of each), by the block's first threads.
+// Centres of a block's own cells (x, y, z of each) in cell widths, by the block's first threads.
 __device__ __forceinline__ void ens_centres(const EnsBlockSys& y, int b, double (&centre)[8][3]) {
     if (threadIdx.x < 24) {
         const int os = threadIdx.x / 3, d = threadIdx.x % 3;
         const int bd = d == 0 ? b % y.nb[0] : (d == 1 ? (b / y.nb[0]) % y.nb[1] : b / (y.nb[0] * y.nb[1]));
-        centre[os][d] = (2 * bd + ((os >> d) & 1) + 0.5) * y.w[d];
+        centre[os][d] = 2 * bd + ((os >> d) & 1) + 0.5;
     }
 }
 
@@ -928,8 +931,9 @@ __device__ __forceinline__ void ens_epilogue(const EnsBlockSys& y, const BatchSt
     Pn.y[g] = yv;
     Pn.z[g] = z;
     const int64_t sl = y.a0 + slot;
-    const float4 q = make_float4(__double2float_rn(x - centre[0]), __double2float_rn(yv - centre[1]),
-                                 __double2float_rn(z - centre[2]), 0.0f);
+    const float4 q = make_float4(__double2float_rn(fma(-centre[0], y.w[0], x)),
+                                 __double2float_rn(fma(-centre[1], y.w[1], yv)),
+                                 __double2float_rn(fma(-centre[2], y.w[2], z)), 0.0f);
     (odd ? ea.xs : ea.xsb)[sl] = q;
     const float4 r = a.ref;
     const float ex = q.x - r.x, ey = q.y - r.y, ez = q.z - r.z;

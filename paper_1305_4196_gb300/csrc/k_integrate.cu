@@ -9,7 +9,7 @@
 // half kick and drift of the next (the same operations, one kernel).
 //
 // Energies use the paper's thread-local accumulators (Sec. II.C) in a fixed
-// order: per-atom shares, then per-CTA FP64 partials, then one CTA.
+// order: per-atom shares, then per-CTA FP64 partials, then the last CTA sums those.
 #include "mdgb_internal.cuh"
 
 #include <algorithm>
