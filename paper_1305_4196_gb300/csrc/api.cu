@@ -301,26 +301,28 @@ int check_err(md_system* s, uint32_t mask) {
     return fail(s, MD_ERR_ARG, "device error 0x%x", e);
 }
 
+// assign, scan, scatter, in-cell order, gather (and copy back), occupied blocks
+int bin_kernels(const md_system* s, bool copy_back) { return 5 + scan_kernels(s->g.ncell) + (copy_back ? 1 : 0); }
+
 // ---- binning: assign, count, scan, scatter, in-cell order, gather.  The permuted state is then in
 // st[1], from where the list builder takes it to `a` (enqueue_lists has to follow; the other
 // builder, of the half lists without atomic operations, does not: copied back here).
-void enqueue_bin(md_system* s, const DevState& a, cudaStream_t st, bool copy_back) {
+// The statistics of the build start at zero.  n_builds: see launch_classify_blocks.
+void enqueue_bin(md_system* s, const DevState& a, cudaStream_t st, bool copy_back, long long* n_builds) {
     const Geometry& g = s->g;
-    cudaMemsetAsync(s->cell_count, 0, sizeof(int32_t) * g.ncell, st);
-    cudaMemsetAsync(s->cursor, 0, sizeof(int32_t) * g.ncell, st);
     launch_bin_assign(a, g, s->atom_cell, s->cell_count, st);
-    launch_scan(s->cell_count, a.cell_start, g.ncell, s->scan_scratch, st);
+    launch_scan(s->cell_count, s->cursor, a.cell_start, g.ncell, s->scan_scratch, st);
     launch_scatter(a, s->atom_cell, a.cell_start, s->cursor, s->slot_key, s->slot_src, st);
     launch_cell_sort(g, a.cell_start, s->slot_key, s->slot_src, s->sorted_src, st);
     launch_gather(a, s->st[1], g, s->sorted_src, s->atom_cell, !mixed(s), copy_back, st);
-    launch_classify_blocks(a, g, st);
+    launch_classify_blocks(a, g, n_builds, st);
 }
 
 int do_bin(md_system* s, int p, bool copy_back) {
     if (s->n == 0) return MD_OK;
-    enqueue_bin(s, view(s, p), s->stream, copy_back);
+    enqueue_bin(s, view(s, p), s->stream, copy_back, nullptr);
     CKL();
-    s->launches += copy_back ? 8 : 7;
+    s->launches += bin_kernels(s, copy_back);
     s->lists_valid = false;
     s->forces_valid = false;
     return MD_OK;
@@ -421,7 +423,7 @@ int do_build(md_system* s, int p = 0) {
     }
     for (int attempt = 0; attempt < 4; ++attempt) {
         const DevState a = view(s, p);
-        CK(cudaMemsetAsync(a.stats, 0, 4 * sizeof(int32_t), s->stream));
+        if (attempt > 0) CK(cudaMemsetAsync(a.stats, 0, 4 * sizeof(int32_t), s->stream));
         CK(cudaMemsetAsync(a.err, 0, sizeof(uint32_t), s->stream));
         if (list_smem(s, s->list_cap, s->tile_cap) > 226 * 1024)
             return fail(s, MD_ERR_CELL_OVERFLOW, "tile (%d atoms) and lists (%d) exceed shared memory",
@@ -672,10 +674,8 @@ int capture_step(md_system* s, int mode, md_system::StepGraph& out) {
     CK(cudaStreamEndCapture(cs, &g));
     // the rebuild body
     CK(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-    enqueue_bin(s, a, cs, af(s));
-    cudaMemsetAsync(a.stats, 0, 4 * sizeof(int32_t), cs);
+    enqueue_bin(s, a, cs, af(s), s->d_ctrl + 1);
     enqueue_lists(s, a, cs);
-    launch_count_build(s->d_ctrl + 1, cs);
     CK(cudaStreamEndCapture(cs, &body));
     CKL();
     CK(cudaGraphInstantiate(&out.exec, g, 0));
@@ -729,10 +729,8 @@ int capture_fused(md_system* s, bool kkd, int p, md_system::StepGraph& out) {
     }
     CK(cudaStreamEndCapture(cs, &g));
     CK(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-    enqueue_bin(s, a, cs, af(s));
-    cudaMemsetAsync(a.stats, 0, 4 * sizeof(int32_t), cs);
+    enqueue_bin(s, a, cs, af(s), s->d_ctrl + 1);
     enqueue_lists(s, a, cs);
-    launch_count_build(s->d_ctrl + 1, cs);
     CK(cudaStreamEndCapture(cs, &body));
     CKL();
     CK(cudaGraphInstantiate(&out.exec, g, 0));
@@ -798,10 +796,8 @@ int capture_fused_multi(md_system* s, md_system::StepGraph& out) {
         tail.assign(deps, deps + ndeps);
         CK(cudaStreamEndCapture(cs, &g));
         CK(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
-        enqueue_bin(s, a, cs, af(s));
-        cudaMemsetAsync(a.stats, 0, 4 * sizeof(int32_t), cs);
+        enqueue_bin(s, a, cs, af(s), s->d_ctrl + 1);
         enqueue_lists(s, a, cs);
-        launch_count_build(s->d_ctrl + 1, cs);
         CK(cudaStreamEndCapture(cs, &body));
     }
     CKL();
@@ -870,10 +866,8 @@ int append_step(md_system* s, cudaGraph_t g, std::vector<cudaGraphNode_t>& tail,
     if ((rc = add_conditional(s, g, tail, h, cudaGraphCondTypeIf, &body))) return rc;
     std::vector<cudaGraphNode_t> none;
     rc = append_captured(s, body, none, [&](cudaStream_t cs) {
-        enqueue_bin(s, a, cs, af(s));
-        cudaMemsetAsync(a.stats, 0, 4 * sizeof(int32_t), cs);
+        enqueue_bin(s, a, cs, af(s), s->d_ctrl + 1);
         enqueue_lists(s, a, cs);
-        launch_count_build(s->d_ctrl + 1, cs);
     });
     if (rc) return rc;
     return append_captured(s, g, tail, [&](cudaStream_t cs) {
@@ -1114,7 +1108,7 @@ int run_chunk_fused(md_system* s, int len, bool first, bool last) {
     if (e & ERR_TILE_OVERFLOW) return MD_ERR_CELL_OVERFLOW;  // the chunk is redone: nothing of it counts
     if (e & ERR_LIST_OVERFLOW) return MD_ERR_LIST_OVERFLOW;
     const long long builds = builds_in_graphs(s);
-    s->launches += builds * (af(s) ? 10 : 9);  // binning (8, or 7 without the copy back), list build, build counter
+    s->launches += builds * (bin_kernels(s, af(s)) + 1);  // binning, list build
     if (builds > 0) {
         s->n_builds += builds;
         s->max_list = (int)s->h_flags[2];
@@ -1166,7 +1160,7 @@ int run_chunk(md_system* s, int len, bool first) {
     if (e & ERR_TILE_OVERFLOW) return MD_ERR_CELL_OVERFLOW;  // the chunk is redone: nothing of it counts
     if (e & ERR_LIST_OVERFLOW) return MD_ERR_LIST_OVERFLOW;
     const long long builds = builds_in_graphs(s);
-    s->launches += builds * (af(s) ? 10 : 9);  // binning (8, or 7 without the copy back), list build, build counter
+    s->launches += builds * (bin_kernels(s, af(s)) + 1);  // binning, list build
     if (builds > 0) {
         s->n_builds += builds;
         s->max_list = (int)s->h_flags[2];
@@ -1382,6 +1376,7 @@ int md_create(int64_t n, const double box[3], double r_cut, double skin, const m
     if (cudaMallocHost(&s->h_ctrl, 3 * sizeof(long long)) != cudaSuccess) return bail(MD_ERR_CUDA);
     if (cudaMemsetAsync(d0.err, 0, STATUS_WORDS * sizeof(uint32_t), s->stream) != cudaSuccess ||
         cudaMemsetAsync(s->parts_done, 0, sizeof(unsigned), s->stream) != cudaSuccess ||
+        cudaMemsetAsync(s->cell_count, 0, sizeof(int32_t) * g.ncell, s->stream) != cudaSuccess ||
         cudaStreamSynchronize(s->stream) != cudaSuccess)
         return bail(MD_ERR_CUDA);
     *out = s;

@@ -125,15 +125,11 @@ void launch_loop_ctrl(long long* passes_left, int done, cudaGraphConditionalHand
     k_loop_ctrl<<<1, 1, 0, st>>>(passes_left, done, handle);
 }
 
-__global__ void k_count_build(long long* n_builds) { *n_builds += 1; }
-
 void launch_step_ctrl(int policy, int every_k, int32_t* rebuild_flag, long long* step_counter,
                       long long* n_builds, uint32_t* err, cudaGraphConditionalHandle handle, cudaStream_t st) {
     (void)n_builds;
     k_step_ctrl<<<1, 1, 0, st>>>(policy, every_k, rebuild_flag, step_counter, err, handle);
 }
-
-void launch_count_build(long long* n_builds, cudaStream_t st) { k_count_build<<<1, 1, 0, st>>>(n_builds); }
 
 // snapshot copy of the permuted state (positions, velocities, images, species, ids)
 __global__ void k_copy_state(DevState d, DevState s) {

@@ -296,7 +296,9 @@ struct DevState {
 // ---- kernel launchers (defined in the .cu files)
 void launch_bin_assign(const DevState& s, const Geometry& g, int32_t* atom_cell, int32_t* cell_count,
                        cudaStream_t st);
-void launch_scan(const int32_t* in, int32_t* out_exclusive, int n, int32_t* scratch, cudaStream_t st);
+constexpr int STATS_WORDS = 5;  // of DevState.stats
+int scan_kernels(int n);
+void launch_scan(int32_t* counts, int32_t* cursor, int32_t* out_exclusive, int n, int32_t* scratch, cudaStream_t st);
 size_t scan_scratch_ints(int n);
 void launch_scatter(const DevState& s, const int32_t* atom_cell, const int32_t* cell_start, int32_t* cursor,
                     int32_t* slot_key, int32_t* slot_src, cudaStream_t st);
@@ -304,11 +306,10 @@ void launch_cell_sort(const Geometry& g, const int32_t* cell_start, const int32_
                       const int32_t* slot_src, int32_t* sorted_src, cudaStream_t st);
 void launch_gather(const DevState& s, const DevState& scratch, const Geometry& g, const int32_t* sorted_src,
                    const int32_t* atom_cell, int fp64, bool copy_back, cudaStream_t st);
-void launch_classify_blocks(const DevState& s, const Geometry& g, cudaStream_t st);
+void launch_classify_blocks(const DevState& s, const Geometry& g, long long* n_builds, cudaStream_t st);
 void launch_step_ctrl(int policy, int every_k, int32_t* rebuild_flag, long long* step_counter,
                       long long* n_builds, uint32_t* err, cudaGraphConditionalHandle handle, cudaStream_t st);
 void launch_loop_ctrl(long long* passes_left, int done, cudaGraphConditionalHandle handle, cudaStream_t st);
-void launch_count_build(long long* n_builds, cudaStream_t st);
 void launch_copy_state(const DevState& dst, const DevState& src, cudaStream_t st);
 void launch_build_lists(const DevState& s, const DevState& d, const Geometry& g, const TileOffsets& to, double rl2, int list_cap,
                         int tile_cap, int half, cudaStream_t st);
