@@ -38,7 +38,7 @@ struct md_system {
     int cur = 0;       // always 0: the state lives in st[0]
     // binning scratch
     int32_t *atom_cell = nullptr, *cell_count = nullptr, *cursor = nullptr, *slot_key = nullptr,
-            *slot_src = nullptr, *sorted_src = nullptr, *scan_scratch = nullptr;
+            *slot_src = nullptr, *scan_scratch = nullptr;
     double *partials = nullptr, *out8 = nullptr;
     unsigned* parts_done = nullptr;  // CTAs of the running energy reduction that have finished
     int nparts = 0;
@@ -301,8 +301,8 @@ int check_err(md_system* s, uint32_t mask) {
     return fail(s, MD_ERR_ARG, "device error 0x%x", e);
 }
 
-// assign, scan, scatter, in-cell order, gather (and copy back), occupied blocks
-int bin_kernels(const md_system* s, bool copy_back) { return 5 + scan_kernels(s->g.ncell) + (copy_back ? 1 : 0); }
+// assign, scan, scatter, in-cell order with gather (and copy back), occupied blocks
+int bin_kernels(const md_system* s, bool copy_back) { return 4 + scan_kernels(s->g.ncell) + (copy_back ? 1 : 0); }
 
 // ---- binning: assign, count, scan, scatter, in-cell order, gather.  The permuted state is then in
 // st[1], from where the list builder takes it to `a` (enqueue_lists has to follow; the other
@@ -313,8 +313,7 @@ void enqueue_bin(md_system* s, const DevState& a, cudaStream_t st, bool copy_bac
     launch_bin_assign(a, g, s->atom_cell, s->cell_count, st);
     launch_scan(s->cell_count, s->cursor, a.cell_start, g.ncell, s->scan_scratch, st);
     launch_scatter(a, s->atom_cell, a.cell_start, s->cursor, s->slot_key, s->slot_src, st);
-    launch_cell_sort(g, a.cell_start, s->slot_key, s->slot_src, s->sorted_src, st);
-    launch_gather(a, s->st[1], g, s->sorted_src, s->atom_cell, !mixed(s), copy_back, st);
+    launch_sort_gather(a, s->st[1], g, s->slot_key, s->slot_src, !mixed(s), copy_back, st);
     launch_classify_blocks(a, g, n_builds, st);
 }
 
@@ -1366,7 +1365,7 @@ int md_create(int64_t n, const double box[3], double r_cut, double skin, const m
     if ((rc = alloc_lists(s, lc))) return bail(rc);
     if ((rc = dalloc(s, &s->atom_cell, n)) || (rc = dalloc(s, &s->cell_count, g.ncell)) ||
         (rc = dalloc(s, &s->cursor, g.ncell)) || (rc = dalloc(s, &s->slot_key, n)) ||
-        (rc = dalloc(s, &s->slot_src, n)) || (rc = dalloc(s, &s->sorted_src, n)) ||
+        (rc = dalloc(s, &s->slot_src, n)) ||
         (rc = dalloc(s, &s->scan_scratch, scan_scratch_ints(g.ncell))))
         return bail(rc);
     s->nparts = 592;
