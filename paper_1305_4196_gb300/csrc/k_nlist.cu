@@ -134,6 +134,8 @@ __global__ void __launch_bounds__(NL_WARPS * 32, 3) k_build_lists_occ(DevState s
     }
 }
 
+static int g_sm_count = 0, g_sm_smem = 0;  // of the device, read at initialisation (never during a stream capture)
+
 // Shared memory of a CTA of `warps` warps.
 static size_t nl_smem_bytes(int tile_cap, int warps) { return nl_tile_bytes(tile_cap) + warps * sizeof(NlWarp); }
 
@@ -158,11 +160,14 @@ void launch_build_lists(const DevState& s, const DevState& d, const Geometry& g,
         else k_build_lists_occ<0><<<s.compact, threads, smem, st>>>(s, d, g, to, rl2, lo, hi, list_cap, tile_cap);
         return;
     }
-    // CTAs per block, each a share of every cell's atoms: while the grid is below two CTAs per SM,
-    // down to shares of about 8 atoms (32,000 atoms, 64 blocks: 150 us with one CTA each, 57 us
-    // with five)
-    const int per_cell = (int)((s.n + g.ncell - 1) / g.ncell);
-    const int split = std::max(1, std::min({(per_cell + 7) / 8, (2 * 152 + g.nblock - 1) / g.nblock, 16}));
+    // CTAs per block, each a share of every cell's atoms: as many as run at once, down to shares of two
+    // atoms (32,000 atoms, 64 blocks, two CTAs per SM: 95 us with one CTA per block, 39 with four, 55
+    // with five, whose last 16 start when the others end; 2,048 atoms, 8 blocks: 43 with one, 16 with
+    // sixteen).
+    const int sms = g_sm_count > 0 ? g_sm_count : 152;
+    const int64_t per_sm = std::min<int64_t>(3, (int64_t)(g_sm_smem > 0 ? g_sm_smem : 233472) / (int64_t)(smem + 1024));
+    const int64_t per_cell = (s.n + g.ncell - 1) / g.ncell;
+    const int split = (int)std::max<int64_t>(1, std::min<int64_t>({per_cell / 2, per_sm * sms / g.nblock, 16}));
     const unsigned grid = (unsigned)g.nblock * (unsigned)split;
     if (half) k_build_lists<1><<<grid, threads, smem, st>>>(s, d, g, to, rl2, lo, hi, list_cap, tile_cap, split);
     else k_build_lists<0><<<grid, threads, smem, st>>>(s, d, g, to, rl2, lo, hi, list_cap, tile_cap, split);
@@ -179,6 +184,11 @@ static void allow_max_smem(K kernel) {
 }
 
 void init_list_kernels(int half) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) {
+        cudaDeviceGetAttribute(&g_sm_count, cudaDevAttrMultiProcessorCount, dev);
+        cudaDeviceGetAttribute(&g_sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+    }
     if (half) {
         allow_max_smem(k_build_lists<1>);
         allow_max_smem(k_build_lists_occ<1>);
