@@ -22,7 +22,8 @@
 // Bound by instruction issue (68 % of cycles at 24 warps per SM; 80 registers, and
 // 42 KB of scan buffers beside the tile).  At 1,048,576 atoms: 590 us and 567 M warp
 // instructions with a lane per own atom that tested every atom of the 27 cells and
-// appended its own hits, 391 us and 322 M with the scan of nl_scan.cuh (other forms of it:
+// appended its own hits, 391 us and 322 M with the scan of nl_scan.cuh, 384 and 309 M with cheaper tile
+// offsets and the copy of the atoms' state (other forms of the scan:
 // 439 us with hit masks turned into entries by a loop over their bits; 551 us with the self
 // pair and the band sieved out of the rows by a lane each).
 #include "nl_scan.cuh"
