@@ -59,6 +59,12 @@ int mdgb_tile_cells(const int32_t nc[3], int32_t block, int32_t cells_out[64]);
  * |r2_fp32 - r2| / r_cut^2, plus the rounding of the FP32 thresholds. */
 int mdgb_cut_band(int32_t frame, double w_max, double half_skin, int32_t R, double r_cut, double *band_out);
 
+/* The shape of md_forces_backward and md_energy_param_grad for n atoms of n_species species on a
+ * grid of nc[3] cells, precision MD_*, on a device of n_sms SMs: CTAs per block, the double
+ * at which the reordered dL/dF starts in the workspace, and the workspace's size in doubles. */
+int mdgb_backward_shape(const int32_t nc[3], int64_t n, int32_t n_species, int32_t precision, int32_t n_sms,
+                        int32_t *split_out, int64_t *grad_at_out, int64_t *doubles_out);
+
 #ifdef __cplusplus
 }
 #endif

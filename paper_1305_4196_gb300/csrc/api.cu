@@ -1234,6 +1234,7 @@ int md_create(int64_t n, const double box[3], double r_cut, double skin, const m
     int rc = validate_params(s, p, r_cut);
     if (rc) return bail(rc);
     cudaGetDevice(&s->device);
+    cudaDeviceGetAttribute(&s->g.sms, cudaDevAttrMultiProcessorCount, s->device);
     s->stream = static_cast<cudaStream_t>(p->stream);
     {
         const char* ng = std::getenv("MDGB_NO_GRAPHS");
@@ -1622,14 +1623,14 @@ static int backward(md_system* s, const double* grad_f, int device_ptrs, double*
         if (rc) return rc;
         const int64_t n = s->n;
         double *G = nullptr, *gx = nullptr;
-        const size_t need = backward_scratch_doubles(s->g, ns, !mixed(s), n);
-        if (need > s->grad_ws_doubles) {  // kept by the system, as its other arrays
+        const BackwardPlan plan = backward_plan(s->g, ns, !mixed(s), n);
+        if (plan.doubles > s->grad_ws_doubles) {  // kept by the system, as its other arrays
             init_grad_kernels(!mixed(s), ns);
             dfree(s, s->grad_ws);
             s->grad_ws = nullptr;
             s->grad_ws_doubles = 0;
-            if ((rc = dalloc(s, &s->grad_ws, need))) return rc;
-            s->grad_ws_doubles = need;
+            if ((rc = dalloc(s, &s->grad_ws, plan.doubles))) return rc;
+            s->grad_ws_doubles = plan.doubles;
         }
         if (grad_f) {
             if (device_ptrs) {
@@ -1645,7 +1646,7 @@ static int backward(md_system* s, const double* grad_f, int device_ptrs, double*
         }
         const size_t smem = backward_smem_bytes(!mixed(s), s->tile_cap);
         if (smem > 226 * 1024) return fail(s, MD_ERR_CELL_OVERFLOW, "tile of %d atoms exceeds shared memory", s->tile_cap);
-        launch_force_backward(s->st[0], s->g, s->pt, s->to, s->tile_cap, !mixed(s), G, gx, s->grad_ws,
+        launch_force_backward(s->st[0], s->g, s->pt, s->to, s->tile_cap, !mixed(s), plan, G, gx, s->grad_ws,
                               s->stream);
         CKL();
         s->launches += (G ? 1 : 0) + 2;

@@ -51,6 +51,20 @@ int mdgb_cut_band(int32_t frame, double w_max, double half_skin, int32_t R, doub
     return MD_OK;
 }
 
+int mdgb_backward_shape(const int32_t nc[3], int64_t n, int32_t n_species, int32_t precision, int32_t n_sms,
+                        int32_t* split_out, int64_t* grad_at_out, int64_t* doubles_out) {
+    Geometry g{};
+    if (!split_out || !grad_at_out || !doubles_out || n < 1 || n_species < 1 || n_species > MAX_SPECIES ||
+        (precision != MD_FP64 && precision != MD_MIXED) || n_sms < 1 || !make_geometry(nc, g))
+        return MD_ERR_ARG;
+    g.sms = n_sms;
+    const BackwardPlan p = backward_plan(g, n_species, precision == MD_FP64, n);
+    *split_out = p.split;
+    *grad_at_out = (int64_t)p.sums;
+    *doubles_out = (int64_t)p.doubles;
+    return MD_OK;
+}
+
 int mdgb_num_blocks(const int32_t nc[3], int32_t* nblock_out) {
     Geometry g{};
     if (!nblock_out || !make_geometry(nc, g)) return MD_ERR_ARG;

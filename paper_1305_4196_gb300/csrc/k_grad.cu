@@ -38,7 +38,6 @@ constexpr int G_LPA = 4;  // lanes per own atom
 constexpr int G_THREADS = 512;
 constexpr int G_ATOMS = G_THREADS / G_LPA;  // own atoms at a time
 constexpr int G_QUANT = 2;                  // per species pair: the derivatives by eps and by sig
-static int g_sm_count = 0;                  // SMs of the device, read at initialisation
 
 // G of one atom in the arithmetic of the pairs.
 template <typename T>
@@ -316,23 +315,16 @@ size_t backward_smem_bytes(int fp64, int tile_cap) {
                     sizeof(double) * G_THREADS);
 }
 
-// CTAs per block: enough for one group of own atoms each, while the grid is below two CTAs
-// per SM (small systems, e.g. force-matching snapshots of a few 10^4 atoms)
-static int backward_split(const Geometry& g, int64_t n) {
-    const int sms = g_sm_count > 0 ? g_sm_count : 152;
+BackwardPlan backward_plan(const Geometry& g, int nsp, int fp64, int64_t n) {
+    BackwardPlan p;
     const int64_t per_block = (n + g.nblock - 1) / g.nblock;
-    const int split = (int)std::min<int64_t>((per_block + G_ATOMS - 1) / G_ATOMS, (2 * sms + g.nblock - 1) / g.nblock);
-    return std::max(1, std::min(split, 8));
-}
-
-// scratch layout: totals (nsp x nsp x 2) | partial sums (the same x CTAs) | G in cell order (n x 4 of T)
-static size_t backward_sums(const Geometry& g, int nsp, int64_t n) {
+    const int64_t split =
+        std::min<int64_t>((per_block + G_ATOMS - 1) / G_ATOMS, (2 * g.sms + g.nblock - 1) / g.nblock);
+    p.split = (int)std::max<int64_t>(1, std::min<int64_t>(split, 8));
     const size_t ncol = (size_t)nsp * nsp * G_QUANT;
-    return (ncol * (1 + (size_t)g.nblock * backward_split(g, n)) + 3) & ~(size_t)3;
-}
-
-size_t backward_scratch_doubles(const Geometry& g, int nsp, int fp64, int64_t n) {
-    return backward_sums(g, nsp, n) + (size_t)n * (fp64 ? 4 : 2);
+    p.sums = (ncol * (1 + (size_t)g.nblock * p.split) + 3) & ~(size_t)3;
+    p.doubles = p.sums + (size_t)n * (fp64 ? 4 : 2);
+    return p;
 }
 
 using Backward = void (*)(DevState, Geometry, PairTable, TileOffsets, int, const void*, double*, double*, int);
@@ -355,12 +347,13 @@ static Backward backward_kernel(int fp64, int energy, int nsp) {
 // With G: dL/deps and dL/dsig (columns 2 t and 2 t + 1 of the totals at the start of the scratch), and
 // dL/dx in the caller's order into gx.  Without: dE/deps and dE/dsig.
 void launch_force_backward(const DevState& s, const Geometry& g, const PairTable& pt, const TileOffsets& to,
-                           int tile_cap, int fp64, const double* G, double* gx, double* scratch, cudaStream_t st) {
+                           int tile_cap, int fp64, const BackwardPlan& plan, const double* G, double* gx,
+                           double* scratch, cudaStream_t st) {
     const int64_t n = s.n;
-    const int ncol = pt.nsp * pt.nsp * G_QUANT, split = backward_split(g, n);
-    const unsigned grid = (unsigned)g.nblock * (unsigned)split;
+    const int ncol = pt.nsp * pt.nsp * G_QUANT;
+    const unsigned grid = (unsigned)g.nblock * (unsigned)plan.split;
     double* part = scratch + ncol;
-    double* Gc = scratch + backward_sums(g, pt.nsp, n);
+    double* Gc = scratch + plan.sums;
     const int bs = 256;
     const unsigned nb = (unsigned)((n + bs - 1) / bs);
     if (G) {
@@ -368,7 +361,7 @@ void launch_force_backward(const DevState& s, const Geometry& g, const PairTable
         else k_grad_in<<<nb, bs, 0, st>>>(s, G, reinterpret_cast<Grad4<float>*>(Gc));
     }
     backward_kernel(fp64, G == nullptr, pt.nsp)<<<grid, G_THREADS, backward_smem_bytes(fp64, tile_cap), st>>>(
-        s, g, pt, to, tile_cap, Gc, gx, part, split);
+        s, g, pt, to, tile_cap, Gc, gx, part, plan.split);
     k_colsum<<<ncol, CS_THREADS, 0, st>>>(part, (int)grid, scratch);
 }
 
@@ -383,8 +376,6 @@ static void allow_max_smem(K kernel) {
 }
 
 void init_grad_kernels(int fp64, int nsp) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&g_sm_count, cudaDevAttrMultiProcessorCount, dev);
     for (int energy = 0; energy < 2; ++energy) allow_max_smem(backward_kernel(fp64, energy, nsp));
 }
 

@@ -50,6 +50,7 @@ struct Geometry {
     int linear;        // 1: linear block numbering (no colour classes)
     int nblock;        // number of 2x2x2 blocks
     int ncell;         // number of cells
+    int sms;           // SMs of the system's device (launch shapes)
 };
 
 // LJ pair constants per species pair (FP32 copies for the mixed path, FP64 for the FP64 path)
@@ -369,9 +370,18 @@ void init_half_af_kernels();
 void init_force_fp64_kernels(int half, int single);
 void init_grad_kernels(int fp64, int nsp);
 size_t backward_smem_bytes(int fp64, int tile_cap);
-size_t backward_scratch_doubles(const Geometry& g, int nsp, int fp64, int64_t n);
+// One derivative pass: CTAs per block (enough for one group of own atoms each, while the grid is below
+// two CTAs per SM: small systems, e.g. force-matching snapshots of a few 10^4 atoms), and
+// its scratch: totals (nsp x nsp x 2) | partial sums (the same x CTAs) | from `sums` on, G in cell order
+// (n x 4 of T).  Made once per call, for the allocation and the launch alike.
+struct BackwardPlan {
+    int split;
+    size_t sums, doubles;
+};
+BackwardPlan backward_plan(const Geometry& g, int nsp, int fp64, int64_t n);
 void launch_force_backward(const DevState& s, const Geometry& g, const PairTable& pt, const TileOffsets& to,
-                           int tile_cap, int fp64, const double* G, double* gx, double* scratch, cudaStream_t st);
+                           int tile_cap, int fp64, const BackwardPlan& plan, const double* G, double* gx,
+                           double* scratch, cudaStream_t st);
 void init_list_kernels(int half);
 
 // integrate modes
