@@ -136,9 +136,9 @@ int md_create(int64_t n, const double box[3], double r_cut, double skin,
 
 /*
  * Load positions, velocities (N x 3, original order) and species ids (N,
- * values in [0, n_species); NULL: all 0).  Positions may lie anywhere; they
- * are mapped into [0, L) at the next neighbour build.  Invalidates forces and
- * lists.  Errors: MD_ERR_ARG (bad species id), MD_ERR_NONFINITE (a position
+ * values in [0, n_species); NULL: all 0).  Positions may lie anywhere (up to 2^30
+ * box lengths away: beyond, the binning returns MD_ERR_NONFINITE); they are
+ * mapped into [0, L) at the next binning.  Invalidates forces and lists.  Errors: MD_ERR_ARG (bad species id), MD_ERR_NONFINITE (a position
  * or velocity is NaN or infinite; the state is not loaded), MD_ERR_CUDA.
  */
 int md_set_state(md_system *s, const double *pos, const double *vel,

@@ -14,8 +14,9 @@ namespace mdgb {
 
 // ---------------------------------------------------------------- assign
 // Map x into [0, L) (one box length at most, counted in the image counters:
-// the same operation the oracle applies at a rebuild) and find the cell.
-__global__ void k_bin_assign(DevState s, Geometry g, int32_t* __restrict__ atom_cell,
+// the same operation the oracle applies at a rebuild) and find the cell.  loaded: the first
+// binning of a state that the caller loaded, whose positions may lie any number of box lengths away.
+__global__ void k_bin_assign(DevState s, Geometry g, int loaded, int32_t* __restrict__ atom_cell,
                              int32_t* __restrict__ cell_count) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= s.n) return;
@@ -37,6 +38,14 @@ __global__ void k_bin_assign(DevState s, Geometry g, int32_t* __restrict__ atom_
         int cc = (int)(x * g.inv_w[d]);
         const long long bits = __double_as_longlong(x);
         if (bits < 0 || cc >= g.nc[d] - 1 || ((bits >> 52) & 0x7ff) == 0x7ff) {
+            if (loaded && !(x >= -L && x < 2.0 * L)) {
+                const double k = floor(x / L);
+                if (fabs(k) < 0x1p30) {  // (what the image counters can hold; else an error below)
+                    x = fma(-k, L, x);
+                    I[d][i] += (int)k;
+                    X[d][i] = x;
+                }
+            }
             if (x >= L) {
                 x = __dsub_rn(x, L);
                 I[d][i] += 1;
@@ -61,11 +70,11 @@ __global__ void k_bin_assign(DevState s, Geometry g, int32_t* __restrict__ atom_
     if ((int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&cell_count[id], __popc(peers));
 }
 
-void launch_bin_assign(const DevState& s, const Geometry& g, int32_t* atom_cell, int32_t* cell_count,
+void launch_bin_assign(const DevState& s, const Geometry& g, int loaded, int32_t* atom_cell, int32_t* cell_count,
                        cudaStream_t st) {
     if (s.n == 0) return;
     int bs = 256;
-    k_bin_assign<<<(unsigned)((s.n + bs - 1) / bs), bs, 0, st>>>(s, g, atom_cell, cell_count);
+    k_bin_assign<<<(unsigned)((s.n + bs - 1) / bs), bs, 0, st>>>(s, g, loaded, atom_cell, cell_count);
 }
 
 // ---------------------------------------------------------------- scan

@@ -295,7 +295,7 @@ struct DevState {
 };
 
 // ---- kernel launchers (defined in the .cu files)
-void launch_bin_assign(const DevState& s, const Geometry& g, int32_t* atom_cell, int32_t* cell_count,
+void launch_bin_assign(const DevState& s, const Geometry& g, int loaded, int32_t* atom_cell, int32_t* cell_count,
                        cudaStream_t st);
 constexpr int STATS_WORDS = 5;  // of DevState.stats
 int scan_kernels(int n);
