@@ -418,6 +418,7 @@ int do_build(md_system* s, int p = 0) {
         ev = take_events(s);
         CK(cudaEventRecord(ev.first, s->stream));
     }
+    CK(cudaMemsetAsync(s->st[0].err, 0, sizeof(uint32_t), s->stream));  // (what the binning reports counts)
     int rc = do_bin(s, p, af(s));
     if (rc) return rc;
     if (s->n == 0) {
@@ -426,8 +427,10 @@ int do_build(md_system* s, int p = 0) {
     }
     for (int attempt = 0; attempt < 4; ++attempt) {
         const DevState a = view(s, p);
-        if (attempt > 0) CK(cudaMemsetAsync(a.stats, 0, 4 * sizeof(int32_t), s->stream));
-        CK(cudaMemsetAsync(a.err, 0, sizeof(uint32_t), s->stream));
+        if (attempt > 0) {
+            CK(cudaMemsetAsync(a.stats, 0, 4 * sizeof(int32_t), s->stream));
+            CK(cudaMemsetAsync(a.err, 0, sizeof(uint32_t), s->stream));
+        }
         if (list_smem(s, s->list_cap, s->tile_cap) > 226 * 1024)
             return fail(s, MD_ERR_CELL_OVERFLOW, "tile (%d atoms) and lists (%d) exceed shared memory",
                         s->tile_cap, s->list_cap);
@@ -442,6 +445,7 @@ int do_build(md_system* s, int p = 0) {
         rc = sync_flags(s);
         if (rc) return rc;
         const uint32_t e = s->h_flags[0];
+        if (e & (ERR_ESCAPE | ERR_NONFINITE)) return check_err(s, ERR_ESCAPE | ERR_NONFINITE);
         const int max_list = (int)s->h_flags[2], max_tile = (int)s->h_flags[3];
         bool again = false;
         if (e & ERR_TILE_OVERFLOW) {
@@ -985,6 +989,7 @@ int run_steps_direct(md_system* s, int len, bool first) {
         CKL();
         s->launches += 1;
         if ((rc = sync_flags(s))) return rc;
+        if ((rc = check_err(s, ERR_NONFINITE | ERR_ESCAPE))) return rc;  // (a build below clears the error word)
         const long long step = s->n_steps + k + 1;
         bool rebuild = s->h_flags[1] != 0;
         if (s->rebuild == MD_REBUILD_EVERY_K) {
@@ -1011,6 +1016,7 @@ int run_steps_direct_fused(md_system* s, int len, bool first, bool last) {
     int p = 0;
     for (int k = 0; k < len; ++k) {
         if ((rc = sync_flags(s))) return rc;
+        if ((rc = check_err(s, ERR_NONFINITE | ERR_ESCAPE))) return rc;  // (a build below clears the error word)
         const long long step = s->n_steps + k + 1;
         bool rebuild = s->h_flags[1] != 0;
         if (s->rebuild == MD_REBUILD_EVERY_K) {

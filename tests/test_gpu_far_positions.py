@@ -1,4 +1,5 @@
-"""Positions any number of box lengths away are mapped into the box at the first binning."""
+"""Positions any number of box lengths away are mapped into the box at the first binning, and an atom
+that later moves by more than one box length between builds is an error on every path that builds."""
 import numpy as np
 import pytest
 
@@ -48,3 +49,32 @@ def test_positions_anywhere(kind, first):
         s.close()
     for a, b in zip(*res):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("x", [2.0 ** 31 * 14.0, -1.0e300])
+def test_positions_beyond_the_image_counters(x):
+    pos, vel = _liquid()
+    pos[9, 1] = x
+    s = M.System(len(pos), np.full(3, 14.0))
+    for call in (s.forces, s.build_neighbors, s.bin_cells, lambda: s.step(1), s.energy_virial):
+        s.set_state(pos, vel)
+        with pytest.raises(M.MDError):
+            call()
+    s.close()
+
+
+@pytest.mark.parametrize("kind", list(KINDS))
+@pytest.mark.parametrize("no_graphs", ["0", "1"])
+@pytest.mark.parametrize("steps", [1, 2, 5])
+def test_an_atom_that_escapes_is_an_error(monkeypatch, kind, no_graphs, steps):
+    """2.5 box lengths in one step: the build in that step reports it, in graphs and launched from the
+    host, also when further steps follow."""
+    monkeypatch.setenv("MDGB_NO_GRAPHS", no_graphs)
+    pos, vel = _liquid()
+    vel[9, 1] = 2.5 * 14.0 / 0.005
+    s = M.System(len(pos), np.full(3, 14.0), dt=0.005, **KINDS[kind])
+    s.set_state(pos, vel)
+    with pytest.raises(M.MDError) as e:
+        s.step(steps)
+    assert e.value.code == M.MD_ERR_NONFINITE
+    s.close()
