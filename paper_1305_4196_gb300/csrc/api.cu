@@ -431,9 +431,15 @@ int do_build(md_system* s, int p = 0) {
             CK(cudaMemsetAsync(a.stats, 0, 4 * sizeof(int32_t), s->stream));
             CK(cudaMemsetAsync(a.err, 0, sizeof(uint32_t), s->stream));
         }
-        if (list_smem(s, s->list_cap, s->tile_cap) > 226 * 1024)
+        if (list_smem(s, s->list_cap, s->tile_cap) > 226 * 1024) {
+            if (attempt == 0 && !af(s)) {  // no list builder takes the state to its new order
+                launch_copy_back(a, s->st[1], s->stream);
+                CKL();
+                s->launches += 1;
+            }
             return fail(s, MD_ERR_CELL_OVERFLOW, "tile (%d atoms) and lists (%d) exceed shared memory",
                         s->tile_cap, s->list_cap);
+        }
         enqueue_lists(s, a, s->stream);
         CKL();
         s->launches += 1;

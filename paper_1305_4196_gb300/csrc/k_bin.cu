@@ -280,6 +280,11 @@ __global__ void k_copy_back(DevState s, DevState d) {
     s.orig[t] = d.orig[t];
 }
 
+void launch_copy_back(const DevState& s, const DevState& scratch, cudaStream_t st) {
+    const int bs = 256;
+    k_copy_back<<<(unsigned)((s.n + bs - 1) / bs), bs, 0, st>>>(s, scratch);
+}
+
 void launch_sort_gather(const DevState& s, const DevState& scratch, const Geometry& g, const int32_t* slot_key,
                         const int32_t* slot_src, int fp64, bool copy_back, cudaStream_t st) {
     if (s.n == 0) return;
@@ -289,7 +294,7 @@ void launch_sort_gather(const DevState& s, const DevState& scratch, const Geomet
     const int64_t threads = (int64_t)g.ncell * 32 * parts;
     k_sort_gather<<<(unsigned)((threads + bs - 1) / bs), bs, 0, st>>>(scratch, s, g, slot_key, slot_src, fp64,
                                                                        parts);
-    if (copy_back) k_copy_back<<<(unsigned)((s.n + bs - 1) / bs), bs, 0, st>>>(s, scratch);
+    if (copy_back) launch_copy_back(s, scratch, st);
 }
 
 // ---------------------------------------------------------------- occupied blocks

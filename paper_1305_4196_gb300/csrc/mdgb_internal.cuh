@@ -305,6 +305,7 @@ void launch_scatter(const DevState& s, const int32_t* atom_cell, const int32_t* 
                     int32_t* slot_key, int32_t* slot_src, cudaStream_t st);
 void launch_sort_gather(const DevState& s, const DevState& scratch, const Geometry& g, const int32_t* slot_key,
                         const int32_t* slot_src, int fp64, bool copy_back, cudaStream_t st);
+void launch_copy_back(const DevState& s, const DevState& scratch, cudaStream_t st);
 void launch_classify_blocks(const DevState& s, const Geometry& g, long long* n_builds, cudaStream_t st);
 void launch_step_ctrl(int policy, int every_k, int32_t* rebuild_flag, long long* step_counter,
                       long long* n_builds, uint32_t* err, cudaGraphConditionalHandle handle, cudaStream_t st);
