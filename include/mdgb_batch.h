@@ -80,6 +80,13 @@ int md_batch_get_state(md_batch *b, double *pos, double *vel, int32_t *image, in
 int md_batch_layout(md_batch *b, int32_t *path, int32_t *threads, int32_t *cell_range);
 
 /*
+ * The launch: form[k] of each system, 0 (one CTA for the whole call), 1 (block tasks), 2 (the
+ * one-CTA operations shared out as tasks) or -1 (no atoms); the CTAs an SM holds at once; the
+ * dynamic shared memory of a CTA.  form: host array of n_systems; any output may be NULL.
+ */
+int md_batch_launch_shape(md_batch *b, int32_t *form, int32_t *ctas_per_sm, int64_t *smem_bytes);
+
+/*
  * Autotuner: times 10 steps of the whole ensemble per candidate (the state is
  * restored afterwards) and keeps the fastest: the CTA size (128, 256, 512), then
  * the largest system run by one CTA (1,024, 2,048, 4,096 atoms), then for each

@@ -16,14 +16,15 @@ _lib.md_batch_forces.argtypes = [_P, _P, C.c_int]
 _lib.md_batch_energies.argtypes = [_P, _P, _P]
 _lib.md_batch_get_state.argtypes = [_P, _P, _P, _P, C.c_int]
 _lib.md_batch_layout.argtypes = [_P, _P, _P, _P]
+_lib.md_batch_launch_shape.argtypes = [_P, _P, _P, _P]
 _lib.md_batch_autotune.argtypes = [_P, C.c_char_p]
 _lib.md_batch_set_wait_budget.argtypes = [_P, C.c_int64, C.c_int32]
 _lib.md_batch_last_error.argtypes = [_P, C.c_char_p, C.c_int64]
 _lib.md_batch_destroy.argtypes = [_P]
 _lib.md_batch_destroy.restype = None
 for _f in ("md_batch_create", "md_batch_set_state", "md_batch_step", "md_batch_forces", "md_batch_energies",
-           "md_batch_get_state", "md_batch_layout", "md_batch_autotune", "md_batch_last_error",
-           "md_batch_set_wait_budget"):
+           "md_batch_get_state", "md_batch_layout", "md_batch_launch_shape", "md_batch_autotune",
+           "md_batch_last_error", "md_batch_set_wait_budget"):
     getattr(_lib, _f).restype = C.c_int
 
 
@@ -93,6 +94,12 @@ class Batch:
         path, th, R = (np.empty(self.nsys, dtype=np.int32) for _ in range(3))
         self._check(_lib.md_batch_layout(self.handle, path.ctypes.data, th.ctypes.data, R.ctypes.data))
         return path, th, R
+
+    def launch_shape(self):
+        """(form of each system, CTAs per SM, dynamic shared memory of a CTA); see md_batch_launch_shape."""
+        form, ctas, smem = np.empty(self.nsys, dtype=np.int32), C.c_int32(), C.c_int64()
+        self._check(_lib.md_batch_launch_shape(self.handle, form.ctypes.data, C.byref(ctas), C.byref(smem)))
+        return form, ctas.value, smem.value
 
     def autotune(self, cache_path=None):
         self._check(_lib.md_batch_autotune(self.handle, cache_path.encode() if cache_path else None))

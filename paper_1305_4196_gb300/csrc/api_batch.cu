@@ -69,7 +69,7 @@ struct md_batch {
     EnsEntry* d_ent = nullptr;
     unsigned long long* d_ctl_init = nullptr;
     int64_t ncell_blk = 0;  // cells of the block systems
-    int nmax = 0, cmax = 0, tile_slots = 0, grid = 0;
+    int nmax = 0, cmax = 0, tile_slots = 0, per_sm = 0, grid = 0;
     size_t smem = 0;
     // test hook: a held entry and a budget (launched without a graph)
     int hold = -1;
@@ -244,12 +244,11 @@ int build_table(md_batch* b) {
     BCK(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, b->device));
     if (smem + 8192 > (size_t)optin)
         return bfail(b, MD_ERR_CELL_OVERFLOW, "an ensemble task needs %zu B of shared memory", smem);
-    b->tile_slots = (int)(smem / sizeof(float4)) - 1;
-    if (!b->blk.empty()) smem += ENS_LIST_EXTRA;
     b->smem = smem;
-    const int per_sm = ensemble_ctas_per_sm(b->threads, smem);
-    if (per_sm < 1) return bfail(b, MD_ERR_CUDA, "the ensemble kernel does not fit an SM at %d threads", b->threads);
-    b->grid = per_sm * b->sms;
+    b->tile_slots = (int)(smem / sizeof(float4)) - 1;
+    b->per_sm = ensemble_ctas_per_sm(b->threads, smem);
+    if (b->per_sm < 1) return bfail(b, MD_ERR_CUDA, "the ensemble kernel does not fit an SM at %d threads", b->threads);
+    b->grid = b->per_sm * b->sms;
     // initial scheduler words: one-CTA systems at their task, the others at START
     std::vector<unsigned long long> init(b->ent.size(), 0ull);
     for (size_t e = 0; e < b->ent.size(); ++e)
@@ -666,6 +665,17 @@ int md_batch_layout(md_batch* b, int32_t* path, int32_t* threads, int32_t* cell_
         if (threads) threads[k] = b->threads;
         if (cell_range) cell_range[k] = one ? b->R[bucket_of(b->n[k])] : 1;
     }
+    return MD_OK;
+}
+
+int md_batch_launch_shape(md_batch* b, int32_t* form, int32_t* ctas_per_sm, int64_t* smem_bytes) {
+    if (!b) return MD_ERR_ARG;
+    if (form) {
+        std::fill(form, form + b->nsys, -1);
+        for (const EnsEntry& en : b->ent) form[en.kind == 1 ? b->blk[en.idx].id : b->one[en.idx].id] = en.kind;
+    }
+    if (ctas_per_sm) *ctas_per_sm = b->per_sm;
+    if (smem_bytes) *smem_bytes = (int64_t)b->smem;
     return MD_OK;
 }
 

@@ -804,11 +804,15 @@ __device__ __forceinline__ void ens_stage(const EnsBlockSys& y, const float4* __
     __syncthreads();
 }
 
-// Shared memory of a LIST task: the scan's buffers and the tile of T atoms.  The host sizes the
-// launch by ens_list_smem and adds ENS_LIST_EXTRA behind what a FORCE tile may take.
+// Shared memory of a LIST task: the tile of T atoms, and in what it leaves the scan's buffers of
+// as many warps as fit, all eight unless the tile comes within some 500 atoms of what the launch is sized for
+// (six then, so a second round over the cells).  Sizing every launch for eight would cost
+// 6 KB, and an ensemble whose tile is near half of an SM's memory its second CTA.
 __host__ __device__ inline size_t ens_list_smem_bytes(int T) {
-    return nl_tile_bytes(T) + NL_WARPS * sizeof(NlWarp);
+    return (size_t)((T + 228) & ~3) * 3 * sizeof(float) + 32768;
 }
+constexpr int ENS_LIST_WARPS_MIN = 6;
+static_assert(ENS_LIST_WARPS_MIN * sizeof(NlWarp) <= 32768 + 224 * 3 * sizeof(float), "a LIST task's buffers");
 
 // LIST: the Verlet lists of the own atoms of block b, by the candidate scan of the main
 // builder (nl_scan.cuh): a warp takes an own cell; entries are tile indices in chunks of 8
@@ -826,7 +830,8 @@ __device__ void ens_list(const EnsBlockSys& y, const BatchState& st, const EnsAr
     for (int d = 0; d < 3; ++d)
 #pragma unroll
         for (int q = 0; q < 4; ++q) to.off[d][q] = y.off[d][q];
-    float* const tx = reinterpret_cast<float*>(smem + NL_WARPS * sizeof(NlWarp));
+    const int lw = min(NL_WARPS, (int)((smem_bytes - nl_tile_bytes(T)) / sizeof(NlWarp)));
+    float* const tx = reinterpret_cast<float*>(smem + lw * sizeof(NlWarp));
     const int stride = (T + 3) & ~3;
     float* const ty = tx + stride;
     float* const tz = ty + stride;
@@ -835,11 +840,11 @@ __device__ void ens_list(const EnsBlockSys& y, const BatchState& st, const EnsAr
     __syncthreads();
     const PosBuf P = ens_pos(st, ea, odd);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    if (warp >= NL_WARPS) return;
+    if (warp >= lw) return;
     NlWarp& w = reinterpret_cast<NlWarp*>(smem)[warp];
     const int cap = ea.list_chunks * 8;
     uint4* nl = ea.nl + y.a0 * (int64_t)ea.list_chunks;
-    for (int oc = warp; oc < 8; oc += min(nw, NL_WARPS)) {
+    for (int oc = warp; oc < 8; oc += min(nw, lw)) {
         const int own_coord = (1 + (oc & 1)) + 4 * (1 + ((oc >> 1) & 1)) + 16 * (1 + (oc >> 2));
         const int count = mt.prefix[oc + 1] - mt.prefix[oc];
         for (int lo_own = 0; lo_own < count; lo_own += 32) {
@@ -886,7 +891,7 @@ __device__ __forceinline__ AtomState ens_load_state(const BatchState& st, const 
 }
 
 // Centres of a block's own cells (x, y, z of each) in cell widths, by the block's first threads.
-__device__ __forceinline__ void ens_centres(const EnsBlockSys& y, int b, double (&centre)[8][3]) {
+__device__ __forceinline__ void ens_centres(const EnsBlockSys& y, int b, double (*centre)[3]) {
     if (threadIdx.x < 24) {
         const int os = threadIdx.x / 3, d = threadIdx.x % 3;
         const int bd = d == 0 ? b % y.nb[0] : (d == 1 ? (b / y.nb[0]) % y.nb[1] : b / (y.nb[0] * y.nb[1]));
@@ -974,8 +979,7 @@ struct EnsList {
 template <bool ENERGY>
 __device__ void ens_force(const EnsBlockSys& y, const BatchState& st, const EnsArrays& ea, const PairTable& pt,
                           float fs2_max, int k, int K, double dt, int b, int bidx, int tile_slots, float4* tile,
-                          EnsTile& mt, uint16_t* queue, int* nqueued) {
-    __shared__ double centre[8][3];
+                          EnsTile& mt, uint16_t* queue, int* nqueued, double (*centre)[3]) {
     const bool odd = (k & 1) != 0;
     if (threadIdx.x == 0) *nqueued = 0;
     ens_meta(y, ea, b, mt);
@@ -1215,7 +1219,8 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS, 1)
     __shared__ double red[BATCH_MAX_THREADS];
     __shared__ int nqueued;
     __shared__ EnsTile mt;
-    const size_t smem_bytes = (size_t)(tile_slots + 1) * sizeof(float4) + ENS_LIST_EXTRA;
+    const size_t smem_bytes = (size_t)(tile_slots + 1) * sizeof(float4);
+    double(*centre)[3] = reinterpret_cast<double(*)[3]>(red);  // (a FORCE task reduces nothing)
     __shared__ uint16_t queue[ENS_QUEUE];
     __shared__ int s_ent, s_task, s_take, s_quit;
     __shared__ uint32_t s_phase;
@@ -1329,10 +1334,10 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS, 1)
                         default:
                             if (energy_call && k == K)
                                 ens_force<true>(y, st, ea, pt, fs2_max, k, K, dt, task, en.idx, tile_slots, tile, mt,
-                                                queue, &nqueued);
+                                                queue, &nqueued, centre);
                             else
                                 ens_force<false>(y, st, ea, pt, fs2_max, k, K, dt, task, en.idx, tile_slots, tile, mt,
-                                                 queue, &nqueued);
+                                                 queue, &nqueued, centre);
                     }
                 }
             }
@@ -1361,8 +1366,7 @@ size_t batch_smem_bytes(int nmax, int cmax) {
 
 size_t ens_tile_smem_bytes(int tile_slots) { return (size_t)(tile_slots + 1) * sizeof(float4); }
 
-static_assert(NL_WARPS * sizeof(NlWarp) <= 32768 + 228 * 12 + ENS_LIST_EXTRA, "a LIST task's buffers");
-size_t ens_list_smem(int T) { return (size_t)((T + 228) & ~3) * 3 * sizeof(float) + 32768; }
+size_t ens_list_smem(int T) { return ens_list_smem_bytes(T); }
 
 void launch_ensemble(const EnsEntry* ent, int nent, const BatchSys* one, const EnsBlockSys* blk,
                      const BatchState& st, const EnsArrays& ea, const PairTable& pt, int n_steps, int flags,

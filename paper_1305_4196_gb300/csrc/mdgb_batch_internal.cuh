@@ -97,9 +97,7 @@ size_t batch_smem_bytes(int nmax, int cmax);
 // Dynamic shared memory of a block task's tile of at most tile_slots slots (float4 each,
 // plus the far slot after the last).
 size_t ens_tile_smem_bytes(int tile_slots);
-// Dynamic shared memory of a block system's list build for a tile of T atoms, without the
-// ENS_LIST_EXTRA bytes that every launch with block systems adds.
-constexpr size_t ENS_LIST_EXTRA = 6272;
+// Dynamic shared memory of a block system's list build for a tile of T atoms.
 size_t ens_list_smem(int T);
 // One persistent launch over every system of the ensemble (k_batch.cu).
 void launch_ensemble(const EnsEntry* ent, int nent, const BatchSys* one, const EnsBlockSys* blk,
