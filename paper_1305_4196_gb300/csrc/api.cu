@@ -46,7 +46,7 @@ struct md_system {
     // [2..9] stats, then the control words (d_ctrl)
     uint32_t* h_flags = nullptr;
     bool has_state = false, lists_valid = false, forces_valid = false;
-    bool loaded = false;  // the state came from md_set_state and has not been binned yet
+    bool far = false;  // md_set_state loaded positions outside the box and no binning has followed
     int64_t n_builds = 0, n_steps = 0, list_entries = 0;
     int max_list = 0, max_tile = 0;
     std::vector<void*> allocs;
@@ -309,11 +309,9 @@ int bin_kernels(const md_system* s, bool copy_back) { return 4 + scan_kernels(s-
 // st[1], from where the list builder takes it to `a` (enqueue_lists has to follow; the other
 // builder, of the half lists without atomic operations, does not: copied back here).
 // The statistics of the build start at zero.  n_builds: see launch_classify_blocks.
-// loaded: see k_bin_assign.
-void enqueue_bin(md_system* s, const DevState& a, cudaStream_t st, bool copy_back, long long* n_builds,
-                 bool loaded = false) {
+void enqueue_bin(md_system* s, const DevState& a, cudaStream_t st, bool copy_back, long long* n_builds) {
     const Geometry& g = s->g;
-    launch_bin_assign(a, g, loaded, s->atom_cell, s->cell_count, st);
+    launch_bin_assign(a, g, s->atom_cell, s->cell_count, st);
     launch_scan(s->cell_count, s->cursor, a.cell_start, g.ncell, s->scan_scratch, st);
     launch_scatter(a, s->atom_cell, a.cell_start, s->cursor, s->slot_key, s->slot_src, st);
     launch_sort_gather(a, s->st[1], g, s->slot_key, s->slot_src, !mixed(s), copy_back, st);
@@ -322,9 +320,13 @@ void enqueue_bin(md_system* s, const DevState& a, cudaStream_t st, bool copy_bac
 
 int do_bin(md_system* s, int p, bool copy_back) {
     if (s->n == 0) return MD_OK;
-    enqueue_bin(s, view(s, p), s->stream, copy_back, nullptr, s->loaded);
+    if (s->far) {
+        launch_map_far(view(s, p), s->g, s->stream);
+        s->launches += 1;
+        s->far = false;
+    }
+    enqueue_bin(s, view(s, p), s->stream, copy_back, nullptr);
     CKL();
-    s->loaded = false;
     s->launches += bin_kernels(s, copy_back);
     s->lists_valid = false;
     s->forces_valid = false;
@@ -1424,7 +1426,7 @@ int md_set_state(md_system* s, const double* pos, const double* vel, const int32
     }
     s->cur = 0;
     CK(cudaMemsetAsync(s->st[0].err, 0, sizeof(uint32_t), s->stream));
-    launch_set_state(s->st[0], dpos, dvel, dsp, s->pt.nsp, s->stream);
+    launch_set_state(s->st[0], s->g, dpos, dvel, dsp, s->pt.nsp, s->stream);
     CKL();
     if (tmp) CK(cudaFreeAsync(tmp, s->stream));
     if (tsp) CK(cudaFreeAsync(tsp, s->stream));
@@ -1436,7 +1438,7 @@ int md_set_state(md_system* s, const double* pos, const double* vel, const int32
     if (s->h_flags[0] & 0x80000000u) return fail(s, MD_ERR_ARG, "species id out of range");
     if (s->h_flags[0] & 0x40000000u) return fail(s, MD_ERR_NONFINITE, "non-finite position or velocity");
     s->has_state = true;
-    s->loaded = true;
+    s->far = (s->h_flags[0] & 0x20000000u) != 0;
     return MD_OK;
 }
 

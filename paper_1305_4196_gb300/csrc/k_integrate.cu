@@ -247,7 +247,7 @@ void launch_reduce_energy(const DevState& s, const PairTable& pt, int mixed, dou
 }
 
 // ---------------------------------------------------------------- state I/O
-__global__ void k_set_state(DevState s, const double* __restrict__ pos, const double* __restrict__ vel,
+__global__ void k_set_state(DevState s, Geometry g, const double* __restrict__ pos, const double* __restrict__ vel,
                             const int32_t* __restrict__ species, int nsp) {
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i >= s.n) return;
@@ -259,6 +259,14 @@ __global__ void k_set_state(DevState s, const double* __restrict__ pos, const do
             atomicOr(s.err, 0x40000000u);
             q[k] = 0.0;
         }
+    // below -L or at 2 L and beyond, by the upper words (a position just above -L counts too): k_map_far
+    bool far = false;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const int h = __double2hiint(q[d]), hL = __double2hiint(g.L[d]);
+        far |= h >= 0 ? h >= hL + (1 << 20) : (h & 0x7fffffff) >= hL;
+    }
+    if (far) atomicOr(s.err, 0x20000000u);
     s.x[i] = q[0];
     s.y[i] = q[1];
     s.z[i] = q[2];
@@ -277,11 +285,11 @@ __global__ void k_set_state(DevState s, const double* __restrict__ pos, const do
     s.orig[i] = (int32_t)i;
 }
 
-void launch_set_state(const DevState& s, const double* pos, const double* vel, const int32_t* species, int nsp,
+void launch_set_state(const DevState& s, const Geometry& g, const double* pos, const double* vel, const int32_t* species, int nsp,
                       cudaStream_t st) {
     if (s.n == 0) return;
     int bs = 256;
-    k_set_state<<<(unsigned)((s.n + bs - 1) / bs), bs, 0, st>>>(s, pos, vel, species, nsp);
+    k_set_state<<<(unsigned)((s.n + bs - 1) / bs), bs, 0, st>>>(s, g, pos, vel, species, nsp);
 }
 
 __global__ void k_get_state(DevState s, double* __restrict__ pos, double* __restrict__ vel,

@@ -295,8 +295,9 @@ struct DevState {
 };
 
 // ---- kernel launchers (defined in the .cu files)
-void launch_bin_assign(const DevState& s, const Geometry& g, int loaded, int32_t* atom_cell, int32_t* cell_count,
+void launch_bin_assign(const DevState& s, const Geometry& g, int32_t* atom_cell, int32_t* cell_count,
                        cudaStream_t st);
+void launch_map_far(const DevState& s, const Geometry& g, cudaStream_t st);
 constexpr int STATS_WORDS = 5;  // of DevState.stats
 int scan_kernels(int n);
 void launch_scan(int32_t* counts, int32_t* cursor, int32_t* out_exclusive, int n, int32_t* scratch, cudaStream_t st);
@@ -350,7 +351,7 @@ void launch_integrate(const DevState& s, const Geometry& g, const PairTable& pt,
                       double dt, double lim2, cudaStream_t st);
 void launch_reduce_energy(const DevState& s, const PairTable& pt, int mixed, double* partials, unsigned* finished,
                           int nparts, double* out8, cudaStream_t st);
-void launch_set_state(const DevState& s, const double* pos, const double* vel, const int32_t* species,
+void launch_set_state(const DevState& s, const Geometry& g, const double* pos, const double* vel, const int32_t* species,
                       int nsp, cudaStream_t st);
 void launch_get_state(const DevState& s, double* pos, double* vel, int32_t* image, cudaStream_t st);
 void launch_forces_out(const DevState& s, int mixed, double* f_out, cudaStream_t st);

@@ -51,6 +51,27 @@ def test_positions_anywhere(kind, first):
         assert np.array_equal(a, b)
 
 
+@pytest.mark.parametrize("L", [14.0, 13.37])
+def test_edges_of_the_mapping(L):
+    """Coordinates at and beside -L, 0, L, 2 L and further: in the box after the binning, and at the place that
+    the image counters give to the last bit of the coordinate."""
+    edges = [e * L for e in (-3.0, -2.0, -1.0, 0.0, 1.0, 2.0, 3.0, 4097.0)]
+    xs = np.array(sorted({f(e) for e in edges for f in (
+        lambda e: e, lambda e: np.nextafter(e, np.inf), lambda e: np.nextafter(e, -np.inf),
+        lambda e: e * (1 + 2.0 ** -21), lambda e: e * (1 - 2.0 ** -21), lambda e: e + 0.3, lambda e: e - 0.3)}))
+    rng = np.random.default_rng(2)
+    pos = rng.uniform(0, L, (len(xs), 3))
+    pos[:, 1] = xs
+    s = M.System(len(xs), np.full(3, L))
+    s.set_state(pos, np.zeros_like(pos))
+    s.bin_cells()
+    x, _, image = s.get_state()
+    assert (x >= 0).all() and (x <= L).all()
+    assert np.array_equal(x[:, ::2], pos[:, ::2]) and not image[:, ::2].any()
+    assert (np.abs(x[:, 1] + image[:, 1] * L - xs) <= 2.0 ** -51 * np.maximum(np.abs(xs), L)).all()
+    s.close()
+
+
 @pytest.mark.parametrize("x", [2.0 ** 31 * 14.0, -1.0e300])
 def test_positions_beyond_the_image_counters(x):
     pos, vel = _liquid()
