@@ -10,9 +10,11 @@
 //
 // Energies use the paper's thread-local accumulators (Sec. II.C) in a fixed
 // order: per-atom shares, then per-CTA FP64 partials, then the last CTA sums those.
+#include "float_sum.cuh"
 #include "mdgb_internal.cuh"
 
 #include <algorithm>
+#include <type_traits>
 
 namespace mdgb {
 
@@ -156,72 +158,85 @@ void launch_copy_state(const DevState& dst, const DevState& src, cudaStream_t st
 
 // ---------------------------------------------------------------- reductions
 // (PE, KE, W_xx, W_yy, W_zz, W_xy, W_xz, W_yz): partial[b][0..7] over a contiguous chunk, each thread
-// summing a fixed strided subset in order, then a fixed-shape tree; the CTA that finishes last
-// sums the partials in the same way.
+// summing a fixed strided subset in order, then the lanes of a warp, then the warps, in a fixed
+// shape; the CTA that finishes last sums the partials.
 //
-// The FP64 pipe bounds this (an SM takes 16 cycles for a warp's FP64 addition or conversion), so a
-// thread adds its atoms' FP32 shares in two floats, hi and lo, with the rounding error of
-// every addition to hi kept in lo (to 2^-46 of the sum of its few atoms), and converts once: 54 -> 29 us
-// for 1,048,576 atoms (with the second launch that it saves).
-constexpr int RED_THREADS = 256;
+// The FP64 pipe would bound this (an SM takes 16 cycles for a warp's FP64 addition or conversion), so
+// FP32 shares are added in three floats up to the warp's sums (FloatSum: no less exact than FP64
+// sums), and the lanes of a warp add each column in a part of the warp only.  At 1,048,576 atoms
+// 54 us with FP64 sums per thread and a second launch, 18 so; at 2,048 atoms 14 and 5.3, at 360,703 in
+// FP64 24.5 (a tree over all threads) and 18.6.
+constexpr int RED_THREADS = 256, RED_WARPS = RED_THREADS / 32;
 
-struct FloatSum {
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float x) {
-        const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
-        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
-        hi = s;
-    }
-    // (a sum that is not finite stays what hi says)
-    __device__ __forceinline__ double get() const { return (double)hi + (isfinite(lo) ? (double)lo : 0.0); }
+struct DoubleSum {
+    double v = 0.0;
+    __device__ __forceinline__ void add(double x) { v += x; }
+    __device__ __forceinline__ void add(const DoubleSum& o) { v += o.v; }
+    __device__ __forceinline__ double get() const { return v; }
 };
 
-__device__ __forceinline__ void reduce_tree(double (&sh)[8][RED_THREADS], const double (&acc)[8]) {
-#pragma unroll
-    for (int c = 0; c < 8; ++c) sh[c][threadIdx.x] = acc[c];
-    __syncthreads();
-    for (int w = RED_THREADS / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
-#pragma unroll
-            for (int c = 0; c < 8; ++c) sh[c][threadIdx.x] += sh[c][threadIdx.x + w];
-        __syncthreads();
-    }
+__device__ __forceinline__ DoubleSum lane_xor(const DoubleSum& s, int o) {
+    return DoubleSum{__shfl_xor_sync(0xffffffffu, s.v, o)};
 }
 
-__global__ void __launch_bounds__(RED_THREADS) k_reduce_energy(DevState s, PairTable pt, int mixed, int64_t chunk,
-                                                               double* __restrict__ partials,
-                                                               unsigned* __restrict__ finished,
-                                                               double* __restrict__ out8) {
-    __shared__ double sh[8][RED_THREADS];
+__device__ __forceinline__ double warp_sum(double v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+template <bool MIXED>
+__global__ void __launch_bounds__(RED_THREADS, 4) k_reduce_energy(DevState s, PairTable pt, int64_t chunk,
+                                                                  double* __restrict__ partials,
+                                                                  unsigned* __restrict__ finished,
+                                                                  double* __restrict__ out8) {
+    __shared__ double sh[RED_WARPS][8];
     __shared__ bool last;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t n = s.n;
     const int64_t lo = blockIdx.x * chunk;
     const int64_t hi = lo + chunk < n ? lo + chunk : n;
-    double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    FloatSum f[7];
+    double ke = 0.0;
+    std::conditional_t<MIXED, FloatSum, DoubleSum> f[8];  // PE, the six of W, one left empty
     for (int64_t i = lo + threadIdx.x; i < hi; i += RED_THREADS) {
         const double vx = s.vx[i], vy = s.vy[i], vz = s.vz[i];
-        if (pt.nsp == 1) acc[1] = fma(vx, vx, fma(vy, vy, fma(vz, vz, acc[1])));
-        else acc[1] += 0.5 * pt.mass[s.species[i]] * (vx * vx + vy * vy + vz * vz);
-        if (mixed) {
+        if (pt.nsp == 1) ke = fma(vx, vx, fma(vy, vy, fma(vz, vz, ke)));
+        else ke += 0.5 * pt.mass[s.species[i]] * (vx * vx + vy * vy + vz * vz);
+        if constexpr (MIXED) {
             f[0].add(s.pe_atom_f[i]);
 #pragma unroll
             for (int c = 0; c < 6; ++c) f[1 + c].add(s.vir_atom_f[c * n + i]);
         } else {
-            acc[0] += s.pe_atom_d[i];
+            f[0].add(s.pe_atom_d[i]);
 #pragma unroll
-            for (int c = 0; c < 6; ++c) acc[2 + c] += s.vir_atom_d[c * n + i];
+            for (int c = 0; c < 6; ++c) f[1 + c].add(s.vir_atom_d[c * n + i]);
         }
     }
-    if (pt.nsp == 1) acc[1] *= 0.5 * pt.mass[0];
-    if (mixed) {
-        acc[0] = f[0].get();
+    if (pt.nsp == 1) ke *= 0.5 * pt.mass[0];
+    // half of the columns to each half of the lanes, three times, then the four lanes of a column
 #pragma unroll
-        for (int c = 0; c < 6; ++c) acc[2 + c] = f[1 + c].get();
+    for (int o = 16, m = 4; m > 0; o >>= 1, m >>= 1) {
+        const bool up = (lane & o) != 0;
+#pragma unroll
+        for (int k = 0; k < m; ++k) {
+            const auto give = up ? f[k] : f[k + m];
+            if (up) f[k] = f[k + m];
+            f[k].add(lane_xor(give, o));
+        }
     }
-    reduce_tree(sh, acc);
+    f[0].add(lane_xor(f[0], 2));
+    f[0].add(lane_xor(f[0], 1));
+    const int c = lane >> 2;  // this lane's column
+    const double t = f[0].get();  // (shares beyond FP32's range come with a force error, so FloatSum suffices)
+    ke = warp_sum(ke);
+    if ((lane & 3) == 0 && c < 7) sh[warp][c == 0 ? 0 : 1 + c] = t;
+    if (lane == 0) sh[warp][1] = ke;
+    __syncthreads();
     if (threadIdx.x < 8) {
-        __stcg(partials + blockIdx.x * 8 + threadIdx.x, sh[threadIdx.x][0]);
+        double v = 0.0;
+#pragma unroll
+        for (int w = 0; w < RED_WARPS; ++w) v += sh[w][threadIdx.x];
+        __stcg(partials + blockIdx.x * 8 + threadIdx.x, v);
         __threadfence();
     }
     __syncthreads();
@@ -229,13 +244,19 @@ __global__ void __launch_bounds__(RED_THREADS) k_reduce_energy(DevState s, PairT
     __syncthreads();
     if (!last) return;
     __threadfence();
+    double v = 0.0;
+    for (int b = threadIdx.x >> 3; b < (int)gridDim.x; b += RED_THREADS / 8)
+        v += __ldcg(partials + b * 8 + (threadIdx.x & 7));
+    v += __shfl_xor_sync(0xffffffffu, v, 8);
+    v += __shfl_xor_sync(0xffffffffu, v, 16);
+    if (lane < 8) sh[warp][lane] = v;
+    __syncthreads();
+    if (threadIdx.x < 8) {
+        double u = 0.0;
 #pragma unroll
-    for (int c = 0; c < 8; ++c) acc[c] = 0.0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += RED_THREADS)
-#pragma unroll
-        for (int c = 0; c < 8; ++c) acc[c] += __ldcg(partials + b * 8 + c);
-    reduce_tree(sh, acc);
-    if (threadIdx.x < 8) out8[threadIdx.x] = sh[threadIdx.x][0];
+        for (int w = 0; w < RED_WARPS; ++w) u += sh[w][threadIdx.x];
+        out8[threadIdx.x] = u;
+    }
 }
 
 void launch_reduce_energy(const DevState& s, const PairTable& pt, int mixed, double* partials, unsigned* finished,
@@ -243,7 +264,8 @@ void launch_reduce_energy(const DevState& s, const PairTable& pt, int mixed, dou
     const int64_t want = (s.n + RED_THREADS - 1) / RED_THREADS;  // small systems: an atom per thread
     const int parts = (int)std::max<int64_t>(1, std::min<int64_t>(nparts, want));
     const int64_t chunk = std::max<int64_t>(1, (s.n + parts - 1) / parts);
-    k_reduce_energy<<<parts, RED_THREADS, 0, st>>>(s, pt, mixed, chunk, partials, finished, out8);
+    (mixed ? k_reduce_energy<true> : k_reduce_energy<false>)<<<parts, RED_THREADS, 0, st>>>(s, pt, chunk, partials,
+                                                                                       finished, out8);
 }
 
 // ---------------------------------------------------------------- state I/O
