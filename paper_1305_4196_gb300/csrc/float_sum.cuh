@@ -9,11 +9,22 @@
 
 namespace mdgb {
 
+// Additions that are never fused with a product before them (a term may be one: with its product unrounded
+// in the sum and rounded in the error, the error is wrong).
+__host__ __device__ __forceinline__ float add_rn(float a, float b) {
+#ifdef __CUDA_ARCH__
+    return __fadd_rn(a, b);
+#else
+    return a + b;
+#endif
+}
+__host__ __device__ __forceinline__ float sub_rn(float a, float b) { return add_rn(a, -b); }
+
 // s + e = a + b exactly, s = a + b rounded (Knuth's two-sum); e does not depend on the order of a and b.
 __host__ __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-    s = a + b;
-    const float t = s - a;
-    e = (a - (s - t)) + (b - t);
+    s = add_rn(a, b);
+    const float t = sub_rn(s, a);
+    e = add_rn(sub_rn(a, sub_rn(s, t)), sub_rn(b, t));
 }
 
 // The sum of FP32 numbers in three floats: the rounding error of every addition to hi goes to mid, that
@@ -28,7 +39,7 @@ struct FloatSum {
         float e1, e2;
         two_sum(hi, x, hi, e1);
         two_sum(mid, e1, mid, e2);
-        lo += e2;
+        lo = add_rn(lo, e2);
     }
 
     // The other of two sums; the same bits whichever of the two takes it.
@@ -37,7 +48,7 @@ struct FloatSum {
         two_sum(hi, o.hi, hi, e1);
         two_sum(mid, o.mid, m, e2);
         two_sum(m, e1, mid, e3);
-        lo = (lo + o.lo) + (e2 + e3);
+        lo = add_rn(add_rn(lo, o.lo), add_rn(e2, e3));
     }
 
     __host__ __device__ __forceinline__ double get() const { return (double)hi + ((double)mid + (double)lo); }

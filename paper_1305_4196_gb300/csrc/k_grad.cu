@@ -30,6 +30,7 @@
 #include <algorithm>
 
 #include "fixpt.cuh"
+#include "float_sum.cuh"
 #include "fp64_math.cuh"
 
 namespace mdgb {
@@ -45,41 +46,69 @@ struct alignas(4 * sizeof(T)) Grad4 {
     T x, y, z, w;
 };
 
-// A lane's sum of parameter terms.  FP64 terms are summed in FP64; FP32 terms in two floats, hi
-// and lo, with the rounding error of every addition to hi kept in lo (to about 2^-45 of the largest
-// partial sum; the terms themselves are rounded at 2^-24): an FP64 addition and the conversion
-// before it would hold a warp as long as some 100 FP32 operations.
+// A lane's sum of parameter terms: FP64 terms in FP64, FP32 terms in three floats (FloatSum: no less
+// exact than FP64 sums; an FP64 addition and the conversion before it would hold a warp as long as
+// some 100 FP32 operations).
 template <typename T>
 struct ParamSum;
 
 template <>
 struct ParamSum<double> {
     double v = 0.0;
-    __device__ __forceinline__ void add(double x, bool take) {
-        if (take) v += x;
-    }
-    __device__ __forceinline__ void merge(int o, bool) { v += __shfl_xor_sync(0xffffffffu, v, o); }
+    __device__ __forceinline__ void add(double x) { v += x; }
+    __device__ __forceinline__ void add(const ParamSum& o) { v += o.v; }
     __device__ __forceinline__ double get() const { return v; }
 };
 
+__device__ __forceinline__ ParamSum<double> lane_xor(const ParamSum<double>& s, int o) {
+    return ParamSum<double>{__shfl_xor_sync(0xffffffffu, s.v, o)};
+}
+
 template <>
-struct ParamSum<float> {
-    float hi = 0.f, lo = 0.f;
-    __device__ __forceinline__ void add(float x, bool take) {
-        x = take ? x : 0.f;
-        const float s = __fadd_rn(hi, x), b = __fsub_rn(s, hi);
-        lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(x, b)));
-        hi = s;
+struct ParamSum<float> : FloatSum {};
+
+__device__ __forceinline__ ParamSum<float> lane_xor(const ParamSum<float>& s, int o) {
+    return ParamSum<float>{lane_xor(static_cast<const FloatSum&>(s), o)};
+}
+
+// The sums of a warp by species pair and quantity, of lanes that hold NV sums each for an atom of species
+// si.  Half of them to each half of an atom's lanes, twice: a lane keeps VPL; then the warp's atoms
+// of one species after the other, whose sums stay with the lanes 4 c .. 4 c + 3 of species c.
+template <int NSP>
+struct WarpColumns {
+    static constexpr int NV = NSP * G_QUANT, VPL = (NV + 3) / 4;
+
+    template <typename S>
+    static __device__ __forceinline__ void get(S (&val)[4 * VPL], int si, double (&out)[VPL]) {
+        const int lane = threadIdx.x & 31;
+        S mine[VPL];
+#pragma unroll
+        for (int o = 2, m = 2 * VPL; o > 0; o >>= 1, m >>= 1) {
+            const bool up = (lane & o) != 0;
+#pragma unroll
+            for (int k = 0; k < m; ++k) {
+                const S give = up ? val[k] : val[k + m];
+                if (up) val[k] = val[k + m];
+                val[k].add(lane_xor(give, o));
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < VPL; ++j) {
+#pragma unroll
+            for (int c = 0; c < NSP; ++c) {
+                S v = NSP == 1 || si == c ? val[j] : S();
+#pragma unroll
+                for (int o = G_LPA; o < 32; o <<= 1) v.add(lane_xor(v, o));
+                if (lane >> 2 == c) mine[j] = v;
+            }
+            out[j] = mine[j].get();
+        }
     }
-    __device__ __forceinline__ void merge(int o, bool upper) {
-        // both lanes add the upper lane's sum to the lower lane's, so that they stay equal
-        const float oh = __shfl_xor_sync(0xffffffffu, hi, o), ol = __shfl_xor_sync(0xffffffffu, lo, o);
-        const float x = upper ? hi : oh;
-        hi = upper ? oh : hi;
-        lo = __fadd_rn(lo, ol);
-        add(x, true);
+    // the column (species pair t, quantity q: 2 t + q) of this lane's j-th sum; negative: none
+    static __device__ __forceinline__ int column(int j) {
+        const int lane = threadIdx.x & 31, c = lane >> 2, v = (lane & 3) * VPL + j;
+        return c < NSP && v < NV ? c * NV + v : -1;
     }
-    __device__ __forceinline__ double get() const { return (double)hi + (double)lo; }
 };
 
 __device__ __forceinline__ float grad_rcp(float x) {
@@ -112,7 +141,7 @@ __global__ void __launch_bounds__(G_THREADS, 2) k_force_backward(DevState s, Geo
                                                                  double* __restrict__ gx_out,
                                                                  double* __restrict__ part_out, int split) {
     constexpr bool FP64 = sizeof(T) == 8;
-    constexpr int NV = NSP * G_QUANT, NC = NSP * NV;  // sums per atom, per CTA
+    constexpr int NC = NSP * NSP * G_QUANT;  // sums per CTA
     static_assert(NC <= 32, "one lane per sum");
     const Grad4<T>* __restrict__ G = reinterpret_cast<const Grad4<T>*>(G_);
     extern __shared__ __align__(16) unsigned char smem[];
@@ -162,7 +191,9 @@ __global__ void __launch_bounds__(G_THREADS, 2) k_force_backward(DevState s, Geo
     const int blk0 = m.start[0];
     const size_t np = s.np;
     const int lq = threadIdx.x % G_LPA;
-    double mine = 0.0;  // lane c of a warp: the warp's sum for column c
+    using Columns = WarpColumns<NSP>;
+    constexpr int VPL = Columns::VPL;
+    double mine[VPL] = {};  // the warp's sums, by the lanes that Columns says
     for (int u0 = part * G_ATOMS; u0 < nown; u0 += split * G_ATOMS) {
         const int ui = u0 + (int)threadIdx.x / G_LPA;
         const bool active = ui < nown;
@@ -180,8 +211,9 @@ __global__ void __launch_bounds__(G_THREADS, 2) k_force_backward(DevState s, Geo
         Grad4<T> Gi{};
         if (!EN) Gi = G[gi];
         T a[3] = {T(0), T(0), T(0)};
-        ParamSum<T> sum[NSP][G_QUANT];
-        const auto visit = [&](int u) {
+        ParamSum<T> sum[4 * VPL];  // species of the neighbour, quantity: 2 k + q
+        // neighbour u; take(its species, the pair's two terms, its part of dL/dx) if it is inside the cutoff
+        const auto visit = [&](int u, auto&& take) {
             T dx, dy, dz;
             int sj;
             if (FP64) {
@@ -204,10 +236,8 @@ __global__ void __launch_bounds__(G_THREADS, 2) k_force_backward(DevState s, Geo
             const T sr2 = tab.sig2[t] * inv;
             const T s6 = sr2 * sr2 * sr2;
             const T v = T(2) * s6 * s6 - s6;
-            T q0, q1;
-            if (EN) {
-                q0 = s6 * s6 - s6;  // dE/deps / 4
-                q1 = v;             // dE/dsig sig / (24 eps)
+            if (EN) {  // dE/deps / 4, dE/dsig sig / (24 eps)
+                take(sj, s6 * s6 - s6, v, T(0), T(0), T(0));
             } else {
                 const Grad4<T> Gj = G[gid[u]];
                 const T wx = Gi.x - Gj.x, wy = Gi.y - Gj.y, wz = Gi.z - Gj.z;
@@ -217,28 +247,31 @@ __global__ void __launch_bounds__(G_THREADS, 2) k_force_backward(DevState s, Geo
                 else e24 = tab.e24[t];
                 const T gq = e24 * v * inv;
                 const T h = T(2) * (e24 * (T(4) * s6 - T(14) * s6 * s6) * inv * inv) * wd;
-                a[0] += gq * wx + h * dx;
-                a[1] += gq * wy + h * dy;
-                a[2] += gq * wz + h * dz;
-                const T wi = wd * inv;
-                q0 = wi * v;                              // dL/deps / 24
-                q1 = wi * (T(4) * s6 * s6 - s6);          // dL/dsig sig / (144 eps)
-            }
-#pragma unroll
-            for (int k = 0; k < NSP; ++k) {
-                sum[k][0].add(q0, NSP == 1 || sj == k);
-                sum[k][1].add(q1, NSP == 1 || sj == k);
+                const T wi = wd * inv;  // dL/deps / 24, dL/dsig sig / (144 eps)
+                take(sj, wi * v, wi * (T(4) * s6 * s6 - s6), gq * wx + h * dx, gq * wy + h * dy, gq * wz + h * dz);
             }
         };
         const int nch = active ? (s.nl_cnt[gi] + 7) >> 3 : 0;
         const unsigned* words = reinterpret_cast<const unsigned*>(s.nl) + (size_t)gi * 4 + lq;
-        unsigned nxt = nch > 0 ? __ldcs(words) : 0u;
-        for (int c = 0; c < nch; ++c) {
-            const unsigned w = nxt;
-            if (c + 1 < nch) nxt = __ldcs(words + (size_t)(c + 1) * np * 4);
-            visit((int)(w & 0xffffu));
-            visit((int)(w >> 16));
-        }
+        const auto walk = [&](auto&& take) {
+            unsigned nxt = nch > 0 ? __ldcs(words) : 0u;
+            for (int c = 0; c < nch; ++c) {
+                const unsigned w = nxt;
+                if (c + 1 < nch) nxt = __ldcs(words + (size_t)(c + 1) * np * 4);
+                visit((int)(w & 0xffffu), take);
+                visit((int)(w >> 16), take);
+            }
+        };
+        walk([&](int sj, T q0, T q1, T ax, T ay, T az) {
+            a[0] += ax;
+            a[1] += ay;
+            a[2] += az;
+#pragma unroll
+            for (int k = 0; k < NSP; ++k) {
+                sum[2 * k].add(NSP == 1 || sj == k ? q0 : T(0));
+                sum[2 * k + 1].add(NSP == 1 || sj == k ? q1 : T(0));
+            }
+        });
         __syncwarp();
         if (!EN) {
 #pragma unroll
@@ -251,30 +284,40 @@ __global__ void __launch_bounds__(G_THREADS, 2) k_force_backward(DevState s, Geo
                 gx_out[3 * (size_t)s.orig[gi] + lq] = (double)v;
             }
         }
-        // the sums of an atom's lanes, then of the warp's atoms by their species
+        double columns[VPL];
+        Columns::get(sum, si, columns);
+        if constexpr (!FP64) {
+            bool bad = false;
 #pragma unroll
-        for (int k = 0; k < NSP; ++k) {
+            for (int j = 0; j < VPL; ++j) bad |= !isfinite(columns[j]);
+            if (__any_sync(0xffffffffu, bad)) {  // (FloatSum) the warp's atoms again, in FP64
+                ParamSum<double> wide[4 * VPL];
+                walk([&](int sj, T q0, T q1, T, T, T) {
 #pragma unroll
-            for (int q = 0; q < G_QUANT; ++q) {
-#pragma unroll
-                for (int o = 1; o < G_LPA; o <<= 1) sum[k][q].merge(o, lane & o);
-#pragma unroll
-                for (int c = 0; c < NSP; ++c) {
-                    ParamSum<T> v = NSP == 1 || si == c ? sum[k][q] : ParamSum<T>();
-#pragma unroll
-                    for (int o = G_LPA; o < 32; o <<= 1) v.merge(o, lane & o);
-                    if (lane == c * NV + k * G_QUANT + q) mine += v.get();
-                }
+                    for (int k = 0; k < NSP; ++k)
+                        if (NSP == 1 || sj == k) {
+                            wide[2 * k].add((double)q0);
+                            wide[2 * k + 1].add((double)q1);
+                        }
+                });
+                __syncwarp();
+                Columns::get(wide, si, columns);
             }
         }
+#pragma unroll
+        for (int j = 0; j < VPL; ++j) mine[j] += columns[j];
     }
     __syncthreads();
-    double* red = reinterpret_cast<double*>(smem);  // the tile is done with
-    red[threadIdx.x] = mine;
+    double* red = reinterpret_cast<double*>(smem);  // the tile is done with: NC sums of each warp
+#pragma unroll
+    for (int j = 0; j < VPL; ++j) {
+        const int c = Columns::column(j);
+        if (c >= 0) red[warp * NC + c] = mine[j];
+    }
     __syncthreads();
     if (threadIdx.x < NC) {
         double v = 0.0;
-        for (int k = 0; k < nw; ++k) v += red[32 * k + threadIdx.x];
+        for (int k = 0; k < nw; ++k) v += red[k * NC + threadIdx.x];
         // the factors left out above, halved
         const int t = threadIdx.x / G_QUANT, q = threadIdx.x % G_QUANT;
         const double f = EN ? (q ? 12.0 * pt.eps_d[t] / pt.sig_d[t] : 2.0)
