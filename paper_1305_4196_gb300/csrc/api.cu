@@ -72,8 +72,8 @@ struct md_system {
     // MULTI_STEPS kick-kick-drift steps from buffer 0 in one graph (even: back in buffer 0),
     // for md_step calls without timing events: fewer graph launches per step
     StepGraph g_multi;
-    // the steps of a chunk in one graph, by what its loop of LOOP_STEPS steps leaves over
-    // (2 * steps + 1 if the closing step of a call follows); see capture_loop
+    // the steps of a chunk in one graph, by whether its loop of LOOP_STEPS steps runs and what it leaves
+    // over (2 * steps + 1 if the closing step of a call follows); see capture_loop
     std::map<int, StepGraph> g_loop;
     float4* xr_alt = nullptr;
     int potential = 0;       // 0: Lennard-Jones pair table; 1: TB-SMA many-body (md_set_tbsma)
@@ -827,7 +827,9 @@ int capture_fused_multi(md_system* s, md_system::StepGraph& out) {
 // while node 5.7 us.  So a chunk of steps is one graph: a while node whose body holds LOOP_STEPS
 // steps, each with its own conditional rebuild, and an if node (always taken) with the steps left
 // over.  Against a graph per step and 8-step graphs of top-level conditions this takes
-// about 7 us off every step.
+// about 7 us off every step.  A chunk without a whole pass has no while node and a single step left
+// over no if node: the call that captures them is the first of its kind, and a node's body costs it
+// some 20 us a step (copper, 16,384 atoms: a first md_step(1) 350 -> 150 us, md_step(4) 500 -> 340).
 constexpr int LOOP_STEPS = 4;  // even: fused steps are back in coordinate buffer 0
 
 // A conditional node behind `tail` (or, while capturing on cs, behind what is captured); its body.
@@ -895,35 +897,38 @@ int append_step(md_system* s, cudaGraph_t g, std::vector<cudaGraphNode_t>& tail,
     });
 }
 
-// The graph of a chunk: d_ctrl[2] passes of LOOP_STEPS mid steps, `left` more of them, and with
-// `closing` a step that is not followed by another.
-int capture_loop(md_system* s, int left, bool closing, md_system::StepGraph& out) {
+// The graph of a chunk: with `loop` d_ctrl[2] passes of LOOP_STEPS mid steps, `left` more of them, and
+// with `closing` a step that is not followed by another.
+int capture_loop(md_system* s, bool loop, int left, bool closing, md_system::StepGraph& out) {
     destroy_graph(out);
     CK(cudaGraphCreate(&out.graph, 0));
     cudaGraph_t g = out.graph;
     // fused steps alternate between the position buffers; the others work in buffer 0
     const auto buffer = [&](int step) { return fused(s) ? step & 1 : 0; };
-    std::vector<cudaGraphNode_t> tail;
-    cudaGraphConditionalHandle hw;
-    CK(cudaGraphConditionalHandleCreate(&hw, g, 0, cudaGraphCondAssignDefault));
-    int rc = append_captured(s, g, tail, [&](cudaStream_t cs) { launch_loop_ctrl(s->d_ctrl + 2, 0, hw, cs); });
-    if (rc) return rc;
+    std::vector<cudaGraphNode_t> tail, btail;
     cudaGraph_t body = nullptr;
-    if ((rc = add_conditional(s, g, tail, hw, cudaGraphCondTypeWhile, &body))) return rc;
-    std::vector<cudaGraphNode_t> btail;
-    for (int j = 0; j < LOOP_STEPS; ++j)
-        if ((rc = append_step(s, body, btail, buffer(j), true))) return rc;
-    if ((rc = append_captured(s, body, btail, [&](cudaStream_t cs) { launch_loop_ctrl(s->d_ctrl + 2, 1, hw, cs); })))
-        return rc;
-    if (left > 0 || closing) {
+    int rc;
+    if (loop) {
+        cudaGraphConditionalHandle hw;
+        CK(cudaGraphConditionalHandleCreate(&hw, g, 0, cudaGraphCondAssignDefault));
+        if ((rc = append_captured(s, g, tail, [&](cudaStream_t cs) { launch_loop_ctrl(s->d_ctrl + 2, 0, hw, cs); })))
+            return rc;
+        if ((rc = add_conditional(s, g, tail, hw, cudaGraphCondTypeWhile, &body))) return rc;
+        for (int j = 0; j < LOOP_STEPS; ++j)
+            if ((rc = append_step(s, body, btail, buffer(j), true))) return rc;
+        if ((rc = append_captured(s, body, btail, [&](cudaStream_t cs) { launch_loop_ctrl(s->d_ctrl + 2, 1, hw, cs); })))
+            return rc;
+    }
+    const int rest = left + (closing ? 1 : 0);
+    body = g;
+    if (rest > 1) {
         cudaGraphConditionalHandle hi;
         CK(cudaGraphConditionalHandleCreate(&hi, g, 1, cudaGraphCondAssignDefault));
         if ((rc = add_conditional(s, g, tail, hi, cudaGraphCondTypeIf, &body))) return rc;
         btail.clear();
-        for (int j = 0; j < left; ++j)
-            if ((rc = append_step(s, body, btail, buffer(j), true))) return rc;
-        if (closing && (rc = append_step(s, body, btail, buffer(left), false))) return rc;
     }
+    for (int j = 0; j < rest; ++j)
+        if ((rc = append_step(s, body, rest > 1 ? btail : tail, buffer(j), j < left))) return rc;
     CKL();
     CK(cudaGraphInstantiate(&out.exec, g, 0));
     return MD_OK;
@@ -944,10 +949,10 @@ int launch_loop(md_system* s, int n_mid, bool closing) {
         s->graph_timing = false;
     }
     const int passes = n_mid / LOOP_STEPS, left = n_mid % LOOP_STEPS;
-    // (a program that varies its step counts meets at most 2 * LOOP_STEPS kinds of rest)
-    md_system::StepGraph& gr = s->g_loop[2 * left + (closing ? 1 : 0)];
+    // (a program that varies its step counts meets at most 4 * LOOP_STEPS kinds)
+    md_system::StepGraph& gr = s->g_loop[(passes > 0 ? 2 * LOOP_STEPS : 0) + 2 * left + (closing ? 1 : 0)];
     if (!gr.exec) {
-        const int rc = capture_loop(s, left, closing, gr);
+        const int rc = capture_loop(s, passes > 0, left, closing, gr);
         if (rc) {
             destroy_loops(s);
             return rc;
@@ -959,7 +964,7 @@ int launch_loop(md_system* s, int n_mid, bool closing) {
     CK(cudaMemcpyAsync(s->d_ctrl, s->h_ctrl, 3 * sizeof(long long), cudaMemcpyHostToDevice, s->stream));
     CK(cudaGraphLaunch(gr.exec, s->stream));
     const int steps = n_mid + (closing ? 1 : 0);
-    s->launches += 1 + passes + (1 + force_kernels(s)) * steps + (fused(s) ? 0 : n_mid);
+    s->launches += (passes > 0 ? 1 + passes : 0) + (1 + force_kernels(s)) * steps + (fused(s) ? 0 : n_mid);
     s->force_evals += steps;
     return MD_OK;
 }
