@@ -213,15 +213,32 @@ def run_reference(args):
     print(json.dumps(line), flush=True)
 
 
+def force_source_sha256(csrc=os.path.join(ROOT, "paper_1305_4196_gb300", "csrc")):
+    """One hash over the sources of the full-list force kernel: k_force.cu and every header
+    of its folder that it includes, directly or through another, in order of their names."""
+    import hashlib
+    import re
+    todo, seen = ["k_force.cu"], set()
+    while todo:
+        name = todo.pop()
+        path = os.path.join(csrc, name)
+        if name in seen or not os.path.exists(path):
+            continue
+        seen.add(name)
+        todo += re.findall(r'^\s*#\s*include\s+"([^"]+)"', open(path).read(), flags=re.M)
+    h = hashlib.sha256()
+    for name in sorted(seen):
+        h.update(name.encode() + b"\0" + open(os.path.join(csrc, name), "rb").read())
+    return h.hexdigest()
+
+
 def measured_force_traffic(n, fused):
     """DRAM bytes per launch of the force kernel (fused: with velocity Verlet) from the
     committed ncu capture (profiles/force_traffic.json), scaled to n atoms; None if the
-    kernel's source changed since the capture."""
-    import hashlib
+    kernel's sources changed since the capture."""
     try:
         rec = json.load(open(os.path.join(ROOT, "profiles", "force_traffic.json")))
-        src = os.path.join(ROOT, "paper_1305_4196_gb300", "csrc", "k_force.cu")
-        if hashlib.sha256(open(src, "rb").read()).hexdigest() != rec["k_force_cu_sha256"]:
+        if force_source_sha256() != rec["sources_sha256"]:
             return None
         r = rec["fused" if fused else "force"]
         return (r["dram_read_bytes"] + r["dram_write_bytes"]) * n / rec["atoms"]
