@@ -1258,6 +1258,7 @@ int md_create(int64_t n, const double box[3], double r_cut, double skin, const m
     if (rc) return bail(rc);
     cudaGetDevice(&s->device);
     cudaDeviceGetAttribute(&s->g.sms, cudaDevAttrMultiProcessorCount, s->device);
+    cudaDeviceGetAttribute(&s->g.sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, s->device);
     s->stream = static_cast<cudaStream_t>(p->stream);
     {
         const char* ng = std::getenv("MDGB_NO_GRAPHS");

@@ -26,6 +26,7 @@
 //
 // A larger system is advanced in phases of tasks that any CTA may take, with Verlet
 // lists (the block systems below).
+#include "launch.cuh"
 #include "mdgb_batch_internal.cuh"
 #include "nl_scan.cuh"
 
@@ -1384,13 +1385,6 @@ int ensemble_ctas_per_sm(int threads, size_t smem) {
     return n;
 }
 
-void init_batch_kernels() {
-    cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, k_ensemble_run) != cudaSuccess) return;
-    int dev = 0, optin = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    cudaFuncSetAttribute(k_ensemble_run, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
-}
+void init_batch_kernels() { allow_max_smem(k_ensemble_run); }
 
 }  // namespace mdgb

@@ -25,6 +25,7 @@
 //
 // FP64: the same structure with FP64 tile coordinates and FP64 sums (k_force_fp64.cu).
 #include "full_task.cuh"
+#include "launch.cuh"
 
 #include <type_traits>
 
@@ -456,16 +457,6 @@ size_t force_smem_bytes(int mixed, int half, int with_energy, int tile_cap) {
 
 // Raise every force kernel's dynamic shared-memory limit to what the SM allows
 // (once per device, before any launch or stream capture).
-template <typename K>
-static void allow_max_smem(K kernel) {
-    cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return;
-    int dev = 0, optin = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
-}
-
 template <bool SINGLE>
 static void init_force_kernels_of(int half) {
     if (half) {
@@ -537,7 +528,7 @@ void launch_forces_mixed(const DevState& s, const Geometry& g, const PairTable& 
     const int per = g.nblock / 8;
     // Four lanes per atom while a colour has fewer than two blocks per SM (296,352 atoms, 216 blocks:
     // 27.7 against 29.8 us a launch; 500,000, 343 blocks: 39.3 against 34.8)
-    const int lpa = with_energy || per >= 2 * 152 ? 1 : 4;
+    const int lpa = with_energy || per >= 2 * g.sms ? 1 : 4;
     using K = void (*)(DevState, Geometry, PairTable, TileOffsets, int, float, int);
     K k;
     if (with_energy) k = single ? (K)k_force_mixed_half<true, true, 1> : (K)k_force_mixed_half<false, true, 1>;

@@ -23,6 +23,7 @@
 // 1.38 ms and one with energy and virial 2.11 ms with 22 operations for each of the 80 padded
 // entries, and takes 0.78 and 1.25 ms; the FP64 pipe is 88 % busy.
 #include "fp64_math.cuh"
+#include "launch.cuh"
 #include "tile.cuh"
 
 #include <algorithm>
@@ -30,7 +31,6 @@
 namespace mdgb {
 
 constexpr int F_THREADS = 256;
-static int g_sm_count = 0;  // SMs of the device, read at initialisation (never during a stream capture)
 
 // ---------------------------------------------------------------- full list
 constexpr int FQ = 16;  // queue slots per lane; the lanes of an atom share theirs
@@ -326,7 +326,7 @@ void launch_forces_fp64(const DevState& s, const Geometry& g, const PairTable& p
         // them.  Against the same split with an own queue and whole 16-byte chunks per lane: 4,000 atoms
         // (8 blocks) 29 us instead of 46, 10,976 (64) 47 / 75, 32,000 (64) 106 / 171, 55,296 (216)
         // 173 / 212, 360,703 (2,016) 776 / 799.
-        const int sms = g_sm_count > 0 ? g_sm_count : 152;
+        const int sms = g.sms;
         const int64_t per_block = (s.n + g.nblock - 1) / g.nblock;
         int64_t split = 1;
         int lpa = 2;
@@ -360,19 +360,7 @@ void launch_forces_fp64(const DevState& s, const Geometry& g, const PairTable& p
     }
 }
 
-template <typename K>
-static void allow_max_smem(K kernel) {
-    cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return;
-    int dev = 0, optin = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
-}
-
 void init_force_fp64_kernels(int half, int single) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&g_sm_count, cudaDevAttrMultiProcessorCount, dev);
     if (half) {
         allow_max_smem(k_force_fp64_half<false>);
         allow_max_smem(k_force_fp64_half<true>);

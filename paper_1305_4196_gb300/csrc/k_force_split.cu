@@ -14,6 +14,7 @@
 // are issued per warp).  Fused step, one CTA per block against this form: 28.4 -> 19.2 us at
 // 32,000 atoms (64 blocks), 21.5 -> 14.8 us at 16,384; forces alone 15.3 -> 7.0 us at 2,048.
 #include "full_task.cuh"
+#include "launch.cuh"
 
 #include <algorithm>
 
@@ -182,23 +183,9 @@ SplitKernel split_kernel(bool single, bool ev, int mode, int lpa) {
     return mode == FM_KICK ? split_of<false, FM_KICK>(lpa) : split_of<false, FM_KKD>(lpa);
 }
 
-template <typename K>
-void allow_max_smem(K kernel) {
-    cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return;
-    int dev = 0, optin = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
-}
-
-int g_sm_count = 0;  // SMs of the device, read at initialisation (never during a stream capture)
-
 }  // namespace
 
 void init_force_split_kernels(int single) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&g_sm_count, cudaDevAttrMultiProcessorCount, dev);
     allow_max_smem(split_kernel(single, true, FM_FORCE, 1));
     for (int mode = FM_FORCE; mode <= FM_KKD; ++mode)
         for (int lpa = 2; lpa <= 8; lpa *= 2) allow_max_smem(split_kernel(single, false, mode, lpa));
@@ -210,7 +197,7 @@ bool launch_forces_mixed_split(const DevState& s, const Geometry& g, const PairT
     // Below two blocks per SM (70,304 atoms, 216 blocks: 26.8 us here, 28.3 with a CTA per block;
     // 108,000 atoms, 512 blocks: 30.6 against 27.0).  The fewest lanes per atom that give every SM
     // a CTA: at 32,000 atoms two lanes (256 CTAs) take 19.2 us, four (512 CTAs) 22.6.
-    const int sms = g_sm_count > 0 ? g_sm_count : 152;
+    const int sms = g.sms;
     if (s.compact || g.nblock >= 2 * sms) return false;
     const int64_t per_block = (s.n + g.nblock - 1) / g.nblock;
     int lpa = with_energy ? 1 : 2;

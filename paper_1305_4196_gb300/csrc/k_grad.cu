@@ -32,6 +32,7 @@
 #include "fixpt.cuh"
 #include "float_sum.cuh"
 #include "fp64_math.cuh"
+#include "launch.cuh"
 
 namespace mdgb {
 
@@ -406,16 +407,6 @@ void launch_force_backward(const DevState& s, const Geometry& g, const PairTable
     backward_kernel(fp64, G == nullptr, pt.nsp)<<<grid, G_THREADS, backward_smem_bytes(fp64, tile_cap), st>>>(
         s, g, pt, to, tile_cap, Gc, gx, part, plan.split);
     k_colsum<<<ncol, CS_THREADS, 0, st>>>(part, (int)grid, scratch);
-}
-
-template <typename K>
-static void allow_max_smem(K kernel) {
-    cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return;
-    int dev = 0, optin = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
 }
 
 void init_grad_kernels(int fp64, int nsp) {

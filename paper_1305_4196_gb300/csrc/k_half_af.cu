@@ -31,6 +31,7 @@
 // than 32 take a second pass per phase, whose atoms keep their sums in lane-private shared
 // memory.
 #include "fixpt.cuh"
+#include "launch.cuh"
 #include "tile.cuh"
 
 namespace mdgb {
@@ -489,22 +490,12 @@ void launch_forces_half_af(const DevState& s, const Geometry& g, const PairTable
     }
 }
 
-template <typename K>
-static void af_allow_max_smem(K kernel) {
-    cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return;
-    int dev = 0, optin = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
-}
-
 void init_half_af_kernels() {
-    af_allow_max_smem(k_build_sched);
-    af_allow_max_smem(k_force_half_af<true, false>);
-    af_allow_max_smem(k_force_half_af<true, true>);
-    af_allow_max_smem(k_force_half_af<false, false>);
-    af_allow_max_smem(k_force_half_af<false, true>);
+    allow_max_smem(k_build_sched);
+    allow_max_smem(k_force_half_af<true, false>);
+    allow_max_smem(k_force_half_af<true, true>);
+    allow_max_smem(k_force_half_af<false, false>);
+    allow_max_smem(k_force_half_af<false, true>);
 }
 
 }  // namespace mdgb

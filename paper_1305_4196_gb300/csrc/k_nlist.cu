@@ -26,6 +26,7 @@
 // offsets and the copy of the atoms' state (other forms of the scan:
 // 439 us with hit masks turned into entries by a loop over their bits; 551 us with the self
 // pair and the band sieved out of the rows by a lane each).
+#include "launch.cuh"
 #include "nl_scan.cuh"
 
 #include <algorithm>
@@ -135,8 +136,6 @@ __global__ void __launch_bounds__(NL_WARPS * 32, 3) k_build_lists_occ(DevState s
     }
 }
 
-static int g_sm_count = 0, g_sm_smem = 0;  // of the device, read at initialisation (never during a stream capture)
-
 // Shared memory of a CTA of `warps` warps.
 static size_t nl_smem_bytes(int tile_cap, int warps) { return nl_tile_bytes(tile_cap) + warps * sizeof(NlWarp); }
 
@@ -165,31 +164,15 @@ void launch_build_lists(const DevState& s, const DevState& d, const Geometry& g,
     // atoms (32,000 atoms, 64 blocks, two CTAs per SM: 95 us with one CTA per block, 39 with four, 55
     // with five, whose last 16 start when the others end; 2,048 atoms, 8 blocks: 43 with one, 16 with
     // sixteen).
-    const int sms = g_sm_count > 0 ? g_sm_count : 152;
-    const int64_t per_sm = std::min<int64_t>(3, (int64_t)(g_sm_smem > 0 ? g_sm_smem : 233472) / (int64_t)(smem + 1024));
+    const int64_t per_sm = std::min<int64_t>(3, (int64_t)g.sm_smem / (int64_t)(smem + 1024));
     const int64_t per_cell = (s.n + g.ncell - 1) / g.ncell;
-    const int split = (int)std::max<int64_t>(1, std::min<int64_t>({per_cell / 2, per_sm * sms / g.nblock, 16}));
+    const int split = (int)std::max<int64_t>(1, std::min<int64_t>({per_cell / 2, per_sm * g.sms / g.nblock, 16}));
     const unsigned grid = (unsigned)g.nblock * (unsigned)split;
     if (half) k_build_lists<1><<<grid, threads, smem, st>>>(s, d, g, to, rl2, lo, hi, list_cap, tile_cap, split);
     else k_build_lists<0><<<grid, threads, smem, st>>>(s, d, g, to, rl2, lo, hi, list_cap, tile_cap, split);
 }
 
-template <typename K>
-static void allow_max_smem(K kernel) {
-    cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return;
-    int dev = 0, optin = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
-}
-
 void init_list_kernels(int half) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess) {
-        cudaDeviceGetAttribute(&g_sm_count, cudaDevAttrMultiProcessorCount, dev);
-        cudaDeviceGetAttribute(&g_sm_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-    }
     if (half) {
         allow_max_smem(k_build_lists<1>);
         allow_max_smem(k_build_lists_occ<1>);

@@ -26,6 +26,7 @@
 // lies in the band around r_cut^2 is decided by the FP64 definition: its atom is
 // finished after the loop by the whole warp, against the tile still in shared memory.
 #include "full_task.cuh"
+#include "launch.cuh"
 
 #include <algorithm>
 
@@ -519,28 +520,14 @@ TbForce tb_force(bool ev, int mode, int lpa) {
                             : (mode == FM_KICK ? tb_force_of<FM_KICK>(lpa) : tb_force_of<FM_KKD>(lpa));
 }
 
-int g_sm_count = 0;  // SMs of the device, read at initialisation (never during a stream capture)
-
 }  // namespace
 
-template <typename K>
-static void tb_allow_max_smem(K kernel) {
-    cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return;
-    int dev = 0, optin = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
-}
-
 void init_tbsma_kernels() {
-    int dev = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&g_sm_count, cudaDevAttrMultiProcessorCount, dev);
-    tb_allow_max_smem(tb_density(true, 1));
-    tb_allow_max_smem(tb_force(true, FM_FORCE, 1));
+    allow_max_smem(tb_density(true, 1));
+    allow_max_smem(tb_force(true, FM_FORCE, 1));
     for (int lpa = 1; lpa <= 8; lpa *= 2) {
-        tb_allow_max_smem(tb_density(false, lpa));
-        for (int mode = FM_FORCE; mode <= FM_KKD; ++mode) tb_allow_max_smem(tb_force(false, mode, lpa));
+        allow_max_smem(tb_density(false, lpa));
+        for (int mode = FM_FORCE; mode <= FM_KKD; ++mode) allow_max_smem(tb_force(false, mode, lpa));
     }
 }
 
@@ -557,7 +544,7 @@ void launch_tbsma(const DevState& s, const Geometry& g, const PairTable& pt, con
     // at least) that give every SM a CTA.  Both passes: 6,912 atoms (27 blocks) 31.9 us with one
     // lane and a CTA per block, 21.4 with eight lanes; 55,296 atoms (216 blocks) 41.2 and 38.0 (two
     // lanes); at 500,000 atoms (2,744 blocks) two lanes take 172, one lane 163.
-    const int sms = g_sm_count > 0 ? g_sm_count : 152;
+    const int sms = g.sms;
     const int64_t per_block = (s.n + g.nblock - 1) / g.nblock;
     int lpa = 1;
     int64_t split = 1;

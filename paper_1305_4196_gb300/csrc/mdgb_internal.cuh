@@ -50,7 +50,7 @@ struct Geometry {
     int linear;        // 1: linear block numbering (no colour classes)
     int nblock;        // number of 2x2x2 blocks
     int ncell;         // number of cells
-    int sms;           // SMs of the system's device (launch shapes)
+    int sms, sm_smem;  // SMs of the system's device, shared memory of one (launch shapes)
 };
 
 // LJ pair constants per species pair (FP32 copies for the mixed path, FP64 for the FP64 path)
