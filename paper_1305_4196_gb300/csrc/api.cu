@@ -25,7 +25,7 @@ struct md_system {
     cudaStream_t stream = nullptr;
     int64_t n = 0;
     int np = 64;
-    Geometry g{};
+    LaunchGeometry g{};
     PairTable pt{};
     TileOffsets to{};
     double box[3] = {0, 0, 0};

@@ -53,7 +53,7 @@ int mdgb_cut_band(int32_t frame, double w_max, double half_skin, int32_t R, doub
 
 int mdgb_backward_shape(const int32_t nc[3], int64_t n, int32_t n_species, int32_t precision, int32_t n_sms,
                         int32_t* split_out, int64_t* grad_at_out, int64_t* doubles_out) {
-    Geometry g{};
+    LaunchGeometry g{};
     if (!split_out || !grad_at_out || !doubles_out || n < 1 || n_species < 1 || n_species > MAX_SPECIES ||
         (precision != MD_FP64 && precision != MD_MIXED) || n_sms < 1 || !make_geometry(nc, g))
         return MD_ERR_ARG;

@@ -504,7 +504,7 @@ static void launch_full(const DevState& s, const Geometry& g, const PairTable& p
                                                                                  out, dt, lim2_f);
 }
 
-void launch_forces_mixed(const DevState& s, const Geometry& g, const PairTable& pt, const TileOffsets& to,
+void launch_forces_mixed(const DevState& s, const LaunchGeometry& g, const PairTable& pt, const TileOffsets& to,
                          int tile_cap, int half, int with_energy, cudaStream_t st) {
     if (s.n == 0) return;
     const size_t smem = force_smem_bytes(1, half, with_energy, tile_cap);
@@ -558,7 +558,7 @@ static void launch_full_mode(const DevState& s, const Geometry& g, const PairTab
     launch_full<SINGLE, false, MODE>(s, g, pt, to, tile_cap, fs2_max, out, dt, lim2_f, smem, st);
 }
 
-void launch_forces_mixed_fused(const DevState& s, const Geometry& g, const PairTable& pt, const TileOffsets& to,
+void launch_forces_mixed_fused(const DevState& s, const LaunchGeometry& g, const PairTable& pt, const TileOffsets& to,
                                int tile_cap, int mode, StepOut out, double dt, double lim2, cudaStream_t st) {
     if (s.n == 0) return;
     const size_t smem = force_smem_bytes(1, 0, 0, tile_cap);

@@ -314,7 +314,7 @@ static void launch_full(const DevState& s, const Geometry& g, const PairTable& p
                                                                                         rc2_test);
 }
 
-void launch_forces_fp64(const DevState& s, const Geometry& g, const PairTable& pt, int tile_cap, int half,
+void launch_forces_fp64(const DevState& s, const LaunchGeometry& g, const PairTable& pt, int tile_cap, int half,
                         int with_energy, cudaStream_t st) {
     if (s.n == 0) return;
     const size_t smem = force_smem_bytes(0, half, with_energy, tile_cap);

@@ -191,7 +191,7 @@ void init_force_split_kernels(int single) {
         for (int lpa = 2; lpa <= 8; lpa *= 2) allow_max_smem(split_kernel(single, false, mode, lpa));
 }
 
-bool launch_forces_mixed_split(const DevState& s, const Geometry& g, const PairTable& pt, const TileOffsets& to,
+bool launch_forces_mixed_split(const DevState& s, const LaunchGeometry& g, const PairTable& pt, const TileOffsets& to,
                                int tile_cap, float fs2_max, bool with_energy, int mode, StepOut out, double dt,
                                float lim2_f, size_t smem, cudaStream_t st) {
     // Below two blocks per SM (70,304 atoms, 216 blocks: 26.8 us here, 28.3 with a CTA per block;

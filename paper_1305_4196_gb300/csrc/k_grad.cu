@@ -359,7 +359,7 @@ size_t backward_smem_bytes(int fp64, int tile_cap) {
                     sizeof(double) * G_THREADS);
 }
 
-BackwardPlan backward_plan(const Geometry& g, int nsp, int fp64, int64_t n) {
+BackwardPlan backward_plan(const LaunchGeometry& g, int nsp, int fp64, int64_t n) {
     BackwardPlan p;
     const int64_t per_block = (n + g.nblock - 1) / g.nblock;
     const int64_t split =

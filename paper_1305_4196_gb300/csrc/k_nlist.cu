@@ -146,7 +146,7 @@ size_t build_lists_smem(int list_cap, int tile_cap) {
     return (size_t)((tile_cap + 227) & ~3) * 3 * sizeof(float) + 32768;
 }
 
-void launch_build_lists(const DevState& s, const DevState& d, const Geometry& g, const TileOffsets& to, double rl2, int list_cap,
+void launch_build_lists(const DevState& s, const DevState& d, const LaunchGeometry& g, const TileOffsets& to, double rl2, int list_cap,
                         int tile_cap, int half, cudaStream_t st) {
     if (s.n == 0) return;
     const int warps = nl_smem_bytes(tile_cap, NL_WARPS) <= 226 * 1024 ? NL_WARPS : NL_WARPS / 2;

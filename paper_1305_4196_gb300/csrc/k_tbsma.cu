@@ -531,7 +531,7 @@ void init_tbsma_kernels() {
     }
 }
 
-void launch_tbsma(const DevState& s, const Geometry& g, const PairTable& pt, const TBTable& tb, const TileOffsets& to,
+void launch_tbsma(const DevState& s, const LaunchGeometry& g, const PairTable& pt, const TBTable& tb, const TileOffsets& to,
                   int tile_cap, float* emb, int with_energy, int mode, StepOut out, double dt, double lim2,
                   cudaStream_t st) {
     if (s.n == 0) return;

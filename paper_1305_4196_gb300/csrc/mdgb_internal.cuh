@@ -50,7 +50,13 @@ struct Geometry {
     int linear;        // 1: linear block numbering (no colour classes)
     int nblock;        // number of 2x2x2 blocks
     int ncell;         // number of cells
-    int sms, sm_smem;  // SMs of the system's device, shared memory of one (launch shapes)
+};
+
+// With what only the rules of launches need, of the system's device.  (Not a part of the kernels' parameter:
+// eight more bytes there took the many-body force kernel from 64 to 70 registers: 7 of 196 us a step at 500,000 atoms.)
+struct LaunchGeometry : Geometry {
+    int sms;      // SMs
+    int sm_smem;  // shared memory of one
 };
 
 // LJ pair constants per species pair (FP32 copies for the mixed path, FP64 for the FP64 path)
@@ -312,10 +318,10 @@ void launch_step_ctrl(int policy, int every_k, int32_t* rebuild_flag, long long*
                       long long* n_builds, uint32_t* err, cudaGraphConditionalHandle handle, cudaStream_t st);
 void launch_loop_ctrl(long long* passes_left, int done, cudaGraphConditionalHandle handle, cudaStream_t st);
 void launch_copy_state(const DevState& dst, const DevState& src, cudaStream_t st);
-void launch_build_lists(const DevState& s, const DevState& d, const Geometry& g, const TileOffsets& to, double rl2, int list_cap,
+void launch_build_lists(const DevState& s, const DevState& d, const LaunchGeometry& g, const TileOffsets& to, double rl2, int list_cap,
                         int tile_cap, int half, cudaStream_t st);
 size_t build_lists_smem(int list_cap, int tile_cap);
-void launch_forces_mixed(const DevState& s, const Geometry& g, const PairTable& pt, const TileOffsets& to,
+void launch_forces_mixed(const DevState& s, const LaunchGeometry& g, const PairTable& pt, const TileOffsets& to,
                          int tile_cap, int half, int with_energy, cudaStream_t st);
 size_t force_smem_bytes(int mixed, int half, int with_energy, int tile_cap);
 // Where a kick-kick-drift step writes the new positions: the other pair of position
@@ -325,19 +331,19 @@ struct StepOut {
     float4* xr;
     double *x, *y, *z;
 };
-void launch_forces_mixed_fused(const DevState& s, const Geometry& g, const PairTable& pt, const TileOffsets& to,
+void launch_forces_mixed_fused(const DevState& s, const LaunchGeometry& g, const PairTable& pt, const TileOffsets& to,
                                int tile_cap, int mode, StepOut out, double dt, double lim2, cudaStream_t st);
 enum { FUSE_FORCE_ONLY = 0, FUSE_KICK = 1, FUSE_KICK_KICK_DRIFT = 2 };  // modes of the fused force launches
 // The same tasks with several CTAs per block and lanes per atom (k_force_split.cu), for systems
 // of few blocks; false where one CTA per block is the better form (nothing is launched).
-bool launch_forces_mixed_split(const DevState& s, const Geometry& g, const PairTable& pt, const TileOffsets& to,
+bool launch_forces_mixed_split(const DevState& s, const LaunchGeometry& g, const PairTable& pt, const TileOffsets& to,
                                int tile_cap, float fs2_max, bool with_energy, int mode, StepOut out, double dt,
                                float lim2_f, size_t smem, cudaStream_t st);
 void init_force_split_kernels(int single);
 // TB-SMA forces (full lists, mixed): the density pass writes emb[i] = 1/sqrt(rho_i) (0 for an
 // atom without neighbours), the force pass the Q31.32 forces; with_energy also writes the
 // per-atom energies and virial shares.  Two launches.
-void launch_tbsma(const DevState& s, const Geometry& g, const PairTable& pt, const TBTable& tb, const TileOffsets& to,
+void launch_tbsma(const DevState& s, const LaunchGeometry& g, const PairTable& pt, const TBTable& tb, const TileOffsets& to,
                   int tile_cap, float* emb, int with_energy, int mode, StepOut out, double dt, double lim2,
                   cudaStream_t st);
 size_t tbsma_smem_bytes(int tile_cap);
@@ -345,7 +351,7 @@ size_t tbsma_smem_bytes(int tile_cap);
 void launch_colour_tags(const DevState& s, const Geometry& g, int block0, int nblocks, int32_t* tags,
                         unsigned long long* conflicts, cudaStream_t st);
 void init_tbsma_kernels();
-void launch_forces_fp64(const DevState& s, const Geometry& g, const PairTable& pt, int tile_cap, int half,
+void launch_forces_fp64(const DevState& s, const LaunchGeometry& g, const PairTable& pt, int tile_cap, int half,
                         int with_energy, cudaStream_t st);
 void launch_integrate(const DevState& s, const Geometry& g, const PairTable& pt, int mode, int mixed,
                       double dt, double lim2, cudaStream_t st);
@@ -380,7 +386,7 @@ struct BackwardPlan {
     int split;
     size_t sums, doubles;
 };
-BackwardPlan backward_plan(const Geometry& g, int nsp, int fp64, int64_t n);
+BackwardPlan backward_plan(const LaunchGeometry& g, int nsp, int fp64, int64_t n);
 void launch_force_backward(const DevState& s, const Geometry& g, const PairTable& pt, const TileOffsets& to,
                            int tile_cap, int fp64, const BackwardPlan& plan, const double* G, double* gx,
                            double* scratch, cudaStream_t st);
