@@ -165,8 +165,8 @@ bool half(const md_system* s) { return s->list_kind != MD_LIST_FULL; }
 // the half list evaluated with no atomic operation (k_half_af.cu)
 bool af(const md_system* s) { return s->list_kind == MD_LIST_HALF_ATOMIC_FREE; }
 // shared memory of the list build / of a force launch for this system's kernels
-size_t list_smem(const md_system* s, int list_cap, int tile_cap) {
-    return af(s) ? af_sched_smem_bytes(tile_cap) : build_lists_smem(list_cap, tile_cap);
+size_t list_smem(const md_system* s, int tile_cap) {
+    return af(s) ? af_sched_smem_bytes(tile_cap) : build_lists_smem(tile_cap);
 }
 size_t fsmem(const md_system* s, int with_energy, int tile_cap) {
     return af(s) ? af_force_smem_bytes(tile_cap) : force_smem_bytes(mixed(s), half(s), with_energy, tile_cap);
@@ -433,7 +433,7 @@ int do_build(md_system* s, int p = 0) {
             CK(cudaMemsetAsync(a.stats, 0, 4 * sizeof(int32_t), s->stream));
             CK(cudaMemsetAsync(a.err, 0, sizeof(uint32_t), s->stream));
         }
-        if (list_smem(s, s->list_cap, s->tile_cap) > 226 * 1024) {
+        if (list_smem(s, s->tile_cap) > 226 * 1024) {
             if (attempt == 0 && !af(s)) {  // no list builder takes the state to its new order
                 launch_copy_back(a, s->st[1], s->stream);
                 CKL();
@@ -632,7 +632,8 @@ int validate_params(md_system* s, const md_params* p, double r_cut) {
     return MD_OK;
 }
 
-// ---- graph-captured time steps
+// ---- graph-captured time steps with event nodes around the forces (md_set_timing; without
+// timing whole chunks are one graph, below)
 //
 // One step = integrate -> step control (sets the IF condition) -> IF(rebuild){binning,
 // gather, copy back, list build} -> forces.  Kernel arguments are fixed at capture,
@@ -656,7 +657,7 @@ int capture_step(md_system* s, int mode, md_system::StepGraph& out) {
     const DevState& a = s->st[0];
     launch_integrate(a, s->g, s->pt, mode, mixed(s), s->dt, s->lim2, cs);
     launch_step_ctrl(s->rebuild == MD_REBUILD_EVERY_K ? 1 : 0, s->rebuild_k, a.rebuild_flag, s->d_ctrl,
-                     s->d_ctrl + 1, a.err, h, cs);
+                     a.err, h, cs);
     cudaStreamCaptureStatus status;
     const cudaGraphNode_t* deps = nullptr;
     size_t ndeps = 0;
@@ -673,19 +674,15 @@ int capture_step(md_system* s, int mode, md_system::StepGraph& out) {
     CK(cudaGraphAddNode(&cnode, cg, deps, nullptr, ndeps, &cp));
     cudaGraph_t body = cp.conditional.phGraph_out[0];
     CK(cudaStreamUpdateCaptureDependencies(cs, &cnode, nullptr, 1, cudaStreamSetCaptureDependencies));
-    if (s->timing) {
-        auto ev = take_events(s);
-        s->ev_free.push_back(ev);
-        CK(cudaEventRecordWithFlags(ev.first, cs, cudaEventRecordExternal));
-        CK(cudaStreamGetCaptureInfo(cs, &status, nullptr, &cg, &deps, nullptr, &ndeps));
-        out.ev_a = ndeps ? deps[0] : nullptr;
-        enqueue_forces(s, 0, cs);
-        CK(cudaEventRecordWithFlags(ev.second, cs, cudaEventRecordExternal));
-        CK(cudaStreamGetCaptureInfo(cs, &status, nullptr, &cg, &deps, nullptr, &ndeps));
-        out.ev_b = ndeps ? deps[0] : nullptr;
-    } else {
-        enqueue_forces(s, 0, cs);
-    }
+    auto ev = take_events(s);
+    s->ev_free.push_back(ev);
+    CK(cudaEventRecordWithFlags(ev.first, cs, cudaEventRecordExternal));
+    CK(cudaStreamGetCaptureInfo(cs, &status, nullptr, &cg, &deps, nullptr, &ndeps));
+    out.ev_a = ndeps ? deps[0] : nullptr;
+    enqueue_forces(s, 0, cs);
+    CK(cudaEventRecordWithFlags(ev.second, cs, cudaEventRecordExternal));
+    CK(cudaStreamGetCaptureInfo(cs, &status, nullptr, &cg, &deps, nullptr, &ndeps));
+    out.ev_b = ndeps ? deps[0] : nullptr;
     CK(cudaStreamEndCapture(cs, &g));
     // the rebuild body
     CK(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
@@ -711,7 +708,7 @@ int capture_fused(md_system* s, bool kkd, int p, md_system::StepGraph& out) {
     CK(cudaStreamBeginCaptureToGraph(cs, g, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
     const DevState a = view(s, p);
     launch_step_ctrl(s->rebuild == MD_REBUILD_EVERY_K ? 1 : 0, s->rebuild_k, a.rebuild_flag, s->d_ctrl,
-                     s->d_ctrl + 1, a.err, h, cs);
+                     a.err, h, cs);
     cudaStreamCaptureStatus status;
     const cudaGraphNode_t* deps = nullptr;
     size_t ndeps = 0;
@@ -729,19 +726,15 @@ int capture_fused(md_system* s, bool kkd, int p, md_system::StepGraph& out) {
     cudaGraph_t body = cp.conditional.phGraph_out[0];
     CK(cudaStreamUpdateCaptureDependencies(cs, &cnode, nullptr, 1, cudaStreamSetCaptureDependencies));
     const int mode = kkd ? FUSE_KICK_KICK_DRIFT : FUSE_KICK;
-    if (s->timing) {
-        auto ev = take_events(s);
-        s->ev_free.push_back(ev);
-        CK(cudaEventRecordWithFlags(ev.first, cs, cudaEventRecordExternal));
-        CK(cudaStreamGetCaptureInfo(cs, &status, nullptr, &cg, &deps, nullptr, &ndeps));
-        out.ev_a = ndeps ? deps[0] : nullptr;
-        enqueue_fused(s, a, mode, step_out(s, 1 - p), cs);
-        CK(cudaEventRecordWithFlags(ev.second, cs, cudaEventRecordExternal));
-        CK(cudaStreamGetCaptureInfo(cs, &status, nullptr, &cg, &deps, nullptr, &ndeps));
-        out.ev_b = ndeps ? deps[0] : nullptr;
-    } else {
-        enqueue_fused(s, a, mode, step_out(s, 1 - p), cs);
-    }
+    auto ev = take_events(s);
+    s->ev_free.push_back(ev);
+    CK(cudaEventRecordWithFlags(ev.first, cs, cudaEventRecordExternal));
+    CK(cudaStreamGetCaptureInfo(cs, &status, nullptr, &cg, &deps, nullptr, &ndeps));
+    out.ev_a = ndeps ? deps[0] : nullptr;
+    enqueue_fused(s, a, mode, step_out(s, 1 - p), cs);
+    CK(cudaEventRecordWithFlags(ev.second, cs, cudaEventRecordExternal));
+    CK(cudaStreamGetCaptureInfo(cs, &status, nullptr, &cg, &deps, nullptr, &ndeps));
+    out.ev_b = ndeps ? deps[0] : nullptr;
     CK(cudaStreamEndCapture(cs, &g));
     CK(cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal));
     enqueue_bin(s, a, cs, af(s), s->d_ctrl + 1);
@@ -771,7 +764,7 @@ int capture_fused_multi(md_system* s, md_system::StepGraph& out) {
                                          cudaStreamCaptureModeThreadLocal));
         const DevState a = view(s, p);
         launch_step_ctrl(s->rebuild == MD_REBUILD_EVERY_K ? 1 : 0, s->rebuild_k, a.rebuild_flag, s->d_ctrl,
-                         s->d_ctrl + 1, a.err, h, cs);
+                         a.err, h, cs);
         cudaStreamCaptureStatus status;
         const cudaGraphNode_t* deps = nullptr;
         size_t ndeps = 0;
@@ -788,10 +781,10 @@ int capture_fused_multi(md_system* s, md_system::StepGraph& out) {
         CK(cudaGraphAddNode(&cnode, cg, deps, nullptr, ndeps, &cp));
         cudaGraph_t body = cp.conditional.phGraph_out[0];
         CK(cudaStreamUpdateCaptureDependencies(cs, &cnode, nullptr, 1, cudaStreamSetCaptureDependencies));
-        // under timing, event nodes around the first step's force kernel (each launch points
+        // event nodes around the first step's force kernel (each launch points
         // them at fresh events): one launch in MULTI_STEPS is timed, so that the events
         // barely change the steps they measure
-        const bool timed = s->timing && j == 0;
+        const bool timed = j == 0;
         if (timed) {
             auto ev = take_events(s);
             s->ev_free.push_back(ev);
@@ -876,7 +869,7 @@ int append_step(md_system* s, cudaGraph_t g, std::vector<cudaGraphNode_t>& tail,
     CK(cudaGraphConditionalHandleCreate(&h, g, 0, cudaGraphCondAssignDefault));
     int rc = append_captured(s, g, tail, [&](cudaStream_t cs) {
         launch_step_ctrl(s->rebuild == MD_REBUILD_EVERY_K ? 1 : 0, s->rebuild_k, a.rebuild_flag, s->d_ctrl,
-                         s->d_ctrl + 1, a.err, h, cs);
+                         a.err, h, cs);
     });
     if (rc) return rc;
     cudaGraph_t body = nullptr;
@@ -1095,15 +1088,13 @@ int run_chunk_fused(md_system* s, int len, bool first, bool last) {
     }
     for (int k = 0; s->timing && k < len; ++k) {  // with timing on: graphs that can hold event nodes
         if (s->g_multi.exec && p == 0 && k + MULTI_STEPS <= n_kkd) {
-            if (s->timing) {
-                const auto& gm = s->g_multi;
-                for (size_t j = 0; j < gm.ev_multi_a.size() && j < gm.ev_multi_b.size(); ++j) {
-                    if (!gm.ev_multi_a[j] || !gm.ev_multi_b[j]) continue;
-                    auto ev = take_events(s);
-                    CK(cudaGraphExecEventRecordNodeSetEvent(gm.exec, gm.ev_multi_a[j], ev.first));
-                    CK(cudaGraphExecEventRecordNodeSetEvent(gm.exec, gm.ev_multi_b[j], ev.second));
-                    s->ev_force.push_back(ev);
-                }
+            const auto& gm = s->g_multi;
+            for (size_t j = 0; j < gm.ev_multi_a.size() && j < gm.ev_multi_b.size(); ++j) {
+                if (!gm.ev_multi_a[j] || !gm.ev_multi_b[j]) continue;
+                auto ev = take_events(s);
+                CK(cudaGraphExecEventRecordNodeSetEvent(gm.exec, gm.ev_multi_a[j], ev.first));
+                CK(cudaGraphExecEventRecordNodeSetEvent(gm.exec, gm.ev_multi_b[j], ev.second));
+                s->ev_force.push_back(ev);
             }
             CK(cudaGraphLaunch(s->g_multi.exec, s->stream));  // MULTI_STEPS steps; back in buffer 0
             s->launches += (1 + force_kernels(s)) * MULTI_STEPS;
@@ -1113,7 +1104,7 @@ int run_chunk_fused(md_system* s, int len, bool first, bool last) {
         }
         const bool kkd = !(last && k == len - 1);
         md_system::StepGraph& gr = s->g_fused[kkd ? 1 : 0][p];
-        if (s->timing && gr.ev_a && gr.ev_b) {
+        if (gr.ev_a && gr.ev_b) {
             auto ev = take_events(s);
             CK(cudaGraphExecEventRecordNodeSetEvent(gr.exec, gr.ev_a, ev.first));
             CK(cudaGraphExecEventRecordNodeSetEvent(gr.exec, gr.ev_b, ev.second));
@@ -1167,7 +1158,7 @@ int run_chunk(md_system* s, int len, bool first) {
     }
     for (int k = 0; s->timing && k < len; ++k) {  // with timing on: graphs that can hold event nodes
         md_system::StepGraph& gr = (first && k == 0) ? s->g_first : s->g_mid;
-        if (s->timing && gr.ev_a && gr.ev_b) {
+        if (gr.ev_a && gr.ev_b) {
             auto ev = take_events(s);
             CK(cudaGraphExecEventRecordNodeSetEvent(gr.exec, gr.ev_a, ev.first));
             CK(cudaGraphExecEventRecordNodeSetEvent(gr.exec, gr.ev_b, ev.second));
@@ -1205,7 +1196,7 @@ int ensure_headroom(md_system* s) {
     }
     if (s->max_tile + std::max(64, s->max_tile / 8) > s->tile_cap) {
         const int cap = std::min(round_up(s->max_tile + s->max_tile / 4 + 64, 32), round_up((int)s->n + 1, 32));
-        if (cap > s->tile_cap && cap <= 32767 && list_smem(s, s->list_cap, cap) <= 226 * 1024 &&
+        if (cap > s->tile_cap && cap <= 32767 && list_smem(s, cap) <= 226 * 1024 &&
             fsmem(s, 0, cap) <= 226 * 1024)
             s->tile_cap = cap;
     }

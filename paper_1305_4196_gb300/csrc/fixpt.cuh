@@ -117,15 +117,6 @@ __device__ __forceinline__ void for_each_neighbour_pair(const uint4* __restrict_
     }
 }
 
-template <typename Body>
-__device__ __forceinline__ void for_each_neighbour(const uint4* __restrict__ lp, size_t stride, int nch,
-                                                   Body&& body) {
-    for_each_neighbour_pair(lp, stride, nch, [&](int u0, int u1) {
-        body(u0);
-        body(u1);
-    });
-}
-
 // One tile entry with a single 128-bit shared-memory load (base = shared address of the tile).
 __device__ __forceinline__ float4 lds_tile(unsigned base, int u) {
     float4 v;

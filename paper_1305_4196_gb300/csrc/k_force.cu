@@ -551,13 +551,6 @@ void launch_forces_mixed(const DevState& s, const LaunchGeometry& g, const PairT
 
 // Full-list mixed forces fused with velocity Verlet (mode FM_KICK: closing half kick;
 // FM_KKD: closing + opening kick and drift, the new positions into out).
-template <bool SINGLE, int MODE>
-static void launch_full_mode(const DevState& s, const Geometry& g, const PairTable& pt, const TileOffsets& to,
-                             int tile_cap, float fs2_max, StepOut out, double dt, float lim2_f, size_t smem,
-                             cudaStream_t st) {
-    launch_full<SINGLE, false, MODE>(s, g, pt, to, tile_cap, fs2_max, out, dt, lim2_f, smem, st);
-}
-
 void launch_forces_mixed_fused(const DevState& s, const LaunchGeometry& g, const PairTable& pt, const TileOffsets& to,
                                int tile_cap, int mode, StepOut out, double dt, double lim2, cudaStream_t st) {
     if (s.n == 0) return;
@@ -571,14 +564,14 @@ void launch_forces_mixed_fused(const DevState& s, const LaunchGeometry& g, const
         return;
     if (mode == FM_KICK) {
         if (single)
-            launch_full_mode<true, FM_KICK>(s, g, pt, to, tile_cap, fs2_max, out, dt, lim2_f, smem, st);
+            launch_full<true, false, FM_KICK>(s, g, pt, to, tile_cap, fs2_max, out, dt, lim2_f, smem, st);
         else
-            launch_full_mode<false, FM_KICK>(s, g, pt, to, tile_cap, fs2_max, out, dt, lim2_f, smem, st);
+            launch_full<false, false, FM_KICK>(s, g, pt, to, tile_cap, fs2_max, out, dt, lim2_f, smem, st);
     } else {
         if (single)
-            launch_full_mode<true, FM_KKD>(s, g, pt, to, tile_cap, fs2_max, out, dt, lim2_f, smem, st);
+            launch_full<true, false, FM_KKD>(s, g, pt, to, tile_cap, fs2_max, out, dt, lim2_f, smem, st);
         else
-            launch_full_mode<false, FM_KKD>(s, g, pt, to, tile_cap, fs2_max, out, dt, lim2_f, smem, st);
+            launch_full<false, false, FM_KKD>(s, g, pt, to, tile_cap, fs2_max, out, dt, lim2_f, smem, st);
     }
 }
 

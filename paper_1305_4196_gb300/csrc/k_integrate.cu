@@ -128,8 +128,7 @@ void launch_loop_ctrl(long long* passes_left, int done, cudaGraphConditionalHand
 }
 
 void launch_step_ctrl(int policy, int every_k, int32_t* rebuild_flag, long long* step_counter,
-                      long long* n_builds, uint32_t* err, cudaGraphConditionalHandle handle, cudaStream_t st) {
-    (void)n_builds;
+                      uint32_t* err, cudaGraphConditionalHandle handle, cudaStream_t st) {
     k_step_ctrl<<<1, 1, 0, st>>>(policy, every_k, rebuild_flag, step_counter, err, handle);
 }
 

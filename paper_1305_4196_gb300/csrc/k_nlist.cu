@@ -141,8 +141,7 @@ static size_t nl_smem_bytes(int tile_cap, int warps) { return nl_tile_bytes(tile
 
 // The size the callers hold against the limit of an SM's shared memory: 12 B per tile atom and
 // about 35 KB (with a tile close to the limit a CTA runs four warps).
-size_t build_lists_smem(int list_cap, int tile_cap) {
-    (void)list_cap;
+size_t build_lists_smem(int tile_cap) {
     return (size_t)((tile_cap + 227) & ~3) * 3 * sizeof(float) + 32768;
 }
 

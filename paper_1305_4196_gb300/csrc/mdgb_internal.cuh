@@ -315,12 +315,12 @@ void launch_sort_gather(const DevState& s, const DevState& scratch, const Geomet
 void launch_copy_back(const DevState& s, const DevState& scratch, cudaStream_t st);
 void launch_classify_blocks(const DevState& s, const Geometry& g, long long* n_builds, cudaStream_t st);
 void launch_step_ctrl(int policy, int every_k, int32_t* rebuild_flag, long long* step_counter,
-                      long long* n_builds, uint32_t* err, cudaGraphConditionalHandle handle, cudaStream_t st);
+                      uint32_t* err, cudaGraphConditionalHandle handle, cudaStream_t st);
 void launch_loop_ctrl(long long* passes_left, int done, cudaGraphConditionalHandle handle, cudaStream_t st);
 void launch_copy_state(const DevState& dst, const DevState& src, cudaStream_t st);
 void launch_build_lists(const DevState& s, const DevState& d, const LaunchGeometry& g, const TileOffsets& to, double rl2, int list_cap,
                         int tile_cap, int half, cudaStream_t st);
-size_t build_lists_smem(int list_cap, int tile_cap);
+size_t build_lists_smem(int tile_cap);
 void launch_forces_mixed(const DevState& s, const LaunchGeometry& g, const PairTable& pt, const TileOffsets& to,
                          int tile_cap, int half, int with_energy, cudaStream_t st);
 size_t force_smem_bytes(int mixed, int half, int with_energy, int tile_cap);

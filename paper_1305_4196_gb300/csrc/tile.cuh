@@ -20,7 +20,6 @@
 namespace mdgb {
 
 struct TileTables {
-    int8_t idx_of_coord[64];  // tile coordinate (tx + 4 ty + 16 tz) -> tile slot
     int8_t coord_of_idx[64];  // tile slot -> tile coordinate
 };
 
@@ -50,7 +49,6 @@ __host__ __device__ constexpr TileTables make_tile_tables() {
         int x = c & 3, y = (c >> 2) & 3, z = c >> 4;
         bool own = x >= 1 && x <= 2 && y >= 1 && y <= 2 && z >= 1 && z <= 2;
         int i = own ? (x - 1) + 2 * (y - 1) + 4 * (z - 1) : (tile_receives(x, y, z) ? k++ : r++);
-        t.idx_of_coord[c] = (int8_t)i;
         t.coord_of_idx[i] = (int8_t)c;
     }
     return t;
@@ -130,35 +128,6 @@ __device__ __forceinline__ void tile_meta(const Geometry& g, const int32_t* __re
     __syncthreads();
 }
 
-// The same meta filled by one warp (lanes take slots lane and lane + 32; ends with __syncwarp).
-__device__ __forceinline__ void tile_meta_warp(const Geometry& g, const int32_t* __restrict__ cell_start, int b,
-                                               TileMeta& m) {
-    const int lane = threadIdx.x & 31;
-    int bx, by, bz;
-    block_coords(g, b, bx, by, bz);
-    int below = 0;  // atoms in slots 0..31
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int t = lane + 32 * h;
-        const int c = tile_coord_of(t);
-        const int id = tile_cell_id(g, bx, by, bz, c);
-        const int st = cell_start[id];
-        int v = cell_start[id + 1] - st;
-        m.start[t] = st;
-        m.coord[t] = (int8_t)c;
-        m.slot[c] = (int8_t)t;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(0xffffffffu, v, o);
-            if (lane >= o) v += y;
-        }
-        m.prefix[t + 1] = v + below;
-        below = __shfl_sync(0xffffffffu, v, 31);
-    }
-    if (lane == 0) m.prefix[0] = 0;
-    __syncwarp();
-}
-
 // Tile slot holding tile index u (binary search in the 65-entry prefix).
 __device__ __forceinline__ int tile_slot_of(const TileMeta& m, int u) {
     int lo = 0, hi = 64;
@@ -187,7 +156,6 @@ __device__ __forceinline__ bool fp64_pair_test(const double* __restrict__ x, con
     return r2 < rl2;
 }
 
-
 // Cell-ordered global index of tile index u.
 __device__ __forceinline__ int tile_global_index(const TileMeta& m, int u) {
     const int slot = tile_slot_of(m, u);
@@ -200,16 +168,6 @@ __device__ __forceinline__ int tile_global_index(const TileMeta& m, int u) {
 __device__ __forceinline__ float pick4(const float (&o)[4], int t) {
     const float a = ((t + 1) & 2) ? o[2] : o[3];  // t = 1, 2: the inner cells
     return __int_as_float(__float_as_int(a) ^ (t < 2 ? (int)0x80000000 : 0));
-}
-
-// Block-frame FP32 coordinates of tile index u, the same additions as the staging below.
-__device__ __forceinline__ float4 tile_coord(const TileMeta& m, const TileOffsets& to, const float4* __restrict__ xr,
-                                             int u) {
-    const int slot = tile_slot_of(m, u);
-    const int c = m.coord[slot];
-    const float4 p = xr[m.start[slot] + (u - m.prefix[slot])];
-    return make_float4(p.x + pick4(to.off[0], c & 3), p.y + pick4(to.off[1], (c >> 2) & 3),
-                       p.z + pick4(to.off[2], c >> 4), p.w);
 }
 
 // Stage the block-frame FP32 coordinates of the tile, one warp per tile cell (lanes
@@ -243,24 +201,6 @@ __device__ __forceinline__ void tile_stage_f32_cells(const TileMeta& m, const fl
             if (e < cnt) tile[u0 + e] = make_float4(p.x + ox, p.y + oy, p.z + oz, p.w);
             if (e < cnt2) tile[v0 + e] = make_float4(q.x + ox2, q.y + oy2, q.z + oz2, q.w);
         }
-    }
-}
-
-// Stage the block-frame FP32 coordinates of the tile (T = m.prefix[64] <= cap).
-__device__ __forceinline__ void tile_stage_f32(const TileMeta& m, const float4* __restrict__ xr,
-                                               const TileOffsets& to, float4* __restrict__ tile,
-                                               int32_t* __restrict__ gidx) {
-    const int T = m.prefix[64];
-    for (int u = threadIdx.x; u < T; u += blockDim.x) {
-        int slot = tile_slot_of(m, u);
-        int c = m.coord[slot];
-        int j = m.start[slot] + (u - m.prefix[slot]);
-        float4 p = xr[j];
-        p.x += pick4(to.off[0], c & 3);
-        p.y += pick4(to.off[1], (c >> 2) & 3);
-        p.z += pick4(to.off[2], c >> 4);
-        tile[u] = p;
-        if (gidx) gidx[u] = j;
     }
 }
 
