@@ -44,12 +44,25 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_force_mixed_split(DevState s,
     constexpr int PER = SPLIT_THREADS / LPA;  // own atoms at a time
     if (part * PER >= nown) return;
     const int64_t n = s.n;
+    const size_t np = s.np;
     const int nsp = pt.nsp;
     const f2_t magic2 = f2_pack(MAGIC, MAGIC);
     const f2_t two21 = f2_pack(TWO21, TWO21);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, lq = threadIdx.x % LPA;
     const unsigned tile_s = (unsigned)__cvta_generic_to_shared(tile);
     const int blk0 = m.start[0];
+    const unsigned pad = (unsigned)T | ((unsigned)T << 16);
+    // A lane's list words: `at` of chunk 0, one 16-byte chunk every np * 4 words; lanes 0..3 take
+    // one word each of every STEP-th chunk (LPA >= 4), lanes 0, 1 two words each (LPA 2)
+    constexpr int STEP = LPA == 8 ? 2 : 1;
+    constexpr int WORDS = LPA == 2 ? 2 : 1;
+    constexpr int AHEAD = LPA == 1 ? 1 : 4;  // chunks on their way together
+    auto list_words = [&](int gi) {
+        return reinterpret_cast<const unsigned*>(s.nl) + (size_t)gi * 4 + (LPA == 2 ? 2 * lq : (lq & 3));
+    };
+    auto load_word = [&](const unsigned* at, int c, int k) {
+        return __ldcs(at + (size_t)c * np * 4 + k);
+    };
     bool staged = false;
     for (int u0 = part * PER; u0 < nown; u0 += split * PER) {
         const int ui = u0 + (int)threadIdx.x / LPA;
@@ -58,7 +71,15 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_force_mixed_split(DevState s,
         // the list's first words before its length is known, and the state of the update: on their
         // way while the tile is staged
         const int cnt = s.nl_cnt[gi];
-        LaneList<LPA> list(s, gi, lq);
+        const unsigned* const words = list_words(gi);
+        const int cq = LPA == 8 ? lq >> 2 : 0;
+        unsigned e[AHEAD][WORDS];
+        if (LPA > 1) {
+#pragma unroll
+            for (int k = 0; k < AHEAD; ++k)
+#pragma unroll
+                for (int h = 0; h < WORDS; ++h) e[k][h] = cq + k * STEP < s.nl_chunks ? load_word(words, cq + k * STEP, h) : pad;
+        }
         LaneState<MODE, LPA> st;
         st.load(s, gi, lq);
         if (!staged) {
@@ -74,18 +95,46 @@ __global__ void __launch_bounds__(SPLIT_THREADS) k_force_mixed_split(DevState s,
         float pe = 0.f, w0 = 0.f, w1 = 0.f, w2 = 0.f, w3 = 0.f, w4 = 0.f, w5 = 0.f;
         bool bad = nch * 8 > FIX_SPLIT_MAX_TERMS;
         float mdist = 3.0e38f, mr2 = 3.0e38f;
-        list.walk(nch, [&](int v0, int v1) {
-            full_pair<SINGLE, EV>(pt, stab, tile_s, pi, si, nsp, fs2_max, magic2, two21, v0, v1, ax, ay, az, pe, w0, w1,
-                                  w2, w3, w4, w5, bad, mdist, mr2);
-        });
-        lanes_sum<LPA>(ax);
-        lanes_sum<LPA>(ay);
-        lanes_sum<LPA>(az);
+        auto pair = [&](unsigned w) {
+            full_pair<SINGLE, EV>(pt, stab, tile_s, pi, si, nsp, fs2_max, magic2, two21, (int)(w & 0xffffu),
+                                  (int)(w >> 16), ax, ay, az, pe, w0, w1, w2, w3, w4, w5, bad, mdist, mr2);
+        };
+        if (LPA == 1) {
+            for_each_neighbour_pair(reinterpret_cast<const uint4*>(s.nl) + gi, np, nch,
+                                    [&](int v0, int v1) { pair((unsigned)v0 | ((unsigned)v1 << 16)); });
+        } else {
+            for (int c0 = cq; c0 < nch; c0 += AHEAD * STEP) {
+                unsigned cur[AHEAD][WORDS];
+#pragma unroll
+                for (int k = 0; k < AHEAD; ++k)
+#pragma unroll
+                    for (int h = 0; h < WORDS; ++h) {
+                        cur[k][h] = c0 + k * STEP < nch ? e[k][h] : pad;
+                        const int c = c0 + (AHEAD + k) * STEP;
+                        if (c < nch) e[k][h] = load_word(words, c, h);
+                    }
+#pragma unroll
+                for (int k = 0; k < AHEAD; ++k)
+                    if (c0 + k * STEP < nch) {
+#pragma unroll
+                        for (int h = 0; h < WORDS; ++h) pair(cur[k][h]);
+                    }
+            }
+        }
+#pragma unroll
+        for (int o = LPA / 2; o > 0; o >>= 1) {
+            ax.hi += __shfl_xor_sync(0xffffffffu, ax.hi, o);
+            ax.lo += __shfl_xor_sync(0xffffffffu, ax.lo, o);
+            ay.hi += __shfl_xor_sync(0xffffffffu, ay.hi, o);
+            ay.lo += __shfl_xor_sync(0xffffffffu, ay.lo, o);
+            az.hi += __shfl_xor_sync(0xffffffffu, az.hi, o);
+            az.lo += __shfl_xor_sync(0xffffffffu, az.lo, o);
+        }
         if (SINGLE) bad |= (mdist <= pt.band_half_f) | (mr2 < pt.r2_wide_f);
         // an atom whose lanes found a pair for the exact finish: once per atom, by the whole warp
         unsigned left = __ballot_sync(0xffffffffu, bad && active);
-        constexpr unsigned GROUP = (1u << LPA) - 1u;
-        const bool mine_bad = lanes_any<LPA>(left, lane);
+        constexpr unsigned GROUP = LPA == 32 ? 0xffffffffu : (1u << LPA) - 1u;
+        const bool mine_bad = (left >> (lane & ~(LPA - 1)) & GROUP) != 0u;
         const int nterms = nch * 8;
         const long long q[3] = {fix_final(ax, nterms), fix_final(ay, nterms), fix_final(az, nterms)};
         const bool write = active && !mine_bad;

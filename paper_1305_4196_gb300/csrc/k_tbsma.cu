@@ -109,6 +109,82 @@ __device__ __forceinline__ bool tb_inside_exact(const DevState& s, const Geometr
     return fp64_pair_test(s.x, s.y, s.z, g.L[0], g.L[1], g.L[2], gi, tile_global_index(m, u), tb.rc2_d);
 }
 
+// What an atom's lanes read of its list: its 16-byte chunks side by side, LPA 2: two words each, 4: one
+// word each, 8: one word of every other chunk.  The first AHEAD chunks are requested by the
+// constructor, before their number is known to the lane.
+template <int LPA>
+struct LaneList {
+    static constexpr int STEP = LPA == 8 ? 2 : 1, WORDS = LPA == 2 ? 2 : 1, AHEAD = 4;
+    const unsigned* words;
+    size_t stride;
+    int cq;
+    unsigned e[AHEAD][WORDS];
+
+    __device__ __forceinline__ unsigned load(int c, int h) const { return __ldcs(words + (size_t)c * stride + h); }
+
+    __device__ __forceinline__ LaneList(const DevState& s, int gi, int lq) {
+        words = reinterpret_cast<const unsigned*>(s.nl) + (size_t)gi * 4 + (LPA == 2 ? 2 * lq : (lq & 3));
+        stride = (size_t)s.np * 4;
+        cq = LPA == 8 ? lq >> 2 : 0;
+#pragma unroll
+        for (int k = 0; k < AHEAD; ++k)
+#pragma unroll
+            for (int h = 0; h < WORDS; ++h) e[k][h] = cq + k * STEP < s.nl_chunks ? load(cq + k * STEP, h) : 0u;
+    }
+
+    // body(u0, u1) for every two entries of the lane's share of nch chunks
+    template <typename Body>
+    __device__ __forceinline__ void walk(int nch, Body&& body) {
+        for (int c0 = cq; c0 < nch; c0 += AHEAD * STEP) {
+            unsigned cur[AHEAD][WORDS];
+#pragma unroll
+            for (int k = 0; k < AHEAD; ++k)
+#pragma unroll
+                for (int h = 0; h < WORDS; ++h) {
+                    cur[k][h] = e[k][h];
+                    const int c = c0 + (AHEAD + k) * STEP;
+                    if (c < nch) e[k][h] = load(c, h);
+                }
+#pragma unroll
+            for (int k = 0; k < AHEAD; ++k)
+                if (c0 + k * STEP < nch) {
+#pragma unroll
+                    for (int h = 0; h < WORDS; ++h) body((int)(cur[k][h] & 0xffffu), (int)(cur[k][h] >> 16));
+                }
+        }
+    }
+};
+
+template <>
+struct LaneList<1> {
+    const uint4* row;
+    size_t stride;
+    __device__ __forceinline__ LaneList(const DevState& s, int gi, int) {
+        row = reinterpret_cast<const uint4*>(s.nl) + gi;
+        stride = s.np;
+    }
+    template <typename Body>
+    __device__ __forceinline__ void walk(int nch, Body&& body) {
+        for_each_neighbour_pair(row, stride, nch, body);
+    }
+};
+
+template <int LPA>
+__device__ __forceinline__ void lanes_sum(FixAcc& a) {
+#pragma unroll
+    for (int o = LPA / 2; o > 0; o >>= 1) {
+        a.hi += __shfl_xor_sync(0xffffffffu, a.hi, o);
+        a.lo += __shfl_xor_sync(0xffffffffu, a.lo, o);
+    }
+}
+
+// The lanes of the warp whose atom has a pair for the exact finish (bad on any of its lanes).
+template <int LPA>
+__device__ __forceinline__ bool lanes_any(unsigned bad, int lane) {
+    constexpr unsigned GROUP = (1u << LPA) - 1u;
+    return (bad >> (lane & ~(LPA - 1)) & GROUP) != 0u;
+}
+
 // The CTA's block and its share of it; false when it has nothing to do (a tile that does not fit is
 // flagged).
 template <int PER>
