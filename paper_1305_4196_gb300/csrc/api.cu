@@ -821,8 +821,8 @@ int capture_fused_multi(md_system* s, md_system::StepGraph& out) {
 // steps, each with its own conditional rebuild, and an if node (always taken) with the steps left
 // over.  Against a graph per step and 8-step graphs of top-level conditions this takes
 // about 7 us off every step.  A chunk without a whole pass has no while node and a single step left
-// over no if node: the call that captures them is the first of its kind, and a node's body costs it
-// some 20 us a step (copper, 16,384 atoms: a first md_step(1) 350 -> 150 us, md_step(4) 500 -> 340).
+// over no if node: the first call of a kind captures them, and a step of a body costs it
+// some 50 us (copper, 16,384 atoms: a first md_step(1) 350 -> 150 us, md_step(4) 500 -> 340).
 constexpr int LOOP_STEPS = 4;  // even: fused steps are back in coordinate buffer 0
 
 // A conditional node behind `tail` (or, while capturing on cs, behind what is captured); its body.
