@@ -24,10 +24,11 @@
 //  * The summation order is fixed, so every result is deterministic.
 // The pass is bound by instruction issue and the latency of the gathered G_j.  For 32,000 atoms of a
 // binary mixture it took 217 us with one lane per atom, 2-byte list reads and FP64 sums, and 47 us
-// for the column sums of a row per atom; it takes 47 us (29 for the energy's derivatives) and 3.
+// for the column sums of a row per atom; it takes 45 us (28 for the energy's derivatives) and 3.
 #include "tile.cuh"
 
 #include <algorithm>
+#include <type_traits>
 
 #include "fixpt.cuh"
 #include "float_sum.cuh"
@@ -47,62 +48,56 @@ struct alignas(4 * sizeof(T)) Grad4 {
     T x, y, z, w;
 };
 
-// A lane's sum of parameter terms: FP64 terms in FP64, FP32 terms in three floats (FloatSum: no less
+// A lane's sums of a pair's two terms: FP64 terms in FP64, FP32 terms in three floats (FloatSum: no less
 // exact than FP64 sums; an FP64 addition and the conversion before it would hold a warp as long as
 // some 100 FP32 operations).
 template <typename T>
-struct ParamSum;
+using ParamSums = std::conditional_t<sizeof(T) == 8, DoubleSum2, FloatSum2>;
 
-template <>
-struct ParamSum<double> {
-    double v = 0.0;
-    __device__ __forceinline__ void add(double x) { v += x; }
-    __device__ __forceinline__ void add(const ParamSum& o) { v += o.v; }
-    __device__ __forceinline__ double get() const { return v; }
-};
-
-__device__ __forceinline__ ParamSum<double> lane_xor(const ParamSum<double>& s, int o) {
-    return ParamSum<double>{__shfl_xor_sync(0xffffffffu, s.v, o)};
-}
-
-template <>
-struct ParamSum<float> : FloatSum {};
-
-__device__ __forceinline__ ParamSum<float> lane_xor(const ParamSum<float>& s, int o) {
-    return ParamSum<float>{lane_xor(static_cast<const FloatSum&>(s), o)};
-}
-
-// The sums of a warp by species pair and quantity, of lanes that hold NV sums each for an atom of species
-// si.  Half of them to each half of an atom's lanes, twice: a lane keeps VPL; then the warp's atoms
-// of one species after the other, whose sums stay with the lanes 4 c .. 4 c + 3 of species c.
+// The sums of a warp by species pair and quantity, of lanes that hold them for an atom of species si by
+// its neighbours' species.  Half of them to each half of an atom's lanes, twice: a lane keeps VPL;
+// then the warp's atoms of one species after the other, whose sums stay with the lanes 4 c .. 4 c + 3
+// of species c.
 template <int NSP>
 struct WarpColumns {
-    static constexpr int NV = NSP * G_QUANT, VPL = (NV + 3) / 4;
+    static constexpr int NV = NSP * G_QUANT, VPL = (NV + 3) / 4, PAIRS = 2 * VPL;
 
     template <typename S>
-    static __device__ __forceinline__ void get(S (&val)[4 * VPL], int si, double (&out)[VPL]) {
+    static __device__ __forceinline__ S over_species(const S& mine, int si) {
         const int lane = threadIdx.x & 31;
-        S mine[VPL];
+        S kept;
 #pragma unroll
-        for (int o = 2, m = 2 * VPL; o > 0; o >>= 1, m >>= 1) {
+        for (int c = 0; c < NSP; ++c) {
+            S v = NSP == 1 || si == c ? mine : S();
+#pragma unroll
+            for (int o = G_LPA; o < 32; o <<= 1) v.add(lane_xor(v, o));
+            if (lane >> 2 == c) kept = v;
+        }
+        return kept;
+    }
+
+    template <typename P>
+    static __device__ __forceinline__ void get(P (&val)[PAIRS], int si, double (&out)[VPL]) {
+        const int lane = threadIdx.x & 31;
+#pragma unroll
+        for (int o = 2, m = VPL; m > 0 && o > 0; o >>= 1, m >>= 1) {
             const bool up = (lane & o) != 0;
 #pragma unroll
             for (int k = 0; k < m; ++k) {
-                const S give = up ? val[k] : val[k + m];
+                const P give = up ? val[k] : val[k + m];
                 if (up) val[k] = val[k + m];
                 val[k].add(lane_xor(give, o));
             }
         }
-#pragma unroll
-        for (int j = 0; j < VPL; ++j) {
-#pragma unroll
-            for (int c = 0; c < NSP; ++c) {
-                S v = NSP == 1 || si == c ? val[j] : S();
-#pragma unroll
-                for (int o = G_LPA; o < 32; o <<= 1) v.add(lane_xor(v, o));
-                if (lane >> 2 == c) mine[j] = v;
-            }
-            out[j] = mine[j].get();
+        if constexpr (VPL == 1) {
+            const bool up = (lane & 1) != 0;
+            auto v = val[0].half(up);
+            v.add(lane_xor(val[0].half(!up), 1));
+            out[0] = over_species(v, si).get();
+        } else {
+            const P v = over_species(val[0], si);
+            out[0] = v.half(false).get();
+            out[1] = v.half(true).get();
         }
     }
     // the column (species pair t, quantity q: 2 t + q) of this lane's j-th sum; negative: none
@@ -215,7 +210,7 @@ __global__ void __launch_bounds__(G_THREADS, 2) k_force_backward(DevState s, Geo
         Grad4<T> Gi{};
         if (!EN) Gi = G[gi];
         T a[3] = {T(0), T(0), T(0)};
-        ParamSum<T> sum[4 * VPL];  // species of the neighbour, quantity: 2 k + q
+        ParamSums<T> sum[Columns::PAIRS];  // by the neighbour's species
         // neighbour u; take(its species, the pair's two terms, its part of dL/dx) if it is inside the cutoff
         const auto visit = [&](int u, auto&& take) {
             T dx, dy, dz;
@@ -272,8 +267,8 @@ __global__ void __launch_bounds__(G_THREADS, 2) k_force_backward(DevState s, Geo
             a[2] += az;
 #pragma unroll
             for (int k = 0; k < NSP; ++k) {
-                sum[2 * k].add(NSP == 1 || sj == k ? q0 : T(0));
-                sum[2 * k + 1].add(NSP == 1 || sj == k ? q1 : T(0));
+                const bool take = NSP == 1 || sj == k;
+                sum[k].add(take ? q0 : T(0), take ? q1 : T(0));
             }
         });
         __syncwarp();
@@ -295,14 +290,11 @@ __global__ void __launch_bounds__(G_THREADS, 2) k_force_backward(DevState s, Geo
 #pragma unroll
             for (int j = 0; j < VPL; ++j) bad |= !isfinite(columns[j]);
             if (__any_sync(0xffffffffu, bad)) {  // (FloatSum) the warp's atoms again, in FP64
-                ParamSum<double> wide[4 * VPL];
+                DoubleSum2 wide[Columns::PAIRS];
                 walk([&](int sj, T q0, T q1, T, T, T) {
 #pragma unroll
                     for (int k = 0; k < NSP; ++k)
-                        if (NSP == 1 || sj == k) {
-                            wide[2 * k].add((double)q0);
-                            wide[2 * k + 1].add((double)q1);
-                        }
+                        if (NSP == 1 || sj == k) wide[k].add((double)q0, (double)q1);
                 });
                 __syncwarp();
                 Columns::get(wide, si, columns);

@@ -163,20 +163,9 @@ void launch_copy_state(const DevState& dst, const DevState& src, cudaStream_t st
 // The FP64 pipe would bound this (an SM takes 16 cycles for a warp's FP64 addition or conversion), so
 // FP32 shares are added in three floats up to the warp's sums (FloatSum: no less exact than FP64
 // sums), and the lanes of a warp add each column in a part of the warp only.  At 1,048,576 atoms
-// 54 us with FP64 sums per thread and a second launch, 18 so; at 2,048 atoms 14 and 5.3, at 360,703 in
-// FP64 24.5 (a tree over all threads) and 18.6.
+// 54 us with FP64 sums per thread and a second launch, 18 so; at 2,048 atoms 14 and 4.9, at 360,703 in
+// FP64 24.5 (a tree over all threads) and 18.7.
 constexpr int RED_THREADS = 256, RED_WARPS = RED_THREADS / 32;
-
-struct DoubleSum {
-    double v = 0.0;
-    __device__ __forceinline__ void add(double x) { v += x; }
-    __device__ __forceinline__ void add(const DoubleSum& o) { v += o.v; }
-    __device__ __forceinline__ double get() const { return v; }
-};
-
-__device__ __forceinline__ DoubleSum lane_xor(const DoubleSum& s, int o) {
-    return DoubleSum{__shfl_xor_sync(0xffffffffu, s.v, o)};
-}
 
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
