@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(F_THREADS * LPA, LPA == 1 ? 3 : 1) k_force_mix
     // through the 32-bit tile sums: they wait here as exact 64-bit values
     constexpr int WQ = 64;
     __shared__ long long wq[WQ][3];
-    __shared__ int wq_u[WQ];
+    __shared__ uint16_t wq_u[WQ];  // (tile indices; with 32 bits a tile of 6,784 atoms would not fit an SM)
     __shared__ int nwq;
     // Reaction sums only for the tile entries a half list reaches (the own cells and their
     // forward neighbours come first in the tile, Sec. II.D.3): 6 x rcap, hx, lx, hy, ly, hz,
@@ -323,11 +323,11 @@ __global__ void __launch_bounds__(F_THREADS * LPA, LPA == 1 ? 3 : 1) k_force_mix
                 fix_add(bz, 0.0f, 0.0f);
                 const int k = atomicAdd(&nwq, 2);
                 if (k + 1 < WQ && k + 2 <= FIX_WIDE_MAX_TERMS) {
-                    wq_u[k] = ui;
+                    wq_u[k] = (uint16_t)ui;
                     wq[k][0] = qx;
                     wq[k][1] = qy;
                     wq[k][2] = qz;
-                    wq_u[k + 1] = u;
+                    wq_u[k + 1] = (uint16_t)u;
                     wq[k + 1][0] = -qx;
                     wq[k + 1][1] = -qy;
                     wq[k + 1][2] = -qz;
