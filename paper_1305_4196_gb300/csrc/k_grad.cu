@@ -32,7 +32,6 @@
 
 #include "fixpt.cuh"
 #include "float_sum.cuh"
-#include "fp64_math.cuh"
 #include "launch.cuh"
 
 namespace mdgb {
@@ -107,14 +106,15 @@ struct WarpColumns {
     }
 };
 
-// 1/x.  FP32: the correctly rounded one (compared over all significands at exponents -30 .. 30); FP64: that
-// but for two numbers in a million, which are one ulp off.  Divisions gave the same digits of every
-// derivative and took 5 and 4 % longer.
+// 1/x, correctly rounded.  FP32: one Newton step from the approximate one (compared with the division over
+// all significands at exponents -30 .. 30), 5 % of the pass's time less than a division; FP64: the division,
+// 2 % (the loss's derivatives) and 4 % (the energy's) more than a cubic step from an FP32 seed, which is an
+// ulp off for two numbers in a million.
 __device__ __forceinline__ float grad_rcp(float x) {
     const float y = rcp_approx(x);
     return __fmaf_rn(y, __fmaf_rn(-x, y, 1.0f), y);
 }
-__device__ __forceinline__ double grad_rcp(double x) { return rcp_cubic(x); }
+__device__ __forceinline__ double grad_rcp(double x) { return 1.0 / x; }
 
 // Per species pair, in shared memory: the lanes of a warp read several entries at once, which the
 // constant bank would serve one after another.  (FP64 keeps 24 eps there: the tile takes the rest.)
