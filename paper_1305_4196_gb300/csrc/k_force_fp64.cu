@@ -21,7 +21,7 @@
 //    exact cutoff test compares bit patterns.
 // Every result is that of FP64 arithmetic throughout.  At 360,703 atoms a force evaluation took
 // 1.38 ms and one with energy and virial 2.11 ms with 22 operations for each of the 80 padded
-// entries, and takes 0.78 and 1.25 ms; the FP64 pipe is 88 % busy.
+// entries, and takes 0.76 and 1.24 ms; the FP64 pipe is 88 % busy.
 #include "fp64_math.cuh"
 #include "launch.cuh"
 #include "tile.cuh"
@@ -88,6 +88,7 @@ __global__ void __launch_bounds__(F_THREADS) k_force_fp64_full(DevState s, Geome
                                                                int split, float rc2_test) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ TileMeta m;
+    __shared__ int needed[65];
     double* tx = reinterpret_cast<double*>(smem);
     double* ty = tx + tile_cap;
     double* tz = ty + tile_cap;
@@ -103,7 +104,8 @@ __global__ void __launch_bounds__(F_THREADS) k_force_fp64_full(DevState s, Geome
     const int nown = m.prefix[8];
     const int per = blockDim.x / LPA;  // own atoms at a time
     if (part * per >= nown) return;
-    tile_stage_f64(s, g, m, b, tx, ty, tz, tsp, split > 1 ? tile_needed(m, part, split, per) : TILE_ALL);
+    if (split > 1) tile_needed_prefix(m, tile_needed(m, part, split, per), needed);
+    tile_stage_f64(s, g, m, b, tx, ty, tz, tsp, split > 1 ? needed : m.prefix);
     __syncthreads();
     const int blk0 = m.start[0];
     const int64_t n = s.n;
@@ -214,7 +216,7 @@ __global__ void __launch_bounds__(F_THREADS) k_force_fp64_half(DevState s, Geome
         if (threadIdx.x == 0) atomicOr(s.err, ERR_TILE_OVERFLOW);
         return;
     }
-    tile_stage_f64(s, g, m, b, tx, ty, tz, tsp);
+    tile_stage_f64(s, g, m, b, tx, ty, tz, tsp, m.prefix);
     for (int u = threadIdx.x; u <= T; u += blockDim.x) {
         acc[u] = 0;
         acc[tile_cap + u] = 0;
@@ -323,7 +325,8 @@ void launch_forces_fp64(const DevState& s, const LaunchGeometry& g, const PairTa
         // than 1.2 times its share of the atoms (64 blocks over 152 SMs: 2 each).  Lanes per atom:
         // eight while a CTA then takes its atoms in one pass, else four below one block per SM
         // (23,328 atoms: 73 us, 89 with two); from there on two, and CTAs for one pass of
-        // them.  Against the same split with an own queue and whole 16-byte chunks per lane: 4,000 atoms
+        // them.  Against the same split with an own queue and whole 16-byte chunks per lane (both with a
+        // warp per tile cell in the staging, which cost 1 to 9 us more than it does now): 4,000 atoms
         // (8 blocks) 29 us instead of 46, 10,976 (64) 47 / 75, 32,000 (64) 106 / 171, 55,296 (216)
         // 173 / 212, 360,703 (2,016) 776 / 799.
         const int sms = g.sms;

@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(G_THREADS, 2) k_force_backward(DevState s, Geo
     float4* tp = reinterpret_cast<float4*>(smem);
     int* gid = FP64 ? tsp + tile_cap : reinterpret_cast<int*>(tp + tile_cap);
     if (FP64) {
-        tile_stage_f64(s, g, m, b, tx, ty, tz, tsp);
+        tile_stage_f64(s, g, m, b, tx, ty, tz, tsp, m.prefix);
     } else {
         tile_stage_f32_cells(m, s.xr, to, tp);
         if (threadIdx.x == 0) tp[T_] = make_float4(1.0e4f, 1.0e4f, 1.0e4f, __int_as_float(0));

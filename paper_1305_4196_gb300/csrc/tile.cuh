@@ -204,7 +204,6 @@ __device__ __forceinline__ void tile_stage_f32_cells(const TileMeta& m, const fl
     }
 }
 
-constexpr unsigned long long TILE_ALL = ~0ull;
 constexpr int STAGE64_AHEAD = 4;
 
 // The tile cells (bit per slot) that the lists of a CTA's own atoms can reach, when CTAs share a block
@@ -226,51 +225,64 @@ __device__ __forceinline__ unsigned long long tile_needed(const TileMeta& m, int
     return half[0] | ((unsigned long long)half[1] << 32);
 }
 
+// The cells of `need` as a prefix over the tile slots, like TileMeta::prefix: pre[64] is the number of their
+// atoms.  By the CTA's first warp; ends with __syncthreads.
+__device__ __forceinline__ void tile_needed_prefix(const TileMeta& m, unsigned long long need, int (&pre)[65]) {
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x, a = 2 * lane;
+        const int c0 = need >> a & 1 ? m.prefix[a + 1] - m.prefix[a] : 0;
+        const int c1 = need >> (a + 1) & 1 ? m.prefix[a + 2] - m.prefix[a + 1] : 0;
+        int v = c0 + c1;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += y;
+        }
+        if (lane == 0) pre[0] = 0;
+        pre[a + 1] = v - c1;
+        pre[a + 2] = v;
+    }
+    __syncthreads();
+}
+
 // Stage the FP64 tile of block b: coordinates relative to the block centre (periodic
 // images shifted by one box length where the tile wraps), species, and a dummy slot T
-// far outside every cutoff.  Only the cells of `need` are filled.  One warp per tile cell, STAGE64_AHEAD
-// rows of 32 atoms on their way together (a CTA with an SM to itself waits for nothing else:
-// 31,000 cycles for the 4,000 atoms of a box of 4 cells per side with one row at a time).
+// far outside every cutoff.  pre: the atoms to stage, by slot (m.prefix: all; tile_needed_prefix).
+// A lane per atom over the cells' borders, as a warp's FP64 addition takes 16 cycles of the SM however few
+// of its lanes take part; STAGE64_AHEAD atoms of a lane on their way together (a CTA with an SM to
+// itself waits for nothing else).  Full-list forces with a warp per cell and so: 62,500 atoms with 2 in a cell
+// 172 -> 49 us (half lists 286 -> 122), 55,296 with 32 176 -> 167, 4,000 with 63 32.9 -> 28.6.
 __device__ __forceinline__ void tile_stage_f64(const DevState& s, const Geometry& g, const TileMeta& m, int b,
                                                double* __restrict__ tx_, double* __restrict__ ty_,
                                                double* __restrict__ tz_, int* __restrict__ tsp,
-                                               unsigned long long need = TILE_ALL) {
+                                               const int (&pre)[65]) {
     int bx, by, bz;
     block_coords(g, b, bx, by, bz);
-    const int T = m.prefix[64];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const int T = m.prefix[64], count = pre[64];
     const double cx = (2.0 * bx + 1.0) * g.w[0], cy = (2.0 * by + 1.0) * g.w[1], cz = (2.0 * bz + 1.0) * g.w[2];
-    // this warp's rows: (cell, first atom), cell by cell
-    int slot = warp, e0 = 0;
-    const auto next_cell = [&]() {
-        while (slot < 64 && !((need >> slot & 1) && e0 < m.prefix[slot + 1] - m.prefix[slot])) slot += nw, e0 = 0;
-    };
-    next_cell();
-    while (slot < 64) {
+    for (int i0 = threadIdx.x; i0 < count; i0 += STAGE64_AHEAD * (int)blockDim.x) {
         double x[STAGE64_AHEAD], y[STAGE64_AHEAD], z[STAGE64_AHEAD];
         int sp[STAGE64_AHEAD], at[STAGE64_AHEAD], coord[STAGE64_AHEAD];
 #pragma unroll
         for (int k = 0; k < STAGE64_AHEAD; ++k) {
+            const int i = i0 + k * (int)blockDim.x;
             at[k] = -1;
-            coord[k] = 21;  // (no wrap)
-            if (slot < 64) {
-                const int u0 = m.prefix[slot], e = e0 + lane;
+            if (i < count) {
+                int slot = 0;
+#pragma unroll
+                for (int h = 32; h > 0; h >>= 1) slot += pre[slot + h] <= i ? h : 0;
+                const int e = i - pre[slot], j = m.start[slot] + e;
+                at[k] = m.prefix[slot] + e;
                 coord[k] = m.coord[slot];
-                if (e < m.prefix[slot + 1] - u0) {
-                    const int j = m.start[slot] + e;
-                    at[k] = u0 + e;
-                    x[k] = s.x[j], y[k] = s.y[j], z[k] = s.z[j];
-                    sp[k] = s.species[j];
-                }
-                e0 += 32;
-                next_cell();
+                x[k] = s.x[j], y[k] = s.y[j], z[k] = s.z[j];
+                sp[k] = s.species[j];
             }
         }
 #pragma unroll
         for (int k = 0; k < STAGE64_AHEAD; ++k) {
+            if (at[k] < 0) continue;
             const int c = coord[k];
             const int rx = 2 * bx - 1 + (c & 3), ry = 2 * by - 1 + ((c >> 2) & 3), rz = 2 * bz - 1 + (c >> 4);
-            if (at[k] < 0) continue;
             if (rx < 0) x[k] -= g.L[0];
             else if (rx >= g.nc[0]) x[k] += g.L[0];
             if (ry < 0) y[k] -= g.L[1];
