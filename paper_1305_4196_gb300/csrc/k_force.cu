@@ -403,28 +403,36 @@ __global__ void __launch_bounds__(F_THREADS * LPA, LPA == 1 ? 3 : 1) k_force_mix
             s.vir_atom_f[5 * n + gi] = w5;
         }
     }
+    // With 1,024 threads, where this thread's first two atoms are (mostly all that it has), before the wait.
+    const int bs = (int)blockDim.x, u0 = threadIdx.x, u1 = u0 + bs;
+    int g0 = 0, g1 = 0;
+    if constexpr (LPA > 1) {
+        if (u0 < recv) g0 = tile_global_index(m, u0);
+        if (u1 < recv) g1 = tile_global_index(m, u1);
+    }
     __syncthreads();
     colour_wait();
-    // add the tile back, a warp per cell: this CTA is the only one of its colour touching these atoms
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int slot = warp; slot < TILE_RECV_CELLS; slot += (int)(blockDim.x >> 5)) {
-        const int u0 = m.prefix[slot], u1 = m.prefix[slot + 1];
-        for (int u = u0 + lane; u < u1; u += 32) {
-            if (count) {
-                const unsigned nt = (cnt2[u >> 1] >> ((u & 1) << 4)) & 0xffffu;
-                if (nt == 0) continue;
-                // more than FIX_SPLIT_MAX_TERMS terms on one atom could wrap its 32-bit sums
-                if (nt > FIX_SPLIT_MAX_TERMS) atomicOr(s.err, ERR_NONFINITE);
-            }
-            const int gj = m.start[slot] + (u - u0);
-            FixAcc fx{acc[0 * rcap + u], acc[1 * rcap + u]};
-            FixAcc fy{acc[2 * rcap + u], acc[3 * rcap + u]};
-            FixAcc fz{acc[4 * rcap + u], acc[5 * rcap + u]};
-            s.fq[gj] += fix_final(fx, 0);
-            s.fq[n + gj] += fix_final(fy, 0);
-            s.fq[2 * n + gj] += fix_final(fz, 0);
+    // add the tile back, an atom per thread: this CTA is the only one of its colour touching these atoms.
+    // (A warp per cell instead: 82 us an evaluation instead of 57 at 70,304 atoms, 41 in a cell, whose second rows
+    // are mostly empty, 383 instead of 263 at 202,612 atoms with 2, as long, 66, at 108,000 with 26.  The
+    // search before the wait takes 2 to 5 us off an evaluation; with 256 threads it cost 16 of 209.)
+    const auto add_back = [&](int u, int gj) {
+        if (count) {
+            const unsigned nt = (cnt2[u >> 1] >> ((u & 1) << 4)) & 0xffffu;
+            if (nt == 0) return;
+            // more than FIX_SPLIT_MAX_TERMS terms on one atom could wrap its 32-bit sums
+            if (nt > FIX_SPLIT_MAX_TERMS) atomicOr(s.err, ERR_NONFINITE);
         }
-    }
+        FixAcc fx{acc[0 * rcap + u], acc[1 * rcap + u]};
+        FixAcc fy{acc[2 * rcap + u], acc[3 * rcap + u]};
+        FixAcc fz{acc[4 * rcap + u], acc[5 * rcap + u]};
+        s.fq[gj] += fix_final(fx, 0);
+        s.fq[n + gj] += fix_final(fy, 0);
+        s.fq[2 * n + gj] += fix_final(fz, 0);
+    };
+    if (LPA > 1 && u0 < recv) add_back(u0, g0);
+    if (LPA > 1 && u1 < recv) add_back(u1, g1);
+    for (int u = LPA > 1 ? u1 + bs : u0; u < recv; u += bs) add_back(u, tile_global_index(m, u));
     __syncthreads();
     if (threadIdx.x == 0) {  // the queued large terms, exact in 64 bits
         const int nq = nwq < WQ ? nwq : WQ;
@@ -526,8 +534,9 @@ void launch_forces_mixed(const DevState& s, const LaunchGeometry& g, const PairT
     }
     cudaMemsetAsync(s.fq, 0, sizeof(long long) * 3 * (size_t)s.n, st);
     const int per = g.nblock / 8;
-    // Four lanes per atom while a colour has fewer than two blocks per SM (296,352 atoms, 216 blocks:
-    // 27.7 against 29.8 us a launch; 500,000, 343 blocks: 39.3 against 34.8)
+    // Four lanes per atom while a colour has fewer than two blocks per SM.  An evaluation with four lanes and
+    // with one: 219,488 atoms (125 blocks) 109 and 126 us, 389,344 (216) 183 and 195, 500,000 (343) 245 and
+    // 209; 296,352 (216 as well, 1,372 atoms each) 155 and 136.
     const int lpa = with_energy || per >= 2 * g.sms ? 1 : 4;
     using K = void (*)(DevState, Geometry, PairTable, TileOffsets, int, float, int);
     K k;
