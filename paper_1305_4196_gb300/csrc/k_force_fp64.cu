@@ -21,7 +21,7 @@
 //    exact cutoff test compares bit patterns.
 // Every result is that of FP64 arithmetic throughout.  At 360,703 atoms a force evaluation took
 // 1.38 ms and one with energy and virial 2.11 ms with 22 operations for each of the 80 padded
-// entries, and takes 0.76 and 1.24 ms; the FP64 pipe is 88 % busy.
+// entries, and takes 0.76 and 1.23 ms; the FP64 pipe is 88 % busy.
 #include "fp64_math.cuh"
 #include "launch.cuh"
 #include "tile.cuh"
